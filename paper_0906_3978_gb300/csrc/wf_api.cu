@@ -1,5 +1,7 @@
 // wf_api.cu -- the C ABI (include/wf.h): context, argument checks, dispatch to the kernels.
+#include <climits>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -123,6 +125,40 @@ wf_status Ctx::tw32(int n, const float2** out) {
   return WF_OK;
 }
 
+// Q62 digits of v, |v| <= 1: v 2^62 = h 2^32 + l, l the signed low word (never -2^31, so that -l exists)
+static void q62_digits(long double v, int& h, int& l) {
+  long long q = std::llrint(v * 4611686018427387904.0L);
+  if ((int)q == INT32_MIN) q += 1;
+  l = (int)q;
+  h = (int)((q - l) >> 32);
+}
+
+wf_status Ctx::fix_tables(int n) {
+  if (fixed_tw.find(n) == fixed_tw.end()) {
+    std::vector<int4> h((size_t)3 * n);
+    const long double pi = 3.14159265358979323846264338327950288L;
+    for (int e = 0; e < 2 * n; ++e) {
+      const long double a = pi * (long double)e / (long double)n;
+      q62_digits(std::cos(a), h[e].x, h[e].y);
+      q62_digits(-std::sin(a), h[e].z, h[e].w);
+    }
+    int p2 = 1;
+    while (2 * p2 <= n) p2 *= 2;
+    const long double f = (long double)p2 / (long double)n;
+    for (int k = 0; k < n; ++k) {
+      const int s = k < n / 2 ? k : (k == n / 2 ? 0 : k - n);
+      const long double a = pi * (long double)s / (long double)n;
+      q62_digits(f * std::cos(a), h[2 * n + k].x, h[2 * n + k].y);
+      q62_digits(-f * std::sin(a), h[2 * n + k].z, h[2 * n + k].w);
+    }
+    int4* d = nullptr;
+    WF_CUDA(cudaMalloc(&d, h.size() * sizeof(int4)));
+    WF_CUDA(cudaMemcpy(d, h.data(), h.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    fixed_tw[n] = d;
+  }
+  return WF_OK;
+}
+
 wf_status Ctx::get_pinned(const std::string& name, size_t bytes, void** out) {
   if (bytes == 0) bytes = 16;
   DevBuf& b = pinned[name];
@@ -187,6 +223,8 @@ void Ctx::release_all() {
   twiddles.clear();
   for (auto& kv : twiddles32) cudaFree(kv.second);
   twiddles32.clear();
+  for (auto& kv : fixed_tw) cudaFree(kv.second);
+  fixed_tw.clear();
   for (auto& kv : pinned)
     if (kv.second.ptr) cudaFreeHost(kv.second.ptr);
   pinned.clear();

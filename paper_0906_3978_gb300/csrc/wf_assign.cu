@@ -5,11 +5,15 @@
 //         exact and independent of the order in which galaxies land.
 // Step 2: the ideal discrete low-pass filter (keep modes with every |k_i| < n/2, drop the
 //         coarse Nyquist planes) and sampling at n^3.  The filter is a box in k and therefore
-//         separable: per axis, a line of 2n samples is transformed (real FFT of length 2n,
-//         computed as a complex FFT of length n), the n/2 lowest modes are kept, and the line
-//         is transformed back at length n (complex FFT of length n/2) and divided by n.
+//         separable.  Per axis, with the even and odd samples e_m, o_m of a line of 2n and
+//         X_k = E_k + exp(-i pi k / n) O_k its low modes,
+//           y_m = e_m - (-1)^m A / n + (1/n) sum_{|k| < n/2} exp(-i pi k / n) O_k exp(2 pi i k m / n),
+//         A = sum (-1)^m e_m: the even samples without their Nyquist mode, plus the odd samples moved
+//         by half a coarse cell.  Only the odd samples are transformed, and as the shift is a
+//         real circulant, two lines go as the real and imaginary part of one complex line of n.
 //         Three passes (z, y, x) each halve one axis: (2n)^3 -> (2n)^2 n -> 2n n^2 -> n^3.
 #include "wf_ctx.h"
+#include "wf_fix.cuh"
 #include "wf_spectral.cuh"
 
 namespace wf {
@@ -121,116 +125,229 @@ __global__ void k_q48_to_double(const unsigned long long* __restrict__ fine, dou
 }
 
 // ------------------------------------------------------------------------------------------
-// step 2: one axis of the ideal low-pass: line of 2N reals -> N reals.
-// AXIS 0: lines along z (contiguous rows), input rows of 2N, (2N)^2 rows.
-// AXIS 1: lines along y of [2N][2N][N]  -> [2N][N][N]; tile = NL consecutive z, fixed x.
-// AXIS 2: lines along x of [2N][N][N]   -> [N][N][N];  tile = NL consecutive z, fixed y.
+// step 2: one axis of the ideal low-pass, line pairs of 2N reals -> N reals, in 64-bit fixed point
+// (wf_fix.cuh).  A pair's z_m = o_m(first) + i o_m(second) is transformed, multiplied by the half-sample
+// shift (bin N/2: -A of the pair, so the inverse also subtracts the even samples' Nyquist mode) and
+// transformed back; the even samples are added last, read again from L2 (a CTA's were read a few
+// microseconds before) instead of being held in registers.  Between the two transforms the line is
+// shifted right by fx_mid bits: the inverse's partial sums are below N ||(e, o)||_2, sqrt(N) times the
+// forward's.  Units: with z scaled by 2^k, the result is 2^(k + a - fx_mid) y, a = floor(log2 N) from
+// the shift table's factor 2^a / N.
 // ------------------------------------------------------------------------------------------
-template <class IN> WF_D double to_real(IN v, double s);
-template <> WF_D double to_real<unsigned long long>(unsigned long long v, double s) { return __ull2double_rn(v) * s; }
-template <> WF_D double to_real<double>(double v, double s) { return v * s; }
+constexpr int kNyqParts = 8;  // partial sums of A that the bin N/2 adds
 
-// lines per CTA: a divisor of N (the y and x passes tile N consecutive z values)
-template <class R, int N> constexpr int lp_lines() { return div_le(N, tile_lines<R>()); }
-template <class R, int N>
-constexpr int lp_threads() { return lp_lines<R, N>() * tpl<R, N>(); }
+// The multiplier between the transforms: bin k of the line (digits ph[k]); bin N/2 takes -A, the sum
+// of the line's kNyqParts partial sums at ny[0], ny[st], ...
+template <int N> struct LpShift {
+  const int4* ph;
+  const fxc* ny;
+  int st;
+  WF_D fxc operator()(int k, fxc X) const {
+    if (k == N / 2) {
+      fxc a{0, 0};
+      for (int g = 0; g < kNyqParts; ++g) a = a + ny[g * st];
+      X = fxc{-a.x, -a.y};
+    }
+    X = fxc{fx_rshift(X.x, fx_mid(N)), fx_rshift(X.y, fx_mid(N))};
+    return fx_twid<-1>(X, __ldg(ph + k));
+  }
+};
 
-template <class R, int N, int AXIS, class IN>
-__global__ void __launch_bounds__(lp_threads<R, N>())
-k_lowpass(const IN* __restrict__ in, double* __restrict__ out, double in_scale,
-          const double2* __restrict__ twtab) {
-  constexpr int M = N, NL = lp_lines<R, N>(), LD = NL + 1;
-  constexpr int TPL = tpl<R, M>(), NT = NL * TPL;
-  static_assert(N % NL == 0, "tile width must divide N");
+// z axis: rows of 2N integers (units of the grid) in pairs -> rows of N doubles.  Thread t of a pair
+// holds elements n1 (N / R1) + t, so a warp reads and writes consecutive 16- and 8-byte pieces of a row.  Pairs
+// of an all-zero CTA (most of the grid outside the survey) are written as zeros at once.  Bound by integer
+// issue: 512^3 survey 32.0 ms (FP64 butterflies over all 2N samples) -> 3.52 ms (3.7 TB/s); asking for three
+// CTAs per SM, where the compiler alone leaves two, took 3.96 to 3.52 (and nothing below 128).
+template <int N> struct LpZ {
+  static constexpr int R1 = fx_plan(N).r1, TPL = N / R1;
+  static constexpr int NP = div_le(2 * N * N, TPL >= 128 ? 1 : 256 / TPL);  // pairs per CTA
+  static constexpr int NT = NP * TPL;
+  static constexpr int LS = fx_padded(N);
+  static constexpr size_t SMEM = (size_t)(NP * LS + N + NP * (TPL + kNyqParts)) * 16;
+};
+template <int N>
+__global__ void __launch_bounds__(LpZ<N>::NT, N >= 128 ? 3 : 0)
+k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out, double unit,
+            const int4* __restrict__ twtab, const int4* __restrict__ phtab) {
+  using G = LpZ<N>;
+  constexpr int R1 = G::R1, N1 = N / R1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
-  cx<R>* tw = tile + M * LD;  // exp(-2 pi i e/(2N)), e < 2N
-  const int tid = threadIdx.x;
-  for (int e = tid; e < 2 * N; e += NT) tw[e] = ld_c<R>(twtab + e);
-  // ---- load 2N reals per line as N complex
-  if constexpr (AXIS == 0) {
-    const size_t r0 = (size_t)blockIdx.x * NL;
-    int nonzero = 0;
-    for (int idx = tid; idx < M * NL; idx += NT) {
-      const int l = idx / M, m = idx % M;
-      const IN* src = in + (r0 + l) * (2 * N) + 2 * m;
-      nonzero |= (src[0] != 0) | (src[1] != 0);
-      tile[m * LD + l] = cx<R>{RT<R>::from_d(to_real(src[0], in_scale)), RT<R>::from_d(to_real(src[1], in_scale))};
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + G::NP * G::LS);
+  fxc* ny = reinterpret_cast<fxc*>(tw + N);  // per pair TPL thread sums, then kNyqParts partial sums
+  __shared__ int s_len[G::NP];
+  __shared__ unsigned s_q[G::NP];
+  const int tid = threadIdx.x, l = tid / G::TPL, t = tid % G::TPL;
+  const size_t row = 2 * ((size_t)blockIdx.x * G::NP + l);
+  const ulonglong2* r0 = reinterpret_cast<const ulonglong2*>(in + row * (2 * N));
+  const ulonglong2* r1 = r0 + N;
+  ulonglong2 a[R1], b[R1];  // (even, odd) of both rows
+  unsigned long long any = 0;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    a[r] = __ldg(r0 + r * N1 + t);
+    b[r] = __ldg(r1 + r * N1 + t);
+  }
+#pragma unroll
+  for (int r = 0; r < R1; ++r) any |= (a[r].x | a[r].y) | (b[r].x | b[r].y);
+  if (tid < G::NP) {
+    s_len[tid] = 0;
+    s_q[tid] = 0;
+  }
+  if (!__syncthreads_or(any != 0)) {
+    double* o = out + 2 * (size_t)blockIdx.x * G::NP * N;
+    for (int e = tid; e < 2 * G::NP * N; e += G::NT) o[e] = 0.0;
+    return;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  if (any) atomicMax(&s_len[l], 64 - __clzll((long long)any));
+  __syncthreads();
+  const int len = s_len[l];  // every value of the pair is below 2^len
+  {
+    unsigned q = 0;
+    auto top = [&](unsigned long long v) {  // v 2^(13 - len), rounded up
+      const unsigned h = v ? (unsigned)(len > 13 ? v >> (len - 13) : v << (13 - len)) + 1u : 0u;
+      q += h * h;  // 4 R1 <= 48 terms of at most 2^26
+    };
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      top(a[r].x);
+      top(a[r].y);
+      top(b[r].x);
+      top(b[r].y);
     }
-    // rows the survey never reaches are all zero: their filtered output is exactly zero
-    if (!__syncthreads_or(nonzero)) {
-      double2* o2 = reinterpret_cast<double2*>(out);
-      for (int idx = tid; idx < (M / 2) * NL; idx += NT)
-        o2[(r0 + idx / (M / 2)) * (N / 2) + idx % (M / 2)] = make_double2(0.0, 0.0);
-      return;
-    }
-  } else {
-    const int z0 = blockIdx.x * NL, c = blockIdx.y;
-    for (int idx = tid; idx < M * NL; idx += NT) {
-      const int m = idx / NL, l = idx % NL;
-      size_t e0, e1;
-      if constexpr (AXIS == 1) {
-        e0 = ((size_t)c * 2 * N + 2 * m) * N + z0 + l;
-        e1 = e0 + N;
-      } else {
-        e0 = ((size_t)(2 * m) * N + c) * N + z0 + l;
-        e1 = e0 + (size_t)N * N;
-      }
-      tile[m * LD + l] = cx<R>{RT<R>::from_d(to_real(in[e0], in_scale)), RT<R>::from_d(to_real(in[e1], in_scale))};
-    }
+    if (q) atomicAdd(&s_q[l], (q >> 7) + 1u);
   }
   __syncthreads();
-  const int l = tid % NL, t = tid / NL;
-  cx<R>* col = tile + l;
-  // forward complex FFT of length N (real FFT of length 2N, packed)
-  fft_line<R, M, TPL, LD, -1, 2>(col, t, tw);
-  // real-2N spectrum X_k, k < N/2, then the length-N C2R pre-step with X_{N/2} = 0
-  const R half = RT<R>::c(0.5);
-  for (int k = t; k <= N / 4; k += TPL) {
-    if (k == 0) {
-      const cx<R> z = col[0];
-      const R x0 = z.x + z.y;
-      col[0] = cx<R>{x0, x0};
-    } else {
-      const int k2 = N / 2 - k;
-      const cx<R> za = col[k * LD], zb = col[(N - k) * LD];
-      const cx<R> zc = col[k2 * LD], zd = col[(N - k2) * LD];
-      // X_k = (Z_k + conj Z_{N-k})/2 - (i/2) W_2N^k (Z_k - conj Z_{N-k})
-      const cx<R> Xa = scale((za + conj(zb)) - mul_i(tw[k] * (za - conj(zb))), half);
-      const cx<R> Xc = scale((zc + conj(zd)) - mul_i(tw[k2] * (zc - conj(zd))), half);
-      // Z'_k = (X_k + conj X_{N/2-k}) + i W_N^{-k}* (X_k - conj X_{N/2-k})
-      col[k * LD] = (Xa + conj(Xc)) + mul_i(conj(tw[2 * k]) * (Xa - conj(Xc)));
-      if (k2 != k) col[k2 * LD] = (Xc + conj(Xa)) + mul_i(conj(tw[2 * k2]) * (Xc - conj(Xa)));
+  // sqrt(N) ||(e, o)|| 2^k <= 2^62
+  const unsigned long long sq = (unsigned long long)s_q[l] * 128ull * (unsigned)N;
+  const int k = 62 + (13 - len) - ((64 - __clzll((long long)sq) + 1) >> 1);
+  auto fix = [&](unsigned long long v) { return (long long)(k >= 0 ? v << k : v >> -k); };
+  fxc v[R1];
+  {
+    fxc e{0, 0};
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const bool odd = (r * N1 + t) & 1;
+      const long long ex = fix(a[r].x), ey = fix(b[r].x);
+      e.x += odd ? -ex : ex;
+      e.y += odd ? -ey : ey;
+      v[r] = fxc{fix(a[r].y), fix(b[r].y)};
     }
+    ny[l * G::TPL + t] = e;
   }
   __syncthreads();
-  fft_line<R, M / 2, TPL, LD, +1, 4>(col, t, tw);
-  // ---- store N reals per line (N/2 complex), divided by N
-  const double inv_n = 1.0 / (double)N;
-  if constexpr (AXIS == 0) {
-    const size_t r0 = (size_t)blockIdx.x * NL;
-    double2* o2 = reinterpret_cast<double2*>(out);
-    for (int idx = tid; idx < (M / 2) * NL; idx += NT) {
-      const int ll = idx / (M / 2), m = idx % (M / 2);
-      const cx<R> v = tile[m * LD + ll];
-      o2[(r0 + ll) * (N / 2) + m] = make_double2(RT<R>::to_d(v.x) * inv_n, RT<R>::to_d(v.y) * inv_n);
+  fxc* parts = ny + G::NP * G::TPL + l * kNyqParts;
+  for (int g = t; g < kNyqParts; g += G::TPL) {
+    fxc e{0, 0};
+    for (int u = g; u < G::TPL; u += kNyqParts) e = e + ny[l * G::TPL + u];
+    parts[g] = e;
+  }
+  fx_convolve<N>(v, slots + l * G::LS, PadMap{}, t, tw, LpShift<N>{phtab, parts, 1});
+  constexpr int A = fx_floor_log2(N) - fx_mid(N);
+  const int ke = k + A;  // the even samples in the result's units
+  auto fixe = [&](unsigned long long w) { return (long long)(ke >= 0 ? w << ke : w >> -ke); };
+  const double c = unit * fx_pow2(-ke);
+  double *o0 = out + row * N, *o1 = o0 + N;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const int m = r * N1 + t;
+    o0[m] = __ll2double_rn(fixe(__ldg(&r0[m].x)) + v[r].x) * c;
+    o1[m] = __ll2double_rn(fixe(__ldg(&r1[m].x)) + v[r].y) * c;
+  }
+}
+
+// y axis (AXIS 1, [2N][2N][N] -> [2N][N][N], fixed x = blockIdx.y) and x axis (AXIS 2, [2N][N][N] -> N^3, fixed
+// y = blockIdx.y): the pairs are the double2 columns of consecutive z, NL of them per CTA.  512^3: y
+// 26.1 -> 3.87 ms, x 13.1 -> 2.10 ms (1.6 TB/s; integer issue and the FP64 pipe's conversions share the
+// time).  Four columns per CTA from 256 up: eight took 4.5 (y) and 2.3 ms, two 4.2 and 2.6.  Three CTAs per
+// SM below 256 (216^3: y 0.34 -> 0.285 ms), which spilled to 4.08 ms at 512^3.
+template <int N> struct LpC {
+  static constexpr int R1 = fx_plan(N).r1, TPL = N / R1;
+    static constexpr int NL = div_le(N / 2, N >= 256 ? 4 : 8);
+  static constexpr int NT = NL * TPL;
+  static constexpr size_t SMEM = (size_t)(N * NL + N + NL * (TPL + kNyqParts)) * 16;
+};
+template <int N, int AXIS>
+__global__ void __launch_bounds__(LpC<N>::NT, N >= 128 && N < 256 ? 3 : 0)
+k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4* __restrict__ twtab,
+            const int4* __restrict__ phtab) {
+  using G = LpC<N>;
+  constexpr int R1 = G::R1, N1 = N / R1, NL = G::NL;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  double2* pa = reinterpret_cast<double2*>(tw + N);       // TPL thread sums per column
+  fxc* parts = reinterpret_cast<fxc*>(pa + NL * G::TPL);  // kNyqParts partial sums per column
+  __shared__ int s_e[NL];
+  __shared__ unsigned s_q[NL];
+  const int tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  const size_t stride = AXIS == 1 ? N : (size_t)N * N;  // of the line, in doubles
+  const size_t first = (AXIS == 1 ? (size_t)blockIdx.y * 2 * N * N : (size_t)blockIdx.y * N) + 2 * ((size_t)blockIdx.x * NL + l);
+  const double* src = in + first;
+  double2 e[R1], o[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const size_t m = r * N1 + t;
+    e[r] = __ldg(reinterpret_cast<const double2*>(src + (2 * m) * stride));
+    o[r] = __ldg(reinterpret_cast<const double2*>(src + (2 * m + 1) * stride));
+  }
+  if (tid < NL) {
+    s_e[tid] = kFxMinExp;
+    s_q[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  {
+    int mx = 0;
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      mx = max(max(mx, max(fx_exp(e[r].x), fx_exp(e[r].y))), max(fx_exp(o[r].x), fx_exp(o[r].y)));
+      const bool odd = (r * N1 + t) & 1;
+      s.x += odd ? -e[r].x : e[r].x;
+      s.y += odd ? -e[r].y : e[r].y;
     }
-  } else {
-    const int z0 = blockIdx.x * NL, c = blockIdx.y;
-    for (int idx = tid; idx < (M / 2) * NL; idx += NT) {
-      const int m = idx / NL, ll = idx % NL;
-      const cx<R> v = tile[m * LD + ll];
-      size_t e0, e1;
-      if constexpr (AXIS == 1) {
-        e0 = ((size_t)c * N + 2 * m) * N + z0 + ll;
-        e1 = e0 + N;
-      } else {
-        e0 = ((size_t)(2 * m) * N + c) * N + z0 + ll;
-        e1 = e0 + (size_t)N * N;
-      }
-      out[e0] = RT<R>::to_d(v.x) * inv_n;
-      out[e1] = RT<R>::to_d(v.y) * inv_n;
+    pa[t * NL + l] = s;
+    if (mx > kFxMinExp) atomicMax(&s_e[l], mx);
+  }
+  __syncthreads();
+  const int emax = s_e[l];
+  {
+    unsigned q = 0;
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const unsigned h0 = fx_top(e[r].x, emax), h1 = fx_top(e[r].y, emax);
+      const unsigned h2 = fx_top(o[r].x, emax), h3 = fx_top(o[r].y, emax);
+      q += h0 * h0 + h1 * h1;  // 4 R1 <= 48 terms of at most 2^26
+      q += h2 * h2 + h3 * h3;
     }
+    if (q) atomicAdd(&s_q[l], (q >> 7) + 1u);
+  }
+  __syncthreads();
+  const int k = fx_scale(emax, s_q[l] + 1u, N);
+  for (int g = t; g < kNyqParts; g += G::TPL) {
+    double2 s = make_double2(0.0, 0.0);
+    for (int u = g; u < G::TPL; u += kNyqParts) {
+      s.x += pa[u * NL + l].x;
+      s.y += pa[u * NL + l].y;
+    }
+    parts[g * NL + l] = fxc{fx_from(s.x, k), fx_from(s.y, k)};
+  }
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fxc{fx_from(o[r].x, k), fx_from(o[r].y, k)};
+  fx_convolve<N>(v, slots + l, ColMap<NL>{}, t, tw, LpShift<N>{phtab, parts + l, NL});
+  constexpr int A = fx_floor_log2(N) - fx_mid(N);
+  const double c = emax == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : fx_pow2(-(k + A));
+  const size_t ostride = AXIS == 1 ? N : (size_t)N * N;
+  double* dst = out + (AXIS == 1 ? (size_t)blockIdx.y * N * N : (size_t)blockIdx.y * N) + 2 * ((size_t)blockIdx.x * NL + l);
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const size_t m = r * N1 + t;
+    const double2 ev = __ldg(reinterpret_cast<const double2*>(src + (2 * m) * stride));
+    *reinterpret_cast<double2*>(dst + m * ostride) =
+        make_double2(fma(__ll2double_rn(v[r].x), c, ev.x), fma(__ll2double_rn(v[r].y), c, ev.y));
   }
 }
 
@@ -239,31 +356,30 @@ static cudaError_t smem_attr(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <class R, int N>
+template <int N>
 static wf_status lowpass_sized(Ctx& c, const unsigned long long* fine, double* n_obs, double unit,
                                cudaStream_t st) {
-  constexpr int NL = lp_lines<R, N>();
-  const size_t smem = (size_t)(N * (NL + 1) + 2 * N) * sizeof(cx<R>);
-  const int nt = lp_threads<R, N>();
-  const double2* tw;
-  WF_TRY(c.tw(N, &tw));
+  using Z = LpZ<N>;
+  using C = LpC<N>;
+  static_assert(2 * N * N % Z::NP == 0 && N / 2 % C::NL == 0 && Z::SMEM <= 227 * 1024 && C::SMEM <= 227 * 1024,
+                "whole tiles");
+  WF_TRY(c.fix_tables(N));
+  const int4 *tw = c.fixed(N), *half = c.fixed_half(N);
   double *t1, *t2;
   WF_TRY(c.get("lp_t1", (size_t)4 * N * N * N * sizeof(double), (void**)&t1));
   WF_TRY(c.get("lp_t2", (size_t)2 * N * N * N * sizeof(double), (void**)&t2));
-  WF_CUDA(smem_attr(k_lowpass<R, N, 0, unsigned long long>, smem));
-  WF_CUDA(smem_attr(k_lowpass<R, N, 1, double>, smem));
-  WF_CUDA(smem_attr(k_lowpass<R, N, 2, double>, smem));
-  const double q48 = unit;
+  WF_CUDA(smem_attr(k_lowpass_z<N>, Z::SMEM));
+  WF_CUDA(smem_attr(k_lowpass_c<N, 1>, C::SMEM));
+  WF_CUDA(smem_attr(k_lowpass_c<N, 2>, C::SMEM));
   const double V = (double)N * N * N;
-  c.launch("lowpass_z", 8 * (8 * V + 4 * V), st, [&] {
-    k_lowpass<R, N, 0, unsigned long long><<<(unsigned)((size_t)4 * N * N / NL), nt, smem, st>>>(fine, t1, q48, tw);
-  });
+  c.launch("lowpass_z", 8 * (8 * V + 4 * V), st,
+           [&] { k_lowpass_z<N><<<2 * N * N / Z::NP, Z::NT, Z::SMEM, st>>>(fine, t1, unit, tw, half); });
   WF_CUDA(cudaGetLastError());
   c.launch("lowpass_y", 8 * (4 * V + 2 * V), st,
-           [&] { k_lowpass<R, N, 1, double><<<dim3(N / NL, 2 * N), nt, smem, st>>>(t1, t2, 1.0, tw); });
+           [&] { k_lowpass_c<N, 1><<<dim3(N / 2 / C::NL, 2 * N), C::NT, C::SMEM, st>>>(t1, t2, tw, half); });
   WF_CUDA(cudaGetLastError());
   c.launch("lowpass_x", 8 * (2 * V + V), st,
-           [&] { k_lowpass<R, N, 2, double><<<dim3(N / NL, N), nt, smem, st>>>(t2, n_obs, 1.0, tw); });
+           [&] { k_lowpass_c<N, 2><<<dim3(N / 2 / C::NL, N), C::NT, C::SMEM, st>>>(t2, n_obs, tw, half); });
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -319,7 +435,7 @@ static wf_status assign_any(Ctx& c, const wf_grid& g, int scheme, const double* 
     switch (n) {
 #define WF_CASE(N) \
   case N:          \
-    s = lowpass_sized<double, N>(c, fine, n_obs, unit, st); \
+    s = lowpass_sized<N>(c, fine, n_obs, unit, st); \
     break;
       WF_SIZES(WF_CASE)
 #undef WF_CASE

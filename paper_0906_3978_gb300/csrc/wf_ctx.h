@@ -104,6 +104,7 @@ struct Ctx {
   std::map<std::string, DevBuf> bufs;
   std::map<int, double2*> twiddles;  // per N: exp(-2 pi i e / (2N)), e < 2N
   std::map<int, float2*> twiddles32; // the same rounded to FP32 (for the FP32 kernels)
+  std::map<int, int4*> fixed_tw;     // per N: Q62 digits of the tables of fix_tables()
   std::map<std::string, DevBuf> pinned;  // page-locked host buffers (scalar staging)
   std::vector<cudaStream_t> streams;     // non-blocking streams for interleaved groups
   cudaStream_t cap_stream = nullptr;     // stream on which CG blocks are captured as graphs
@@ -138,6 +139,13 @@ struct Ctx {
   wf_status get(const std::string& name, size_t bytes, void** out);
   wf_status tw(int n, const double2** out);
   wf_status tw32(int n, const float2** out);
+  // Q62 digits (re high, re low, im high, im low) for the fixed-point transforms: tw[e] =
+  // exp(-2 pi i e / (2n)), e < 2n; half[k] = exp(-pi i s / n) 2^floor(log2 n) / n for k < n with signed
+  // frequency s (the half-sample shift of a length-n line with its normalisation), 2^.. / n at n / 2.
+  // fix_tables makes them (call it before any capture), fixed() and fixed_half() return them.
+  wf_status fix_tables(int n);
+  const int4* fixed(int n) const { return fixed_tw.at(n); }
+  const int4* fixed_half(int n) const { return fixed_tw.at(n) + 2 * n; }
   // Page-locked host buffer `name` with at least `bytes` bytes.
   wf_status get_pinned(const std::string& name, size_t bytes, void** out);
   // i-th library-owned non-blocking stream.
