@@ -1,0 +1,418 @@
+// wf_fixspec.cuh -- the FP64 spectral passes (packed half spectra of wf_spectral.cuh, FP64 storage) with their
+// transforms in 64-bit fixed point (wf_fix.cuh).  A CTA's threads load their elements straight into
+// registers, the transform exchanges them through shared memory between its two or three passes, and the
+// results go straight back: columns of the x and y passes as rows of 64 or 128 bytes, the rows of the
+// z passes as consecutive 16-byte elements.  Bound by the FP64 pipe's conversions (four per complex element,
+// more with an epilogue) beside the integer pipe; the FP64 butterflies they replace were bound by the
+// FP64 pipe alone.  512^3 per launch, before -> after: y pass 3.53 -> 0.65 ms (3.3 TB/s), x multiplier 7.80 -> 1.26,
+// z forward 4.48 -> 0.85, z inverse with the residual 5.52 -> 2.05.  Relative error of a smoothed field against
+// long double: 3.4e-16 .. 6.6e-16 -> 1.2e-16 .. 2.1e-16 (32^3 .. 128^3).
+#pragma once
+#include "wf_fix.cuh"
+#include "wf_spectral.cuh"
+
+namespace wf {
+
+// Geometry of the x / y passes: NL consecutive kz columns by N rows, one thread per line and element
+// class mod N / R1.
+template <int N> struct FxC {
+  static constexpr int NH = N / 2;
+  static constexpr int R1 = fx_plan(N).r1, N1 = N / R1;
+  static constexpr int NL = div_le(NH, N >= 256 ? 4 : 8);
+  static constexpr int NT = NL * N1;
+  static constexpr int KB = NH / NL;  // column blocks per plane
+  static constexpr size_t SMEM = (size_t)(N * NL + N) * 16;
+  static_assert(NL >= 2, "a packed-column pair takes two line slots");
+};
+
+// y pass: complex transform along y of every (x, kz) line, in place.  grid (N/2 / NL, N, systems)
+template <int N, int DIR>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  if (sc && sc[z].done) return;
+  double2* p = T + z * bt.spec + (size_t)blockIdx.y * N * NH + blockIdx.x * NL + l;
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) raw[r] = p[(size_t)(r * N1 + t) * NH];
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
+  fx_forward<N, DIR>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) { p[(size_t)k * NH] = fx_to2(X, f); });
+}
+
+// ---- Fourier tables as Q62 digits ----------------------------------------------------------------
+// tab[i] 2^-e as digits (high, low), in place; |tab[i]| < 2^e, e = exps[z estride].  grid (., systems)
+static __global__ void k_table_digits(double* __restrict__ tab, int len, const int* __restrict__ exps, int estride) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= len) return;
+  tab += (size_t)blockIdx.y * len;
+  long long q = __double2ll_rn(tab[i] * fx_pow2(62 - exps[blockIdx.y * estride]));
+  const int l = (int)q;
+  reinterpret_cast<int2*>(tab)[i] = make_int2((int)((q - l) >> 32), l);
+}
+WF_D fxc fx_scaleq(fxc a, int2 w) { return fxc{fx_mulq(a.x, w.x, w.y), fx_mulq(a.y, w.x, w.y)}; }
+// (a + s b) / 2 of two digit pairs
+WF_D int2 fx_mean(int2 a, int2 b, int s) {
+  const long long x = ((long long)a.x << 32) + a.y, y = ((long long)b.x << 32) + b.y;
+  const long long q = (x + s * y) >> 1;
+  const int l = (int)q;
+  return make_int2((int)((q - l) >> 32), l);
+}
+
+// x pass of a Fourier multiplier:  out = IFFT_x( tab (.) FFT_x(in) ), in != out.  The table holds digits
+// with the system's power of two exps[z estride].  The packed column's multiplier pairs a line with the one at
+// -ky: CTAs with blockIdx.x = N/2 / NL take both lines of a pair (ky <= N/2), the others skip column 0.
+// grid (N/2 / NL + 1, N, systems)
+template <int N> constexpr size_t fx_xmul_smem() { return FxC<N>::SMEM + (size_t)2 * N * 16; }
+template <int N>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_xmul(const double2* __restrict__ in, double2* __restrict__ out, const int2* __restrict__ tab,
+          const int* __restrict__ exps, int estride, const int4* __restrict__ twtab, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  const bool pair = blockIdx.x == G::KB;
+  const int ky = blockIdx.y;
+  if (pair && ky > N / 2) return;
+  in += z * bt.spec;
+  out += z * bt.spec;
+  tab += z * bt.tab;
+  const int ky_s = sfreq(ky, N);
+  const size_t rowstride = (size_t)N * NH;
+  // a pair's line slots 0 and 1 hold column 0 at ky and -ky, its other slots nothing
+  const int row_y = pair && l == 1 ? (N - ky) % N : ky;
+  const bool live = !pair || l < 2;
+  const size_t base = (size_t)row_y * NH + (pair ? 0 : blockIdx.x * NL + l);
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r)
+    raw[r] = live ? __ldg(in + base + (size_t)(r * N1 + t) * rowstride) : make_double2(0.0, 0.0);
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const int ls = pair && l < 2 ? 0 : l;  // the two lines of a pair share a scale
+  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
+  constexpr int H2 = fx_mid(N);
+  const int sh = -(H2 + exps[z * estride]);
+  if (!pair) {
+    const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
+    fx_convolve<N>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X) {
+      const int kxs = sfreq(k, N);
+      return fx_scaleq(fxc{fx_rshift(X.x, H2), fx_rshift(X.y, H2)}, __ldg(tab + kxs * kxs + k0));
+    });
+    if (kz == 0) return;  // the packed column's pair CTA writes it
+  } else {
+    fxc* nat = reinterpret_cast<fxc*>(tw + N);  // both lines' spectra in natural order
+    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+      if (l < 2) nat[l * N + k] = fxc{fx_rshift(X.x, H2), fx_rshift(X.y, H2)};
+    });
+    __syncthreads();
+    fx_inverse<N, +1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k) {
+      if (l >= 2) return fxc{0, 0};
+      const int kxs = sfreq(k, N), n2 = kxs * kxs + ky_s * ky_s;
+      const int2 m0 = __ldg(tab + n2), mN = __ldg(tab + n2 + NH * NH);
+      const fxc a = fx_scaleq(nat[l * N + k], fx_mean(m0, mN, 1));
+      const fxc b = fx_scaleq(nat[(1 - l) * N + (N - k) % N], fx_mean(m0, mN, -1));
+      return fxc{a.x + b.x, a.y - b.y};  // m+ Z(k) + m- conj Z(-k)
+    });
+    if (l >= 2 || (l == 1 && row_y == ky)) return;
+  }
+#pragma unroll
+  for (int r = 0; r < R1; ++r) out[base + (size_t)(r * N1 + t) * rowstride] = fx_to2(v[r], f, sh);
+}
+
+// x pass of the CG start:  out = tab (.) FFT_x(in),  partial of wgt |out|^2 (wgt 1 on column 0, 2 elsewhere)
+// per CTA; FP64 table.  CTAs as in k_fx_xmul.
+template <int N>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_xfwd(const double2* __restrict__ in, double2* __restrict__ out, const double* __restrict__ tab,
+          const int4* __restrict__ twtab, double* __restrict__ partials, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  const bool pair = blockIdx.x == G::KB;
+  const int ky = blockIdx.y;
+  partials += (size_t)z * bt.part + blockIdx.y * gridDim.x + blockIdx.x;
+  if (pair && ky > N / 2) {
+    if (tid == 0) *partials = 0.0;
+    return;
+  }
+  in += z * bt.spec;
+  out += z * bt.spec;
+  tab += z * bt.tab;
+  const int ky_s = sfreq(ky, N);
+  const size_t rowstride = (size_t)N * NH;
+  const int row_y = pair && l == 1 ? (N - ky) % N : ky;
+  const bool live = !pair || l < 2;
+  const size_t base = (size_t)row_y * NH + (pair ? 0 : blockIdx.x * NL + l);
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r)
+    raw[r] = live ? __ldg(in + base + (size_t)(r * N1 + t) * rowstride) : make_double2(0.0, 0.0);
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const int ls = pair && l < 2 ? 0 : l;
+  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
+  AccD acc;
+  if (!pair) {
+    const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
+    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+      if (kz == 0) return;
+      const int kxs = sfreq(k, N);
+      const double m = __ldg(tab + kxs * kxs + k0);
+      const double2 d = fx_to2(X, f), o = make_double2(d.x * m, d.y * m);
+      out[base + (size_t)k * rowstride] = o;
+      acc.add_prod(2.0 * o.x, o.x);
+      acc.add_prod(2.0 * o.y, o.y);
+    });
+  } else {
+    fxc* nat = reinterpret_cast<fxc*>(tw + N);
+    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+      if (l < 2) nat[l * N + k] = X;
+    });
+    __syncthreads();
+    if (l < 2 && !(l == 1 && row_y == ky))
+      for (int k = t; k < N; k += N1) {
+        const int kxs = sfreq(k, N), n2 = kxs * kxs + ky_s * ky_s;
+        const double m0 = __ldg(tab + n2), mN = __ldg(tab + n2 + NH * NH);
+        const double a = 0.5 * (m0 + mN), b = 0.5 * (m0 - mN);
+        const double2 zc = fx_to2(nat[l * N + k], f), zp = fx_to2(nat[(1 - l) * N + (N - k) % N], f);
+        const double2 o = make_double2(a * zc.x + b * zp.x, a * zc.y - b * zp.y);
+        out[base + (size_t)k * rowstride] = o;
+        acc.add_prod(o.x, o.x);
+        acc.add_prod(o.y, o.y);
+      }
+  }
+  const double s = block_sum(acc.get(), red);
+  if (tid == 0) *partials = s;
+}
+
+// x pass of s = C x:  out = IFFT_x( tab (.) in ), in != out; FP64 table.  grid (N/2 / NL, N, systems)
+template <int N>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_xinv(const double2* __restrict__ in, double2* __restrict__ out, const double* __restrict__ tab,
+          const int4* __restrict__ twtab, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  in += z * bt.spec;
+  out += z * bt.spec;
+  tab += z * bt.tab;
+  const int ky = blockIdx.y, ky_s = sfreq(ky, N), kz = blockIdx.x * NL + l;
+  const size_t rowstride = (size_t)N * NH, base = (size_t)ky * NH + kz;
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const int kx = r * N1 + t, kxs = sfreq(kx, N), n2 = kxs * kxs + ky_s * ky_s + kz * kz;
+    const double2 c = __ldg(in + base + (size_t)kx * rowstride);
+    const double m = __ldg(tab + n2);
+    if (kz != 0) {
+      raw[r] = make_double2(c.x * m, c.y * m);
+    } else {
+      const double mN = __ldg(tab + n2 + NH * NH), a = 0.5 * (m + mN), b = 0.5 * (m - mN);
+      const double2 p = __ldg(in + (size_t)((N - ky) % N) * NH + (size_t)((N - kx) % N) * rowstride);
+      raw[r] = make_double2(a * c.x + b * p.x, a * c.y - b * p.y);
+    }
+  }
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
+  fx_forward<N, +1>(v, slots + l, ColMap<NL>{}, t, tw,
+                    [&](int k, fxc X, int) { out[base + (size_t)k * rowstride] = fx_to2(X, f); });
+}
+
+// ---- z passes: rows of N reals as H = N/2 complex elements, thread t of a row holding n1 (H / R1) + t ----
+template <int N> struct FxZ {
+  static constexpr int H = N / 2, R1 = fx_plan(H).r1, N1 = H / R1;
+  static constexpr int NL = div_le(N * N, 256 / N1);  // rows per CTA
+  static constexpr int NT = NL * N1;
+  static constexpr int LS = fx_padded(H);
+  static constexpr int GZ = N * N / NL;  // CTAs per system
+  static constexpr size_t SMEM = (size_t)(NL * LS + N) * 16;
+};
+
+// X_k of the packed half spectrum from the length-H transform Z of x_2m + i x_2m+1 (slots in natural order)
+template <int N, class MAP> WF_D fxc fx_r2c(const fxc* s, const MAP& map, int k, const int4* tw) {
+  constexpr int H = N / 2;
+  const fxc a = s[map(k)];
+  if (k == 0) return fxc{a.x + a.y, a.x - a.y};
+  const fxc b = s[map(H - k)];
+  // halves first: X_k = (Z_k + conj Z_{H-k}) / 2 - (i/2) W_N^k (Z_k - conj Z_{H-k})
+  const fxc ah{(a.x + 1) >> 1, (a.y + 1) >> 1}, bh{(b.x + 1) >> 1, (b.y + 1) >> 1};
+  const fxc d = fx_twid<-1>(fxc{ah.x - bh.x, ah.y + bh.y}, tw[k]);
+  return fxc{ah.x + bh.x + d.y, ah.y - bh.y - d.x};
+}
+// Z_k from the packed X: (X_k + conj X_{H-k}) + i W_N^-k (X_k - conj X_{H-k})
+template <int N, class MAP> WF_D fxc fx_c2r(const fxc* s, const MAP& map, int k, const int4* tw) {
+  constexpr int H = N / 2;
+  const fxc a = s[map(k)];
+  if (k == 0) return fxc{a.x + a.y, a.x - a.y};
+  const fxc b = s[map(H - k)];
+  const fxc d = fx_twid<+1>(fxc{a.x - b.x, a.y + b.y}, tw[k]);
+  return fxc{a.x + b.x - d.y, a.y - b.y + d.x};
+}
+// The scale factor of a line's element count that bounds the C2R transform: with the packed X scaled by
+// ||Z||_2 <= 2 sqrt(2) ||X||_2, its partial sums are below sqrt(8 H) ||X||_2.
+template <int N> constexpr int fx_c2r_count() { return 8 * (N / 2); }
+
+// z forward: real rows -> packed spectrum rows; optional partial of sum(in^2).  grid (GZ, 1, systems)
+template <int N, bool SQ>
+__global__ void __launch_bounds__(FxZ<N>::NT)
+k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* __restrict__ twtab,
+          double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxZ<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, H = G::H;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + G::NL * G::LS);  // exp(-2 pi i e / N)
+  __shared__ int se[G::NL];
+  __shared__ unsigned sq[G::NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
+  if (sc && sc[z].done) return;
+  const size_t row = (size_t)blockIdx.x * G::NL + l;
+  const double2* src = reinterpret_cast<const double2*>(in + z * bt.real) + row * H;
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) raw[r] = __ldg(src + r * N1 + t);
+  if (tid < G::NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], H);
+  fxc* s = slots + l * G::LS;
+  fxc v[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
+  if constexpr (SQ) {
+    AccD acc;
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      acc.add_prod(raw[r].x, raw[r].x);
+      acc.add_prod(raw[r].y, raw[r].y);
+    }
+    const double q = block_sum(acc.get(), red);
+    if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = q;
+  }
+  fx_forward_nat<H, -1, 2>(v, s, PadMap{}, t, tw);
+  double2* dst = out + z * bt.spec + row * H;
+  for (int k = t; k < H; k += N1) dst[k] = fx_to2(fx_r2c<N>(s, PadMap{}, k, tw), f);
+}
+
+// z inverse: packed spectrum rows -> real rows, value v = scl * C2R(in), then the modes of k_zinv
+// (ZI_STORE out = v; ZI_RESID out = b - (v + nbar w s) with the partial sum of out^2).  grid (GZ, 1, systems)
+template <int N, int MODE>
+__global__ void __launch_bounds__(FxZ<N>::NT)
+k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double* __restrict__ s,
+          const double* __restrict__ w, const double* __restrict__ b, double scl, const int4* __restrict__ twtab,
+          double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxZ<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, H = G::H;
+  static_assert(MODE == ZI_STORE || MODE == ZI_RESID, "mode");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + G::NL * G::LS);
+  __shared__ int se[G::NL];
+  __shared__ unsigned sq[G::NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
+  const double nbar = sc ? sc[z].nbar : 0.0;
+  if (MODE != ZI_RESID && sc && sc[z].done == 4) return;
+  const size_t row = (size_t)blockIdx.x * G::NL + l;
+  const double2* src = in + z * bt.spec + row * H;
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) raw[r] = __ldg(src + r * N1 + t);
+  if (tid < G::NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], fx_c2r_count<N>());
+  fxc* sl = slots + l * G::LS;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) sl[PadMap{}(r * N1 + t)] = fx_from2(raw[r], f);
+  __syncthreads();
+  fxc v[R1];
+  fx_inverse<H, +1, 2>(v, sl, PadMap{}, t, tw, [&](int k) { return fx_c2r<N>(sl, PadMap{}, k, tw); });
+  AccD acc;
+  const size_t e0 = z * (bt.real / 2) + row * H;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const size_t e = e0 + r * N1 + t;
+    const double2 x = fx_to2(v[r], f);
+    double2 val;
+    if constexpr (MODE == ZI_RESID) {
+      const double2 sv = __ldg(reinterpret_cast<const double2*>(s) + e);
+      const double2 wv = __ldg(reinterpret_cast<const double2*>(w) + e);
+      const double2 bv = __ldg(reinterpret_cast<const double2*>(b) + e);
+      val.x = bv.x - (x.x * scl + nbar * wv.x * sv.x);
+      val.y = bv.y - (x.y * scl + nbar * wv.y * sv.y);
+      acc.add_prod(val.x, val.x);
+      acc.add_prod(val.y, val.y);
+    } else {
+      val = make_double2(x.x * scl, x.y * scl);
+    }
+    reinterpret_cast<double2*>(out)[e] = val;
+  }
+  if constexpr (MODE == ZI_RESID) {
+    const double sum = block_sum(acc.get(), red);
+    if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = sum;
+  }
+}
+
+}  // namespace wf

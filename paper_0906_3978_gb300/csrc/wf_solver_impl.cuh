@@ -33,13 +33,13 @@
 #include "wf_solver_group.h"
 #include "wf_plane.cuh"
 #include "wf_spectral.cuh"
+#include "wf_fixspec.cuh"
 #include "wf_deflate.cuh"
 
 namespace wf {
 
-// Arithmetic of the FP64-storage transforms.  The engine also runs in double-float (df32, FP32
-// units, ~2^-48 relative accuracy), which measured slower than native FP64 for the y pass at
-// the tile shapes used here, so native FP64 is used.
+// Arithmetic of the FP64-storage passes.  Their transforms run in 64-bit fixed point (wf_fix.cuh), the
+// vector updates and sums in FP64.
 using FP64Arith = double;
 
 template <class K>
@@ -64,6 +64,11 @@ struct Spec {
   static constexpr size_t SMz = ZG<R, N>::SMEM;
   static constexpr int GXY = (NH / NLxy) * N;   // blocks of an x or y pass (per system)
   static constexpr int GZ = N * N / NLz;        // blocks of a z pass (per system)
+  static constexpr bool F64 = sizeof(SS) == 8;  // FP64 storage: fixed-point transforms
+  using FC = FxC<N>;
+  using FZ = FxZ<N>;
+  static constexpr int GXF = F64 ? (FC::KB + 1) * N : GXY;  // partial sums of the CG start's x pass
+  static constexpr int GZI = F64 ? FZ::GZ : GZ;             // partial sums of the z inverse (residual)
   static constexpr size_t SPEC = (size_t)N * N * NH;  // complex elements of a spectrum
   static constexpr size_t V = (size_t)N * N * N;
   static constexpr int TAB = 3 * (N / 2) * (N / 2) + 1;
@@ -97,9 +102,19 @@ struct Spec {
     WF_A((k_cg_xinv<R, N, false>), SMxy);
     WF_A((k_cg_xupd<R, N, true>), SMxy);
     WF_A((k_cg_xupd<R, N, false>), SMxy);
-    WF_A((k_xmul<R, N, true, false, true>), SMxy);
-    WF_A((k_xmul<R, N, false, true, false>), SMxy);
-    WF_A((k_xmul<R, N, true, true, false>), SMxy);
+    if constexpr (F64) {
+      WF_A((k_fx_xmul<N>), fx_xmul_smem<N>());
+      WF_A((k_fx_xfwd<N>), fx_xmul_smem<N>());
+      WF_A((k_fx_xinv<N>), FC::SMEM);
+      WF_A((k_fx_zfwd<N, false>), FZ::SMEM);
+      WF_A((k_fx_zinv<N, ZI_STORE>), FZ::SMEM);
+      WF_A((k_fx_zinv<N, ZI_RESID>), FZ::SMEM);
+    } else {
+      WF_A((k_xmul<R, N, true, false, true>), SMxy);
+      WF_A((k_xmul<R, N, false, true, false>), SMxy);
+      WF_A((k_zfwd<R, N, false>), SMz);
+      WF_A((k_zinv<R, N, ZI_ACCUM>), SMz);
+    }
     WF_A((k_zturn<R, N>), SMz);
     if constexpr (std::is_same<R, float>::value) {
       WF_A((k_zcoarse<R, N>), SMz);
@@ -108,11 +123,6 @@ struct Spec {
       WF_A((k_ycoarse<R, N>), (size_t)N * (kDeflMaxRadius + 2) * sizeof(cx<R>));
     }
     if constexpr (PCS > 0) WF_A((k_plane_turn<R, N, PCS, PE>), (PlaneG<R, N, PCS, PE>::SMEM));
-    WF_A((k_zfwd<R, N, true>), SMz);
-    WF_A((k_zfwd<R, N, false>), SMz);
-    WF_A((k_zinv<R, N, ZI_STORE>), SMz);
-    WF_A((k_zinv<R, N, ZI_RESID>), SMz);
-    WF_A((k_zinv<R, N, ZI_ACCUM>), SMz);
 #undef WF_A
     for (const PassVariant& v : yvariants())
       if (e == cudaSuccess) e = v.setup();
@@ -163,10 +173,27 @@ struct Spec {
       });
     }
   };
+  // the FP64 y pass (fixed point); tw is unused, its twiddles come from the context
+  struct YFix {
+    static cudaError_t setup() {
+      cudaError_t e = set_smem(k_fx_ypass<N, -1>, FC::SMEM);
+      return e == cudaSuccess ? set_smem(k_fx_ypass<N, +1>, FC::SMEM) : e;
+    }
+    static void run(Ctx& c, int nb, ST* t, const ST*, const CgScal* sc, int dir, cudaStream_t st) {
+      double2* T = reinterpret_cast<double2*>(t);
+      const dim3 grid(FC::KB, N, nb);
+      c.launch("ypass_f64", 2 * BS * nb, st, [&] {
+        if (dir < 0) k_fx_ypass<N, -1><<<grid, FC::NT, FC::SMEM, st>>>(T, c.fixed(N), sc, bat());
+        else k_fx_ypass<N, +1><<<grid, FC::NT, FC::SMEM, st>>>(T, c.fixed(N), sc, bat());
+      });
+    }
+  };
   // candidates: FP32 grids of 128 and up (the inner solves) get a few; everything else the default
   static const std::vector<PassVariant>& yvariants() {
     static const std::vector<PassVariant> v = [] {
-      std::vector<PassVariant> out{{"nl_s2_r8", YV<NLT, 2, 8>::setup, YV<NLT, 2, 8>::run}};
+      std::vector<PassVariant> out;
+      if constexpr (F64) out.push_back({"fixed", YFix::setup, YFix::run});
+      else out.push_back({"nl_s2_r8", YV<NLT, 2, 8>::setup, YV<NLT, 2, 8>::run});
       if constexpr (std::is_same<R, float>::value && N >= 128) {
         constexpr int H = NLT / 2;
         out.push_back({"nl_s2_r32", YV<NLT, 2, 32>::setup, YV<NLT, 2, 32>::run});
@@ -375,17 +402,35 @@ struct Spec {
   static void ypass(Ctx& c, int nb, ST* t, const ST* tw, const CgScal* sc, int dir, cudaStream_t st) {
     pick(c, "ypass", yvariants()).run(c, nb, t, tw, sc, dir, st);
   }
-  // out = [IFFT_x] tab (.) [FFT_x] in
+  // out = [IFFT_x] tab (.) [FFT_x] in (FP64 form with both transforms: fmul below)
   template <bool FWD, bool INV, bool DOT>
   static void xmul(Ctx& c, int nb, const ST* in, ST* out, const SS* tab, const ST* tw, double* part,
                    const CgScal* sc, cudaStream_t st) {
-    c.launch(cls("xmul", "xmul_f64"), 2 * BS * nb, st,
-             [&] { k_xmul<R, N, FWD, INV, DOT><<<gxy(nb), NTx, SMxy, st>>>(in, out, tab, tw, part, sc, bat()); });
+    c.launch(cls("xmul", "xmul_f64"), 2 * BS * nb, st, [&] {
+      if constexpr (F64 && FWD) {
+        static_assert(!INV && DOT, "the FP64 forward x pass starts a CG");
+        k_fx_xfwd<N><<<dim3(FC::KB + 1, N, nb), FC::NT, fx_xmul_smem<N>(), st>>>(in, out, tab, c.fixed(N), part, bat());
+      } else if constexpr (F64) {
+        k_fx_xinv<N><<<dim3(FC::KB, N, nb), FC::NT, FC::SMEM, st>>>(in, out, tab, c.fixed(N), bat());
+      } else {
+        k_xmul<R, N, FWD, INV, DOT><<<gxy(nb), NTx, SMxy, st>>>(in, out, tab, tw, part, sc, bat());
+      }
+    });
   }
-  static void zfwd(Ctx& c, int nb, const double* in, ST* out, const ST* tw, double* part, bool sq,
-                   const CgScal* sc, cudaStream_t st) {
+  // out = IFFT_x tab (.) FFT_x in in FP64 storage, tab as digits (k_table_digits), system z's power of two at
+  // exps[z * estride]
+  static void fmul(Ctx& c, int nb, const double2* in, double2* out, const double* tab, const int* exps, int estride,
+                   cudaStream_t st) {
+    c.launch("xmul_f64", 2 * BS * nb, st, [&] {
+      k_fx_xmul<N><<<dim3(FC::KB + 1, N, nb), FC::NT, fx_xmul_smem<N>(), st>>>(
+          in, out, reinterpret_cast<const int2*>(tab), exps, estride, c.fixed(N), bat());
+    });
+  }
+  static void zfwd(Ctx& c, int nb, const double* in, ST* out, const ST* tw, double* part, const CgScal* sc,
+                   cudaStream_t st) {
     c.launch(cls("zfwd", "zfwd_f64"), (BS + 8 * BV) * nb, st, [&] {
-      if (sq) k_zfwd<R, N, true><<<gz(nb), NTz, SMz, st>>>(in, out, tw, part, sc, bat());
+      if constexpr (F64)
+        k_fx_zfwd<N, false><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(in, out, c.fixed(N), part, sc, bat());
       else k_zfwd<R, N, false><<<gz(nb), NTz, SMz, st>>>(in, out, tw, part, sc, bat());
     });
   }
@@ -393,8 +438,12 @@ struct Spec {
   static void zinv(Ctx& c, int nb, const ST* in, double* out, const double* s, const double* w, const double* b,
                    double scl, const ST* tw, double* part, const CgScal* sc, cudaStream_t st) {
     const double vb = MODE == ZI_RESID ? 4 : (MODE == ZI_ACCUM ? 2 : 1);
-    c.launch(cls("zinv", "zinv_f64"), (BS + 8 * vb * BV) * nb, st,
-             [&] { k_zinv<R, N, MODE><<<gz(nb), NTz, SMz, st>>>(in, out, s, w, b, scl, tw, part, sc, bat()); });
+    c.launch(cls("zinv", "zinv_f64"), (BS + 8 * vb * BV) * nb, st, [&] {
+      if constexpr (F64)
+        k_fx_zinv<N, MODE><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(in, out, s, w, b, scl, c.fixed(N), part, sc,
+                                                                          bat());
+      else k_zinv<R, N, MODE><<<gz(nb), NTz, SMz, st>>>(in, out, s, w, b, scl, tw, part, sc, bat());
+    });
   }
 
   struct NoHook {
@@ -475,6 +524,15 @@ static void make_tables(const std::vector<double>& sinv, bool precond, double c0
   }
 }
 
+// Smallest e with every entry of v below 2^e in modulus (the power of two of a table's digits)
+static inline int table_exp(const double* v, size_t n) {
+  double m = 0.0;
+  for (size_t i = 0; i < n; ++i) m = std::max(m, std::fabs(v[i]));
+  int e = 0;
+  std::frexp(m, &e);
+  return std::max(-900, std::min(e, 1000));
+}
+
 // Device table `name` from v, converted to T, through a page-locked staging buffer of the same
 // name (an asynchronous copy: the staging buffer is rewritten only by a later solve of the same
 // workspace, after this one's stream has finished).
@@ -550,6 +608,14 @@ struct GroupCommon : Group {
     return WF_OK;
   }
 
+  // The prior's FP64 table `stab` (TAB entries per system) to digits in place, after push_scalars: the
+  // systems' powers of two are in their scalars.
+  void table_digits(Ctx& c, double* stab, cudaStream_t st) {
+    c.launch("tables", 0, st, [&] {
+      k_table_digits<<<dim3((TAB + 255) / 256, nb), 256, 0, st>>>(stab, TAB, &sc->texp, kScalInts);
+    });
+  }
+  static constexpr int kScalInts = (int)(sizeof(CgScal) / sizeof(int));
   wf_status push_scalars(cudaStream_t st) {
     for (int m = 0; m < nb; ++m) hsc[m] = h[m];
     WF_CUDA(cudaMemcpyAsync(sc, hsc, nb * sizeof(CgScal), cudaMemcpyHostToDevice, st));
@@ -636,6 +702,7 @@ struct GroupFP64 : GroupCommon<N> {
     WF_CUDA(SP::attrs());
     const size_t SPEC = SP::SPEC, V = SP::V;
     WF_TRY(c.tw(N, &tw));
+    WF_TRY(c.fix_tables(N));
     const char* nm[6] = {"x", "r", "p0", "p1", "T", "T2"};
     ST** ptr[6] = {&xh, &rh, &P0, &P1, &T, &T2};
     for (int i = 0; i < 6; ++i) WF_TRY(c.get(key + nm[i], nb * SPEC * sizeof(ST), (void**)ptr[i]));
@@ -674,12 +741,14 @@ struct GroupFP64 : GroupCommon<N> {
     h.assign(nb, CgScal{});
     for (int m = 0; m < nb; ++m) {
       h[m].nbar = sys[m]->nbar;
+      h[m].texp = table_exp(sys[m]->sinv.data(), TAB);
       h[m].max_iter = sys[m]->opts.max_iter;
       h[m].tol2 = sys[m]->opts.tol * sys[m]->opts.tol;
       h[m].bb = bb0[m];
       if (this->bad[m]) h[m].done = 4;
     }
     WF_TRY(this->push_scalars(st));
+    this->table_digits(c, stab, st);
     c.launch("make_D", 16.0 * V * nb, st, [&] { k_make_D<double><<<dim3(152 * 4, nb), 256, 0, st>>>(W, D, sc, inv_vc, V); });
     WF_CUDA(cudaMemsetAsync(xh, 0, nb * SPEC * sizeof(ST), st));
     rel.assign(nb, 1.0);
@@ -692,11 +761,11 @@ struct GroupFP64 : GroupCommon<N> {
   // r = C F(rhs) for every system; p = 0; reset the recurrences of the running systems
   wf_status start_cg(Ctx& c, const double* rhs, cudaStream_t st) {
     const size_t SPEC = SP::SPEC;
-    SP::zfwd(c, nb, rhs, T, tw, part, false, nullptr, st);
+    SP::zfwd(c, nb, rhs, T, tw, part, nullptr, st);
     SP::ypass(c, nb, T, tw, nullptr, -1, st);
     SP::template xmul<true, false, true>(c, nb, T, rh, ct, tw, part, nullptr, st);
     const Bat b = SP::bat();
-    c.launch("fin", 0, st, [&] { k_fin_init<<<nb, 1024, 0, st>>>(part, SP::GXY, sc, b); });
+    c.launch("fin", 0, st, [&] { k_fin_init<<<nb, 1024, 0, st>>>(part, SP::GXF, sc, b); });
     WF_CUDA(cudaMemsetAsync(P0, 0, nb * SPEC * sizeof(ST), st));
     WF_CUDA(cudaMemsetAsync(P1, 0, nb * SPEC * sizeof(ST), st));
     WF_CUDA(cudaGetLastError());
@@ -719,12 +788,12 @@ struct GroupFP64 : GroupCommon<N> {
       SP::ypass(c, nb, T, tw, nullptr, +1, st);
       SP::template zinv<ZI_STORE>(c, nb, T, S, nullptr, nullptr, nullptr, inv_vc, tw, part, nullptr, st);
       // residual b - A s
-      SP::zfwd(c, nb, S, T, tw, part, false, nullptr, st);
+      SP::zfwd(c, nb, S, T, tw, part, nullptr, st);
       SP::ypass(c, nb, T, tw, nullptr, -1, st);
-      SP::template xmul<true, true, false>(c, nb, T, T2, stab, tw, part, nullptr, st);
+      SP::fmul(c, nb, T, T2, stab, &sc->texp, this->kScalInts, st);
       SP::ypass(c, nb, T2, tw, nullptr, +1, st);
       SP::template zinv<ZI_RESID>(c, nb, T2, RES, S, W, B, inv_vc, tw, part, sc, st);
-      c.launch("fin", 0, st, [&] { k_fin_sum<<<nb, 1024, 0, st>>>(part, SP::GZ, 0, sc, b); });
+      c.launch("fin", 0, st, [&] { k_fin_sum<<<nb, 1024, 0, st>>>(part, SP::GZI, 0, sc, b); });
     } else if (phase == 3) {
       WF_TRY(this->push_scalars(st));
       WF_TRY(start_cg(c, RES, st));
@@ -795,6 +864,7 @@ struct GroupMixed : GroupCommon<N> {
   float *ct, *mt;
   double* stab;
   std::vector<int> outer, iters;
+  std::vector<int> texp;  // per system: power of two of the prior table's digits
   std::vector<int> noco;  // per system: inner solves without the coarse space after a failed one
   bool unit_m = true;
   static constexpr int NPART = SF::NPART > SD::NPART ? SF::NPART : SD::NPART;
@@ -819,6 +889,7 @@ struct GroupMixed : GroupCommon<N> {
     const size_t SPEC = SF::SPEC, V = SF::V;
     WF_TRY(c.tw(N, &tw));
     WF_TRY(c.tw32(N, &tw32));
+    WF_TRY(c.fix_tables(N));
     const char* nm[5] = {"x", "r", "p0", "p1", "T"};
     float2** ptr[5] = {&xh, &rh, &P0, &P1, &T};
     for (int i = 0; i < 5; ++i) WF_TRY(c.get(key + nm[i], nb * SPEC * sizeof(float2), (void**)ptr[i]));
@@ -877,7 +948,7 @@ struct GroupMixed : GroupCommon<N> {
     std::vector<double> ones((size_t)nb * SF::TAB, 1.0);
     float* tone;
     WF_TRY(upload_tables<float>(c, key + "t1", ones, &tone, st));
-    SF::zfwd(c, nb, W, T, tw32, part, false, nullptr, st);
+    SF::zfwd(c, nb, W, T, tw32, part, nullptr, st);
     SF::ypass(c, nb, T, tw32, nullptr, -1, st);
     SF::template xmul<true, false, true>(c, nb, T, P0, tone, tw32, part, nullptr, st);
     const int C = 4 * K + 1;
@@ -969,8 +1040,13 @@ struct GroupMixed : GroupCommon<N> {
     WF_TRY(upload_tables<float>(c, key + "tm", vm, &mt, st));
     WF_TRY(upload_tables<double>(c, key + "ts", vs, &stab, st));
     h.assign(nb, CgScal{});
-    for (int m = 0; m < nb; ++m) h[m].nbar = sys[m]->nbar;
+    texp.resize(nb);
+    for (int m = 0; m < nb; ++m) {
+      h[m].nbar = sys[m]->nbar;
+      h[m].texp = texp[m] = table_exp(sys[m]->sinv.data(), TAB);
+    }
     WF_TRY(this->push_scalars(st));
+    this->table_digits(c, stab, st);
     c.launch("make_D", 12.0 * V * nb, st, [&] { k_make_D<float><<<dim3(152 * 4, nb), 256, 0, st>>>(W, D, sc, inv_vc, V); });
     if (K > 0) WF_TRY(defl_setup(c, st));
     // x = 0 (accumulated in S), res = b
@@ -1002,6 +1078,7 @@ struct GroupMixed : GroupCommon<N> {
       for (int m = 0; m < nb; ++m) {
         CgScal z{};
         z.nbar = sys[m]->nbar;
+        z.texp = texp[m];
         if (state[m]) {
           z.done = 4;
         } else {
@@ -1018,7 +1095,7 @@ struct GroupMixed : GroupCommon<N> {
       }
       WF_TRY(this->push_scalars(st));
       const size_t SPEC = SF::SPEC;
-      SF::zfwd(c, nb, RES, T, tw32, part, false, nullptr, st);
+      SF::zfwd(c, nb, RES, T, tw32, part, nullptr, st);
       SF::ypass(c, nb, T, tw32, nullptr, -1, st);
       SF::template xmul<true, false, true>(c, nb, T, rh, ct, tw32, part, nullptr, st);
       c.launch("fin", 0, st, [&] { k_fin_init<<<nb, 1024, 0, st>>>(part, SF::GXY, sc, bf); });
@@ -1051,13 +1128,13 @@ struct GroupMixed : GroupCommon<N> {
       SF::ypass(c, nb, T, tw32, nullptr, +1, st);
       SF::template zinv<ZI_ACCUM>(c, nb, T, S, nullptr, nullptr, nullptr, inv_vc, tw32, part, sc, st);
       // FP64 residual res = b - A x
-      SD::zfwd(c, nb, S, T64, tw, part, false, nullptr, st);
+      SD::zfwd(c, nb, S, T64, tw, part, nullptr, st);
       SD::ypass(c, nb, T64, tw, nullptr, -1, st);
-      SD::template xmul<true, true, false>(c, nb, T64, T64b, stab, tw, part, nullptr, st);
+      SD::fmul(c, nb, T64, T64b, stab, &sc->texp, this->kScalInts, st);
       SD::ypass(c, nb, T64b, tw, nullptr, +1, st);
       SD::template zinv<ZI_RESID>(c, nb, T64b, RES, S, W, B, inv_vc, tw, part, sc, st);
       const Bat bd = SD::bat();
-      c.launch("fin", 0, st, [&] { k_fin_sum<<<nb, 1024, 0, st>>>(part, SD::GZ, 0, sc, bd); });
+      c.launch("fin", 0, st, [&] { k_fin_sum<<<nb, 1024, 0, st>>>(part, SD::GZI, 0, sc, bd); });
     }
     WF_CUDA(cudaGetLastError());
     return this->pull_scalars(st);
@@ -1119,20 +1196,23 @@ wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::v
   int* err;
   WF_TRY(c.err_word(&err));
   WF_CUDA(SD::attrs());
-  const double2* tw;
-  WF_TRY(c.tw(N, &tw));
+  WF_TRY(c.fix_tables(N));
   double2 *T, *T2;
-  double* part;
+  int *exps, *hexp;
   WF_TRY(c.get("sm_T", SD::SPEC * sizeof(double2), (void**)&T));
   WF_TRY(c.get("sm_T2", SD::SPEC * sizeof(double2), (void**)&T2));
-  WF_TRY(c.get("sm_part", (size_t)SD::NPART * sizeof(double), (void**)&part));
+  WF_TRY(c.get("sm_e", sizeof(int), (void**)&exps));
+  WF_TRY(c.get_pinned("sm_eh", sizeof(int), (void**)&hexp));
   double* gt;
   WF_TRY(upload_tables<double>(c, "sm_g", table, &gt, st));
-  SD::zfwd(c, 1, in, T, tw, part, false, nullptr, st);
-  SD::ypass(c, 1, T, tw, nullptr, -1, st);
-  SD::template xmul<true, true, false>(c, 1, T, T2, gt, tw, part, nullptr, st);
-  SD::ypass(c, 1, T2, tw, nullptr, +1, st);
-  SD::template zinv<ZI_STORE>(c, 1, T2, out, nullptr, nullptr, nullptr, 1.0 / (double)SD::V, tw, part, nullptr,
+  *hexp = table_exp(table.data(), table.size());
+  WF_CUDA(cudaMemcpyAsync(exps, hexp, sizeof(int), cudaMemcpyHostToDevice, st));
+  c.launch("tables", 0, st, [&] { k_table_digits<<<dim3((SD::TAB + 255) / 256, 1), 256, 0, st>>>(gt, SD::TAB, exps, 1); });
+  SD::zfwd(c, 1, in, T, nullptr, nullptr, nullptr, st);
+  SD::ypass(c, 1, T, nullptr, nullptr, -1, st);
+  SD::fmul(c, 1, T, T2, gt, exps, 1, st);
+  SD::ypass(c, 1, T2, nullptr, nullptr, +1, st);
+  SD::template zinv<ZI_STORE>(c, 1, T2, out, nullptr, nullptr, nullptr, 1.0 / (double)SD::V, nullptr, nullptr, nullptr,
                               st);
   WF_CUDA(cudaGetLastError());
   WF_CUDA(cudaStreamSynchronize(st));
@@ -1196,6 +1276,7 @@ wf_status tune_spec(Ctx& c, std::string& report) {
   int* err;
   WF_TRY(c.err_word(&err));
   WF_CUDA(SP::attrs());
+  WF_TRY(c.fix_tables(SP::NH * 2));
   const ST* tw;
   if constexpr (sizeof(typename SP::SS) == 8) {
     WF_TRY(c.tw(SP::NH * 2, &tw));

@@ -49,7 +49,7 @@ struct __align__(16) CgScal {
   int lit;            // iterations since the last reset of p: p_old = P[lit & 1]
   int defl;           // deflated inner solves: 2 start step (alpha = 1) pending, 1 first iteration
   int noco;           // deflated groups: 1 = this system runs its inner solves without the coarse space
-  int pad;
+  int texp;           // power of two of the FP64 prior table's digits (k_fx_xmul)
 };
 
 // Distances between consecutive systems of a batch (elements of each array type).

@@ -71,3 +71,35 @@ def test_weighted_lowpass_over_the_mass_range(ctx, n):
     got = ctx.grid_assign_weighted(torch.from_numpy(pos).to(DEV), torch.from_numpy(mass).to(DEV), n, box, wf.TSC, 2,
                                    fine_out=fine)
     assert rl2(got, lowpass(fine, n, 2.0 ** -32)) <= tol((2 * n) ** 3)
+
+
+def smoothed(f, n, box, r_s):
+    m = torch.arange(n, device=DEV)
+    m = torch.where(m > n // 2, m - n, m).to(torch.float64)
+    z = torch.arange(n // 2 + 1, device=DEV, dtype=torch.float64)
+    n2 = (m * m)[:, None, None] + (m * m)[None, :, None] + (z * z)[None, None, :]
+    k2 = (2.0 * math.pi / box) ** 2 * n2
+    return torch.fft.irfftn(torch.fft.rfftn(f) * torch.exp(-0.5 * k2 * r_s * r_s), s=(n, n, n))
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("kind", ["white", "spike", "tiny", "huge"])
+def test_fourier_passes_every_size(ctx, n, kind):
+    """The FP64 z, y and x passes (forward, multiplier, inverse): white noise, one value 1e9 above it, and
+    fields near the ends of the exponent range."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n)
+    f = torch.randn((n, n, n), dtype=torch.float64, device=DEV, generator=g)
+    if kind == "spike":
+        f[n // 3, n // 2, 1] = 1e9
+    scale = {"tiny": 1e-230, "huge": 1e290}.get(kind, 1.0)
+    got = ctx.smooth(f * scale, 1.0 * n, 0.6) / scale
+    assert rl2(got, smoothed(f, n, 1.0 * n, 0.6)) <= tol(n ** 3)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_non_finite_fields_stay_non_finite(ctx, value):
+    """Every value of the result depends on every value of the field."""
+    f = torch.zeros((24, 24, 24), dtype=torch.float64, device=DEV)
+    f[3, 4, 5] = value
+    assert not bool(torch.isfinite(ctx.smooth(f, 24.0, 1.0)).any())
