@@ -162,7 +162,7 @@ template <int N> struct LpZ {
   static constexpr int R1 = fx_plan(N).r1, TPL = N / R1;
   static constexpr int NP = div_le(2 * N * N, TPL >= 128 ? 1 : 256 / TPL);  // pairs per CTA
   static constexpr int NT = NP * TPL;
-  static constexpr int LS = fx_padded(N);
+  static constexpr int LS = ln_padded(N, 3, TPL, 8);
   static constexpr size_t SMEM = (size_t)(NP * LS + N + NP * (TPL + kNyqParts)) * 16;
 };
 template <int N>
@@ -243,7 +243,7 @@ k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out,
     for (int u = g; u < G::TPL; u += kNyqParts) e = e + ny[l * G::TPL + u];
     parts[g] = e;
   }
-  fx_convolve<N>(v, slots + l * G::LS, PadMap{}, t, tw, LpShift<N>{phtab, parts, 1});
+  ln_convolve<N, FxPlan<N>>(v, slots + l * G::LS, PadMap{}, t, tw, LpShift<N>{phtab, parts, 1});
   constexpr int A = fx_floor_log2(N) - fx_mid(N);
   const int ke = k + A;  // the even samples in the result's units
   auto fixe = [&](unsigned long long w) { return (long long)(ke >= 0 ? w << ke : w >> -ke); };
@@ -337,7 +337,7 @@ k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4*
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fxc{fx_from(o[r].x, k), fx_from(o[r].y, k)};
-  fx_convolve<N>(v, slots + l, ColMap<NL>{}, t, tw, LpShift<N>{phtab, parts + l, NL});
+  ln_convolve<N, FxPlan<N>>(v, slots + l, ColMap<NL>{}, t, tw, LpShift<N>{phtab, parts + l, NL});
   constexpr int A = fx_floor_log2(N) - fx_mid(N);
   const double c = emax == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : fx_pow2(-(k + A));
   const size_t ostride = AXIS == 1 ? N : (size_t)N * N;

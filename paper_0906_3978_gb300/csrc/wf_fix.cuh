@@ -16,7 +16,7 @@
 // largest value lies below 2^-800 keep an absolute resolution of about 2^-860 only, and a line with an
 // infinity or NaN becomes NaN throughout (FP64 butterflies spread either over the line as well).
 #pragma once
-#include "wf_common.cuh"
+#include "wf_line.cuh"
 
 namespace wf {
 
@@ -76,315 +76,49 @@ WF_D int4 fx_w9(int m) {
                   : make_int4(-1008987269, 1537591498, -367241333, 1978927779);
 }
 
-// ---- small DFTs in registers ---------------------------------------------------------------
-template <int DIR> WF_D void fx_dft2(fxc& a, fxc& b) {
-  const fxc s = a + b;
-  b = a - b;
-  a = s;
-}
-template <int DIR> WF_D void fx_dft3(fxc& a, fxc& b, fxc& c) {
-  const fxc t = b + c, u = b - c;
-  const fxc m{a.x - ((t.x + 1) >> 1), a.y - ((t.y + 1) >> 1)};
-  const fxc ju = fx_mul_i<DIR>(fxc{fx_mulq(u.x, kFxS3h, kFxS3l), fx_mulq(u.y, kFxS3h, kFxS3l)});
-  a = a + t;
-  b = m + ju;
-  c = m - ju;
-}
-template <int DIR> WF_D void fx_dft4(fxc& a, fxc& b, fxc& c, fxc& d) {
-  const fxc t0 = a + c, t1 = a - c, t2 = b + d, t3 = fx_mul_i<DIR>(b - d);
-  a = t0 + t2;
-  b = t1 + t3;
-  c = t0 - t2;
-  d = t1 - t3;
-}
-// v[0..RAD) -> its DFT in natural order
-template <int RAD, int DIR> WF_D void fx_dft(fxc* v) {
-  if constexpr (RAD == 2) {
-    fx_dft2<DIR>(v[0], v[1]);
-  } else if constexpr (RAD == 3) {
-    fx_dft3<DIR>(v[0], v[1], v[2]);
-  } else if constexpr (RAD == 4) {
-    fx_dft4<DIR>(v[0], v[1], v[2], v[3]);
-  } else if constexpr (RAD == 6) {
-    // 2 x 3 without twiddles: n = 3 n1 + 2 n2, k = 3 k1 + 4 k2 (mod 6)
-    fxc a0 = v[0], a1 = v[2], a2 = v[4], b0 = v[3], b1 = v[5], b2 = v[1];
-    fx_dft3<DIR>(a0, a1, a2);
-    fx_dft3<DIR>(b0, b1, b2);
-    v[0] = a0 + b0;
-    v[3] = a0 - b0;
-    v[4] = a1 + b1;
-    v[1] = a1 - b1;
-    v[2] = a2 + b2;
-    v[5] = a2 - b2;
-  } else if constexpr (RAD == 8) {
-    fx_dft4<DIR>(v[0], v[2], v[4], v[6]);
-    fx_dft4<DIR>(v[1], v[3], v[5], v[7]);
-    // W8^1 = (1 + DIR i)/sqrt2, W8^2 = DIR i, W8^3 = (-1 + DIR i)/sqrt2
-    const fxc p = v[3] + fx_mul_i<DIR>(v[3]), q = fx_mul_i<DIR>(v[7]) - v[7];
-    const fxc o1{fx_mulq(p.x, kFxR2h, kFxR2l), fx_mulq(p.y, kFxR2h, kFxR2l)};
-    const fxc o2 = fx_mul_i<DIR>(v[5]);
-    const fxc o3{fx_mulq(q.x, kFxR2h, kFxR2l), fx_mulq(q.y, kFxR2h, kFxR2l)};
-    const fxc e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
-    v[0] = e0 + o0;
-    v[4] = e0 - o0;
-    v[1] = e1 + o1;
-    v[5] = e1 - o1;
-    v[2] = e2 + o2;
-    v[6] = e2 - o2;
-    v[3] = e3 + o3;
-    v[7] = e3 - o3;
-  } else if constexpr (RAD == 9) {
-    // 3 x 3: columns n = 3 n1 + n2, twiddles W9^(n2 k1), rows; k = k1 + 3 k2
-    fx_dft3<DIR>(v[0], v[3], v[6]);
-    fx_dft3<DIR>(v[1], v[4], v[7]);
-    fx_dft3<DIR>(v[2], v[5], v[8]);
-    v[4] = fx_twid<DIR>(v[4], fx_w9(1));
-    v[5] = fx_twid<DIR>(v[5], fx_w9(2));
-    v[7] = fx_twid<DIR>(v[7], fx_w9(2));
-    v[8] = fx_twid<DIR>(v[8], fx_w9(4));
-    fx_dft3<DIR>(v[0], v[1], v[2]);
-    fx_dft3<DIR>(v[3], v[4], v[5]);
-    fx_dft3<DIR>(v[6], v[7], v[8]);
-    fxc t = v[1];  // transpose the 3 x 3 result
-    v[1] = v[3];
-    v[3] = t;
-    t = v[2];
-    v[2] = v[6];
-    v[6] = t;
-    t = v[5];
-    v[5] = v[7];
-    v[7] = t;
-  } else {
-    static_assert(RAD == 12, "radix");
-    // 4 x 3 without twiddles: n = 3 n1 + 4 n2, k = 9 k1 + 4 k2 (mod 12)
-    fxc a[3][4];
-#pragma unroll
-    for (int n2 = 0; n2 < 3; ++n2) {
-#pragma unroll
-      for (int n1 = 0; n1 < 4; ++n1) a[n2][n1] = v[(3 * n1 + 4 * n2) % 12];
-      fx_dft4<DIR>(a[n2][0], a[n2][1], a[n2][2], a[n2][3]);
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-      fx_dft3<DIR>(a[0][k1], a[1][k1], a[2][k1]);
-#pragma unroll
-      for (int k2 = 0; k2 < 3; ++k2) v[(9 * k1 + 4 * k2) % 12] = a[k2][k1];
-    }
-  }
-}
-
-// ---- radix plans: M = R1 R2 R3 (R3 = 1: two passes), butterflies small enough for registers ------
+// ---- radix plans: M = R1 R2 R3 (R3 = 1: two passes), butterflies of up to 12 points ------
 struct FxRad {
   int r1, r2, r3;
 };
+// (the last radix no smaller than the first, or a divisor of it, so that no pass runs a nearly empty round)
 constexpr FxRad fx_plan(int m) {
   switch (m) {
     case 8: return {4, 2, 1};
-    case 12: return {4, 3, 1};
+    case 12: return {3, 4, 1};
     case 16: return {4, 4, 1};
-    case 24: return {6, 4, 1};
+    case 24: return {4, 6, 1};
     case 32: return {8, 4, 1};
     case 36: return {6, 6, 1};
-    case 48: return {8, 6, 1};
-    case 54: return {9, 6, 1};
+    case 48: return {6, 8, 1};
+    case 54: return {6, 9, 1};
     case 64: return {8, 8, 1};
-    case 72: return {12, 6, 1};
-    case 96: return {12, 8, 1};
-    case 108: return {12, 9, 1};
+    case 72: return {8, 9, 1};
+    case 96: return {8, 12, 1};
+    case 108: return {9, 12, 1};
     case 128: return {8, 4, 4};
     case 144: return {12, 12, 1};
     case 192: return {8, 6, 4};
     case 216: return {6, 6, 6};
     case 256: return {8, 8, 4};
-    case 288: return {8, 6, 6};
-    case 384: return {8, 8, 6};
+    case 288: return {6, 6, 8};
+    case 384: return {6, 8, 8};
     case 512: return {8, 8, 8};
     default: return {0, 0, 0};
   }
 }
 
-// Forward transform, a multiplier at each k, and the inverse transform (unnormalised) of one line held
-// by TPL = M / R1 threads: thread t enters with v[n1] = z[n1 (M / R1) + t] and leaves with the same
-// elements of the result.  n = n1 R2 R3 + n2 R3 + n3, k = k1 + R1 k2 + R1 R2 k3; every pass writes the
-// slots it read, so one barrier stands between two passes.  s: the line's M slots (slot p at
-// s[map(p)]); tw[e] = digits of exp(-2 pi i e / M); ph(k, X): the multiplier.  Every thread of the CTA
-// calls it; all of the CTA's lines are done together.
-template <int M, class MAP, class PH>
-WF_D void fx_convolve(fxc (&v)[fx_plan(M).r1], fxc* s, const MAP& map, int t, const int4* tw, const PH& ph) {
-  constexpr int R1 = fx_plan(M).r1, R2 = fx_plan(M).r2, R3 = fx_plan(M).r3, N1 = M / R1;
-  static_assert(R1 * R2 * R3 == M, "plan");
-  fx_dft<R1, -1>(v);
-  s[map(t)] = v[0];
-#pragma unroll
-  for (int k1 = 1; k1 < R1; ++k1) s[map(k1 * N1 + t)] = fx_twid<-1>(v[k1], tw[t * k1]);
-  __syncthreads();
-  if constexpr (R3 > 1) {
-    for (int j = t; j < M / R2; j += N1) {
-      const int k1 = j / R3, n3 = j % R3, base = k1 * R2 * R3 + n3;
-      fxc a[R2];
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) a[n2] = s[map(base + n2 * R3)];
-      fx_dft<R2, -1>(a);
-      s[map(base)] = a[0];
-#pragma unroll
-      for (int k2 = 1; k2 < R2; ++k2) s[map(base + k2 * R3)] = fx_twid<-1>(a[k2], tw[R1 * n3 * k2]);
-    }
-    __syncthreads();
-    for (int j = t; j < M / R3; j += N1) {
-      const int k1 = j / R2, k2 = j % R2, base = j * R3;
-      fxc a[R3];
-#pragma unroll
-      for (int n3 = 0; n3 < R3; ++n3) a[n3] = s[map(base + n3)];
-      fx_dft<R3, -1>(a);
-#pragma unroll
-      for (int k3 = 0; k3 < R3; ++k3) a[k3] = ph(k1 + R1 * k2 + R1 * R2 * k3, a[k3]);
-      fx_dft<R3, +1>(a);
-      s[map(base)] = a[0];
-#pragma unroll
-      for (int n3 = 1; n3 < R3; ++n3) s[map(base + n3)] = fx_twid<+1>(a[n3], tw[R1 * n3 * k2]);
-    }
-    __syncthreads();
-    for (int j = t; j < M / R2; j += N1) {
-      const int k1 = j / R3, n3 = j % R3, base = k1 * R2 * R3 + n3;
-      fxc a[R2];
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) a[k2] = s[map(base + k2 * R3)];
-      fx_dft<R2, +1>(a);
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) s[map(base + n2 * R3)] = fx_twid<+1>(a[n2], tw[(n2 * R3 + n3) * k1]);
-    }
-  } else {
-    for (int j = t; j < R1; j += N1) {  // j = k1
-      fxc a[R2];
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) a[n2] = s[map(j * R2 + n2)];
-      fx_dft<R2, -1>(a);
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) a[k2] = ph(j + R1 * k2, a[k2]);
-      fx_dft<R2, +1>(a);
-      s[map(j * R2)] = a[0];
-#pragma unroll
-      for (int n2 = 1; n2 < R2; ++n2) s[map(j * R2 + n2)] = fx_twid<+1>(a[n2], tw[n2 * j]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k1 = 0; k1 < R1; ++k1) v[k1] = s[map(k1 * N1 + t)];
-  fx_dft<R1, +1>(v);
-}
+// the operations of the line engine (wf_line.cuh) on fixed-point values
+template <int DIR> WF_D fxc ln_mul_i(fxc a) { return fx_mul_i<DIR>(a); }
+template <int DIR> WF_D fxc ln_twid(fxc a, int4 w) { return fx_twid<DIR>(a, w); }
+WF_D fxc ln_r2(fxc a) { return fxc{fx_mulq(a.x, kFxR2h, kFxR2l), fx_mulq(a.y, kFxR2h, kFxR2l)}; }
+WF_D fxc ln_s3(fxc a) { return fxc{fx_mulq(a.x, kFxS3h, kFxS3l), fx_mulq(a.y, kFxS3h, kFxS3l)}; }
+WF_D fxc ln_half(fxc a) { return fxc{(a.x + 1) >> 1, (a.y + 1) >> 1}; }
+template <int DIR> WF_D fxc ln_rot9(fxc a, int m) { return fx_twid<DIR>(a, fx_w9(m)); }
 
-// The forward half alone, in either direction (DIR = +1: conjugate twiddles): enters like fx_convolve
-// and hands every Z_k the thread ends with to out(k, Z_k, i), i = 0, 1, ... its number in the thread.  TWS: W_M^e = tw[TWS e].
-template <int M, int DIR, int TWS = 1, class MAP, class OUT>
-WF_D void fx_forward(fxc (&v)[fx_plan(M).r1], fxc* s, const MAP& map, int t, const int4* tw, const OUT& out) {
-  constexpr int R1 = fx_plan(M).r1, R2 = fx_plan(M).r2, R3 = fx_plan(M).r3, N1 = M / R1;
-  fx_dft<R1, DIR>(v);
-  s[map(t)] = v[0];
-#pragma unroll
-  for (int k1 = 1; k1 < R1; ++k1) s[map(k1 * N1 + t)] = fx_twid<DIR>(v[k1], tw[TWS * t * k1]);
-  __syncthreads();
-  if constexpr (R3 > 1) {
-    for (int j = t; j < M / R2; j += N1) {
-      const int k1 = j / R3, n3 = j % R3, base = k1 * R2 * R3 + n3;
-      fxc a[R2];
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) a[n2] = s[map(base + n2 * R3)];
-      fx_dft<R2, DIR>(a);
-      s[map(base)] = a[0];
-#pragma unroll
-      for (int k2 = 1; k2 < R2; ++k2) s[map(base + k2 * R3)] = fx_twid<DIR>(a[k2], tw[TWS * R1 * n3 * k2]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < (M / R3 + N1 - 1) / N1; ++m) {
-      const int j = t + m * N1;
-      if ((M / R3) % N1 == 0 || j < M / R3) {
-        fxc a[R3];
-#pragma unroll
-        for (int n3 = 0; n3 < R3; ++n3) a[n3] = s[map(j * R3 + n3)];
-        fx_dft<R3, DIR>(a);
-#pragma unroll
-        for (int k3 = 0; k3 < R3; ++k3) out(j / R2 + R1 * (j % R2) + R1 * R2 * k3, a[k3], m * R3 + k3);
-      }
-    }
-  } else {
-#pragma unroll
-    for (int m = 0; m < (R1 + N1 - 1) / N1; ++m) {
-      const int j = t + m * N1;
-      if (R1 % N1 == 0 || j < R1) {
-        fxc a[R2];
-#pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) a[n2] = s[map(j * R2 + n2)];
-        fx_dft<R2, DIR>(a);
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) out(j + R1 * k2, a[k2], m * R2 + k2);
-      }
-    }
-  }
-}
-
-// The same with the result left in the line's slots in natural order (a barrier after it).
-template <int M, int DIR, int TWS, class MAP>
-WF_D void fx_forward_nat(fxc (&v)[fx_plan(M).r1], fxc* s, const MAP& map, int t, const int4* tw) {
-  constexpr int R1 = fx_plan(M).r1, R2 = fx_plan(M).r2, R3 = fx_plan(M).r3, N1 = M / R1;
-  constexpr int RL = R3 > 1 ? R3 : R2, NB = M / RL, PER = (NB + N1 - 1) / N1;
-  fxc res[PER * RL];
-  fx_forward<M, DIR, TWS>(v, s, map, t, tw, [&](int, fxc X, int i) { res[i] = X; });
-  __syncthreads();
-#pragma unroll
-  for (int m = 0; m < PER; ++m) {
-    const int j = t + m * N1;
-    if (NB % N1 == 0 || j < NB)
-#pragma unroll
-      for (int r = 0; r < RL; ++r) s[map(R3 > 1 ? j / R2 + R1 * (j % R2) + R1 * R2 * r : j + R1 * r)] = res[m * RL + r];
-  }
-  __syncthreads();
-}
-
-// The mirror image: takes Z_k from in(k) (which may read the line's own slots: a barrier stands before
-// the first write) and leaves v[n1] = z[n1 (M / R1) + t], z_n = sum_k Z_k exp(DIR 2 pi i k n / M).
-template <int M, int DIR, int TWS = 1, class MAP, class IN>
-WF_D void fx_inverse(fxc (&v)[fx_plan(M).r1], fxc* s, const MAP& map, int t, const int4* tw, const IN& in) {
-  constexpr int R1 = fx_plan(M).r1, R2 = fx_plan(M).r2, R3 = fx_plan(M).r3, N1 = M / R1;
-  constexpr int RL = R3 > 1 ? R3 : R2, NB = M / RL, PER = (NB + N1 - 1) / N1;
-  fxc a[PER][RL];
-#pragma unroll
-  for (int m = 0; m < PER; ++m) {
-    const int j = t + m * N1;
-    if (NB % N1 == 0 || j < NB)
-#pragma unroll
-      for (int r = 0; r < RL; ++r)
-        a[m][r] = R3 > 1 ? in(j / R2 + R1 * (j % R2) + R1 * R2 * r) : in(j + R1 * r);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int m = 0; m < PER; ++m) {
-    const int j = t + m * N1;
-    if (NB % N1 == 0 || j < NB) {
-      fx_dft<RL, DIR>(a[m]);
-      const int e = R3 > 1 ? R1 * (j % R2) : j;  // twiddle step of output r
-      s[map(j * RL)] = a[m][0];
-#pragma unroll
-      for (int r = 1; r < RL; ++r) s[map(j * RL + r)] = fx_twid<DIR>(a[m][r], tw[TWS * r * e]);
-    }
-  }
-  __syncthreads();
-  if constexpr (R3 > 1) {
-    for (int j = t; j < M / R2; j += N1) {
-      const int k1 = j / R3, n3 = j % R3, base = k1 * R2 * R3 + n3;
-      fxc b[R2];
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) b[k2] = s[map(base + k2 * R3)];
-      fx_dft<R2, DIR>(b);
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) s[map(base + n2 * R3)] = fx_twid<DIR>(b[n2], tw[TWS * (n2 * R3 + n3) * k1]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int k1 = 0; k1 < R1; ++k1) v[k1] = s[map(k1 * N1 + t)];
-  fx_dft<R1, DIR>(v);
-}
+// radix plan of a fixed-point line: butterflies of at most 12 points
+template <int M> struct FxPlan {
+  static constexpr int r1 = fx_plan(M).r1, r2 = fx_plan(M).r2, r3 = fx_plan(M).r3;
+};
 
 // ---- scaling -----------------------------------------------------------------------------------
 WF_D int fx_exp(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
@@ -455,16 +189,6 @@ constexpr int fx_floor_log2(int n) { return n < 2 ? 0 : 1 + fx_floor_log2(n / 2)
 // the shift between a forward transform and the inverse that follows: ceil(log2(n) / 2), since the inverse's
 // partial sums are below n ||z||_2, sqrt(n) times the forward's
 constexpr int fx_mid(int n) { return (fx_floor_log2(n - 1) + 2) / 2; }
-
-// slots of a tile of NL lines side by side; slots of one line with a pad per 8 (strided passes of
-// neighbouring threads then fall on different banks)
-template <int NL> struct ColMap {
-  WF_D int operator()(int p) const { return p * NL; }
-};
-struct PadMap {
-  WF_D int operator()(int p) const { return p + (p >> 3); }
-};
-constexpr int fx_padded(int m) { return m + m / 8; }
 
 // twiddles exp(-2 pi i e / N), e < N, of the table exp(-2 pi i e / 2N) in shared memory
 template <int N> WF_D void fx_load_tw(int4* tw, const int4* __restrict__ tab, int tid, int nt) {

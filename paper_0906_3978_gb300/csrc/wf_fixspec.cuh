@@ -18,7 +18,8 @@ namespace wf {
 template <int N> struct FxC {
   static constexpr int NH = N / 2;
   static constexpr int R1 = fx_plan(N).r1, N1 = N / R1;
-  static constexpr int NL = div_le(NH, N >= 256 ? 4 : 8);
+  // up to 256 threads, but at small sizes eight columns, so that N (N/2) / NL CTAs cover the chip
+  static constexpr int NL = div_le(NH, N >= 96 ? 256 / N1 : 8);
   static constexpr int NT = NL * N1;
   static constexpr int KB = NH / NL;  // column blocks per plane
   static constexpr size_t SMEM = (size_t)(N * NL + N) * 16;
@@ -52,7 +53,7 @@ k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, const CgScal
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
-  fx_forward<N, DIR>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) { p[(size_t)k * NH] = fx_to2(X, f); });
+  ln_forward<N, FxPlan<N>, DIR>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) { p[(size_t)k * NH] = fx_to2(X, f); });
 }
 
 // ---- Fourier tables as Q62 digits ----------------------------------------------------------------
@@ -122,18 +123,18 @@ k_fx_xmul(const double2* __restrict__ in, double2* __restrict__ out, const int2*
   const int sh = -(H2 + exps[z * estride]);
   if (!pair) {
     const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
-    fx_convolve<N>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X) {
+    ln_convolve<N, FxPlan<N>>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X) {
       const int kxs = sfreq(k, N);
       return fx_scaleq(fxc{fx_rshift(X.x, H2), fx_rshift(X.y, H2)}, __ldg(tab + kxs * kxs + k0));
     });
     if (kz == 0) return;  // the packed column's pair CTA writes it
   } else {
     fxc* nat = reinterpret_cast<fxc*>(tw + N);  // both lines' spectra in natural order
-    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+    ln_forward<N, FxPlan<N>, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
       if (l < 2) nat[l * N + k] = fxc{fx_rshift(X.x, H2), fx_rshift(X.y, H2)};
     });
     __syncthreads();
-    fx_inverse<N, +1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k) {
+    ln_inverse<N, FxPlan<N>, +1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k) {
       if (l >= 2) return fxc{0, 0};
       const int kxs = sfreq(k, N), n2 = kxs * kxs + ky_s * ky_s;
       const int2 m0 = __ldg(tab + n2), mN = __ldg(tab + n2 + NH * NH);
@@ -195,7 +196,7 @@ k_fx_xfwd(const double2* __restrict__ in, double2* __restrict__ out, const doubl
   AccD acc;
   if (!pair) {
     const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
-    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+    ln_forward<N, FxPlan<N>, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
       if (kz == 0) return;
       const int kxs = sfreq(k, N);
       const double m = __ldg(tab + kxs * kxs + k0);
@@ -206,7 +207,7 @@ k_fx_xfwd(const double2* __restrict__ in, double2* __restrict__ out, const doubl
     });
   } else {
     fxc* nat = reinterpret_cast<fxc*>(tw + N);
-    fx_forward<N, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+    ln_forward<N, FxPlan<N>, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
       if (l < 2) nat[l * N + k] = X;
     });
     __syncthreads();
@@ -268,7 +269,7 @@ k_fx_xinv(const double2* __restrict__ in, double2* __restrict__ out, const doubl
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
-  fx_forward<N, +1>(v, slots + l, ColMap<NL>{}, t, tw,
+  ln_forward<N, FxPlan<N>, +1>(v, slots + l, ColMap<NL>{}, t, tw,
                     [&](int k, fxc X, int) { out[base + (size_t)k * rowstride] = fx_to2(X, f); });
 }
 
@@ -277,7 +278,7 @@ template <int N> struct FxZ {
   static constexpr int H = N / 2, R1 = fx_plan(H).r1, N1 = H / R1;
   static constexpr int NL = div_le(N * N, 256 / N1);  // rows per CTA
   static constexpr int NT = NL * N1;
-  static constexpr int LS = fx_padded(H);
+  static constexpr int LS = ln_padded(H, 3, N1, 8);
   static constexpr int GZ = N * N / NL;  // CTAs per system
   static constexpr size_t SMEM = (size_t)(NL * LS + N) * 16;
 };
@@ -347,7 +348,7 @@ k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* 
     const double q = block_sum(acc.get(), red);
     if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = q;
   }
-  fx_forward_nat<H, -1, 2>(v, s, PadMap{}, t, tw);
+  ln_forward_nat<H, FxPlan<H>, -1, 2>(v, s, PadMap{}, t, tw);
   double2* dst = out + z * bt.spec + row * H;
   for (int k = t; k < H; k += N1) dst[k] = fx_to2(fx_r2c<N>(s, PadMap{}, k, tw), f);
 }
@@ -388,7 +389,7 @@ k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double
   for (int r = 0; r < R1; ++r) sl[PadMap{}(r * N1 + t)] = fx_from2(raw[r], f);
   __syncthreads();
   fxc v[R1];
-  fx_inverse<H, +1, 2>(v, sl, PadMap{}, t, tw, [&](int k) { return fx_c2r<N>(sl, PadMap{}, k, tw); });
+  ln_inverse<H, FxPlan<H>, +1, 2>(v, sl, PadMap{}, t, tw, [&](int k) { return fx_c2r<N>(sl, PadMap{}, k, tw); });
   AccD acc;
   const size_t e0 = z * (bt.real / 2) + row * H;
 #pragma unroll
@@ -413,6 +414,298 @@ k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double
     const double sum = block_sum(acc.get(), red);
     if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = sum;
   }
+}
+
+// ==========================================================================================
+// The FP64 CG passes (the work of k_cg_xinv, k_cg_xupd and k_zturn): vector updates and sums in FP64,
+// transforms in fixed point.  UNIT_M (every system preconditioned): m = 1 but at k = 0, where it is 0,
+// and the m table holds 1 / c^2 instead, which the residual estimate would otherwise divide for.  108^3 per
+// launch (events, with ~5 us of bracketing), FP64 butterflies -> here: x pass 1 58.8 -> 43 us, x pass 2 87 -> 43,
+// z turn 103 -> 37, y pass 43 -> 16; the FP64 pipe's updates and conversions (about 55 per complex element and
+// iteration) and the loads' latency at this size share the rest.  Each round's operands are requested
+// before they are needed: with the loads between the stores, x pass 1 took 65 us.
+// ==========================================================================================
+template <bool UNIT_M> WF_D double cg_m(const double* mtab, int n2) {
+  return UNIT_M ? (n2 == 0 ? 0.0 : 1.0) : __ldg(mtab + n2);
+}
+template <bool UNIT_M> WF_D double cg_ic2(const double* mtab, int n2, double c) {
+  return UNIT_M ? __ldg(mtab + n2) : 1.0 / (c * c);
+}
+
+// x pass 1: p_new = r + beta p_old;  x += alpha_prev p_old;  T = IFFT_x(c (.) p_new);  partial of <p_new, m p_new>.
+// The packed column takes its partner element from -ky in registers.  grid (N/2 / NL, N, systems)
+template <int N, bool UNIT_M>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_cg_xinv(const double2* __restrict__ r, double2* P0, double2* P1, double2* __restrict__ x, double2* __restrict__ T,
+             const double* __restrict__ ctab, const double* __restrict__ mtab, const int4* __restrict__ twtab,
+             double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  sc += z;
+  if (sc->done) return;
+  const double2* __restrict__ pold = ((sc->lit & 1) ? P1 : P0) + z * bt.spec;
+  double2* __restrict__ pnew = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;
+  r += z * bt.spec;
+  x += z * bt.spec;
+  T += z * bt.spec;
+  ctab += z * bt.tab;
+  mtab += z * bt.tab;
+  const double beta = sc->beta, alpha = sc->alpha_prev;
+  const int ky = blockIdx.y, ky_s = sfreq(ky, N), kz = blockIdx.x * NL + l;
+  const size_t rowstride = (size_t)N * NH, base = (size_t)ky * NH + kz;
+  double2 raw[R1];
+  double acc = 0.0;  // half of the sum: the columns kz != 0 weigh 2
+  constexpr int CH = R1 % 4 == 0 ? 4 : 3;  // elements whose loads are in flight together
+  static_assert(R1 % CH == 0, "chunks");
+#pragma unroll
+  for (int q0 = 0; q0 < R1; q0 += CH) {
+    double2 rv[CH], po[CH], xv[CH];
+    double cv[CH];
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      const int kx = (q0 + j) * N1 + t, kxs = sfreq(kx, N);
+      const size_t e = base + (size_t)kx * rowstride;
+      rv[j] = __ldg(r + e);
+      po[j] = __ldg(pold + e);
+      xv[j] = x[e];
+      cv[j] = __ldg(ctab + kxs * kxs + ky_s * ky_s + kz * kz);
+    }
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      const int kx = (q0 + j) * N1 + t;
+      const size_t e = base + (size_t)kx * rowstride;
+      const double2 p = make_double2(rv[j].x + beta * po[j].x, rv[j].y + beta * po[j].y);
+      pnew[e] = p;
+      x[e] = make_double2(xv[j].x + alpha * po[j].x, xv[j].y + alpha * po[j].y);
+      if (kz != 0) {
+        if (UNIT_M) {
+          acc = fma(p.x, p.x, fma(p.y, p.y, acc));
+        } else {
+          const int kxs = sfreq(kx, N);
+          acc = fma(__ldg(mtab + kxs * kxs + ky_s * ky_s + kz * kz), p.x * p.x + p.y * p.y, acc);
+        }
+        raw[q0 + j] = make_double2(cv[j] * p.x, cv[j] * p.y);
+      } else {
+        raw[q0 + j] = p;  // raw for the pair below
+      }
+    }
+  }
+  if (kz == 0) {  // packed column: c and m act on the planes P0 = (Z + conj Z(-k)) / 2, PN = (Z - conj Z(-k)) / 2i
+#pragma unroll
+    for (int q0 = 0; q0 < R1; q0 += CH) {
+      double2 rq[CH], pq[CH];
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        const int kx = (q0 + j) * N1 + t;
+        const size_t eq = (size_t)((N - ky) % N) * NH + (size_t)((N - kx) % N) * rowstride;
+        rq[j] = __ldg(r + eq);
+        pq[j] = __ldg(pold + eq);
+      }
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        const int kxs = sfreq((q0 + j) * N1 + t, N), n2 = kxs * kxs + ky_s * ky_s;
+        const double2 p = raw[q0 + j];
+        const double qx = rq[j].x + beta * pq[j].x, qy = rq[j].y + beta * pq[j].y;
+        const double a0 = 0.5 * (p.x + qx), b0 = 0.5 * (p.y - qy), aN = 0.5 * (p.y + qy), bN = 0.5 * (qx - p.x);
+        acc += 0.5 * (cg_m<UNIT_M>(mtab, n2) * (a0 * a0 + b0 * b0) + cg_m<UNIT_M>(mtab, n2 + NH * NH) * (aN * aN + bN * bN));
+        const double c = __ldg(ctab + n2), cN = __ldg(ctab + n2 + NH * NH), a = 0.5 * (c + cN), b = 0.5 * (c - cN);
+        raw[q0 + j] = make_double2(a * p.x + b * qx, a * p.y - b * qy);
+      }
+    }
+  }
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  fxc v[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q) v[q] = fx_from2(raw[q], f);
+  ln_forward<N, FxPlan<N>, +1>(v, slots + l, ColMap<NL>{}, t, tw,
+                    [&](int k, fxc X, int) { T[base + (size_t)k * rowstride] = fx_to2(X, f); });
+  const double sum = block_sum(2.0 * acc, red);
+  if (tid == 0) partials[(size_t)z * bt.part + blockIdx.y * gridDim.x + blockIdx.x] = sum;
+}
+
+// x pass 2:  T^ = FFT_x(T);  q = m p + c T^;  r -= alpha q;  partials of <r, r> and an upper estimate of
+// V_c ||C^-1 r||^2 (two per CTA).  CTAs as in k_fx_xmul.
+template <int N, bool UNIT_M>
+__global__ void __launch_bounds__(FxC<N>::NT)
+k_fx_cg_xupd(const double2* __restrict__ T, double2* __restrict__ r, const double2* P0, const double2* P1,
+             const double* __restrict__ ctab, const double* __restrict__ mtab, const int4* __restrict__ twtab,
+             double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxC<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + N * NL);
+  __shared__ int se[NL];
+  __shared__ unsigned sq[NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  sc += z;
+  if (sc->done) return;
+  const bool pair = blockIdx.x == G::KB;
+  const int ky = blockIdx.y;
+  partials += (size_t)z * bt.part + 2 * (size_t)(blockIdx.y * gridDim.x + blockIdx.x);
+  if (pair && ky > N / 2) {
+    if (tid < 2) partials[tid] = 0.0;
+    return;
+  }
+  const double2* __restrict__ p = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;  // this iteration's p_new
+  T += z * bt.spec;
+  r += z * bt.spec;
+  ctab += z * bt.tab;
+  mtab += z * bt.tab;
+  const double alpha = sc->alpha;
+  const int ky_s = sfreq(ky, N);
+  const size_t rowstride = (size_t)N * NH;
+  const int row_y = pair && l == 1 ? (N - ky) % N : ky;
+  const bool live = !pair || l < 2;
+  const size_t base = (size_t)row_y * NH + (pair ? 0 : blockIdx.x * NL + l);
+  double2 raw[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q)
+    raw[q] = live ? __ldg(T + base + (size_t)(q * N1 + t) * rowstride) : make_double2(0.0, 0.0);
+  if (tid < NL) {
+    se[tid] = kFxMinExp;
+    sq[tid] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const int ls = pair && l < 2 ? 0 : l;
+  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  fxc v[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q) v[q] = fx_from2(raw[q], f);
+  double rr = 0.0, rc = 0.0;
+  if (!pair) {
+    const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
+    // r and p of a round's results are requested before its butterfly
+    constexpr int RL = FxPlan<N>::r3 > 1 ? FxPlan<N>::r3 : FxPlan<N>::r2;
+    double2 rpre[RL], ppre[RL];
+    auto request = [&](int m) {
+#pragma unroll
+      for (int i = 0; i < RL; ++i) {
+        const size_t e = base + (size_t)ln_index<N, FxPlan<N>>(t, m * RL + i) * rowstride;
+        rpre[i] = r[e];
+        ppre[i] = __ldg(p + e);
+      }
+    };
+    ln_forward<N, FxPlan<N>, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int i) {
+      if (kz == 0) return;
+      const int kxs = sfreq(k, N), n2 = kxs * kxs + k0;
+      const size_t e = base + (size_t)k * rowstride;
+      double2 rv = rpre[i % RL];
+      const double2 pv = ppre[i % RL], tv = fx_to2(X, f);
+      const double c = __ldg(ctab + n2);
+      double2 q;
+      if (UNIT_M) {
+        q = make_double2(fma(c, tv.x, pv.x), fma(c, tv.y, pv.y));
+      } else {
+        const double m = __ldg(mtab + n2);
+        q = make_double2(m * pv.x + c * tv.x, m * pv.y + c * tv.y);
+      }
+      rv.x -= alpha * q.x;
+      rv.y -= alpha * q.y;
+      r[e] = rv;
+      const double m2 = rv.x * rv.x + rv.y * rv.y;
+      rr += m2;
+      rc = fma(cg_ic2<UNIT_M>(mtab, n2, c), m2, rc);
+    }, request);
+    rr *= 2.0;
+    rc *= 2.0;
+  } else {
+    fxc* nat = reinterpret_cast<fxc*>(tw + N);  // both lines' T^ in natural order
+    ln_forward<N, FxPlan<N>, -1>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) {
+      if (l < 2) nat[l * N + k] = X;
+    });
+    __syncthreads();
+    if (l < 2 && !(l == 1 && row_y == ky))
+      for (int k = t; k < N; k += N1) {
+        const int kxs = sfreq(k, N), n2 = kxs * kxs + ky_s * ky_s;
+        const size_t e = base + (size_t)k * rowstride;
+        const double c0 = __ldg(ctab + n2), cN = __ldg(ctab + n2 + NH * NH);
+        const double m0 = cg_m<UNIT_M>(mtab, n2), mN = cg_m<UNIT_M>(mtab, n2 + NH * NH);
+        const double ca = 0.5 * (c0 + cN), cb = 0.5 * (c0 - cN), ma = 0.5 * (m0 + mN), mb = 0.5 * (m0 - mN);
+        const double2 zc = fx_to2(nat[l * N + k], f), zp = fx_to2(nat[(1 - l) * N + (N - k) % N], f);
+        const double2 pv = __ldg(p + e);
+        double2 pp = make_double2(0.0, 0.0);
+        if (mb != 0.0) pp = __ldg(p + (size_t)((N - row_y) % N) * NH + (size_t)((N - k) % N) * rowstride);
+        double2 rv = r[e];
+        rv.x -= alpha * (ma * pv.x + mb * pp.x + (ca * zc.x + cb * zp.x));
+        rv.y -= alpha * (ma * pv.y - mb * pp.y + (ca * zc.y - cb * zp.y));
+        r[e] = rv;
+        const double m2 = rv.x * rv.x + rv.y * rv.y;
+        rr += m2;
+        rc = fma(fmax(cg_ic2<UNIT_M>(mtab, n2, c0), cg_ic2<UNIT_M>(mtab, n2 + NH * NH, cN)), m2, rc);
+      }
+  }
+  const double s1 = block_sum(rr, red);
+  const double s2 = block_sum(rc, red);
+  if (tid == 0) {
+    partials[0] = s1;
+    partials[1] = s2;
+  }
+}
+
+// z turn: each (x, y) line packed -> real, times D, -> packed; partial of D T^2.  grid (GZ, 1, systems)
+template <int N>
+__global__ void __launch_bounds__(FxZ<N>::NT)
+k_fx_zturn(double2* __restrict__ spec, const double* __restrict__ D, const int4* __restrict__ twtab,
+           double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+  using G = FxZ<N>;
+  constexpr int R1 = G::R1, N1 = G::N1, H = G::H;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fxc* slots = reinterpret_cast<fxc*>(smem_raw);
+  int4* tw = reinterpret_cast<int4*>(slots + G::NL * G::LS);
+  __shared__ int se[2 * G::NL];
+  __shared__ unsigned sq[2 * G::NL];
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
+  if (sc && sc[z].done) return;
+  const size_t row = (size_t)blockIdx.x * G::NL + l;
+  double2* line = spec + z * bt.spec + row * H;
+  double2 raw[R1];
+#pragma unroll
+  for (int r = 0; r < R1; ++r) raw[r] = line[r * N1 + t];
+  for (int i = tid; i < 2 * G::NL; i += G::NT) {
+    se[i] = kFxMinExp;
+    sq[i] = 0;
+  }
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  __syncthreads();
+  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], fx_c2r_count<N>());
+  fxc* sl = slots + l * G::LS;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) sl[PadMap{}(r * N1 + t)] = fx_from2(raw[r], f);
+  __syncthreads();
+  fxc v[R1];
+  ln_inverse<H, FxPlan<H>, +1, 2>(v, sl, PadMap{}, t, tw, [&](int k) { return fx_c2r<N>(sl, PadMap{}, k, tw); });
+  const double2* d = reinterpret_cast<const double2*>(D + z * bt.real) + row * H;
+  double acc = 0.0;
+#pragma unroll
+  for (int r = 0; r < R1; ++r) {
+    const double2 dv = __ldg(d + r * N1 + t), T = fx_to2(v[r], f);
+    raw[r] = make_double2(T.x * dv.x, T.y * dv.y);
+    acc = fma(raw[r].x, T.x, fma(raw[r].y, T.y, acc));
+  }
+  const FxScale g = fx_line_scale(raw, &se[G::NL + l], &sq[G::NL + l], H);
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], g);
+  ln_forward_nat<H, FxPlan<H>, -1, 2>(v, sl, PadMap{}, t, tw);
+  for (int k = t; k < H; k += N1) line[k] = fx_to2(fx_r2c<N>(sl, PadMap{}, k, tw), g);
+  const double sum = block_sum(acc, red);
+  if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = sum;
 }
 
 }  // namespace wf

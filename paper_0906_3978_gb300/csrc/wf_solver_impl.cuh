@@ -68,7 +68,7 @@ struct Spec {
   using FC = FxC<N>;
   using FZ = FxZ<N>;
   static constexpr int GXF = F64 ? (FC::KB + 1) * N : GXY;  // partial sums of the CG start's x pass
-  static constexpr int GZI = F64 ? FZ::GZ : GZ;             // partial sums of the z inverse (residual)
+  static constexpr int GZI = F64 ? FZ::GZ : GZ;             // partial sums of the z turn and the z inverse
   static constexpr size_t SPEC = (size_t)N * N * NH;  // complex elements of a spectrum
   static constexpr size_t V = (size_t)N * N * N;
   static constexpr int TAB = 3 * (N / 2) * (N / 2) + 1;
@@ -98,10 +98,6 @@ struct Spec {
     if (done) return cudaSuccess;
     cudaError_t e = cudaSuccess;
 #define WF_A(k, b) if (e == cudaSuccess) e = set_smem(k, b)
-    WF_A((k_cg_xinv<R, N, true>), SMxy);
-    WF_A((k_cg_xinv<R, N, false>), SMxy);
-    WF_A((k_cg_xupd<R, N, true>), SMxy);
-    WF_A((k_cg_xupd<R, N, false>), SMxy);
     if constexpr (F64) {
       WF_A((k_fx_xmul<N>), fx_xmul_smem<N>());
       WF_A((k_fx_xfwd<N>), fx_xmul_smem<N>());
@@ -115,7 +111,6 @@ struct Spec {
       WF_A((k_zfwd<R, N, false>), SMz);
       WF_A((k_zinv<R, N, ZI_ACCUM>), SMz);
     }
-    WF_A((k_zturn<R, N>), SMz);
     if constexpr (std::is_same<R, float>::value) {
       WF_A((k_zcoarse<R, N>), SMz);
       WF_A((k_xcr<R, N, 32>), SMxy);
@@ -331,6 +326,43 @@ struct Spec {
       return (N / 2 / NL) * N;
     }
   };
+  // the FP64 CG x passes (fixed point)
+  struct XFix {
+    static cudaError_t setup() {
+      cudaError_t e = set_smem(k_fx_cg_xinv<N, true>, FC::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_fx_cg_xinv<N, false>, FC::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_fx_cg_xupd<N, true>, fx_xmul_smem<N>());
+      if (e == cudaSuccess) e = set_smem(k_fx_cg_xupd<N, false>, fx_xmul_smem<N>());
+      return e;
+    }
+    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* ctab, const SS* mtab, bool unit_m,
+                    const ST*, double* part, CgScal* sc, cudaStream_t st) {
+      if constexpr (F64) {
+        const dim3 grid(FC::KB, N, nb);
+        c.launch("cg_xinv_f64", 6 * BS * nb, st, [&] {
+          if (unit_m)
+            k_fx_cg_xinv<N, true><<<grid, FC::NT, FC::SMEM, st>>>(r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
+          else
+            k_fx_cg_xinv<N, false><<<grid, FC::NT, FC::SMEM, st>>>(r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
+        });
+      }
+      return FC::KB * N;
+    }
+    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
+                    const ST*, double* part, CgScal* sc, cudaStream_t st) {
+      if constexpr (F64) {
+        const dim3 grid(FC::KB + 1, N, nb);
+        const size_t sm = fx_xmul_smem<N>();
+        c.launch("cg_xupd_f64", 4 * BS * nb, st, [&] {
+          if (unit_m)
+            k_fx_cg_xupd<N, true><<<grid, FC::NT, sm, st>>>(T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
+          else
+            k_fx_cg_xupd<N, false><<<grid, FC::NT, sm, st>>>(T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
+        });
+      }
+      return (FC::KB + 1) * N;
+    }
+  };
   static constexpr int NLX = xtma_lines<R, N, 3, 2>();
   static const std::vector<XVariant>& xvariants() {
     static const std::vector<XVariant> v = [] {
@@ -338,7 +370,9 @@ struct Spec {
       // 0.58 ms against 1.23-1.83 ms for the staged forms, whose single resident CTA per SM
       // serialises each tile's table gathers, transform and epilogue); the staged forms stay
       // candidates for the tuner on the FP32 grids of 128 and up
-      std::vector<XVariant> out{{"registers", XReg<8>::setup, XReg<8>::xinv, XReg<8>::xupd}};
+      std::vector<XVariant> out;
+      if constexpr (F64) out.push_back({"fixed", XFix::setup, XFix::xinv, XFix::xupd});
+      else out.push_back({"registers", XReg<8>::setup, XReg<8>::xinv, XReg<8>::xupd});
       if constexpr (std::is_same<R, float>::value && N >= 128) {
         out.push_back({"registers_r16", XReg<16>::setup, XReg<16>::xinv, XReg<16>::xupd});
         out.push_back({"registers_r32", XReg<32>::setup, XReg<32>::xinv, XReg<32>::xupd});
@@ -377,10 +411,20 @@ struct Spec {
       });
     }
   };
+  struct ZFix {  // FP64 (fixed point)
+    static cudaError_t setup() { return set_smem(k_fx_zturn<N>, FZ::SMEM); }
+    static void run(Ctx& c, int nb, ST* T, const SS* D, const ST*, double* part, const CgScal* sc, cudaStream_t st) {
+      if constexpr (F64)
+        c.launch("zturn_f64", (2 * BS + sizeof(SS) * BV) * nb, st,
+                 [&] { k_fx_zturn<N><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(T, D, c.fixed(N), part, sc, bat()); });
+    }
+  };
   static const std::vector<ZVariant>& zvariants() {
     static const std::vector<ZVariant> v = [] {
       constexpr int E0 = z_elems<R, N>();
-      std::vector<ZVariant> out{{"e_default", ZV<E0>::setup, ZV<E0>::run}};
+      std::vector<ZVariant> out;
+      if constexpr (F64) out.push_back({"fixed", ZFix::setup, ZFix::run});
+      else out.push_back({"e_default", ZV<E0>::setup, ZV<E0>::run});
       if constexpr (std::is_same<R, float>::value && N >= 128) {
         if constexpr (E0 / 2 >= 4 && (N / 2) % (E0 / 2) == 0) out.push_back({"e/2", ZV<E0 / 2>::setup, ZV<E0 / 2>::run});
         if constexpr (E0 / 4 >= 4 && (N / 2) % (E0 / 4) == 0) out.push_back({"e/4", ZV<E0 / 4>::setup, ZV<E0 / 4>::run});
@@ -459,7 +503,7 @@ struct Spec {
     const int n1 = pick(c, "xinv", xvariants())
                        .xinv(c, nb, rin ? rin : r, P0, P1, x, T, ctab, mtab, unit_m, tw, part, sc, st);
     after_xinv(st);
-    int nmid = GZ;  // blocks that sum the data term of <p, A p> into part[NX ...]
+    int nmid = GZI;  // blocks that sum the data term of <p, A p> into part[NX ...]
     bool fused = false;
     if constexpr (PCS > 0) {
       if (c.fused_planes) {
@@ -734,6 +778,8 @@ struct GroupFP64 : GroupCommon<N> {
       make_tables(sys[m]->sinv, pre, c0, vc.data() + (size_t)m * TAB, vm.data() + (size_t)m * TAB);
       std::copy(sys[m]->sinv.begin(), sys[m]->sinv.end(), vs.begin() + (size_t)m * TAB);
     }
+    if (unit_m)  // the FP64 CG passes take 1 / c^2 from the m table, whose values they know
+      for (size_t i = 0; i < vm.size(); ++i) vm[i] = 1.0 / (vc[i] * vc[i]);
     WF_TRY(upload_tables<double>(c, key + "tc", vc, &ct, st));
     WF_TRY(upload_tables<double>(c, key + "tm", vm, &mt, st));
     WF_TRY(upload_tables<double>(c, key + "ts", vs, &stab, st));
