@@ -173,16 +173,30 @@ struct AccF {
 template <class S> struct AccFor { using T = AccD; };
 template <> struct AccFor<float> { using T = AccF; };
 
+// the lanes of this thread's warp that exist (a CTA's last warp may be partial)
+WF_D int warp_lanes() {
+  const int left = (int)blockDim.x - (int)(threadIdx.x & ~31u);
+  return left < 32 ? left : 32;
+}
+WF_D unsigned lane_mask(int lanes) { return lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u; }
+
 // Block-wide sum of a double; result valid in thread 0.  `red` holds >= 32 doubles.
 WF_D double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nl = warp_lanes();
+  const unsigned mask = lane_mask(nl);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double t = __shfl_down_sync(mask, v, o);
+    if (l + o < nl) v += t;
+  }
   __syncthreads();
   if (l == 0) red[w] = v;
   __syncthreads();
   const int nw = (blockDim.x + 31) >> 5;
   v = (threadIdx.x < nw) ? red[threadIdx.x] : 0.0;
   if (w == 0)
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) {
+      const double t = __shfl_down_sync(mask, v, o);
+      if (l + o < nl) v += t;
+    }
   return v;
 }

@@ -363,4 +363,47 @@ constexpr int ln_padded(int m, int sh, int n1, int banks) {
   return l;
 }
 
+// Sum over the CTA of the threads' double-float accumulators; valid in thread 0.  Each warp adds its 32 values
+// exactly, as integers in units of 2^-57 of the largest (three reductions of limbs), and only the warps' sums
+// meet in FP64: a tree of FP64 shuffles over all threads keeps GB300's FP64 pipe busy for ~1 us per CTA.
+// The result does not depend on any order.  red holds >= 32 doubles.
+WF_D long long acc_fixed(float f, int E) {  // f 2^(33 - (E - 150)) truncated, for exponents up to E
+  const unsigned u = __float_as_uint(f);
+  const int e = (u >> 23) & 0xff, sh = 33 - (E - e);
+  const long long m = e ? (long long)((u & 0x7fffffu) | 0x800000u) : 0;
+  const long long v = sh >= 0 ? m << sh : (sh > -24 ? m >> -sh : 0);
+  return (int)u < 0 ? -v : v;
+}
+WF_D double block_sum_acc(const AccF& a, double* red) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5, nl = warp_lanes();
+  const unsigned mask = lane_mask(nl);
+  const int E = (int)(__reduce_max_sync(mask, __float_as_uint(a.hi) & 0x7fffffffu) >> 23);
+  const long long v = acc_fixed(a.hi, E) + acc_fixed(a.lo, E);
+  const int s0 = __reduce_add_sync(mask, (int)(v & 0x1fffff));
+  const int s1 = __reduce_add_sync(mask, (int)((v >> 21) & 0x1fffff));
+  const int s2 = __reduce_add_sync(mask, (int)(v >> 42));
+  long long* sums = reinterpret_cast<long long*>(red);
+  __shared__ int exps[32];
+  __syncthreads();
+  if (l == 0) {
+    sums[w] = (long long)s0 + ((long long)s1 << 21) + ((long long)s2 << 42);
+    exps[w] = E;
+  }
+  __syncthreads();
+  double r = 0.0;
+  if (w == 0) {
+    for (int i = l; i < nw; i += nl) {  // one round but in a CTA of a single partial warp
+      const int k = exps[i] - 150 - 33;  // the units; a non-finite accumulator makes the sum a NaN
+      r += exps[i] == 0xff ? __longlong_as_double(0x7ff8000000000000ll)
+                           : __ll2double_rn(sums[i]) * __hiloint2double((k + 1023) << 20, 0);
+    }
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < nw) {
+        const double t = __shfl_down_sync(mask, r, o);
+        if (l + o < nl) r += t;
+      }
+  }
+  return r;
+}
+
 }  // namespace wf

@@ -34,6 +34,7 @@
 #include "wf_plane.cuh"
 #include "wf_spectral.cuh"
 #include "wf_fixspec.cuh"
+#include "wf_lines32.cuh"
 #include "wf_deflate.cuh"
 
 namespace wf {
@@ -88,8 +89,16 @@ struct Spec {
   // algorithmic bytes of one launch per system (DRAM traffic the pass cannot avoid)
   static constexpr double BS = (double)SPEC * sizeof(ST);
   static constexpr double BV = (double)V;
+  // Geometries of the FP32 line passes: rows of 16 columns (128 bytes; rows of 64 bytes at the x lines' stride
+  // copy at half the rate), 1024 threads per SM (64 registers: with one CTA of 512 threads per SM x pass 1
+  // takes 0.81 ms at 512^3, with two 0.61), rows of the z passes by CTAs of 128 threads
+  using GX = LX<N, 16, 512, -1024, typename F32XPlan<N>::T, 8>;
+  using GY = LX<N, 16, 512>;
+  using GZ1 = LZ<N, 128>;
+  using GZ2 = LZ<N, 256>;
   // cluster size of the fused y / z / y plane kernel (0: not available at this size)
   static constexpr int PCS = plane_cs<R, N>(), PE = plane_e<R, N>();
+  static constexpr size_t OCT = (size_t)(NH + 1) * (NH + 1) * NH;  // entries of the octant table of c
   // the persistent passes with tensor copies: tile lines and buffers in flight
   static constexpr int NLT = tma_lines<R, N>();
 
@@ -112,8 +121,8 @@ struct Spec {
       WF_A((k_zinv<R, N, ZI_ACCUM>), SMz);
     }
     if constexpr (std::is_same<R, float>::value) {
-      WF_A((k_zcoarse<R, N>), SMz);
-      WF_A((k_xcr<R, N, 32>), SMxy);
+      WF_A((k_ln_zcoarse<GZ1>), GZ1::SMEM);
+      WF_A((k_ln_xcr<GX>), GX::SMEM);
       WF_A(k_gj_update, kUpdSmem);
       WF_A((k_ycoarse<R, N>), (size_t)N * (kDeflMaxRadius + 2) * sizeof(cx<R>));
     }
@@ -168,6 +177,20 @@ struct Spec {
       });
     }
   };
+  template <class G>
+  struct YLn {  // the line engine with geometry G
+    static cudaError_t setup() {
+      cudaError_t e = set_smem(k_ln_ypass<G, -1>, G::SMEM);
+      return e == cudaSuccess ? set_smem(k_ln_ypass<G, +1>, G::SMEM) : e;
+    }
+    static void run(Ctx& c, int nb, ST* t, const ST* tw, const CgScal* sc, int dir, cudaStream_t st) {
+      const dim3 grid(G::KB, N, nb);
+      c.launch("ypass", 2 * BS * nb, st, [&] {
+        if (dir < 0) k_ln_ypass<G, -1><<<grid, G::NT, G::SMEM, st>>>(t, tw, sc, bat());
+        else k_ln_ypass<G, +1><<<grid, G::NT, G::SMEM, st>>>(t, tw, sc, bat());
+      });
+    }
+  };
   // the FP64 y pass (fixed point); tw is unused, its twiddles come from the context
   struct YFix {
     static cudaError_t setup() {
@@ -183,147 +206,99 @@ struct Spec {
       });
     }
   };
-  // candidates: FP32 grids of 128 and up (the inner solves) get a few; everything else the default
   static const std::vector<PassVariant>& yvariants() {
     static const std::vector<PassVariant> v = [] {
       std::vector<PassVariant> out;
-      if constexpr (F64) out.push_back({"fixed", YFix::setup, YFix::run});
-      else out.push_back({"nl_s2_r8", YV<NLT, 2, 8>::setup, YV<NLT, 2, 8>::run});
-      if constexpr (std::is_same<R, float>::value && N >= 128) {
-        constexpr int H = NLT / 2;
-        out.push_back({"nl_s2_r32", YV<NLT, 2, 32>::setup, YV<NLT, 2, 32>::run});
-        out.push_back({"nl_s3_r32", YV<NLT, 3, 32>::setup, YV<NLT, 3, 32>::run});
-        out.push_back({"nl/2_s2_r32", YV<H, 2, 32>::setup, YV<H, 2, 32>::run});
-        out.push_back({"nl/2_s3_r16", YV<H, 3, 16>::setup, YV<H, 3, 16>::run});
+      if constexpr (F64) {
+        out.push_back({"fixed", YFix::setup, YFix::run});
+      } else {
+        // lines up to 288 (128^3: 94 -> 80 us for 32 systems, 288^3: 191 -> 100 for 3), where a CTA of 512 threads
+        // holds whole 128-byte rows (96 at some ragged sizes); above, two or three tensor-copied tiles in
+        // flight (384^3: 142 against 156, 512^3: 173 against 195)
+        using L = YLn<GY>;
+        using T = YV<NLT, N < 512 ? 2 : 3, 32>;
+        if constexpr (N <= 288) out.push_back({"lines", L::setup, L::run});
+        if constexpr (N >= 128) out.push_back({"tma_r32", T::setup, T::run});
+        if constexpr (N > 288) out.push_back({"lines", L::setup, L::run});
       }
       return out;
     }();
     return v;
   }
-  // ---- x-pass variants: the two CG x passes, staged by tensor copies (<NL, STG, RMAX>) or the
-  // register-staged kernels; each launcher returns the number of partial sums it wrote -------
-  using XinvRun = int (*)(Ctx&, int, ST*, ST*, ST*, ST*, ST*, const SS*, const SS*, bool, const ST*, double*,
-                          CgScal*, cudaStream_t);
-  using XupdRun = int (*)(Ctx&, int, const ST*, ST*, ST*, ST*, const SS*, const SS*, bool, const ST*, double*,
-                          CgScal*, cudaStream_t);
+  // ---- x-pass variants: the two CG x passes; each launcher returns the number of partial sums it wrote
+  using XinvRun = int (*)(Ctx&, int, ST*, ST*, ST*, ST*, ST*, const SS*, const SS*, const SS*, bool, const ST*,
+                          double*, CgScal*, cudaStream_t);
+  using XupdRun = int (*)(Ctx&, int, const ST*, ST*, ST*, ST*, const SS*, const SS*, const SS*, bool, const ST*,
+                          double*, CgScal*, cudaStream_t);
   struct XVariant {
     const char* name;
     cudaError_t (*setup)();
     XinvRun xinv;
     XupdRun xupd;
   };
-  template <int NL, int STG, int RMAX, int EX = elems_for<R>(N, NL), int COPY = 0>
-  struct XV {
-    using G = TG<R, N, NL, STG, EX>;
-    static constexpr size_t SM = TXG<R, N, NL, STG, 3>::SMEM;
-    static inline int occ = 1;
-    static cudaError_t setup() {
-      cudaError_t e = set_smem(k_cg_xinv_tma<R, N, true, NL, STG, RMAX, EX, COPY>, SM);
-      if (e == cudaSuccess) e = set_smem(k_cg_xinv_tma<R, N, false, NL, STG, RMAX, EX, COPY>, SM);
-      if (e == cudaSuccess) e = set_smem(k_cg_xupd_tma<R, N, true, NL, STG, RMAX, EX, COPY>, SM);
-      if (e == cudaSuccess) e = set_smem(k_cg_xupd_tma<R, N, false, NL, STG, RMAX, EX, COPY>, SM);
-      if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_xinv_tma<R, N, true, NL, STG, RMAX, EX, COPY>,
-                                                          G::NT, SM);
-      if (occ < 1) occ = 1;
-      return e;
-    }
-    // tensor maps for the tensor-copy form; the row-copy form passes zeroed (unused) maps
-    static bool map(Ctx& c, CUtensorMap* m, const void* p, int nb) {
-      if (COPY == 1) {
-        std::memset(m, 0, sizeof(*m));
-        return true;
-      }
-      if (make_spectrum_map(m, const_cast<void*>(p), N, nb, sizeof(SS) == 8, NL, 1, G::BR)) return true;
-      c.map_failed = true;
-      return false;
-    }
-    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* ctab, const SS* mtab, bool unit_m,
-                    const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
-      CUtensorMap mr, m0, m1, mx, mt;
-      if (!map(c, &mr, r, nb) || !map(c, &m0, P0, nb) || !map(c, &m1, P1, nb) || !map(c, &mx, x, nb) ||
-          !map(c, &mt, T, nb))
-        return G::TPS;
-      const unsigned grid = persistent_grid(c, occ, (long long)nb * G::TPS);
-      c.launch(cls("cg_xinv", "cg_xinv_f64"), 6 * BS * nb, st, [&] {
-        if (unit_m)
-          k_cg_xinv_tma<R, N, true, NL, STG, RMAX, EX, COPY><<<grid, G::NT, SM, st>>>(
-              mr, m0, m1, mx, mt, r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat(), nb, c.dev_err);
-        else
-          k_cg_xinv_tma<R, N, false, NL, STG, RMAX, EX, COPY><<<grid, G::NT, SM, st>>>(
-              mr, m0, m1, mx, mt, r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat(), nb, c.dev_err);
-      });
-      return G::TPS;
-    }
-    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
-                    const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
-      CUtensorMap mt, mr, m0, m1;
-      if (!map(c, &mt, T, nb) || !map(c, &mr, r, nb) || !map(c, &m0, P0, nb) || !map(c, &m1, P1, nb)) return G::TPS;
-      const unsigned grid = persistent_grid(c, occ, (long long)nb * G::TPS);
-      c.launch(cls("cg_xupd", "cg_xupd_f64"), 4 * BS * nb, st, [&] {
-        if (unit_m)
-          k_cg_xupd_tma<R, N, true, NL, STG, RMAX, EX, COPY><<<grid, G::NT, SM, st>>>(
-              mt, mr, m0, m1, T, P0, P1, r, ctab, mtab, tw, part, sc, bat(), nb, c.dev_err);
-        else
-          k_cg_xupd_tma<R, N, false, NL, STG, RMAX, EX, COPY><<<grid, G::NT, SM, st>>>(
-              mt, mr, m0, m1, T, P0, P1, r, ctab, mtab, tw, part, sc, bat(), nb, c.dev_err);
-      });
-      return G::TPS;
-    }
-  };
-  // the register-staged kernels (one CTA per tile, loads through registers), radix cap RMAX, at
-  // least MINB resident CTAs per SM (the register cap that allows them: 128 for 2, 85 for 3)
-  template <int RMAX, int MINB = 0>
+  // the register-staged kernels (one CTA per tile, loads through registers), radix cap RMAX
+  template <int RMAX>
   struct XReg {
     static cudaError_t setup() {
-      cudaError_t e = set_smem(k_cg_xinv<R, N, true, RMAX, MINB>, SMxy);
-      if (e == cudaSuccess) e = set_smem(k_cg_xinv<R, N, false, RMAX, MINB>, SMxy);
-      if (e == cudaSuccess) e = set_smem(k_cg_xupd<R, N, true, RMAX, MINB>, SMxy);
-      if (e == cudaSuccess) e = set_smem(k_cg_xupd<R, N, false, RMAX, MINB>, SMxy);
+      cudaError_t e = set_smem(k_cg_xinv<R, N, true, RMAX>, SMxy);
+      if (e == cudaSuccess) e = set_smem(k_cg_xinv<R, N, false, RMAX>, SMxy);
+      if (e == cudaSuccess) e = set_smem(k_cg_xupd<R, N, true, RMAX>, SMxy);
+      if (e == cudaSuccess) e = set_smem(k_cg_xupd<R, N, false, RMAX>, SMxy);
       return e;
     }
-    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* ctab, const SS* mtab, bool unit_m,
+    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* oct, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
       c.launch(cls("cg_xinv", "cg_xinv_f64"), 6 * BS * nb, st, [&] {
         if (unit_m)
-          k_cg_xinv<R, N, true, RMAX, MINB><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
+          k_cg_xinv<R, N, true, RMAX><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
         else
-          k_cg_xinv<R, N, false, RMAX, MINB><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
+          k_cg_xinv<R, N, false, RMAX><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
       });
       return GXY;
     }
-    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
+    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* oct, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
       c.launch(cls("cg_xupd", "cg_xupd_f64"), 4 * BS * nb, st, [&] {
         if (unit_m)
-          k_cg_xupd<R, N, true, RMAX, MINB><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
+          k_cg_xupd<R, N, true, RMAX><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
         else
-          k_cg_xupd<R, N, false, RMAX, MINB><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
+          k_cg_xupd<R, N, false, RMAX><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
       });
       return GXY;
     }
   };
-  // x pass 2 with its r and p rows prefetched into shared memory (NL lines, EX elements per thread)
-  template <int RMAX, int NL, int EX>
-  struct XPf {
-    using G = XYP<R, N, NL, EX>;
+  // the line-engine kernels with geometry G
+  template <class G>
+  struct XLn {
     static cudaError_t setup() {
-      cudaError_t e = set_smem(k_cg_xupd_pf<R, N, true, RMAX, NL, EX>, G::SMEM);
-      if (e == cudaSuccess) e = set_smem(k_cg_xupd_pf<R, N, false, RMAX, NL, EX>, G::SMEM);
+      cudaError_t e = set_smem(k_ln_xinv<G, true>, G::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_ln_xinv<G, false>, G::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_ln_xupd<G, true>, G::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_ln_xupd<G, false>, G::SMEM);
       return e;
     }
-    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
-                    const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
-      const dim3 grid(N / 2 / NL, N, nb);
-      c.launch(cls("cg_xupd", "cg_xupd_f64"), 4 * BS * nb, st, [&] {
+    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* oct, const SS* ctab, const SS* mtab,
+                    bool unit_m, const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
+      const dim3 grid(G::KB, N, nb);
+      c.launch("cg_xinv", 6 * BS * nb, st, [&] {
         if (unit_m)
-          k_cg_xupd_pf<R, N, true, RMAX, NL, EX><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc,
-                                                                              bat());
+          k_ln_xinv<G, true><<<grid, G::NT, G::SMEM, st>>>(r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
         else
-          k_cg_xupd_pf<R, N, false, RMAX, NL, EX><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, ctab, mtab, tw, part,
-                                                                               sc, bat());
+          k_ln_xinv<G, false><<<grid, G::NT, G::SMEM, st>>>(r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
       });
-      return (N / 2 / NL) * N;
+      return G::KB * N;
+    }
+    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* oct, const SS* ctab, const SS* mtab,
+                    bool unit_m, const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
+      const dim3 grid(G::KB, N + G::YP, nb);
+      static_assert(2 * G::KB * (N + G::YP) <= NPART, "partial sums");
+      c.launch("cg_xupd", 4 * BS * nb, st, [&] {
+        if (unit_m)
+          k_ln_xupd<G, true><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
+        else
+          k_ln_xupd<G, false><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
+      });
+      return G::KB * (N + G::YP);
     }
   };
   // the FP64 CG x passes (fixed point)
@@ -335,7 +310,7 @@ struct Spec {
       if (e == cudaSuccess) e = set_smem(k_fx_cg_xupd<N, false>, fx_xmul_smem<N>());
       return e;
     }
-    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* ctab, const SS* mtab, bool unit_m,
+    static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* oct, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST*, double* part, CgScal* sc, cudaStream_t st) {
       if constexpr (F64) {
         const dim3 grid(FC::KB, N, nb);
@@ -348,7 +323,7 @@ struct Spec {
       }
       return FC::KB * N;
     }
-    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
+    static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* oct, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST*, double* part, CgScal* sc, cudaStream_t st) {
       if constexpr (F64) {
         const dim3 grid(FC::KB + 1, N, nb);
@@ -363,71 +338,54 @@ struct Spec {
       return (FC::KB + 1) * N;
     }
   };
-  static constexpr int NLX = xtma_lines<R, N, 3, 2>();
   static const std::vector<XVariant>& xvariants() {
     static const std::vector<XVariant> v = [] {
-      // variant 0: the register-staged kernels, measured fastest at every size (512^3 FP32: 0.72 and
-      // 0.58 ms against 1.23-1.83 ms for the staged forms, whose single resident CTA per SM
-      // serialises each tile's table gathers, transform and epilogue); the staged forms stay
-      // candidates for the tuner on the FP32 grids of 128 and up
       std::vector<XVariant> out;
-      if constexpr (F64) out.push_back({"fixed", XFix::setup, XFix::xinv, XFix::xupd});
-      else out.push_back({"registers", XReg<8>::setup, XReg<8>::xinv, XReg<8>::xupd});
-      if constexpr (std::is_same<R, float>::value && N >= 128) {
-        out.push_back({"registers_r16", XReg<16>::setup, XReg<16>::xinv, XReg<16>::xupd});
-        out.push_back({"registers_r32", XReg<32>::setup, XReg<32>::xinv, XReg<32>::xupd});
-        // x pass 2 only (its x pass 1 entry is the radix-32 register kernel again)
-        if constexpr ((N / 2) % 8 == 0 && N % 16 == 0) {
-          using P1 = XPf<32, 8, 16>;
-          using P2 = XPf<16, 8, 16>;
-          out.push_back({"prefetch_nl8_e16_r32", P1::setup, XReg<32>::xinv, P1::xupd});
-          out.push_back({"prefetch_nl8_e16_r16", P2::setup, XReg<32>::xinv, P2::xupd});
-        }
-      }
-      if constexpr (std::is_same<R, float>::value && N >= 128 && N % 8 == 0 && NLX * (N / 8) <= 512) {
-        using E8 = XV<NLX, 2, 8, 8, 1>;  // per-thread row copies, 8 elements per thread
-        using T8 = XV<NLX, 2, 8, 8, 0>;  // tensor copies, 8 elements per thread
-        out.push_back({"rows_s2_e8", E8::setup, E8::xinv, E8::xupd});
-        out.push_back({"tensor_s2_e8", T8::setup, T8::xinv, T8::xupd});
+      if constexpr (F64) {
+        out.push_back({"fixed", XFix::setup, XFix::xinv, XFix::xupd});
+      } else {
+        // the line engine first: faster from 64 to 512 but for x pass 1 at 128, 192 and 288 (1-5% behind the
+        // register-staged form), which the tuner may pick
+        out.push_back({"lines", XLn<GX>::setup, XLn<GX>::xinv, XLn<GX>::xupd});
+        if constexpr (N >= 128) out.push_back({"registers_r32", XReg<32>::setup, XReg<32>::xinv, XReg<32>::xupd});
       }
       return out;
     }();
     return v;
   }
-  // ---- z-turn variants: elements per thread (threads per CTA) ------------------------------
-  using ZRun = void (*)(Ctx&, int, ST*, const SS*, const ST*, double*, const CgScal*, cudaStream_t);
+  // ---- z-turn variants: threads per CTA ----------------------------------------------------
+  using ZRun = int (*)(Ctx&, int, ST*, const SS*, const ST*, double*, const CgScal*, cudaStream_t);  // partial sums written
   struct ZVariant {
     const char* name;
     cudaError_t (*setup)();
     ZRun run;
   };
-  template <int EZ>
-  struct ZV {
-    static cudaError_t setup() { return set_smem(k_zturn<R, N, EZ>, ZG<R, N, EZ>::SMEM); }
-    static void run(Ctx& c, int nb, ST* T, const SS* D, const ST* tw, double* part, const CgScal* sc,
-                    cudaStream_t st) {
-      c.launch(cls("zturn", "zturn_f64"), (2 * BS + sizeof(SS) * BV) * nb, st, [&] {
-        k_zturn<R, N, EZ><<<gz(nb), ZG<R, N, EZ>::NT, ZG<R, N, EZ>::SMEM, st>>>(T, D, tw, part, sc, bat());
-      });
+  template <class G>
+  struct ZLn {  // the line engine with geometry G
+    static cudaError_t setup() { return set_smem(k_ln_zturn<G>, G::SMEM); }
+    static int run(Ctx& c, int nb, ST* T, const SS* D, const ST* tw, double* part, const CgScal* sc, cudaStream_t st) {
+      c.launch("zturn", (2 * BS + sizeof(SS) * BV) * nb, st,
+               [&] { k_ln_zturn<G><<<dim3(G::GZ, 1, nb), G::NT, G::SMEM, st>>>(T, D, tw, part, sc, bat()); });
+      return G::GZ;
     }
   };
   struct ZFix {  // FP64 (fixed point)
     static cudaError_t setup() { return set_smem(k_fx_zturn<N>, FZ::SMEM); }
-    static void run(Ctx& c, int nb, ST* T, const SS* D, const ST*, double* part, const CgScal* sc, cudaStream_t st) {
+    static int run(Ctx& c, int nb, ST* T, const SS* D, const ST*, double* part, const CgScal* sc, cudaStream_t st) {
       if constexpr (F64)
         c.launch("zturn_f64", (2 * BS + sizeof(SS) * BV) * nb, st,
                  [&] { k_fx_zturn<N><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(T, D, c.fixed(N), part, sc, bat()); });
+      return FZ::GZ;
     }
   };
   static const std::vector<ZVariant>& zvariants() {
     static const std::vector<ZVariant> v = [] {
-      constexpr int E0 = z_elems<R, N>();
       std::vector<ZVariant> out;
-      if constexpr (F64) out.push_back({"fixed", ZFix::setup, ZFix::run});
-      else out.push_back({"e_default", ZV<E0>::setup, ZV<E0>::run});
-      if constexpr (std::is_same<R, float>::value && N >= 128) {
-        if constexpr (E0 / 2 >= 4 && (N / 2) % (E0 / 2) == 0) out.push_back({"e/2", ZV<E0 / 2>::setup, ZV<E0 / 2>::run});
-        if constexpr (E0 / 4 >= 4 && (N / 2) % (E0 / 4) == 0) out.push_back({"e/4", ZV<E0 / 4>::setup, ZV<E0 / 4>::run});
+      if constexpr (F64) {
+        out.push_back({"fixed", ZFix::setup, ZFix::run});
+      } else {
+        out.push_back({"lines128", ZLn<GZ1>::setup, ZLn<GZ1>::run});
+        if constexpr (N >= 128) out.push_back({"lines256", ZLn<GZ2>::setup, ZLn<GZ2>::run});
       }
       return out;
     }();
@@ -496,14 +454,14 @@ struct Spec {
   // One CG iteration of every unfinished system (no host synchronisation).  The first x pass forms
   // p from rin (default r); after_xinv(st) is enqueued right after it.
   template <class H = NoHook>
-  static void iteration(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* D, const SS* ctab,
-                        const SS* mtab, bool unit_m, const ST* tw, double* part, CgScal* sc, double inv_vc,
+  static void iteration(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* D, const SS* oct,
+                        const SS* ctab, const SS* mtab, bool unit_m, const ST* tw, double* part, CgScal* sc, double inv_vc,
                         cudaStream_t st, ST* rin = nullptr, H after_xinv = H()) {
     const Bat b = bat();
     const int n1 = pick(c, "xinv", xvariants())
-                       .xinv(c, nb, rin ? rin : r, P0, P1, x, T, ctab, mtab, unit_m, tw, part, sc, st);
+                       .xinv(c, nb, rin ? rin : r, P0, P1, x, T, oct, ctab, mtab, unit_m, tw, part, sc, st);
     after_xinv(st);
-    int nmid = GZI;  // blocks that sum the data term of <p, A p> into part[NX ...]
+    int nmid = 0;  // blocks that sum the data term of <p, A p> into part[NX ...]
     bool fused = false;
     if constexpr (PCS > 0) {
       if (c.fused_planes) {
@@ -515,11 +473,11 @@ struct Spec {
     }
     if (!fused) {
       ypass(c, nb, T, tw, sc, +1, st);
-      pick(c, "zturn", zvariants()).run(c, nb, T, D, tw, part + NX, sc, st);
+      nmid = pick(c, "zturn", zvariants()).run(c, nb, T, D, tw, part + NX, sc, st);
       ypass(c, nb, T, tw, sc, -1, st);
     }
     c.launch("fin", 0, st, [&] { k_fin_alpha<<<nb, 1024, 0, st>>>(part, n1, NX, nmid, sc, b); });
-    const int n3 = pick(c, "xupd", xvariants()).xupd(c, nb, T, r, P0, P1, ctab, mtab, unit_m, tw, part, sc, st);
+    const int n3 = pick(c, "xupd", xvariants()).xupd(c, nb, T, r, P0, P1, oct, ctab, mtab, unit_m, tw, part, sc, st);
     c.launch("fin", 0, st, [&] { k_fin_beta<<<nb, 1024, 0, st>>>(part, n3, inv_vc, sc, b); });
   }
 };
@@ -820,7 +778,7 @@ struct GroupFP64 : GroupCommon<N> {
   wf_status block(Ctx& c, cudaStream_t st) {
     return this->run_block(c, st, [&](cudaStream_t s2) {
       for (int i = 0; i < check_every<N>(); ++i)
-        SP::iteration(c, nb, rh, P0, P1, xh, T, D, ct, mt, unit_m, tw, part, sc, inv_vc, s2);
+        SP::iteration(c, nb, rh, P0, P1, xh, T, D, nullptr, ct, mt, unit_m, tw, part, sc, inv_vc, s2);
     });
   }
   wf_status enqueue(Ctx& c, cudaStream_t st) override {
@@ -907,7 +865,7 @@ struct GroupMixed : GroupCommon<N> {
   float* D;
   double2 *T64, *T64b;
   const float2* tw32 = nullptr;  // FP32 copy of the twiddle table for the FP32 passes
-  float *ct, *mt;
+  float *ct, *mt, *coct = nullptr;
   double* stab;
   std::vector<int> outer, iters;
   std::vector<int> texp;  // per system: power of two of the prior table's digits
@@ -1031,7 +989,8 @@ struct GroupMixed : GroupCommon<N> {
       defl_xr(c, st);
       SF::ypass(c, nb, T, tw32, sc, +1, st);
       c.launch("defl_z", (SF::BS + 4 * SF::BV) * nb, st, [&] {
-        k_zcoarse<float, N><<<SF::gz(nb), SF::NTz, SF::SMz, st>>>(T, D, tw32, Gz, K, sc, bf, gzs);
+        using G = typename SF::GZ1;
+        k_ln_zcoarse<G><<<dim3(G::GZ, 1, nb), G::NT, G::SMEM, st>>>(T, D, tw32, Gz, K, sc, bf, gzs);
       });
       const size_t ysm = ((size_t)N * (K + 1) + N) * sizeof(float2);
       c.launch("defl_y", 8.0 * gzs * nb, st, [&] {
@@ -1053,7 +1012,8 @@ struct GroupMixed : GroupCommon<N> {
   void defl_xr(Ctx& c, cudaStream_t st) {
     const Bat bf = SF::bat();
     c.launch("defl_xr", 2 * SF::BS * nb, st, [&] {
-      k_xcr<float, N, 32><<<SF::gxy(nb), SF::NTx, SF::SMxy, st>>>(rh, T, ct, tw32, sc, bf);
+      using G = typename SF::GX;
+      k_ln_xcr<G><<<dim3(G::KB, N, nb), G::NT, G::SMEM, st>>>(rh, T, coct, ct, tw32, sc, bf);
     });
   }
   // one deflated inner iteration: p = (r - Z mu) + beta p with mu from the coarse projection
@@ -1061,7 +1021,7 @@ struct GroupMixed : GroupCommon<N> {
     const Bat bf = SF::bat();
     defl_project<1>(c, rh, st);
     c.launch("fin", 0, st, [&] { k_fin_defl<<<nb, 256, 0, st>>>(dpart, nh, sc); });
-    SF::iteration(c, nb, rh, P0, P1, xh, T, D, ct, mt, unit_m, tw32, part, sc, inv_vc, st, nullptr,
+    SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, st, nullptr,
                   [&](cudaStream_t s) {
                     c.launch("defl_restore", 0, s, [&] {
                       k_defl_restore<float, N><<<dim3((nh + 1 + 255) / 256, nb), 256, 0, s>>>(rh, rsave, dmodes, nh,
@@ -1141,6 +1101,11 @@ struct GroupMixed : GroupCommon<N> {
       }
       WF_TRY(this->push_scalars(st));
       const size_t SPEC = SF::SPEC;
+      // c over the octant of wavenumbers, in the FP64 scratch spectrum (idle until the residual)
+      coct = reinterpret_cast<float*>(T64b);
+      c.launch("tables", 4.0 * SF::OCT * nb, st, [&] {
+        k_oct<N><<<dim3(N / 2 + 1, N / 2 + 1, nb), N / 2 < 128 ? N / 2 : 128, 0, st>>>(ct, coct, SF::OCT, SF::TAB, sc);
+      });
       SF::zfwd(c, nb, RES, T, tw32, part, nullptr, st);
       SF::ypass(c, nb, T, tw32, nullptr, -1, st);
       SF::template xmul<true, false, true>(c, nb, T, rh, ct, tw32, part, nullptr, st);
@@ -1155,7 +1120,7 @@ struct GroupMixed : GroupCommon<N> {
         WF_CUDA(cudaMemsetAsync(Rc, 0, nb * SPEC * sizeof(float2), st));
         c.launch("fin", 0, st, [&] { k_defl_arm<<<nb, 32, 0, st>>>(sc); });
         defl_project<0>(c, Rc, st);
-        SF::iteration(c, nb, rh, P0, P1, xh, T, D, ct, mt, unit_m, tw32, part, sc, inv_vc, st, Rc);
+        SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, st, Rc);
       }
       phase = 1;
     }
@@ -1163,7 +1128,7 @@ struct GroupMixed : GroupCommon<N> {
       WF_TRY(this->run_block(c, st, [&](cudaStream_t s2) {
         for (int i = 0; i < check_every<N>(); ++i) {
           if (K > 0) defl_iteration(c, s2);
-          else SF::iteration(c, nb, rh, P0, P1, xh, T, D, ct, mt, unit_m, tw32, part, sc, inv_vc, s2);
+          else SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, s2);
         }
       }));
     } else if (phase == 2) {
@@ -1350,13 +1315,15 @@ wf_status tune_spec(Ctx& c, std::string& report) {
   double* part;
   CgScal* sc;
   WF_TRY(c.get("tune_x", (size_t)5 * nb * SPEC * sizeof(ST), (void**)&xb));
-  WF_TRY(c.get("tune_xtab", (size_t)nb * SP::TAB * sizeof(SS), (void**)&tab));
+  // tables of ones: c and m by n^2, and c over the octant, in one buffer
+  const size_t ntab = (size_t)nb * (SP::OCT > SP::TAB ? SP::OCT : SP::TAB);
+  WF_TRY(c.get("tune_xtab", ntab * sizeof(SS), (void**)&tab));
   WF_TRY(c.get("tune_xpart", (size_t)nb * SP::NPART * sizeof(double), (void**)&part));
   WF_TRY(c.get("tune_xsc", (size_t)nb * sizeof(CgScal), (void**)&sc));
   WF_CUDA(cudaMemsetAsync(xb, 0, (size_t)5 * nb * SPEC * sizeof(ST), st));
   WF_CUDA(cudaMemsetAsync(sc, 0, (size_t)nb * sizeof(CgScal), st));
   {
-    std::vector<SS> ones((size_t)nb * SP::TAB, (SS)1);
+    std::vector<SS> ones(ntab, (SS)1);
     WF_CUDA(cudaMemcpyAsync(tab, ones.data(), ones.size() * sizeof(SS), cudaMemcpyHostToDevice, st));
     WF_CUDA(cudaStreamSynchronize(st));
   }
@@ -1367,8 +1334,8 @@ wf_status tune_spec(Ctx& c, std::string& report) {
     const char* name;
     void run(Ctx& c, int nb, cudaStream_t st, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* tab, const ST* tw,
              double* part, CgScal* sc, int, int) const {
-      if (inv) v->xinv(c, nb, r, P0, P1, x, T, tab, tab, true, tw, part, sc, st);
-      else v->xupd(c, nb, T, r, P0, P1, tab, tab, true, tw, part, sc, st);
+      if (inv) v->xinv(c, nb, r, P0, P1, x, T, tab, tab, tab, true, tw, part, sc, st);
+      else v->xupd(c, nb, T, r, P0, P1, tab, tab, tab, true, tw, part, sc, st);
     }
   };
   for (int inv = 1; inv >= 0; --inv) {

@@ -360,8 +360,8 @@ WF_D void tile_mul(cx<R>* tile, int kz0, int ky_s, const TAB* tab, int tid) {
 // P0 = (Z + conj Z(-k)) / 2 and PN = (Z - conj Z(-k)) / 2i (Z(-k) from the partner line).
 // UNIT_M: m = 1 at every k != 0 (the preconditioned system), so m is read only on column 0.
 // ------------------------------------------------------------------------------------------
-template <class R, int N, bool UNIT_M, int RMAX = 8, int MINB = 0>
-__global__ void __launch_bounds__(XYG<R, N>::NT, MINB)
+template <class R, int N, bool UNIT_M, int RMAX = 8>
+__global__ void __launch_bounds__(XYG<R, N>::NT)
 k_cg_xinv(const typename Store<R>::T* __restrict__ r, typename Store<R>::T* P0, typename Store<R>::T* P1,
           typename Store<R>::T* __restrict__ x, typename Store<R>::T* __restrict__ T,
           const typename Store<R>::S* __restrict__ ctab, const typename Store<R>::S* __restrict__ mtab,
@@ -501,8 +501,8 @@ k_cg_xinv(const typename Store<R>::T* __restrict__ r, typename Store<R>::T* P0, 
 // weights, without 1/V_c) and an upper estimate of V_c ||C^-1 r||^2 (the canonical residual): on
 // column 0 the larger of the two planes' 1/c^2 is used.  grid (N/2 / NL, N).
 // ------------------------------------------------------------------------------------------
-template <class R, int N, bool UNIT_M, int RMAX = 8, int MINB = 0>
-__global__ void __launch_bounds__(XYG<R, N>::NT, MINB)
+template <class R, int N, bool UNIT_M, int RMAX = 8>
+__global__ void __launch_bounds__(XYG<R, N>::NT)
 k_cg_xupd(const typename Store<R>::T* __restrict__ T, typename Store<R>::T* __restrict__ r,
           const typename Store<R>::T* P0, const typename Store<R>::T* P1,
           const typename Store<R>::S* __restrict__ ctab, const typename Store<R>::S* __restrict__ mtab,
@@ -619,606 +619,6 @@ k_cg_xupd(const typename Store<R>::T* __restrict__ T, typename Store<R>::T* __re
     partials[2 * bid] = s1;
     partials[2 * bid + 1] = s2;
   }
-}
-
-// ------------------------------------------------------------------------------------------
-// CG x pass 2 with its r and p tiles prefetched: the same work as k_cg_xupd, but the tile's r and p
-// rows are requested (per-thread asynchronous 16-byte copies into shared memory) before T is loaded
-// and transformed, so the epilogue reads them from shared memory instead of waiting on HBM.  One
-// tile per CTA, NL lines (8 leaves shared memory for two CTAs per SM).  grid (N/2 / NL, N).
-// ------------------------------------------------------------------------------------------
-template <class R, int N, int NL_, int EX>
-struct XYP {
-  using ST = typename Store<R>::T;
-  static constexpr int M = N, NH = N / 2, NL = NL_;
-  static constexpr int E = EX;
-  static constexpr int TPL = M / E >= 1 ? M / E : 1;
-  static constexpr int NT = NL * TPL;
-  static constexpr int LD = NL + 1;  // padded transform tile
-  static constexpr int VW = (sizeof(ST) == 8 && NL % 2 == 0) ? 2 : 1;
-  static constexpr int NV = NL / VW;
-  static constexpr int NVEC = M * NV;
-  static constexpr int PER = (NVEC + NT - 1) / NT;
-  static constexpr bool EVEN = NVEC % NT == 0;
-  using VT = typename std::conditional<VW == 2, float4, ST>::type;
-  // transform tile, twiddles, then the dense r and p tiles (16-byte aligned)
-  static constexpr size_t TILE = (size_t)M * LD * sizeof(cx<R>), TWB = (size_t)M * sizeof(cx<R>);
-  static constexpr size_t OFF_R = ((TILE + TWB + 127) / 128) * 128;
-  static constexpr size_t DENSE = (size_t)M * NL * sizeof(ST);
-  static constexpr size_t SMEM = OFF_R + 2 * DENSE;
-  static_assert(NH % NL == 0 && (NL * sizeof(ST)) % 16 == 0, "whole 16-byte pieces per row");
-};
-
-template <class R, int N, bool UNIT_M, int RMAX, int NL, int EX>
-__global__ void __launch_bounds__(XYP<R, N, NL, EX>::NT)
-k_cg_xupd_pf(const typename Store<R>::T* __restrict__ T, typename Store<R>::T* __restrict__ r,
-             const typename Store<R>::T* P0, const typename Store<R>::T* P1,
-             const typename Store<R>::S* __restrict__ ctab, const typename Store<R>::S* __restrict__ mtab,
-             const typename Store<R>::T* __restrict__ twtab, double* __restrict__ partials,
-             const CgScal* __restrict__ sc, Bat bt) {
-  using G = XYP<R, N, NL, EX>;
-  using ST = typename Store<R>::T;
-  using SS = typename Store<R>::S;
-  constexpr int NH = G::NH;
-  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
-  cx<R>* tw = tile + G::M * G::LD;
-  cx<R>* rt = reinterpret_cast<cx<R>*>(smem_raw + G::OFF_R);  // r rows, dense
-  cx<R>* pt = rt + G::M * NL;                                  // p rows, dense
-  __shared__ double red[32];
-  const int z = blockIdx.z;
-  sc += z;
-  if (sc->done) return;
-  const ST* __restrict__ p = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;  // this iteration's p_new
-  T += z * bt.spec;
-  r += z * bt.spec;
-  ctab += z * bt.tab;
-  mtab += z * bt.tab;
-  partials += z * bt.part;
-  const int tid = threadIdx.x;
-  const int kz0 = blockIdx.x * NL, ky = blockIdx.y;
-  const int ky_s = sfreq(ky, N);
-  const int pky = (N - ky) % N;
-  const size_t rowstride = (size_t)N * NH;
-  const size_t base = (size_t)ky * NH + kz0;
-  // r and p rows first: they arrive while T is loaded and transformed
-  {
-    constexpr int PV = 16 / (int)sizeof(ST), NVR = NL / PV;
-    for (int idx = tid; idx < G::M * NVR; idx += G::NT) {
-      const int i = idx / NVR, v = (idx % NVR) * PV;
-      cp_async16(rt + i * NL + v, r + base + (size_t)i * rowstride + v);
-      cp_async16(pt + i * NL + v, p + base + (size_t)i * rowstride + v);
-    }
-    cp_async_commit();
-  }
-  const SS alpha = (SS)sc->alpha;
-  load_tw<R, G::M, 2 * N>(tw, twtab, tid, G::NT);
-  tile_load<G>(tile, T + base, rowstride, tid);
-  if (kz0 == 0)
-    for (int i = tid; i < G::M; i += G::NT) tile[i * G::LD + NL] = ld_c<R>(T + (size_t)pky * NH + (size_t)i * rowstride);
-  __syncthreads();
-  fft_line<R, G::M, G::TPL, G::LD, -1, 1, cmin(RMAX, rmax_for(G::M, G::TPL))>(tile + tid % NL, tid / NL, tw);
-  if (kz0 == 0) {  // transform the partner line too, then apply c to column 0 as a packed pair
-    fft_line<R, G::M, G::TPL, G::LD, -1, 1, cmin(RMAX, rmax_for(G::M, G::TPL))>(tile + NL, tid / NL, tw,
-                                                                                 tid % NL == 0);
-    combine_col0<R, N, G::LD, NL>(tile, ky_s, ctab, tid, G::NT);
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  // epilogue: r -= alpha (m p + c T^), two elements of a row per step, stored as one vector
-  typename AccFor<SS>::T a_rr, a_rc;
-  constexpr int W = G::VW;
-#pragma unroll 4
-  for (int idx = tid; idx < G::M * (NL / W); idx += G::NT) {
-    const int i = idx / (NL / W), c0 = (idx % (NL / W)) * W;
-    const int kxs = sfreq(i, N);
-    cx<R> out[W];
-    SS s_rr = 0, s_rc = 0;
-#pragma unroll
-    for (int u = 0; u < W; ++u) {
-      const int kz = kz0 + c0 + u;
-      const int n2 = kxs * kxs + ky_s * ky_s + kz * kz;
-      const cx<R> t = tile[i * G::LD + c0 + u], pv = pt[i * NL + c0 + u];
-      cx<R> rv = rt[i * NL + c0 + u];
-      const SS c = ctab[n2];
-      SS ic2 = (SS)1 / (c * c);
-      SS q0, q1;
-      if (kz == 0) {
-        const SS cN = ctab[n2 + NH * NH];
-        const SS i2 = (SS)1 / (cN * cN);
-        ic2 = ic2 > i2 ? ic2 : i2;
-        const SS m0 = mtab[n2], mN = mtab[n2 + NH * NH];
-        const SS a = (SS)0.5 * (m0 + mN), b = (SS)0.5 * (m0 - mN);
-        ST pp = ST{};
-        if (b != (SS)0) pp = p[(size_t)((N - i) % N) * rowstride + (size_t)pky * NH];
-        q0 = a * pv.x + b * pp.x + t.x;
-        q1 = a * pv.y - b * pp.y + t.y;
-      } else {
-        const SS m = UNIT_M ? (SS)1 : mtab[n2];
-        q0 = m * pv.x + c * t.x;
-        q1 = m * pv.y + c * t.y;
-      }
-      rv.x -= alpha * q0;
-      rv.y -= alpha * q1;
-      out[u] = rv;
-      const SS wgt = kz == 0 ? (SS)1 : (SS)2;
-      const SS m2 = wgt * (rv.x * rv.x + rv.y * rv.y);
-      s_rr += m2;
-      s_rc += ic2 * m2;
-    }
-    *reinterpret_cast<typename G::VT*>(r + base + (size_t)i * rowstride + c0) = *reinterpret_cast<const typename G::VT*>(out);
-    a_rr.add(s_rr);
-    a_rc.add(s_rc);
-  }
-  const double s1 = block_sum(a_rr.get(), red);
-  const double s2 = block_sum(a_rc.get(), red);
-  if (tid == 0) {
-    const int bid = blockIdx.y * gridDim.x + blockIdx.x;
-    partials[2 * bid] = s1;
-    partials[2 * bid + 1] = s2;
-  }
-}
-
-// ------------------------------------------------------------------------------------------
-// Persistent CG x passes with tensor copies.  A stage holds NS tiles (one per staged stream), all
-// loaded by tensor copies along x (box {2 NL, 1, BR, 1}) and completed on the stage's barrier.
-// The packed column's partner line (-ky) is read with plain loads into its own buffer, only by
-// the tiles that hold column kz = 0.  Partial sums are written per tile, at index
-// ky * (N/2 / NL) + kz0 / NL of the system, so the finishers sum them in a fixed order.
-// ------------------------------------------------------------------------------------------
-// lines per tile of the staged x passes: the largest divisor of N/2 up to the 128-byte row that
-// keeps the copies 16-byte aligned and lets STG stages of NS tiles fit in shared memory
-template <class R, int N, int NS, int STG> constexpr int xtma_lines() {
-  int d = cmin(N / 2, tile_lines<R>());
-  while (d > 1 && ((N / 2) % d != 0 || (2 * d * (int)sizeof(typename Store<R>::S)) % 16 != 0 ||
-                   (long)STG * NS * N * d * (long)sizeof(cx<R>) + 2L * N * (long)sizeof(cx<R>) > 200L * 1024))
-    --d;
-  return d;
-}
-
-// shared memory of a staged x pass: STG stages of NS tiles, the twiddles, the partner line, one
-// tile of Fourier-table entries and the barriers
-template <class R, int N, int NL, int STG, int NS>
-struct TXG {
-  using G = TG<R, N, NL, STG>;
-  static constexpr size_t SMEM = 128 + (size_t)STG * NS * G::SSTR * sizeof(cx<R>) + 2 * (size_t)N * sizeof(cx<R>) +
-                                 (size_t)N * NL * sizeof(typename Store<R>::S) + 16 * STG;
-};
-
-// Row copies of a dense x-pass tile (M rows of NL elements, row i at g + i rowstride) as 16-byte
-// pieces, each thread a fixed share: per-thread asynchronous copies in, plain vector stores out.
-template <class G, class R, class ST>
-WF_D void tile_rows_async(cx<R>* tile, const ST* g, size_t rowstride, int tid) {
-  constexpr int VW = 16 / (int)sizeof(ST), NV = G::NL / VW, NVEC = G::M * NV;
-  static_assert(G::NL % VW == 0, "whole 16-byte pieces per row");
-#pragma unroll 4
-  for (int idx = tid; idx < NVEC; idx += G::NT) {
-    const int i = idx / NV, v = (idx % NV) * VW;
-    cp_async16(tile + i * G::NL + v, g + (size_t)i * rowstride + v);
-  }
-}
-template <class G, class R, class ST>
-WF_D void tile_rows_store(const cx<R>* tile, ST* g, size_t rowstride, int tid) {
-  constexpr int VW = 16 / (int)sizeof(ST), NV = G::NL / VW, NVEC = G::M * NV;
-#pragma unroll 4
-  for (int idx = tid; idx < NVEC; idx += G::NT) {
-    const int i = idx / NV, v = (idx % NV) * VW;
-    *reinterpret_cast<float4*>(g + (size_t)i * rowstride + v) = *reinterpret_cast<const float4*>(tile + i * G::NL + v);
-  }
-}
-
-// The multiplier pair of the packed column (slot 0 of each row) with its partner line held in
-// `part` (element kx at part[kx]).  Must be called by all threads; synchronises.
-template <class R, int N, int LD, class TAB>
-WF_D void combine_col0_sep(cx<R>* tile, const cx<R>* part, int ky_s, const TAB* tab, int tid, int nt) {
-  constexpr int NH = N / 2;
-  for (int kx = tid; kx < N; kx += nt) {
-    const int kxs = sfreq(kx, N);
-    const int n2 = kxs * kxs + ky_s * ky_s;
-    const R m0 = tab_to<R>(tab[n2]);
-    const R mN = tab_to<R>(tab[n2 + NH * NH]);
-    const R h = RT<R>::c(0.5);
-    const R a = (m0 + mN) * h, b = (m0 - mN) * h;
-    const cx<R> zc = tile[kx * LD];
-    const cx<R> zp = conj(part[(N - kx) % N]);
-    tile[kx * LD] = scale(zc, a) + scale(zp, b);
-  }
-  __syncthreads();
-}
-
-// x pass 1, staged (the work of k_cg_xinv):  p_new = r + beta p_old;  x += alpha_prev p_old;
-// T = IFFT_x(c (.) p_new);  partial of <p_new, m p_new>.  Stage tiles: r (becomes p_new), p_old
-// (becomes c p_new, then T), x.  COPY 0: tensor copies (maps mR, mP0, mP1, mX, mT) completed on
-// the stage's barrier, tensor stores; COPY 1: per-thread asynchronous row copies completed by
-// copy groups, plain stores (the maps are unused).
-template <class R, int N, bool UNIT_M, int NL, int STG, int RMAX, int EX, int COPY>
-__global__ void __launch_bounds__(TG<R, N, NL, STG, EX>::NT)
-k_cg_xinv_tma(const __grid_constant__ CUtensorMap mR, const __grid_constant__ CUtensorMap mP0,
-              const __grid_constant__ CUtensorMap mP1, const __grid_constant__ CUtensorMap mX,
-              const __grid_constant__ CUtensorMap mT, const typename Store<R>::T* __restrict__ r,
-              typename Store<R>::T* P0, typename Store<R>::T* P1, typename Store<R>::T* __restrict__ xg,
-              typename Store<R>::T* __restrict__ Tg,
-              const typename Store<R>::S* __restrict__ ctab, const typename Store<R>::S* __restrict__ mtab,
-              const typename Store<R>::T* __restrict__ twtab, double* __restrict__ partials,
-              const CgScal* __restrict__ sc, Bat bt, int nb, int* __restrict__ err) {
-  using G = TG<R, N, NL, STG, EX>;
-  using ST = typename Store<R>::T;
-  using SS = typename Store<R>::S;
-  constexpr int NS = 3, M = N, NH = N / 2;
-  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ double red[32];
-  cx<R>* buf = reinterpret_cast<cx<R>*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
-  cx<R>* tw = buf + STG * NS * G::SSTR;
-  cx<R>* pl = tw + M;  // partner line of the packed column
-  uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<typename Store<R>::S*>(pl + M) + M * NL);
-  const int tid = threadIdx.x;
-  const TileSeq<G> seq{sc, nb * G::TPS};
-  if (tid == 0) {
-    prefetch_tensormap(&mR);
-    prefetch_tensormap(&mX);
-    prefetch_tensormap(&mT);
-    for (int s = 0; s < STG; ++s) mbar_init(&bar[s], 1);
-    mbar_init_fence();
-  }
-  __syncthreads();
-  load_tw<R, M, 2 * N>(tw, twtab, tid, G::NT);
-  const size_t rowstride = (size_t)N * NH;
-  auto issue = [&](int id, int s) {
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kz0 = (rem % G::KB) * NL;
-    if constexpr (COPY == 0) {
-      const CUtensorMap* mpo = (sc[z].lit & 1) ? &mP1 : &mP0;  // p_old
-      mbar_expect_tx(&bar[s], NS * G::TILE_BYTES);
-      for (int q = 0; q < G::NBOX; ++q) {
-        const int off = q * G::BR * NL;
-        tma_load_4d(buf + (s * NS + 0) * G::SSTR + off, &mR, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-        tma_load_4d(buf + (s * NS + 1) * G::SSTR + off, mpo, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-        tma_load_4d(buf + (s * NS + 2) * G::SSTR + off, &mX, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-      }
-    } else {
-      const size_t o = z * bt.spec + (size_t)ky * NH + kz0;
-      const ST* po = ((sc[z].lit & 1) ? P1 : P0) + o;
-      tile_rows_async<G>(buf + (s * NS + 0) * G::SSTR, r + o, rowstride, tid);
-      tile_rows_async<G>(buf + (s * NS + 1) * G::SSTR, po, rowstride, tid);
-      tile_rows_async<G>(buf + (s * NS + 2) * G::SSTR, xg + o, rowstride, tid);
-    }
-  };
-  int ids[STG];
-  ids[0] = seq.next(blockIdx.x, gridDim.x);
-  for (int j = 1; j < STG; ++j) ids[j] = seq.next(ids[j - 1] < seq.total ? ids[j - 1] + gridDim.x : seq.total, gridDim.x);
-  unsigned pending = 0, phase = 0;
-  for (int j = 0; j < STG - 1; ++j) {
-    if (COPY == 0 && tid == 0 && ids[j] < seq.total) {
-      issue(ids[j], j);
-      pending |= 1u << j;
-    }
-    if constexpr (COPY == 1) {
-      if (ids[j] < seq.total) issue(ids[j], j);
-      cp_async_commit();
-    }
-  }
-  // Fourier-table entries of this thread's elements, one tile ahead: the next tile's are gathered
-  // while the current one is processed, so their latency overlaps the work
-  constexpr int PER = G::E;  // elements per thread: M NL / NT
-  SS cv[PER], mv[PER], cn[PER], mn[PER];
-  auto gather = [&](int id, SS* c, SS* m) {
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kz0 = (rem % G::KB) * NL;
-    const int ky_s = sfreq(ky, N);
-    const SS* ctz = ctab + z * bt.tab;
-    const SS* mtz = mtab + z * bt.tab;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int e = tid + k * G::NT, i = e / NL, kz = kz0 + e % NL;
-      const int kxs = sfreq(i, N);
-      const int n2 = kxs * kxs + ky_s * ky_s + kz * kz;
-      c[k] = ctz[n2];
-      m[k] = UNIT_M ? (SS)1 : mtz[n2];
-    }
-  };
-  if (ids[0] < seq.total) gather(ids[0], cv, mv);
-  bool ok = true;
-  for (int k = 0; ids[0] < seq.total; ++k) {
-    const int s = k % STG;
-    if constexpr (COPY == 0) {
-      if (tid == 0 && ids[STG - 1] < seq.total) {
-        bulk_wait_read<0>();
-        issue(ids[STG - 1], (k + STG - 1) % STG);
-        pending |= 1u << ((k + STG - 1) % STG);
-      }
-    } else {
-      if (ids[STG - 1] < seq.total) issue(ids[STG - 1], (k + STG - 1) % STG);
-      cp_async_commit();
-    }
-    const int id = ids[0];
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kb = rem % G::KB, kz0 = kb * NL;
-    const int ky_s = sfreq(ky, N);
-    const CgScal& S = sc[z];
-    const SS beta = (SS)S.beta, alpha_prev = (SS)S.alpha_prev;
-    const size_t o = z * bt.spec + (size_t)ky * NH + kz0;
-    const SS* ct = ctab + z * bt.tab;
-    const SS* mt = mtab + z * bt.tab;
-    // partner line of column 0: p_new at (kx, -ky, 0), recomputed from the inputs (plain loads,
-    // in flight while the tiles arrive)
-    if (kz0 == 0) {
-      const ST* pold = ((S.lit & 1) ? P1 : P0) + z * bt.spec;
-      const ST* rz = r + z * bt.spec;
-      const size_t pb = (size_t)((N - ky) % N) * NH;
-      for (int i = tid; i < M; i += G::NT) {
-        const size_t e = pb + (size_t)i * N * NH;
-        const ST rv = rz[e], po = pold[e];
-        pl[i] = cx<R>{rv.x + beta * po.x, rv.y + beta * po.y};
-      }
-    }
-    if (STG > 1 && ids[1] < seq.total) gather(ids[1], cn, mn);
-    if constexpr (COPY == 0) {
-      ok = tile_arrived<STG>(bar, s, phase, pending, err);
-      if (!ok) break;
-    } else {
-      cp_async_wait<STG - 1>();
-      __syncthreads();
-    }
-    cx<R>* tr = buf + (s * NS + 0) * G::SSTR;  // r -> p_new
-    cx<R>* tp = buf + (s * NS + 1) * G::SSTR;  // p_old -> c p_new -> T
-    cx<R>* tx = buf + (s * NS + 2) * G::SSTR;  // x
-    typename AccFor<SS>::T acc;  // <p_new, m p_new> over the columns kz != 0 (weight 2)
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int e = tid + k * G::NT, kz = kz0 + e % NL;
-      const cx<R> rv = tr[e], po = tp[e], xv = tx[e];
-      const cx<R> pn = cx<R>{rv.x + beta * po.x, rv.y + beta * po.y};
-      tx[e] = cx<R>{xv.x + alpha_prev * po.x, xv.y + alpha_prev * po.y};
-      tr[e] = pn;
-      if (kz != 0) {
-        acc.add((SS)2 * mv[k] * (pn.x * pn.x + pn.y * pn.y));
-        tp[e] = cx<R>{pn.x * cv[k], pn.y * cv[k]};
-      } else {
-        tp[e] = pn;  // the packed column stays raw for the pair combine
-      }
-    }
-    if constexpr (COPY == 0) {
-      fence_proxy_async();
-      __syncthreads();
-      if (tid == 0) {  // p_new and x are final: store them while T is transformed
-        const CUtensorMap* mpn = (S.lit & 1) ? &mP0 : &mP1;
-        for (int q = 0; q < G::NBOX; ++q) {
-          tma_store_4d(mpn, 2 * kz0, ky, q * G::BR, z, tr + q * G::BR * NL);
-          tma_store_4d(&mX, 2 * kz0, ky, q * G::BR, z, tx + q * G::BR * NL);
-        }
-      }
-    } else {
-      __syncthreads();
-      tile_rows_store<G>(tr, ((S.lit & 1) ? P0 : P1) + o, rowstride, tid);
-      tile_rows_store<G>(tx, xg + o, rowstride, tid);
-    }
-    if (kz0 == 0) {
-      // m term of the packed column (weight 1): m0 |P0|^2 + mN |PN|^2 of its two planes
-      for (int kx = tid; kx < N; kx += G::NT) {
-        const int kxs = sfreq(kx, N);
-        const int n2 = kxs * kxs + ky_s * ky_s;
-        const cx<R> zc = tp[kx * NL];
-        const cx<R> zp = pl[(N - kx) % N];
-        const SS h = (SS)0.5;
-        const SS a0 = h * (zc.x + zp.x), b0 = h * (zc.y - zp.y);
-        const SS aN = h * (zc.y + zp.y), bN = h * (zp.x - zc.x);
-        acc.add(mt[n2] * (a0 * a0 + b0 * b0) + mt[n2 + NH * NH] * (aN * aN + bN * bN));
-      }
-      combine_col0_sep<R, N, NL>(tp, pl, ky_s, ct, tid, G::NT);
-    }
-    fft_line<R, M, G::TPL, NL, +1, 1, cmin(RMAX, rmax_for(M, G::TPL))>(tp + tid % NL, tid / NL, tw);
-    if constexpr (COPY == 0) {
-      fence_proxy_async();
-      __syncthreads();
-      if (tid == 0) {
-        for (int q = 0; q < G::NBOX; ++q) tma_store_4d(&mT, 2 * kz0, ky, q * G::BR, z, tp + q * G::BR * NL);
-        bulk_commit();
-      }
-    } else {
-      tile_rows_store<G>(tp, Tg + o, rowstride, tid);
-    }
-    const double sum = block_sum(acc.get(), red);
-    if (tid == 0) partials[z * bt.part + ky * G::KB + kb] = sum;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      cv[j] = cn[j];
-      mv[j] = mn[j];
-    }
-    for (int j = 0; j < STG - 1; ++j) ids[j] = ids[j + 1];
-    ids[STG - 1] = seq.next(ids[STG - 2] < seq.total ? ids[STG - 2] + gridDim.x : seq.total, gridDim.x);
-  }
-  if (COPY == 0 && tid == 0) tiles_drain<STG>(bar, phase, pending, ok);
-  if constexpr (COPY == 1) cp_async_wait<0>();
-}
-
-// x pass 2, staged (the work of k_cg_xupd):  T^ = FFT_x(T);  q = m p + c T^;  r -= alpha q;
-// partials of <r, r> and ||C^-1 r||^2 (two per tile).  Stage tiles: T, r, p_new.  COPY as for
-// x pass 1.
-template <class R, int N, bool UNIT_M, int NL, int STG, int RMAX, int EX, int COPY>
-__global__ void __launch_bounds__(TG<R, N, NL, STG, EX>::NT)
-k_cg_xupd_tma(const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mR,
-              const __grid_constant__ CUtensorMap mP0, const __grid_constant__ CUtensorMap mP1,
-              const typename Store<R>::T* __restrict__ T, const typename Store<R>::T* P0,
-              const typename Store<R>::T* P1, typename Store<R>::T* __restrict__ rg,
-              const typename Store<R>::S* __restrict__ ctab,
-              const typename Store<R>::S* __restrict__ mtab, const typename Store<R>::T* __restrict__ twtab,
-              double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt, int nb, int* __restrict__ err) {
-  using G = TG<R, N, NL, STG, EX>;
-  using ST = typename Store<R>::T;
-  using SS = typename Store<R>::S;
-  constexpr int NS = 3, M = N, NH = N / 2;
-  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ double red[32];
-  cx<R>* buf = reinterpret_cast<cx<R>*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
-  cx<R>* tw = buf + STG * NS * G::SSTR;
-  cx<R>* pl = tw + M;  // partner line of the packed column
-  typename Store<R>::S* ctile = reinterpret_cast<typename Store<R>::S*>(pl + M);  // c(k) of the tile
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ctile + M * NL);
-  const int tid = threadIdx.x;
-  const TileSeq<G> seq{sc, nb * G::TPS};
-  if (tid == 0) {
-    prefetch_tensormap(&mT);
-    prefetch_tensormap(&mR);
-    for (int s = 0; s < STG; ++s) mbar_init(&bar[s], 1);
-    mbar_init_fence();
-  }
-  __syncthreads();
-  load_tw<R, M, 2 * N>(tw, twtab, tid, G::NT);
-  const size_t rowstride = (size_t)N * NH;
-  auto issue = [&](int id, int s) {
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kz0 = (rem % G::KB) * NL;
-    if constexpr (COPY == 0) {
-      const CUtensorMap* mp = (sc[z].lit & 1) ? &mP0 : &mP1;  // this iteration's p_new
-      mbar_expect_tx(&bar[s], NS * G::TILE_BYTES);
-      for (int q = 0; q < G::NBOX; ++q) {
-        const int off = q * G::BR * NL;
-        tma_load_4d(buf + (s * NS + 0) * G::SSTR + off, &mT, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-        tma_load_4d(buf + (s * NS + 1) * G::SSTR + off, &mR, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-        tma_load_4d(buf + (s * NS + 2) * G::SSTR + off, mp, 2 * kz0, ky, q * G::BR, z, &bar[s]);
-      }
-    } else {
-      const size_t o = z * bt.spec + (size_t)ky * NH + kz0;
-      tile_rows_async<G>(buf + (s * NS + 0) * G::SSTR, T + o, rowstride, tid);
-      tile_rows_async<G>(buf + (s * NS + 1) * G::SSTR, rg + o, rowstride, tid);
-      tile_rows_async<G>(buf + (s * NS + 2) * G::SSTR, ((sc[z].lit & 1) ? P0 : P1) + o, rowstride, tid);
-    }
-  };
-  int ids[STG];
-  ids[0] = seq.next(blockIdx.x, gridDim.x);
-  for (int j = 1; j < STG; ++j) ids[j] = seq.next(ids[j - 1] < seq.total ? ids[j - 1] + gridDim.x : seq.total, gridDim.x);
-  unsigned pending = 0, phase = 0;
-  for (int j = 0; j < STG - 1; ++j) {
-    if (COPY == 0 && tid == 0 && ids[j] < seq.total) {
-      issue(ids[j], j);
-      pending |= 1u << j;
-    }
-    if constexpr (COPY == 1) {
-      if (ids[j] < seq.total) issue(ids[j], j);
-      cp_async_commit();
-    }
-  }
-  // c(k) of this thread's elements, one tile ahead (gathered while the current tile is processed)
-  constexpr int PER = G::E;  // elements per thread: M NL / NT
-  SS cv[PER], cn[PER];
-  auto gather = [&](int id, SS* c) {
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kz0 = (rem % G::KB) * NL;
-    const int ky_s = sfreq(ky, N);
-    const SS* ctz = ctab + z * bt.tab;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int e = tid + k * G::NT, i = e / NL, kz = kz0 + e % NL;
-      const int kxs = sfreq(i, N);
-      c[k] = ctz[kxs * kxs + ky_s * ky_s + kz * kz];
-    }
-  };
-  if (ids[0] < seq.total) gather(ids[0], cv);
-  bool ok = true;
-  for (int k = 0; ids[0] < seq.total; ++k) {
-    const int s = k % STG;
-    if constexpr (COPY == 0) {
-      if (tid == 0 && ids[STG - 1] < seq.total) {
-        bulk_wait_read<0>();
-        issue(ids[STG - 1], (k + STG - 1) % STG);
-        pending |= 1u << ((k + STG - 1) % STG);
-      }
-    } else {
-      if (ids[STG - 1] < seq.total) issue(ids[STG - 1], (k + STG - 1) % STG);
-      cp_async_commit();
-    }
-    const int id = ids[0];
-    const int z = id / G::TPS, rem = id % G::TPS, ky = rem / G::KB, kb = rem % G::KB, kz0 = kb * NL;
-    const int ky_s = sfreq(ky, N), pky = (N - ky) % N;
-    const CgScal& S = sc[z];
-    const SS alpha = (SS)S.alpha;
-    const SS* ct = ctab + z * bt.tab;
-    const SS* mt = mtab + z * bt.tab;
-    const ST* p = ((S.lit & 1) ? P0 : P1) + z * bt.spec;
-    if (kz0 == 0) {  // partner line of T at -ky, column 0 (plain loads)
-      const ST* Tz = T + z * bt.spec;
-      for (int i = tid; i < M; i += G::NT) pl[i] = ld_c<R>(Tz + (size_t)pky * NH + (size_t)i * N * NH);
-    }
-    if (STG > 1 && ids[1] < seq.total) gather(ids[1], cn);
-    if constexpr (COPY == 0) {
-      ok = tile_arrived<STG>(bar, s, phase, pending, err);
-      if (!ok) break;
-    } else {
-      cp_async_wait<STG - 1>();
-      __syncthreads();
-    }
-    cx<R>* tt = buf + (s * NS + 0) * G::SSTR;
-    cx<R>* tr = buf + (s * NS + 1) * G::SSTR;
-    const cx<R>* tp = buf + (s * NS + 2) * G::SSTR;
-    fft_line<R, M, G::TPL, NL, -1, 1, cmin(RMAX, rmax_for(M, G::TPL))>(tt + tid % NL, tid / NL, tw);
-    if (kz0 == 0) {  // transform the partner line too, then apply c to column 0 as a packed pair
-      // (by all threads, a few elements each: a separate, small instance of the transform keeps
-      // the main one's register budget)
-      fft_line_map<R, M, G::NT, -1, 1, 8>(pl, Strided<1>{}, tid, tw);
-      combine_col0_sep<R, N, NL>(tt, pl, ky_s, ct, tid, G::NT);
-    }
-    typename AccFor<SS>::T a_rr, a_rc;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int e = tid + k * G::NT, i = e / NL, kz = kz0 + e % NL;
-      const cx<R> t = tt[e], pv = tp[e];
-      cx<R> rv = tr[e];
-      const SS c = cv[k];
-      SS ic2 = (SS)1 / (c * c);
-      SS q0, q1;
-      if (kz == 0) {
-        const int kxs = sfreq(i, N);
-        const int n2 = kxs * kxs + ky_s * ky_s;
-        // packed column: T^ already carries c; the m term combines p with p(-kx, -ky, 0) (in the
-        // storage type: FP64 here would run on GB300's 1/64-rate unit)
-        const SS cN = ct[n2 + NH * NH];
-        const SS i2 = (SS)1 / (cN * cN);
-        ic2 = ic2 > i2 ? ic2 : i2;
-        const SS m0 = mt[n2], mN = mt[n2 + NH * NH];
-        const SS a = (SS)0.5 * (m0 + mN), b = (SS)0.5 * (m0 - mN);
-        ST pp = ST{};
-        if (b != (SS)0) pp = p[(size_t)((N - i) % N) * N * NH + (size_t)pky * NH];
-        q0 = a * pv.x + b * pp.x + t.x;
-        q1 = a * pv.y - b * pp.y + t.y;
-      } else {
-        SS m = (SS)1;
-        if constexpr (!UNIT_M) {
-          const int kxs = sfreq(i, N);
-          m = mt[kxs * kxs + ky_s * ky_s + kz * kz];
-        }
-        q0 = m * pv.x + c * t.x;
-        q1 = m * pv.y + c * t.y;
-      }
-      rv.x -= alpha * q0;
-      rv.y -= alpha * q1;
-      tr[e] = rv;
-      const SS wgt = kz == 0 ? (SS)1 : (SS)2;
-      const SS m2 = wgt * (rv.x * rv.x + rv.y * rv.y);
-      a_rr.add(m2);
-      a_rc.add(ic2 * m2);
-    }
-    if constexpr (COPY == 0) {
-      fence_proxy_async();
-      __syncthreads();
-      if (tid == 0) {
-        for (int q = 0; q < G::NBOX; ++q) tma_store_4d(&mR, 2 * kz0, ky, q * G::BR, z, tr + q * G::BR * NL);
-        bulk_commit();
-      }
-    } else {
-      __syncthreads();
-      tile_rows_store<G>(tr, rg + z * bt.spec + (size_t)ky * NH + kz0, rowstride, tid);
-    }
-    const double s1 = block_sum(a_rr.get(), red);
-    const double s2 = block_sum(a_rc.get(), red);
-    if (tid == 0) {
-      partials[z * bt.part + 2 * (ky * G::KB + kb)] = s1;
-      partials[z * bt.part + 2 * (ky * G::KB + kb) + 1] = s2;
-    }
-#pragma unroll
-    for (int j = 0; j < PER; ++j) cv[j] = cn[j];
-    for (int j = 0; j < STG - 1; ++j) ids[j] = ids[j + 1];
-    ids[STG - 1] = seq.next(ids[STG - 2] < seq.total ? ids[STG - 2] + gridDim.x : seq.total, gridDim.x);
-  }
-  if (COPY == 0 && tid == 0) tiles_drain<STG>(bar, phase, pending, ok);
-  if constexpr (COPY == 1) cp_async_wait<0>();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1401,80 +801,6 @@ WF_D void zrows_store(const cx<R>* tile, typename G::ST* g, size_t row0, int tid
     }
     *reinterpret_cast<VT*>(g + (row0 + l) * G::H + i) = v;
   }
-}
-
-// ------------------------------------------------------------------------------------------
-// z turn (middle of A p): each (x, y) line: packed -> real (C2R), times D(x, y, z), -> packed.
-// D = nbar w / V_c carries the 1/V_c of the inverse transform.  grid (N*N / NL).
-// ------------------------------------------------------------------------------------------
-template <class R, int N, int EZ = z_elems<R, N>()>
-__global__ void __launch_bounds__(ZG<R, N, EZ>::NT)
-k_zturn(typename Store<R>::T* __restrict__ spec, const typename Store<R>::S* __restrict__ D,
-        const typename Store<R>::T* __restrict__ twtab, double* __restrict__ partials, const CgScal* __restrict__ sc,
-        Bat bt) {
-  using G = ZG<R, N, EZ>;
-  using SS = typename Store<R>::S;
-  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
-  cx<R>* tw = tile + G::M * G::LD;  // 2N entries
-  __shared__ double red[32];
-  const int z = blockIdx.z;
-  if (sc && sc[z].done) return;
-  spec += z * bt.spec;
-  D += z * bt.real;
-  partials += z * bt.part;
-  const int tid = threadIdx.x;
-  const size_t row0 = (size_t)blockIdx.x * G::NL;
-  // the D rows go to L2 while the rows are transformed
-  if (tid < G::NL) prefetch_l2(D + (row0 + tid) * N, N * sizeof(SS));
-  for (int e = tid; e < 2 * N; e += G::NT) tw[e] = ld_c<R>(twtab + e);
-  zrows_load<G>(tile, spec, row0, tid);
-  __syncthreads();
-  const int l = tid % G::NL, t = tid / G::NL;
-  c2r_prep<R, N, G::LD>(tile + l, t, G::TPL, tw);
-  __syncthreads();
-  fft_line<R, G::M, G::TPL, G::LD, +1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
-  // real samples 2i, 2i+1 of line l sit in element i: multiply by D, VW elements at a time,
-  // and sum D T^2 (the <c p, D (c p)> term of <p, A p>)
-  using DV = typename std::conditional<G::VW == 2, float4, double2>::type;  // 2 VW reals of D
-  typename AccFor<SS>::T acc;
-#pragma unroll 4
-  for (int k = 0; k < G::PER; ++k) {
-    const int idx = tid + k * G::NT;
-    if (!(G::EVEN || idx < G::NVEC)) continue;
-    const int ll = idx / G::NV, i = (idx % G::NV) * G::VW;
-    const SS* dp = D + (row0 + ll) * N + 2 * i;
-    if constexpr (G::VW == 2) {
-      const float4 d = *reinterpret_cast<const float4*>(dp);
-      cx<R> a = tile[i * G::LD + ll], b = tile[(i + 1) * G::LD + ll];
-      const cx<R> a0 = a, b0 = b;
-      a.x = a.x * RT<R>::from_f(d.x);
-      a.y = a.y * RT<R>::from_f(d.y);
-      b.x = b.x * RT<R>::from_f(d.z);
-      b.y = b.y * RT<R>::from_f(d.w);
-      // D T^2 >= 0: the vector's four terms are summed first (in R = the storage type)
-      acc.add((SS)(a.x * a0.x + a.y * a0.y + b.x * b0.x + b.y * b0.y));
-      tile[i * G::LD + ll] = a;
-      tile[(i + 1) * G::LD + ll] = b;
-    } else {
-      const double2 d = *reinterpret_cast<const double2*>(dp);
-      cx<R> a = tile[i * G::LD + ll];
-      const cx<R> a0 = a;
-      a.x = a.x * RT<R>::c(d.x);
-      a.y = a.y * RT<R>::c(d.y);
-      acc.add((SS)(a.x * a0.x + a.y * a0.y));
-      tile[i * G::LD + ll] = a;
-    }
-  }
-  (void)sizeof(DV);
-  __syncthreads();
-  fft_line<R, G::M, G::TPL, G::LD, -1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
-  r2c_post<R, N, G::LD>(tile + l, t, G::TPL, tw);
-  __syncthreads();
-  zrows_store<G>(tile, spec, row0, tid);
-  const double sum = block_sum(acc.get(), red);
-  if (tid == 0) partials[blockIdx.x] = sum;
 }
 
 // ------------------------------------------------------------------------------------------
