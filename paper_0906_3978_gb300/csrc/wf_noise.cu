@@ -17,6 +17,7 @@
 #include <utility>
 
 #include "wf_ctx.h"
+#include "wf_fp64fn.cuh"
 #include "wf_spectral.cuh"
 
 namespace wf {
@@ -60,23 +61,90 @@ WF_D double sel_value(const SelParams& s, const double4* __restrict__ holes, dou
   return val;
 }
 
+// The window at the nodes.  The plain formula costs ~75 FP64 operations a node, all on the 1/64-rate pipe
+// (256^3: 1.97 ms, here 0.82).  The cone and hole tests are first taken in FP32: a node whose margin exceeds
+// 2^-20 r (|a_x| + |a_y| + |a_z| + |cos|), more than twice the FP32 error of dot and cos r (each a few
+// 2^-24 relative, the approximate square root 2^-22), is decided there, and only the others repeat the exact
+// test of sel_value, operation by operation.  What depends on one axis alone (offset, its square, its term of
+// the axis product, each rounded as in the definition) comes from tables of the CTA, and the value of an
+// observed node takes the FP64 functions of wf_fp64fn.cuh (~30 operations).  Lengths beyond 1e12 or below
+// 1e-12 and exponents beyond +-700 go through the plain formula.
+struct AxisTab {
+  double d, d2, da;  // i H - o, its square, its product with the cone's axis component
+  float f;           // d in FP32
+  int pad;
+};
+constexpr int kWindowMaxN = 512;  // largest grid: the shared-memory limit is set for it, whatever the call's size
+constexpr size_t window_smem(int n) { return sizeof(FnTables) + 3 * (size_t)n * sizeof(AxisTab); }
 __global__ void __launch_bounds__(256)
 k_window(int n, SelParams s, const double4* __restrict__ holes, double* __restrict__ w,
          double* __restrict__ partials) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
-  const size_t V = (size_t)n * n * n;
+  FnTables& fn = *reinterpret_cast<FnTables*>(smem_raw);
+  AxisTab* tab = reinterpret_cast<AxisTab*>(smem_raw + sizeof(FnTables));
+  const int tid = threadIdx.x, lane = tid & 31;
+  make_fn_tables(fn, tid, blockDim.x);
+  for (int e = tid; e < 3 * n; e += blockDim.x) {
+    const int a = e / n, i = e - a * n;
+    const double d = __dsub_rn(__dmul_rn((double)i, s.H), a == 0 ? s.ox : a == 1 ? s.oy : s.oz);
+    tab[e] = AxisTab{d, __dmul_rn(d, d), __dmul_rn(d, a == 0 ? s.ax : a == 1 ? s.ay : s.az), (float)d, 0};
+  }
+  __syncthreads();
+  const float axf = (float)s.ax, ayf = (float)s.ay, azf = (float)s.az, chf = (float)s.cos_half;
+  const float eps = 9.5367431640625e-7f;  // 2^-20
+  const float ceps = eps * (fabsf(axf) + fabsf(ayf) + fabsf(azf) + fabsf(chf));
+  const double ip0 = s.kind ? 1.0 / s.p0 : 0.0;
+  const bool p0_ok = s.kind == 0 || (s.p0 > 1e-100 && s.p0 < 1e100);
   AccD acc;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < V; e += (size_t)gridDim.x * blockDim.x) {
-    const int iz = (int)(e % n), iy = (int)((e / n) % n), ix = (int)(e / ((size_t)n * n));
-    const double val = sel_value(s, holes, __dsub_rn(__dmul_rn((double)ix, s.H), s.ox),
-                                 __dsub_rn(__dmul_rn((double)iy, s.H), s.oy),
-                                 __dsub_rn(__dmul_rn((double)iz, s.H), s.oz));
-    w[e] = val;
-    acc.add(val);
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  for (int row = blockIdx.x * (blockDim.x >> 5) + (tid >> 5); row < n * n; row += nw) {  // a warp per (x, y) row
+    const AxisTab X = tab[row / n], Y = tab[n + row % n];
+    const double r2xy = __dadd_rn(X.d2, Y.d2), dxy = __dadd_rn(X.da, Y.da);
+    const float f2 = fmaf(X.f, X.f, Y.f * Y.f), fd = fmaf(X.f, axf, Y.f * ayf);
+    double* out = w + (size_t)row * n;
+    for (int iz = lane; iz < n; iz += 32) {
+      const AxisTab& Z = tab[2 * n + iz];
+      const float r2f = fmaf(Z.f, Z.f, f2), rf = r2f * rsqrtf(r2f);
+      double val = 0.0;
+      if (!(rf > 1e-12f && rf < 1e12f) || !p0_ok) {
+        val = sel_value(s, holes, X.d, Y.d, Z.d);
+        acc.add(val);
+      } else {
+        const double r2 = __dadd_rn(r2xy, Z.d2);
+        const float side = fmaf(Z.f, azf, fd) - chf * rf;
+        bool inside = side > ceps * rf;
+        if (!inside && !(side < -ceps * rf)) inside = __dadd_rn(dxy, Z.da) >= __dmul_rn(s.cos_half, __dsqrt_rn(r2));
+        for (int h = 0; h < s.n_holes && inside; ++h) {
+          const double4 hv = holes[h];
+          const float hx = (float)hv.x, hy = (float)hv.y, hz = (float)hv.z, hw = (float)hv.w;
+          const float in = fmaf(X.f, hx, fmaf(Y.f, hy, Z.f * hz)) - hw * rf;
+          const float m = eps * (fabsf(hx) + fabsf(hy) + fabsf(hz) + fabsf(hw)) * rf;
+          if (in > m) inside = false;
+          else if (!(in < -m))
+            inside = !(__dadd_rn(__dadd_rn(__dmul_rn(X.d, hv.x), __dmul_rn(Y.d, hv.y)), __dmul_rn(Z.d, hv.z)) >
+                       __dmul_rn(hv.w, __dsqrt_rn(r2)));
+        }
+        if (inside) {
+          if (s.kind == 0) {
+            val = 1.0;
+          } else {
+            const double r = sqrt_fast(r2);
+            double t = r * ip0;
+            t = fma(fma(-t, s.p0, r), ip0, t);
+            const double x = s.kind == 1 ? -(t * t) : s.p1 * (log_fast(t, fn.lg) + (1.0 - t));
+            val = fabs(x) < 700.0 ? exp_fast(x, fn.ex) : exp(x);
+          }
+          acc.add(val);
+        }
+      }
+      out[iz] = val;
+    }
   }
   const double sum = block_sum(acc.get(), red);
   if (threadIdx.x == 0) partials[blockIdx.x] = sum;
 }
+constexpr int kWindowBlocks = 152 * 4;
 
 // The selection at arbitrary positions pos[3 i] (the completeness at a galaxy), or its
 // reciprocal (0 where w = 0), the galaxy mass of the inverse-weighting estimator.
@@ -428,14 +496,15 @@ wf_status noise_run(Ctx& c, const wf_grid& g, const wf_selection& sel, const dou
   double4* dh;
   WF_TRY(c.get("holes", hh.size() * sizeof(double4), (void**)&dh));
   WF_CUDA(cudaMemcpyAsync(dh, hh.data(), hh.size() * sizeof(double4), cudaMemcpyHostToDevice, st));
-  const int grid = 152 * 8;
+  const int grid = 152 * 8, wgrid = kWindowBlocks;
   double *part, *scal;
   WF_TRY(c.get("noise_part", grid * sizeof(double), (void**)&part));
   WF_TRY(c.get("noise_scal", 4 * sizeof(double), (void**)&scal));
   const size_t V = (size_t)n * n * n;
-  c.launch("window", 8.0 * V, st, [&] { k_window<<<grid, 256, 0, st>>>(n, s, dh, w, part); });
+  WF_CUDA(cudaFuncSetAttribute(k_window, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)window_smem(kWindowMaxN)));
+  c.launch("window", 8.0 * V, st, [&] { k_window<<<wgrid, 256, window_smem(n), st>>>(n, s, dh, w, part); });
   WF_CUDA(cudaGetLastError());
-  c.launch("fin", 0, st, [&] { k_nbar<<<1, 1024, 0, st>>>(part, grid, (double)n_gal, scal); });
+  c.launch("fin", 0, st, [&] { k_nbar<<<1, 1024, 0, st>>>(part, wgrid, (double)n_gal, scal); });
   WF_CUDA(cudaGetLastError());
   c.launch("data", 8.0 * V * (d ? 4 : 3), st, [&] { k_data<<<grid, 256, 0, st>>>(n_obs, w, scal, d, b, V); });
   WF_CUDA(cudaGetLastError());
@@ -567,9 +636,11 @@ extern "C" wf_status wf_build_noise_noalloc(const wf_grid* grid, const wf_select
   // every partial and scalar below is written before it is read: nothing in the scratch
   // needs clearing between calls
   const size_t V = (size_t)n * n * n;
-  k_window<<<kNoallocParts, 256, 0, st>>>(n, s, dh, w, part);
+  static_assert(kWindowBlocks <= kNoallocParts, "partial sums");
+  WF_CUDA(cudaFuncSetAttribute(k_window, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)window_smem(kWindowMaxN)));
+  k_window<<<kWindowBlocks, 256, window_smem(n), st>>>(n, s, dh, w, part);
   WF_CUDA(cudaGetLastError());
-  k_nbar<<<1, 1024, 0, st>>>(part, kNoallocParts, (double)n_gal, scal);
+  k_nbar<<<1, 1024, 0, st>>>(part, kWindowBlocks, (double)n_gal, scal);
   WF_CUDA(cudaGetLastError());
   k_data<<<kNoallocParts, 256, 0, st>>>(n_obs, w, scal, d, b, V);
   WF_CUDA(cudaGetLastError());
