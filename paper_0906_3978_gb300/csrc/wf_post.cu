@@ -11,9 +11,11 @@
 // definition gives; counts are integer atomics (exact whatever the order); every sum is
 // per-block partials plus a fixed-order single-CTA finisher (deterministic).
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "wf_ctx.h"
+#include "wf_fp64fn.cuh"
 #include "wf_solver_group.h"
 #include "wf_spectral.cuh"
 
@@ -24,12 +26,43 @@ constexpr int kPostBlocks = 152 * 4;  // grid of the sweeps (per-block partials)
 // ------------------------------------------------------------------------------------------
 // Sec. 4.1: sums of t r, t^2, r^2, (r - t)^2, (1 + r) log((1 + r) / (1 + t)) (where both
 // 1 + delta > 0) and the count of the cells left out of the last one.  6 partials per block.
+// Bound by the FP64 pipe: the library's quotient and logarithm made it 55 operations a cell
+// (256^3: 1.46 ms, now 0.76).
+// The table-driven logarithm (wf_fp64fn.cuh) is taken of the quotient directly: with k and the table's c
+// for an FP32 estimate of a / b, log(a / b) = k log 2 - log c + log1p((a 2^-k c - b) / b), where the
+// difference is one fused operation on a short product, so b's reciprocal needs one Newton step and the
+// quotient one correction; 24 a cell.
 // ------------------------------------------------------------------------------------------
+WF_D bool plain_range(double d) {  // positive and between 2^-500 and 2^500
+  const int hi = __double2hiint(d);
+  return hi > ((1023 - 500) << 20) && hi < ((1023 + 500) << 20);
+}
+// log(a / b) for a, b in the plain range
+WF_D double log_ratio(double a, double b, const double2* __restrict__ lg) {
+  int ea, eb;
+  const float fa = lead(a, ea), fb = lead(b, eb);
+  const float y = __frcp_rn(fb);
+  float q = fa * y;  // (1/2, 2): q 2^(ea - eb) estimates a / b
+  const int ix = __float_as_int(q) + (0x3f800000 - 0x3f400000);  // m in [3/4, 3/2)
+  const int dk = (ix >> 23) - 127, k = ea - eb + dk;
+  const double2 t = lg[(ix >> 16) & (kLogTab - 1)];
+  // a and b with their exponents taken off, a 2^-dk c - b
+  const double am = times_pow2(a, -ea - dk), bm = times_pow2(b, -eb);
+  double yb = widen(y);
+  yb = fma(fma(-bm, yb, 1.0), yb, yb);
+  const double u = fma(am, t.x, -bm);
+  double r = u * yb;
+  r = fma(fma(-bm, r, u), yb, r);  // to full precision beside a = b, where the logarithm is small
+  return fma(small_int(k), 0.69314718055994530942, t.y + log1p_short(r));
+}
 __global__ void __launch_bounds__(256)
 k_compare(const double* __restrict__ rec, const double* __restrict__ tru, size_t n, double* __restrict__ partials) {
   __shared__ double red[32];
+  __shared__ FnTables fn;
+  make_fn_tables(fn, threadIdx.x, blockDim.x);
+  __syncthreads();
   AccD tr, tt, rr, d2, kl;
-  double excl = 0.0;
+  int excl = 0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     const double r = rec[e], t = tru[e];
     tr.add_prod(t, r);
@@ -38,10 +71,11 @@ k_compare(const double* __restrict__ rec, const double* __restrict__ tru, size_t
     const double d = r - t;
     d2.add_prod(d, d);
     const double a = 1.0 + r, b = 1.0 + t;
-    if (a > 0.0 && b > 0.0) kl.add(a * log(a / b));
-    else excl += 1.0;
+    if (plain_range(a) && plain_range(b)) kl.add_prod(a, log_ratio(a, b, fn.lg));
+    else if (a > 0.0 && b > 0.0) kl.add(a * log(a / b));
+    else ++excl;
   }
-  const double v[6] = {tr.get(), tt.get(), rr.get(), d2.get(), kl.get(), excl};
+  const double v[6] = {tr.get(), tt.get(), rr.get(), d2.get(), kl.get(), (double)excl};
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
     const double s = block_sum(v[j], red);
@@ -69,38 +103,72 @@ __global__ void k_compare_fin(const double* __restrict__ partials, int nblk, dou
 // ------------------------------------------------------------------------------------------
 struct DensArgs {
   int n, n_shells, n_bins;
-  double H, ox, oy, oz, lo, width;
-  double shells[16];
+  double H, ox, oy, oz, lo, width, inv_width;
+  double shells[16];     // the shells' radii
+  long long r2_from[16]; // bits of the smallest double whose square root is at least that radius
 };
 
+// Bound by the FP64 pipe: a division, a floor and a square root a node made it 55 operations (256^3: 1.46 ms); 8
+// remain (0.25 ms).  The bin floor(fl(x / width)) is that of x (1 / width) unless the latter lies within 2^-40 of
+// an integer (relative to its size), where the division is repeated.  A shell's r >= s is taken on r^2: the
+// square root is monotone, so it holds from one double on, found on the host; r^2 is one addition, since
+// (dx^2 + dy^2) belongs to the row and dz^2 to a table.
 __global__ void __launch_bounds__(256)
 k_density_hist(const double* __restrict__ delta, const double* __restrict__ w, DensArgs a,
                unsigned long long* __restrict__ hist) {
-  extern __shared__ unsigned int cnt[];  // [n_shells][2][n_bins + 2]
-  const int nb2 = a.n_bins + 2, tot = a.n_shells * 2 * nb2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* sqr = reinterpret_cast<double*>(smem_raw);                    // [3][n]: squared offsets per axis
+  unsigned int* cnt = reinterpret_cast<unsigned int*>(sqr + 3 * a.n);   // [n_shells][2][n_bins + 2]
+  const int nb2 = a.n_bins + 2, tot = a.n_shells * 2 * nb2, n = a.n;
   for (int i = threadIdx.x; i < tot; i += blockDim.x) cnt[i] = 0u;
+  for (int e = threadIdx.x; e < 3 * n; e += blockDim.x) {
+    const int ax = e / n;
+    const double d = __dsub_rn(__dmul_rn((double)(e - ax * n), a.H), ax == 0 ? a.ox : ax == 1 ? a.oy : a.oz);
+    sqr[e] = __dmul_rn(d, d);
+  }
   __syncthreads();
-  const unsigned un = (unsigned)a.n, V = un * un * un;
-  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < V; e += gridDim.x * blockDim.x) {
-    const double q = floor(__ddiv_rn(__dsub_rn(__dadd_rn(1.0, delta[e]), a.lo), a.width));
-    int slot;
-    if (q < 0.0) slot = a.n_bins;
-    else if (q >= (double)a.n_bins) slot = a.n_bins + 1;
-    else if (q >= 0.0) slot = (int)q;
-    else continue;  // NaN: in no bin
-    const unsigned row = e / un;
-    const int iz = (int)(e - row * un), iy = (int)(row % un), ix = (int)(row / un);
-    const double dx = __dsub_rn(__dmul_rn((double)ix, a.H), a.ox);
-    const double dy = __dsub_rn(__dmul_rn((double)iy, a.H), a.oy);
-    const double dz = __dsub_rn(__dmul_rn((double)iz, a.H), a.oz);
-    const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
-    const int g = w[e] > 0.0 ? 0 : 1;
-    for (int s = 0; s < a.n_shells; ++s)
-      if (r >= a.shells[2 * s] && r < a.shells[2 * s + 1]) atomicAdd(&cnt[(s * 2 + g) * nb2 + slot], 1u);
+  const double magic = 6755399441055744.0;  // 2^52 + 2^51: adding it leaves the nearest integer in the low word
+  const int nw = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
+  for (int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n * n; row += nw) {  // a warp per (x, y)
+    const double xy2 = __dadd_rn(sqr[row / n], sqr[n + row % n]);
+    const size_t e0 = (size_t)row * n;
+    for (int iz = lane; iz < n; iz += 32) {
+      const double x = __dsub_rn(__dadd_rn(1.0, delta[e0 + iz]), a.lo), p = x * a.inv_width;
+      const long long wb = __double_as_longlong(w[e0 + iz]);
+      const double f = p + magic, dist = p - (f - magic);  // distance from the nearest integer (|p| < 2^31)
+      const int near = __double2loint(f), ep = (__double2hiint(p) >> 20) & 0x7ff, ed = (__double2hiint(dist) >> 20) & 0x7ff;
+      int slot;
+      // |p| < 2^30, and dist is no smaller than 2^-40 max(1, |p|): the floor is decided
+      if (ep < 1023 + 30 && ed >= max(ep, 1023) - 40) {
+        const int q = near - (__double2hiint(dist) < 0 ? 1 : 0);
+        slot = q < 0 ? a.n_bins : (q >= a.n_bins ? a.n_bins + 1 : q);
+      } else {
+        const double q = floor(__ddiv_rn(x, a.width));
+        if (q < 0.0) slot = a.n_bins;
+        else if (q >= (double)a.n_bins) slot = a.n_bins + 1;
+        else if (q >= 0.0) slot = (int)q;
+        else continue;  // NaN: in no bin
+      }
+      const long long r2 = __double_as_longlong(__dadd_rn(xy2, sqr[2 * n + iz]));
+      const int g = wb > 0 && wb <= 0x7ff0000000000000ll ? 0 : 1;  // w > 0
+      for (int s = 0; s < a.n_shells; ++s)
+        if (r2 >= a.r2_from[2 * s] && r2 < a.r2_from[2 * s + 1]) atomicAdd(&cnt[(s * 2 + g) * nb2 + slot], 1u);
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < tot; i += blockDim.x)
     if (cnt[i]) atomicAdd(&hist[i], (unsigned long long)cnt[i]);
+}
+// bits of the smallest double r2 >= 0 with sqrt(r2) >= s (comparable as integers; s is no NaN)
+static long long shell_from(double s) {
+  double t = s > 0.0 ? s * s : 0.0;
+  if (s > 0.0) {
+    while (t > 0.0 && std::sqrt(std::nextafter(t, 0.0)) >= s) t = std::nextafter(t, 0.0);
+    while (std::sqrt(t) < s) t = std::nextafter(t, INFINITY);
+  }
+  long long b;
+  std::memcpy(&b, &t, sizeof b);
+  return b;
 }
 
 // One CTA per (shell, region): N, mean, mu2..mu4, skewness, kurtosis, Pearson's skewness from the
@@ -292,9 +360,11 @@ wf_status density_run(Ctx& c, const wf_grid& g, const double* delta, const doubl
   a.oz = observer[2];
   a.lo = lo;
   a.width = width;
+  a.inv_width = std::isnormal(1.0 / width) ? 1.0 / width : NAN;  // NAN: every bin by division
   for (int i = 0; i < 16; ++i) a.shells[i] = i < 2 * n_shells ? shells[i] : 0.0;
   for (int i = 0; i < 2 * n_shells; ++i)
     if (std::isnan(shells[i])) return WF_ERR_ARG;
+  for (int i = 0; i < 16; ++i) a.r2_from[i] = shell_from(a.shells[i]);
   const int nb2 = n_bins + 2, slots = n_shells * 2 * nb2;
   unsigned long long *dh, *hh;
   double *dm, *hm;
@@ -304,7 +374,10 @@ wf_status density_run(Ctx& c, const wf_grid& g, const double* delta, const doubl
   WF_TRY(c.get_pinned("post_mom_h", (size_t)n_shells * 2 * 8 * sizeof(double), (void**)&hm));
   WF_CUDA(cudaMemsetAsync(dh, 0, (size_t)slots * sizeof(unsigned long long), st));
   const size_t V = (size_t)g.n * g.n * g.n;
-  const size_t smem = (size_t)slots * sizeof(unsigned int);
+  const size_t smem = (size_t)slots * sizeof(unsigned int) + 3 * (size_t)g.n * sizeof(double);
+  // the limit for every call (2 x 6144 counters, 512 nodes an axis): calls of other sizes may set it meanwhile
+  constexpr int smem_max = 2 * 6144 * (int)sizeof(unsigned int) + 3 * 512 * (int)sizeof(double);
+  WF_CUDA(cudaFuncSetAttribute(k_density_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   c.launch("density_hist", 16.0 * (double)V, st,
            [&] { k_density_hist<<<kPostBlocks, 256, smem, st>>>(delta, w, a, dh); });
   c.launch("fin", 0, st, [&] { k_density_moments<<<n_shells * 2, 256, 0, st>>>(dh, n_bins, lo, width, dm); });
