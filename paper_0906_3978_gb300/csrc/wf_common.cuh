@@ -200,3 +200,29 @@ WF_D double block_sum(double v, double* red) {
     }
   return v;
 }
+
+// ------------------------------------------------------------------------------------------
+// Chained launches.  A kernel launched with programmatic stream serialisation (Ctx::chain) starts as soon as the
+// last CTA of its predecessor is done, before that one's memory is flushed and its completion signalled;
+// chain_start() waits for the latter.  Only constants (twiddles, tensor maps) may be touched before it.  Launched
+// plainly it does nothing.  (Letting the successor start earlier still, griddepcontrol.launch_dependents at the
+// start of each kernel, is slower: its waiting CTAs crowd the SMs that drain first.  Mixed solve at 64^3: 4.54 ms
+// plain, 4.33 here, 4.72 with early starts; at 512^3 290, 290, 328.)
+// ------------------------------------------------------------------------------------------
+WF_D void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The last CTA of a grid (of `total` CTAs that all call this, after thread 0 has written the CTA's partial
+// sums) gets true, with every other CTA's partial sums visible; *ticket is 0 before and after.
+WF_D bool last_cta(unsigned* ticket, unsigned total) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == total - 1;
+    if (last) {
+      *ticket = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last;
+}

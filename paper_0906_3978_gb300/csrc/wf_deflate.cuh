@@ -24,8 +24,9 @@
 //   k_xcoarse   DFT along x at the coarse modes; g = coords of (m - 1) r + c Gc, and coords of r
 //   k_defl_mu   mu = E^-1 g (one warp per mode); r -= Z mu kept aside for the x pass, which forms
 //               p = (r - Z mu) + beta p; partials of <r, Z mu>
-//   k_fin_defl  <r, z> = <r, r> - <r, Z mu>; beta = <r, z> / <r, z>_prev; alpha's numerator
-//   (x pass 1)  then k_defl_restore puts the saved coarse entries of r back
+//               and, by its last CTA, <r, z> = <r, r> - <r, Z mu>; beta = <r, z> / <r, z>_prev; alpha's
+//               numerator
+//   (x pass 1)  then the forward y pass (or k_defl_restore) puts the saved coarse entries of r back
 #pragma once
 #include "wf_spectral.cuh"
 
@@ -51,12 +52,13 @@ k_ycoarse(const typename Store<R>::T* __restrict__ gz, const typename Store<R>::
   cx<R>* a = reinterpret_cast<cx<R>*>(smem_raw);  // [N][K+1]
   cx<R>* tw = a + N * KZ;                          // tw[e] = exp(-2 pi i e / N)
   const int z = blockIdx.y;
-  if (sc[z].done) return;
+  for (int e = threadIdx.x; e < N; e += blockDim.x) tw[e] = ld_c<R>(twtab + 2 * e);
+  chain_start();
+  if (finished(sc + z)) return;
   const int x = blockIdx.x;
   gz += z * gzs + (size_t)x * N * KZ;
   gy += z * gys;
   for (int e = threadIdx.x; e < N * KZ; e += blockDim.x) a[e] = ld_c<R>(gz + e);
-  for (int e = threadIdx.x; e < N; e += blockDim.x) tw[e] = ld_c<R>(twtab + 2 * e);
   __syncthreads();
   const int nout = (2 * K + 1) * KZ;
   for (int o = threadIdx.x; o < nout; o += blockDim.x) {
@@ -91,7 +93,8 @@ k_xcoarse(const typename Store<R>::T* __restrict__ gy, const typename Store<R>::
           float* __restrict__ gco, float* __restrict__ rco, const CgScal* __restrict__ sc, Bat bt, size_t gys,
           int ncp) {
   const int z = blockIdx.y;
-  if (sc[z].done) return;
+  chain_start();
+  if (finished(sc + z)) return;
   const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (warp > nh) return;
   r += z * bt.spec;
@@ -146,6 +149,35 @@ k_xcoarse(const typename Store<R>::T* __restrict__ gy, const typename Store<R>::
   }
 }
 
+// the coarse entries of r as they were before k_defl_mu<MODE 1> (where the y pass does not put them back);
+// grid (ceil((nh + 1) / 256), systems)
+template <class R, int N>
+__global__ void k_defl_restore(typename Store<R>::T* __restrict__ r, const typename Store<R>::T* __restrict__ rsave,
+                               const int4* __restrict__ modes, int nh, const CgScal* __restrict__ sc, Bat bt) {
+  const int z = blockIdx.y;
+  chain_start();
+  if (finished(sc + z)) return;
+  const int u = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (u <= nh) restore_entry<N>(r + z * bt.spec, rsave + (size_t)z * (2 * nh + 1), modes, nh, u);
+}
+
+// <r, z> = <r, r> - <r, Z mu> (sc->rr holds <r, r> from the last x pass 2); beta = <r, z> over its
+// previous value (0 on the first iteration after the start step); alpha's numerator becomes <r, z>.
+WF_D void fin_defl(const double* dpart, int nh, CgScal* sc, double* red) {
+  const double s = sum_fresh(dpart, nh + 1, 1, red);
+  if (threadIdx.x == 0) {
+    const double rz = sc->rr - s;
+    if (!(rz > 0.0) || !isfinite(rz)) {
+      sc->done = 3;
+      return;
+    }
+    sc->beta = sc->defl == 1 ? 0.0 : rz / sc->rzo;
+    if (sc->defl == 1) sc->defl = 0;
+    sc->rzo = rz;
+    sc->rr = rz;
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // mu = E^-1 g, one warp per half-space mode (rows 1 + 2j, 2 + 2j; warp nh: row 0), and its use
 // (mu = 0 for a system with off[z] or its noco set):
@@ -159,13 +191,15 @@ template <class R, int N, int MODE>
 __global__ void __launch_bounds__(256)
 k_defl_mu(const float* __restrict__ Einv, const float* __restrict__ gco, const float* __restrict__ rco,
           const int4* __restrict__ modes, int nh, int ncp, typename Store<R>::T* __restrict__ vec,
-          typename Store<R>::T* __restrict__ rsave, double* __restrict__ dpart, const CgScal* __restrict__ sc,
+          typename Store<R>::T* __restrict__ rsave, double* __restrict__ dpart, CgScal* __restrict__ sc,
           Bat bt, const int* __restrict__ off) {
+  __shared__ double red[32];
   using ST = typename Store<R>::T;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* gs = reinterpret_cast<float*>(smem_raw);
   const int z = blockIdx.y;
-  if (sc[z].done) return;
+  chain_start();
+  if (finished(sc + z)) return;
   Einv += (size_t)z * ncp * ncp;
   gco += (size_t)z * ncp;
   rco += (size_t)z * ncp;
@@ -175,6 +209,7 @@ k_defl_mu(const float* __restrict__ Einv, const float* __restrict__ gco, const f
   for (int e = threadIdx.x; e < ncp; e += blockDim.x) gs[e] = gco[e];
   __syncthreads();
   const int warp = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  auto product = [&] {
   if (warp > nh) return;
   const int ra = warp < nh ? 1 + 2 * warp : 0;
   const float4* rowa = reinterpret_cast<const float4*>(Einv + (size_t)ra * ncp);
@@ -256,45 +291,11 @@ k_defl_mu(const float* __restrict__ Einv, const float* __restrict__ gco, const f
       st_c(vec, ld_c<R>(&o) - v);
     }
   }
-}
-
-// the coarse entries of r as they were before k_defl_mu<MODE 1>; grid (ceil((nh + 1) / 256), systems)
-template <class R, int N>
-__global__ void k_defl_restore(typename Store<R>::T* __restrict__ r, const typename Store<R>::T* __restrict__ rsave,
-                               const int4* __restrict__ modes, int nh, const CgScal* __restrict__ sc, Bat bt) {
-  const int z = blockIdx.y;
-  if (sc[z].done) return;
-  const int u = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (u > nh) return;
-  r += z * bt.spec;
-  rsave += (size_t)z * (2 * nh + 1);
-  if (u == nh) {
-    r[0] = rsave[2 * nh];
-    return;
-  }
-  const int4 md = modes[u];
-  r[dslot<N>(md.x, md.y, md.z)] = rsave[2 * u];
-  if (md.z == 0) r[dslot<N>(-md.x, -md.y, 0)] = rsave[2 * u + 1];
-}
-
-// <r, z> = <r, r> - <r, Z mu> (sc->rr holds <r, r> from the last x pass 2); beta = <r, z> over its
-// previous value (0 on the first iteration after the start step); alpha's numerator becomes
-// <r, z>.  grid = systems.
-static __global__ void k_fin_defl(const double* __restrict__ dpart, int nh, CgScal* sc) {
-  __shared__ double red[32];
-  sc += blockIdx.x;
-  if (sc->done) return;
-  const double s = sum_partials(dpart + (size_t)blockIdx.x * (nh + 1), nh + 1, 1, 0, red);
-  if (threadIdx.x == 0) {
-    const double rz = sc->rr - s;
-    if (!(rz > 0.0) || !isfinite(rz)) {
-      sc->done = 3;
-      return;
-    }
-    sc->beta = sc->defl == 1 ? 0.0 : rz / sc->rzo;
-    if (sc->defl == 1) sc->defl = 0;
-    sc->rzo = rz;
-    sc->rr = rz;
+  };
+  product();
+  if constexpr (MODE == 1) {  // the last CTA takes <r, z> and beta
+    __syncthreads();          // every warp's entry of dpart
+    if (last_cta(&sc[z].tick[2], gridDim.x)) fin_defl(dpart, nh, sc + z, red);
   }
 }
 
@@ -341,27 +342,27 @@ __global__ void k_dh_gather(const typename Store<R>::T* __restrict__ what, float
 //   (a h, b h') c c' (Im Dh(h + h') - Im Dh(h - h'))
 //   (b h, a h') c c' (Im Dh(h - h') + Im Dh(h + h'))
 //   (b h, b h') m_h [h = h'] + c c' (Re Dh(h - h') - Re Dh(h + h'))
-// grid (ncp / 16, ncp / 16, systems), 16 x 16 threads
+// E is symmetric to the last bit: the tiles above the diagonal are computed (their FP64 products bound the kernel) and
+// written twice.  grid (ncp / 16, ncp / 16, systems), 16 x 16 threads
 template <class S>
 __global__ void k_ebuild(const float2* __restrict__ dh, const S* __restrict__ ctab, const S* __restrict__ mtab,
                          const int4* __restrict__ modes, int nh, int ncp, int K, float* __restrict__ E, int tabs) {
   const int z = blockIdx.z;
   const int C = 4 * K + 1;
+  if (blockIdx.y > blockIdx.x) return;
+  __shared__ float tile[16][17];
   const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
   dh += (size_t)z * C * C * C;
   ctab += (size_t)z * tabs;
   mtab += (size_t)z * tabs;
   E += (size_t)z * ncp * ncp;
   const int nc = 2 * nh + 1;
-  if (i >= ncp || j >= ncp) return;
-  if (i >= nc || j >= nc) {
-    E[(size_t)i * ncp + j] = i == j ? 1.f : 0.f;
-    return;
-  }
   auto D = [&](int x, int y, int w) { return dh[((x + 2 * K) * C + (y + 2 * K)) * C + (w + 2 * K)]; };
   const double s2 = 1.41421356237309505;
   double v;
-  if (i == 0 && j == 0) {
+  if (i >= nc || j >= nc) {
+    v = i == j ? 1.0 : 0.0;
+  } else if (i == 0 && j == 0) {
     v = (double)mtab[0] + (double)ctab[0] * (double)ctab[0] * (double)D(0, 0, 0).x;
   } else if (i == 0 || j == 0) {
     const int c = i == 0 ? j : i;
@@ -380,6 +381,10 @@ __global__ void k_ebuild(const float2* __restrict__ dh, const S* __restrict__ ct
     else v = dg + cc * ((double)A.x - (double)B.x);
   }
   E[(size_t)i * ncp + j] = (float)v;
+  if (blockIdx.y == blockIdx.x) return;
+  tile[threadIdx.y][threadIdx.x] = (float)v;
+  __syncthreads();
+  E[(size_t)(blockIdx.x * 16 + threadIdx.y) * ncp + blockIdx.y * 16 + threadIdx.x] = tile[threadIdx.x][threadIdx.y];
 }
 
 // Condition guard.  A coarse block built and inverted in FP32 cannot hold a condition number far
@@ -559,6 +564,7 @@ WF_D void gj_tile_mma(const float (*As)[68], const float (*Bs)[68], float acc[8]
   }
 }
 
+WF_D void l2_hint(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // load a 64 x 64 block (row stride ld) into shared memory, transposed (T = true: S[c][r] = G(r, c))
 // or not, as float4 rows
 template <bool T>
@@ -644,6 +650,9 @@ static __global__ void __launch_bounds__(256) k_gj_update(float* __restrict__ M,
   Rp += (size_t)z * B * ncp;
   Cp += (size_t)z * ncp * B;
   const int tid = threadIdx.x;
+  // the tile itself, read at the end: asked into L2 now (M is larger than L2)
+  for (int e = tid; e < T2 * T2 / 32; e += 256)
+    l2_hint(M + ((size_t)ti * T2 + e / (T2 / 32)) * ncp + (size_t)tj * T2 + (e % (T2 / 32)) * 32);
   // A: the old block columns of the tile's two block rows (Cp rows), transposed into As
   for (int e = tid; e < T2 * B / 4; e += 256) {
     const int r = e / (B / 4), c = (e % (B / 4)) * 4;  // r < 128: row of the tile, c: k

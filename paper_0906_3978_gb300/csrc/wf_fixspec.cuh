@@ -26,10 +26,11 @@ template <int N> struct FxC {
   static_assert(NL >= 2, "a packed-column pair takes two line slots");
 };
 
-// y pass: complex transform along y of every (x, kz) line, in place.  grid (N/2 / NL, N, systems)
+// y pass: complex transform along y of every (x, kz) line, in place.  With fin.n1 > 0 the first row of CTAs takes alpha
+// (YFin).  grid (N/2 / NL, N + (fin.n1 > 0), systems)
 template <int N, int DIR>
 __global__ void __launch_bounds__(FxC<N>::NT)
-k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, const CgScal* __restrict__ sc, Bat bt) {
+k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, CgScal* __restrict__ sc, Bat bt, YFin fin) {
   using G = FxC<N>;
   constexpr int R1 = G::R1, N1 = G::N1, NL = G::NL, NH = G::NH;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -38,8 +39,18 @@ k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, const CgScal
   __shared__ int se[NL];
   __shared__ unsigned sq[NL];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
-  if (sc && sc[z].done) return;
-  double2* p = T + z * bt.spec + (size_t)blockIdx.y * N * NH + blockIdx.x * NL + l;
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (sc && finished(sc + z)) return;
+  int x = blockIdx.y;
+  if constexpr (DIR < 0) {
+    if (fin.n1 > 0 && x-- == 0) {
+      if (blockIdx.x == 0)
+        fin_alpha(fin.part + (size_t)z * bt.part, fin.n1, fin.off, fin.n2, sc + z, reinterpret_cast<double*>(smem_raw));
+      return;
+    }
+  }
+  double2* p = T + z * bt.spec + (size_t)x * N * NH + blockIdx.x * NL + l;
   double2 raw[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) raw[r] = p[(size_t)(r * N1 + t) * NH];
@@ -47,7 +58,6 @@ k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, const CgScal
     se[tid] = kFxMinExp;
     sq[tid] = 0;
   }
-  fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
   fxc v[R1];
@@ -448,8 +458,10 @@ k_fx_cg_xinv(const double2* __restrict__ r, double2* P0, double2* P1, double2* _
   __shared__ unsigned sq[NL];
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   const double2* __restrict__ pold = ((sc->lit & 1) ? P1 : P0) + z * bt.spec;
   double2* __restrict__ pnew = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;
   r += z * bt.spec;
@@ -524,7 +536,6 @@ k_fx_cg_xinv(const double2* __restrict__ r, double2* P0, double2* P1, double2* _
     se[tid] = kFxMinExp;
     sq[tid] = 0;
   }
-  fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
   fxc v[R1];
@@ -552,8 +563,10 @@ k_fx_cg_xupd(const double2* __restrict__ T, double2* __restrict__ r, const doubl
   __shared__ unsigned sq[NL];
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   const bool pair = blockIdx.x == G::KB;
   const int ky = blockIdx.y;
   partials += (size_t)z * bt.part + 2 * (size_t)(blockIdx.y * gridDim.x + blockIdx.x);
@@ -580,7 +593,6 @@ k_fx_cg_xupd(const double2* __restrict__ T, double2* __restrict__ r, const doubl
     se[tid] = kFxMinExp;
     sq[tid] = 0;
   }
-  fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const int ls = pair && l < 2 ? 0 : l;
   const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
@@ -672,7 +684,9 @@ k_fx_zturn(double2* __restrict__ spec, const double* __restrict__ D, const int4*
   __shared__ unsigned sq[2 * G::NL];
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
-  if (sc && sc[z].done) return;
+  fx_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (sc && finished(sc + z)) return;
   const size_t row = (size_t)blockIdx.x * G::NL + l;
   double2* line = spec + z * bt.spec + row * H;
   double2 raw[R1];
@@ -682,7 +696,6 @@ k_fx_zturn(double2* __restrict__ spec, const double* __restrict__ D, const int4*
     se[i] = kFxMinExp;
     sq[i] = 0;
   }
-  fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const FxScale f = fx_line_scale(raw, &se[l], &sq[l], fx_c2r_count<N>());
   fxc* sl = slots + l * G::LS;

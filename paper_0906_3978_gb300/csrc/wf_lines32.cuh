@@ -125,8 +125,10 @@ k_ln_xinv(const float2* __restrict__ r, float2* P0, float2* P1, float2* __restri
   float2* tw = reinterpret_cast<float2*>(slots + N * NL);
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   const float2* __restrict__ pold = ((sc->lit & 1) ? P1 : P0) + z * bt.spec;
   float2* __restrict__ pnew = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;
   r += z * bt.spec;
@@ -136,7 +138,6 @@ k_ln_xinv(const float2* __restrict__ r, float2* P0, float2* P1, float2* __restri
   ctab += z * bt.tab;
   mtab += z * bt.tab;
   const float beta = (float)sc->beta, alpha = (float)sc->alpha_prev;
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
   const int ky = blockIdx.y, ky_s = sfreq(ky, N), kz = blockIdx.x * NL + l;
   const size_t rowstride = (size_t)N * NH, base = (size_t)ky * NH + kz;
   AccF acc;  // the terms are >= 0: a chunk's terms are summed in FP32 first
@@ -207,24 +208,33 @@ k_ln_xinv(const float2* __restrict__ r, float2* P0, float2* P1, float2* __restri
   if (tid == 0) partials[(size_t)z * bt.part + blockIdx.y * gridDim.x + blockIdx.x] = sum;
 }
 
-// x stage of the coarse projection:  T = IFFT_x(c (.) r).  grid (N/2 / NL, N, systems)
+// x stage of the coarse projection:  T = IFFT_x(c (.) r).  With n3 > 0 the first row of CTAs takes beta and the stop
+// test of the iteration before from its n3 pairs of partial sums.  grid (N/2 / NL, N + (n3 > 0), systems)
 template <class G>
 __global__ void __launch_bounds__(G::NT, G::MINB)
 k_ln_xcr(const float2* __restrict__ r, float2* __restrict__ T, const float* __restrict__ oct,
-         const float* __restrict__ ctab, const float2* __restrict__ twtab, const CgScal* __restrict__ sc, Bat bt) {
+         const float* __restrict__ ctab, const float2* __restrict__ twtab, CgScal* __restrict__ sc, Bat bt,
+         const double* __restrict__ part, int n3, double inv_vc) {
   using C = cx<float>;
   constexpr int N = G::N, NH = G::NH, NL = G::NL, R1 = G::R1, N1 = G::N1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* slots = reinterpret_cast<C*>(smem_raw);
   float2* tw = reinterpret_cast<float2*>(slots + N * NL);
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
-  if (sc[z].done) return;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (finished(sc + z)) return;
+  int ky = blockIdx.y;
+  if (n3 > 0 && ky-- == 0) {
+    if (blockIdx.x == 0)
+      fin_beta(part + (size_t)z * bt.part, n3, inv_vc, sc + z, reinterpret_cast<double*>(smem_raw));
+    return;
+  }
   r += z * bt.spec;
   T += z * bt.spec;
   oct += z * G::OCT;
   ctab += z * bt.tab;
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
-  const int ky = blockIdx.y, ky_s = sfreq(ky, N), kz = blockIdx.x * NL + l;
+  const int ky_s = sfreq(ky, N), kz = blockIdx.x * NL + l;
   const size_t rowstride = (size_t)N * NH, base = (size_t)ky * NH + kz;
   C v[R1];
   float cv[R1];
@@ -273,11 +283,13 @@ k_ln_xupd(const float2* __restrict__ T, float2* __restrict__ r, const float2* P0
   float2* tw = reinterpret_cast<float2*>(slots + N * NL);
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   const bool pair = blockIdx.y >= N;
   const int first = ((blockIdx.y - N) * G::KB + blockIdx.x) * (NL / 2);  // a pair CTA's first ky
-  partials += (size_t)z * bt.part + 2 * (size_t)(blockIdx.y * G::KB + blockIdx.x);
+  partials += (size_t)z * bt.part + 2 * (blockIdx.y * G::KB + blockIdx.x);
   if (pair && first > N / 2) {
     if (tid < 2) partials[tid] = 0.0;
     return;
@@ -292,7 +304,6 @@ k_ln_xupd(const float2* __restrict__ T, float2* __restrict__ r, const float2* P0
   ctab += z * bt.tab;
   mtab += z * bt.tab;
   const float alpha = (float)sc->alpha;
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
   const int ky_s = sfreq(ky, N);
   const size_t rowstride = (size_t)N * NH;
   const int row_y = pair && l % 2 == 1 ? (N - ky) % N : ky;
@@ -373,22 +384,46 @@ k_ln_xupd(const float2* __restrict__ T, float2* __restrict__ r, const float2* P0
   }
 }
 
-// y pass: complex transform along y of every (x, kz) line, in place.  grid (N/2 / NL, N, systems)
+template <int N> WF_D size_t dslot(int kx, int ky, int kz);
+// entry u (u = nh: k = 0) of r and, on the kz = 0 plane, its conjugate's
+template <int N> WF_D void restore_entry(float2* r, const float2* rsave, const int4* modes, int nh, int u) {
+  if (u == nh) {
+    r[0] = rsave[2 * nh];
+    return;
+  }
+  const int4 md = modes[u];
+  r[dslot<N>(md.x, md.y, md.z)] = rsave[2 * u];
+  if (md.z == 0) r[dslot<N>(-md.x, -md.y, 0)] = rsave[2 * u + 1];
+}
+
+// y pass: complex transform along y of every (x, kz) line, in place.  With fin.n1 > 0 the first row of CTAs takes alpha
+// (YFin).  grid (N/2 / NL, N + (fin.n1 > 0), systems)
 template <class G, int DIR>
 __global__ void __launch_bounds__(G::NT, G::MINB)
-k_ln_ypass(float2* __restrict__ T, const float2* __restrict__ twtab, const CgScal* __restrict__ sc, Bat bt) {
+k_ln_ypass(float2* __restrict__ T, const float2* __restrict__ twtab, CgScal* __restrict__ sc, Bat bt, YFin fin) {
   using C = cx<float>;
   constexpr int N = G::N, NH = G::NH, NL = G::NL, R1 = G::R1, N1 = G::N1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* slots = reinterpret_cast<C*>(smem_raw);
   float2* tw = reinterpret_cast<float2*>(slots + N * NL);
   const int z = blockIdx.z, tid = threadIdx.x, l = tid % NL, t = tid / NL;
-  if (sc && sc[z].done) return;
-  float2* p = T + z * bt.spec + (size_t)blockIdx.y * N * NH + blockIdx.x * NL + l;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (sc && finished(sc + z)) return;
+  int x = blockIdx.y;
+  if constexpr (DIR < 0) {
+    if (fin.n1 > 0 && x-- == 0) {
+      if (blockIdx.x != 0) return;
+      for (int u = tid; u <= fin.nh; u += G::NT)
+        restore_entry<N>(fin.r + z * bt.spec, fin.rsave + (size_t)z * (2 * fin.nh + 1), fin.modes, fin.nh, u);
+      fin_alpha(fin.part + (size_t)z * bt.part, fin.n1, fin.off, fin.n2, sc + z, reinterpret_cast<double*>(smem_raw));
+      return;
+    }
+  }
+  float2* p = T + z * bt.spec + (size_t)x * N * NH + blockIdx.x * NL + l;
   C v[R1];
 #pragma unroll
   for (int q = 0; q < R1; ++q) v[q] = ld2(p + (size_t)(q * N1 + t) * NH);
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   ln_forward<N, typename G::PL, DIR>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, C X, int) { st2(p + (size_t)k * NH, X); });
 }
@@ -472,13 +507,14 @@ k_ln_zturn(float2* __restrict__ spec, const float* __restrict__ D, const float2*
   float2* tw = reinterpret_cast<float2*>(slots + G::NL * G::LS);
   __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
-  if (sc && sc[z].done) return;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (sc && finished(sc + z)) return;
   const size_t row = (size_t)blockIdx.x * G::NL + l;
   float2* line = spec + z * bt.spec + row * H;
   C v[R1];
 #pragma unroll
   for (int q = 0; q < R1; ++q) v[q] = ld2(line + q * N1 + t);
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
   AccF acc;
   C* s = slots + l * G::LS;
   ln_turn<G>(v, s, t, tw, reinterpret_cast<const float2*>(D + z * bt.real) + row * H, &acc);
@@ -501,13 +537,14 @@ k_ln_zcoarse(const float2* __restrict__ spec, const float* __restrict__ D, const
   C* slots = reinterpret_cast<C*>(smem_raw);
   float2* tw = reinterpret_cast<float2*>(slots + G::NL * G::LS);
   const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
-  if (sc[z].done) return;
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (finished(sc + z)) return;
   const size_t row0 = (size_t)blockIdx.x * G::NL, row = row0 + l;
   const float2* line = spec + z * bt.spec + row * H;
   C v[R1];
 #pragma unroll
   for (int q = 0; q < R1; ++q) v[q] = ld2(line + q * N1 + t);
-  ln_load_tw<N>(tw, twtab, tid, G::NT);
   ln_turn<G>(v, slots + l * G::LS, t, tw, reinterpret_cast<const float2*>(D + z * bt.real) + row * H, nullptr);
   gz += z * gzs + row0 * (K + 1);
   for (int e = tid; e < G::NL * (K + 1); e += G::NT) {

@@ -145,12 +145,30 @@ struct Spec {
   }
   // ---- launch variants of a pass (tile lines, buffers in flight, radix cap); the context's
   // tuning table picks one per (pass, precision, size), variant 0 by default ------------------
-  using PassRun = void (*)(Ctx&, int, ST*, const ST*, const CgScal*, int, cudaStream_t);
+  using PassRun = void (*)(Ctx&, int, ST*, const ST*, CgScal*, int, cudaStream_t, const YFin&);
   struct PassVariant {
     const char* name;
     cudaError_t (*setup)();
-    PassRun run;
+    PassRun go;
+    void run(Ctx& c, int nb, ST* t, const ST* tw, CgScal* sc, int dir, cudaStream_t st) const {
+      go(c, nb, t, tw, sc, dir, st, YFin{});
+    }
   };
+  // alpha (and the coarse entries of r back) in launches of their own, for a middle pass that does not take them along
+  static void finish_alpha(Ctx& c, int nb, CgScal* sc, const YFin& fin, cudaStream_t st) {
+    if (fin.n1 <= 0) return;
+    if constexpr (!F64)
+      if (fin.nh >= 0)
+        c.launch("defl_restore", 0, st, [&] {
+          Ctx::chain(k_defl_restore<float, N>, dim3((fin.nh + 1 + 255) / 256, nb), 256, 0, st, fin.r, fin.rsave,
+                     fin.modes, fin.nh, sc, bat());
+        });
+    c.launch("fin", 0, st,
+             [&] { Ctx::chain(k_fin_alpha, nb, 1024, 0, st, fin.part, fin.n1, fin.off, fin.n2, sc, bat()); });
+  }
+  static void finish_beta(Ctx& c, int nb, double* part, int n3, double inv_vc, CgScal* sc, cudaStream_t st) {
+    c.launch("fin", 0, st, [&] { Ctx::chain(k_fin_beta, nb, 1024, 0, st, part, n3, inv_vc, sc, bat()); });
+  }
   // y pass variant <NL, STG, RMAX>: complex FFT along y of every (x, kz) line, in place
   template <int NL, int STG, int RMAX>
   struct YV {
@@ -164,16 +182,17 @@ struct Spec {
       if (occ < 1) occ = 1;
       return e;
     }
-    static void run(Ctx& c, int nb, ST* t, const ST* tw, const CgScal* sc, int dir, cudaStream_t st) {
+    static void run(Ctx& c, int nb, ST* t, const ST* tw, CgScal* sc, int dir, cudaStream_t st, const YFin& fin) {
       CUtensorMap m;
       if (!make_spectrum_map(&m, t, N, nb, sizeof(SS) == 8, NL, G::BR, 1)) {
         c.map_failed = true;
         return;
       }
       const unsigned grid = persistent_grid(c, occ, (long long)nb * G::TPS);
+      finish_alpha(c, nb, sc, fin, st);
       c.launch(cls("ypass", "ypass_f64"), 2 * BS * nb, st, [&] {
-        if (dir < 0) k_ypass_tma<R, N, -1, NL, STG, RMAX><<<grid, G::NT, G::SMEM, st>>>(m, tw, sc, nb, c.dev_err);
-        else k_ypass_tma<R, N, +1, NL, STG, RMAX><<<grid, G::NT, G::SMEM, st>>>(m, tw, sc, nb, c.dev_err);
+        if (dir < 0) Ctx::chain(k_ypass_tma<R, N, -1, NL, STG, RMAX>, grid, G::NT, G::SMEM, st, m, tw, sc, nb, c.dev_err);
+        else Ctx::chain(k_ypass_tma<R, N, +1, NL, STG, RMAX>, grid, G::NT, G::SMEM, st, m, tw, sc, nb, c.dev_err);
       });
     }
   };
@@ -183,11 +202,11 @@ struct Spec {
       cudaError_t e = set_smem(k_ln_ypass<G, -1>, G::SMEM);
       return e == cudaSuccess ? set_smem(k_ln_ypass<G, +1>, G::SMEM) : e;
     }
-    static void run(Ctx& c, int nb, ST* t, const ST* tw, const CgScal* sc, int dir, cudaStream_t st) {
-      const dim3 grid(G::KB, N, nb);
+    static void run(Ctx& c, int nb, ST* t, const ST* tw, CgScal* sc, int dir, cudaStream_t st, const YFin& fin) {
+      const dim3 grid(G::KB, N + (fin.n1 > 0), nb);
       c.launch("ypass", 2 * BS * nb, st, [&] {
-        if (dir < 0) k_ln_ypass<G, -1><<<grid, G::NT, G::SMEM, st>>>(t, tw, sc, bat());
-        else k_ln_ypass<G, +1><<<grid, G::NT, G::SMEM, st>>>(t, tw, sc, bat());
+        if (dir < 0) Ctx::chain(k_ln_ypass<G, -1>, grid, G::NT, G::SMEM, st, t, tw, sc, bat(), fin);
+        else Ctx::chain(k_ln_ypass<G, +1>, grid, G::NT, G::SMEM, st, t, tw, sc, bat(), fin);
       });
     }
   };
@@ -197,12 +216,12 @@ struct Spec {
       cudaError_t e = set_smem(k_fx_ypass<N, -1>, FC::SMEM);
       return e == cudaSuccess ? set_smem(k_fx_ypass<N, +1>, FC::SMEM) : e;
     }
-    static void run(Ctx& c, int nb, ST* t, const ST*, const CgScal* sc, int dir, cudaStream_t st) {
+    static void run(Ctx& c, int nb, ST* t, const ST*, CgScal* sc, int dir, cudaStream_t st, const YFin& fin) {
       double2* T = reinterpret_cast<double2*>(t);
-      const dim3 grid(FC::KB, N, nb);
+      const dim3 grid(FC::KB, N + (fin.n1 > 0), nb);
       c.launch("ypass_f64", 2 * BS * nb, st, [&] {
-        if (dir < 0) k_fx_ypass<N, -1><<<grid, FC::NT, FC::SMEM, st>>>(T, c.fixed(N), sc, bat());
-        else k_fx_ypass<N, +1><<<grid, FC::NT, FC::SMEM, st>>>(T, c.fixed(N), sc, bat());
+        if (dir < 0) Ctx::chain(k_fx_ypass<N, -1>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
+        else Ctx::chain(k_fx_ypass<N, +1>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
       });
     }
   };
@@ -225,7 +244,7 @@ struct Spec {
     }();
     return v;
   }
-  // ---- x-pass variants: the two CG x passes; each launcher returns the number of partial sums it wrote
+  // ---- x-pass variants: the two CG x passes.  each launcher returns the number of partial sums it wrote
   using XinvRun = int (*)(Ctx&, int, ST*, ST*, ST*, ST*, ST*, const SS*, const SS*, const SS*, bool, const ST*,
                           double*, CgScal*, cudaStream_t);
   using XupdRun = int (*)(Ctx&, int, const ST*, ST*, ST*, ST*, const SS*, const SS*, const SS*, bool, const ST*,
@@ -250,9 +269,9 @@ struct Spec {
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
       c.launch(cls("cg_xinv", "cg_xinv_f64"), 6 * BS * nb, st, [&] {
         if (unit_m)
-          k_cg_xinv<R, N, true, RMAX><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_cg_xinv<R, N, true, RMAX>, gxy(nb), NTx, SMxy, st, r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
         else
-          k_cg_xinv<R, N, false, RMAX><<<gxy(nb), NTx, SMxy, st>>>(r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_cg_xinv<R, N, false, RMAX>, gxy(nb), NTx, SMxy, st, r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
       });
       return GXY;
     }
@@ -260,9 +279,9 @@ struct Spec {
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
       c.launch(cls("cg_xupd", "cg_xupd_f64"), 4 * BS * nb, st, [&] {
         if (unit_m)
-          k_cg_xupd<R, N, true, RMAX><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_cg_xupd<R, N, true, RMAX>, gxy(nb), NTx, SMxy, st, T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
         else
-          k_cg_xupd<R, N, false, RMAX><<<gxy(nb), NTx, SMxy, st>>>(T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_cg_xupd<R, N, false, RMAX>, gxy(nb), NTx, SMxy, st, T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
       });
       return GXY;
     }
@@ -282,9 +301,9 @@ struct Spec {
       const dim3 grid(G::KB, N, nb);
       c.launch("cg_xinv", 6 * BS * nb, st, [&] {
         if (unit_m)
-          k_ln_xinv<G, true><<<grid, G::NT, G::SMEM, st>>>(r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_ln_xinv<G, true>, grid, G::NT, G::SMEM, st, r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
         else
-          k_ln_xinv<G, false><<<grid, G::NT, G::SMEM, st>>>(r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_ln_xinv<G, false>, grid, G::NT, G::SMEM, st, r, P0, P1, x, T, oct, ctab, mtab, tw, part, sc, bat());
       });
       return G::KB * N;
     }
@@ -294,9 +313,9 @@ struct Spec {
       static_assert(2 * G::KB * (N + G::YP) <= NPART, "partial sums");
       c.launch("cg_xupd", 4 * BS * nb, st, [&] {
         if (unit_m)
-          k_ln_xupd<G, true><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_ln_xupd<G, true>, grid, G::NT, G::SMEM, st, T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
         else
-          k_ln_xupd<G, false><<<grid, G::NT, G::SMEM, st>>>(T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
+          Ctx::chain(k_ln_xupd<G, false>, grid, G::NT, G::SMEM, st, T, r, P0, P1, oct, ctab, mtab, tw, part, sc, bat());
       });
       return G::KB * (N + G::YP);
     }
@@ -316,9 +335,9 @@ struct Spec {
         const dim3 grid(FC::KB, N, nb);
         c.launch("cg_xinv_f64", 6 * BS * nb, st, [&] {
           if (unit_m)
-            k_fx_cg_xinv<N, true><<<grid, FC::NT, FC::SMEM, st>>>(r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
+            Ctx::chain(k_fx_cg_xinv<N, true>, grid, FC::NT, FC::SMEM, st, r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
           else
-            k_fx_cg_xinv<N, false><<<grid, FC::NT, FC::SMEM, st>>>(r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
+            Ctx::chain(k_fx_cg_xinv<N, false>, grid, FC::NT, FC::SMEM, st, r, P0, P1, x, T, ctab, mtab, c.fixed(N), part, sc, bat());
         });
       }
       return FC::KB * N;
@@ -330,9 +349,9 @@ struct Spec {
         const size_t sm = fx_xmul_smem<N>();
         c.launch("cg_xupd_f64", 4 * BS * nb, st, [&] {
           if (unit_m)
-            k_fx_cg_xupd<N, true><<<grid, FC::NT, sm, st>>>(T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
+            Ctx::chain(k_fx_cg_xupd<N, true>, grid, FC::NT, sm, st, T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
           else
-            k_fx_cg_xupd<N, false><<<grid, FC::NT, sm, st>>>(T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
+            Ctx::chain(k_fx_cg_xupd<N, false>, grid, FC::NT, sm, st, T, r, P0, P1, ctab, mtab, c.fixed(N), part, sc, bat());
         });
       }
       return (FC::KB + 1) * N;
@@ -365,7 +384,7 @@ struct Spec {
     static cudaError_t setup() { return set_smem(k_ln_zturn<G>, G::SMEM); }
     static int run(Ctx& c, int nb, ST* T, const SS* D, const ST* tw, double* part, const CgScal* sc, cudaStream_t st) {
       c.launch("zturn", (2 * BS + sizeof(SS) * BV) * nb, st,
-               [&] { k_ln_zturn<G><<<dim3(G::GZ, 1, nb), G::NT, G::SMEM, st>>>(T, D, tw, part, sc, bat()); });
+               [&] { Ctx::chain(k_ln_zturn<G>, dim3(G::GZ, 1, nb), G::NT, G::SMEM, st, T, D, tw, part, sc, bat()); });
       return G::GZ;
     }
   };
@@ -374,7 +393,7 @@ struct Spec {
     static int run(Ctx& c, int nb, ST* T, const SS* D, const ST*, double* part, const CgScal* sc, cudaStream_t st) {
       if constexpr (F64)
         c.launch("zturn_f64", (2 * BS + sizeof(SS) * BV) * nb, st,
-                 [&] { k_fx_zturn<N><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(T, D, c.fixed(N), part, sc, bat()); });
+                 [&] { Ctx::chain(k_fx_zturn<N>, dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st, T, D, c.fixed(N), part, sc, bat()); });
       return FZ::GZ;
     }
   };
@@ -401,8 +420,8 @@ struct Spec {
     return vs[i >= 0 && i < (int)vs.size() ? i : 0];
   }
   // complex FFT along y of every (x, kz) line of nb spectra, in place
-  static void ypass(Ctx& c, int nb, ST* t, const ST* tw, const CgScal* sc, int dir, cudaStream_t st) {
-    pick(c, "ypass", yvariants()).run(c, nb, t, tw, sc, dir, st);
+  static void ypass(Ctx& c, int nb, ST* t, const ST* tw, CgScal* sc, int dir, cudaStream_t st, const YFin& fin = YFin{}) {
+    pick(c, "ypass", yvariants()).go(c, nb, t, tw, sc, dir, st, fin);
   }
   // out = [IFFT_x] tab (.) [FFT_x] in (FP64 form with both transforms: fmul below)
   template <bool FWD, bool INV, bool DOT>
@@ -448,37 +467,34 @@ struct Spec {
     });
   }
 
-  struct NoHook {
-    void operator()(cudaStream_t) const {}
-  };
   // One CG iteration of every unfinished system (no host synchronisation).  The first x pass forms
-  // p from rin (default r); after_xinv(st) is enqueued right after it.
-  template <class H = NoHook>
-  static void iteration(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* D, const SS* oct,
-                        const SS* ctab, const SS* mtab, bool unit_m, const ST* tw, double* part, CgScal* sc, double inv_vc,
-                        cudaStream_t st, ST* rin = nullptr, H after_xinv = H()) {
-    const Bat b = bat();
-    const int n1 = pick(c, "xinv", xvariants())
-                       .xinv(c, nb, rin ? rin : r, P0, P1, x, T, oct, ctab, mtab, unit_m, tw, part, sc, st);
-    after_xinv(st);
-    int nmid = 0;  // blocks that sum the data term of <p, A p> into part[NX ...]
+  // p from rin (default r); fin: the coarse entries of r to put back (nh < 0: none), the rest is filled in here.
+  // The number of partial sums of <r, r> and the estimate is returned; with `beta` they are taken here.
+  static int iteration(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* D, const SS* oct,
+                       const SS* ctab, const SS* mtab, bool unit_m, const ST* tw, double* part, CgScal* sc, double inv_vc,
+                       cudaStream_t st, ST* rin = nullptr, YFin fin = YFin{}, bool beta = true) {
+    fin.part = part;
+    fin.off = NX;
+    fin.n1 = pick(c, "xinv", xvariants())
+                 .xinv(c, nb, rin ? rin : r, P0, P1, x, T, oct, ctab, mtab, unit_m, tw, part, sc, st);
     bool fused = false;
     if constexpr (PCS > 0) {
       if (c.fused_planes) {
         c.launch("plane_turn", (2 * BS + sizeof(SS) * BV) * nb, st,
-                 [&] { plane_turn_launch<R, N, PCS, PE>(T, D, tw, part + NX, sc, b, nb, st); });
-        nmid = N * PCS;
+                 [&] { plane_turn_launch<R, N, PCS, PE>(T, D, tw, part + NX, sc, bat(), nb, st); });
+        fin.n2 = N * PCS;
+        finish_alpha(c, nb, sc, fin, st);
         fused = true;
       }
     }
     if (!fused) {
       ypass(c, nb, T, tw, sc, +1, st);
-      nmid = pick(c, "zturn", zvariants()).run(c, nb, T, D, tw, part + NX, sc, st);
-      ypass(c, nb, T, tw, sc, -1, st);
+      fin.n2 = pick(c, "zturn", zvariants()).run(c, nb, T, D, tw, part + NX, sc, st);
+      ypass(c, nb, T, tw, sc, -1, st, fin);
     }
-    c.launch("fin", 0, st, [&] { k_fin_alpha<<<nb, 1024, 0, st>>>(part, n1, NX, nmid, sc, b); });
     const int n3 = pick(c, "xupd", xvariants()).xupd(c, nb, T, r, P0, P1, oct, ctab, mtab, unit_m, tw, part, sc, st);
-    c.launch("fin", 0, st, [&] { k_fin_beta<<<nb, 1024, 0, st>>>(part, n3, inv_vc, sc, b); });
+    if (beta) finish_beta(c, nb, part, n3, inv_vc, sc, st);
+    return n3;
   }
 };
 
@@ -676,8 +692,9 @@ static void group_sums_end(GroupCommon<N>& g) {
 // converged to 1e-10, too close to the mixed path's 1e-6 bound.
 constexpr double kInnerMargin = 0.5;
 
-// Check interval: grids of 256^3 and up check the device flags every 4 iterations.
-template <int N> constexpr int check_every() { return N >= 256 ? 4 : (N >= 128 ? 8 : 16); }
+// Check interval: grids of 256^3 and up check the device flags every 4 iterations, smaller ones every 8 (a block
+// of finished iterations still launches; a check costs ~15 us).
+template <int N> constexpr int check_every() { return N >= 256 ? 4 : 8; }
 
 // ------------------------------------------------------------------------------------------
 // FP64 group: FP64 storage, spectral arithmetic R.
@@ -982,52 +999,53 @@ struct GroupMixed : GroupCommon<N> {
   // coordinates of A' r - r and of r, and r -= Z E^-1 g kept aside (MODE 1); or the start vector
   // Z E^-1 Z^T r into `out` (MODE 0)
   template <int MODE>
-  void defl_project(Ctx& c, float2* out, cudaStream_t st) {
+  void defl_project(Ctx& c, float2* out, cudaStream_t st, int n3 = 0) {
     const Bat bf = SF::bat();
     const int gw = (nh + 1 + 7) / 8;
     if constexpr (MODE == 1) {
-      defl_xr(c, st);
+      defl_xr(c, st, n3);
       SF::ypass(c, nb, T, tw32, sc, +1, st);
       c.launch("defl_z", (SF::BS + 4 * SF::BV) * nb, st, [&] {
         using G = typename SF::GZ1;
-        k_ln_zcoarse<G><<<dim3(G::GZ, 1, nb), G::NT, G::SMEM, st>>>(T, D, tw32, Gz, K, sc, bf, gzs);
+        Ctx::chain(k_ln_zcoarse<G>, dim3(G::GZ, 1, nb), G::NT, G::SMEM, st, T, D, tw32, Gz, K, sc, bf, gzs);
       });
       const size_t ysm = ((size_t)N * (K + 1) + N) * sizeof(float2);
       c.launch("defl_y", 8.0 * gzs * nb, st, [&] {
-        k_ycoarse<float, N><<<dim3(N, nb), 256, ysm, st>>>(Gz, tw32, Gy, K, sc, gzs, gys);
+        Ctx::chain(k_ycoarse<float, N>, dim3(N, nb), 256, ysm, st, Gz, tw32, Gy, K, sc, gzs, gys);
       });
     }
     c.launch("defl_x", 8.0 * gys * nb, st, [&] {
-      k_xcoarse<float, N, MODE><<<dim3(gw, nb), 256, 0, st>>>(Gy, rh, ct, mt, tw32, dmodes, nh, K, gco, rco, sc, bf,
-                                                              gys, ncp);
+      Ctx::chain(k_xcoarse<float, N, MODE>, dim3(gw, nb), 256, 0, st, Gy, rh, ct, mt, tw32, dmodes, nh, K, gco, rco, sc,
+                 bf, gys, ncp);
     });
     c.launch("defl_mu", 4.0 * ncp * ncp * nb, st, [&] {
-      k_defl_mu<float, N, MODE><<<dim3(gw, nb), 256, ncp * sizeof(float), st>>>(Einv, gco, rco, dmodes, nh, ncp,
-                                                                                 out, rsave, dpart, sc, bf, doff);
+      Ctx::chain(k_defl_mu<float, N, MODE>, dim3(gw, nb), 256, ncp * sizeof(float), st, Einv, gco, rco, dmodes, nh, ncp,
+                 out, rsave, dpart, sc, bf, doff);
     });
   }
   // T = IFFT_x(c r), register-staged (a persistent form on tensor copies along x, the y pass's tile
   // walk with the table multiply and partner column added, took 0.52 ms at 512^3 against 0.42: one
   // CTA per SM cannot hide the table gathers and the strided partner loads)
-  void defl_xr(Ctx& c, cudaStream_t st) {
+  void defl_xr(Ctx& c, cudaStream_t st, int n3) {
     const Bat bf = SF::bat();
     c.launch("defl_xr", 2 * SF::BS * nb, st, [&] {
       using G = typename SF::GX;
-      k_ln_xcr<G><<<dim3(G::KB, N, nb), G::NT, G::SMEM, st>>>(rh, T, coct, ct, tw32, sc, bf);
+      Ctx::chain(k_ln_xcr<G>, dim3(G::KB, N + (n3 > 0), nb), G::NT, G::SMEM, st, rh, T, coct, ct, tw32, sc, bf, part, n3,
+                 inv_vc);
     });
   }
-  // one deflated inner iteration: p = (r - Z mu) + beta p with mu from the coarse projection
-  void defl_iteration(Ctx& c, cudaStream_t st) {
-    const Bat bf = SF::bat();
-    defl_project<1>(c, rh, st);
-    c.launch("fin", 0, st, [&] { k_fin_defl<<<nb, 256, 0, st>>>(dpart, nh, sc); });
-    SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, st, nullptr,
-                  [&](cudaStream_t s) {
-                    c.launch("defl_restore", 0, s, [&] {
-                      k_defl_restore<float, N><<<dim3((nh + 1 + 255) / 256, nb), 256, 0, s>>>(rh, rsave, dmodes, nh,
-                                                                                               sc, bf);
-                    });
-                  });
+  // one deflated inner iteration: p = (r - Z mu) + beta p with mu from the coarse projection.  n3 > 0: beta and the stop
+  // test of the iteration before are still to be taken, by the coarse x stage; the same is left to the caller here
+  // unless this is the last one before the host looks (the return value).
+  int defl_iteration(Ctx& c, cudaStream_t st, int n3, bool last) {
+    defl_project<1>(c, rh, st, n3);
+    YFin fin;
+    fin.nh = nh;
+    fin.r = rh;
+    fin.rsave = rsave;
+    fin.modes = dmodes;
+    n3 = SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, st, nullptr, fin, last);
+    return last ? 0 : n3;
   }
   wf_status prepare_end(Ctx& c, cudaStream_t st) override {
     const size_t V = SF::V;
@@ -1126,8 +1144,9 @@ struct GroupMixed : GroupCommon<N> {
     }
     if (phase == 1) {
       WF_TRY(this->run_block(c, st, [&](cudaStream_t s2) {
+        int n3 = 0;
         for (int i = 0; i < check_every<N>(); ++i) {
-          if (K > 0) defl_iteration(c, s2);
+          if (K > 0) n3 = defl_iteration(c, s2, n3, i == check_every<N>() - 1);
           else SF::iteration(c, nb, rh, P0, P1, xh, T, D, coct, ct, mt, unit_m, tw32, part, sc, inv_vc, s2);
         }
       }));

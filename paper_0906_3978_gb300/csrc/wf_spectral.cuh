@@ -50,7 +50,11 @@ struct __align__(16) CgScal {
   int defl;           // deflated inner solves: 2 start step (alpha = 1) pending, 1 first iteration
   int noco;           // deflated groups: 1 = this system runs its inner solves without the coarse space
   int texp;           // power of two of the FP64 prior table's digits (k_fx_xmul)
+  unsigned tick[4];   // arrivals of the CTAs of a kernel that ends with a finisher (0 between kernels)
 };
+// sc->done, read after chain_start(): a volatile read, which is not moved across the wait (the loads that follow
+// the test of it are then not moved either)
+WF_D bool finished(const CgScal* sc) { return *(const volatile int*)&sc->done != 0; }
 
 // Distances between consecutive systems of a batch (elements of each array type).
 struct Bat {
@@ -220,7 +224,7 @@ struct TG {
 template <class G> struct TileSeq {
   const CgScal* sc;
   int total;
-  WF_D bool live(int id) const { return !(sc && sc[id / G::TPS].done); }
+  WF_D bool live(int id) const { return !(sc && finished(sc + id / G::TPS)); }
   // the first live tile at or after id in steps of `step` (total if none)
   WF_D int next(int id, int step) const {
     while (id < total && !live(id)) id += step;
@@ -274,8 +278,9 @@ k_ypass_tma(const __grid_constant__ CUtensorMap tm, const typename Store<R>::T* 
     for (int s = 0; s < STG; ++s) mbar_init(&bar[s], 1);
     mbar_init_fence();
   }
-  __syncthreads();
   load_tw<R, G::M, 2 * N>(tw, twtab, tid, G::NT);
+  chain_start();
+  __syncthreads();
   auto issue = [&](int id, int s) {
     const int z = id / G::TPS, rem = id % G::TPS, x = rem / G::KB, kz0 = (rem % G::KB) * NL;
     mbar_expect_tx(&bar[s], G::TILE_BYTES);
@@ -377,9 +382,10 @@ k_cg_xinv(const typename Store<R>::T* __restrict__ r, typename Store<R>::T* P0, 
   cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
   cx<R>* tw = tile + G::M * G::LD;
   __shared__ double red[32];
+  chain_start();
   const int z = blockIdx.z;
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   // p_old / p_new alternate between P0 and P1 with this system's iteration count
   const ST* __restrict__ pold = ((sc->lit & 1) ? P1 : P0) + z * bt.spec;
   ST* __restrict__ pnew = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;
@@ -518,9 +524,10 @@ k_cg_xupd(const typename Store<R>::T* __restrict__ T, typename Store<R>::T* __re
   cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
   cx<R>* tw = tile + G::M * G::LD;
   __shared__ double red[32];
+  chain_start();
   const int z = blockIdx.z;
   sc += z;
-  if (sc->done) return;
+  if (finished(sc)) return;
   const ST* __restrict__ p = ((sc->lit & 1) ? P0 : P1) + z * bt.spec;  // this iteration's p_new
   T += z * bt.spec;
   r += z * bt.spec;
@@ -967,16 +974,24 @@ static __global__ void k_fin_init(const double* __restrict__ partials, int n, Cg
   }
 }
 
-// <p, A p> = partials [0, n1) (the m term, from the x pass) + [off2, off2 + n2) (the data term,
-// from the z turn); alpha = rr / <p, A p>.
-// (the first n1 partials of the system, and n2 from offset off2)
-static __global__ void k_fin_alpha(const double* __restrict__ partials, int n1, int off2, int n2, CgScal* sc, Bat bt) {
-  __shared__ double red[32];
-  sc += blockIdx.x;
-  if (sc->done) return;
-  const double pm = sum_partials(partials + blockIdx.x * bt.part, n1, 1, 0, red);
-  const double pd = sum_partials(partials + blockIdx.x * bt.part + off2, n2, 1, 0, red);
-  const double pq = pm + pd;
+// The sums and scalar updates at the end of a CG iteration's halves, by the threads of one CTA: the last to
+// finish of the pass that produced the partial sums (last_cta), or a kernel of its own (k_fin_*, after the
+// passes that have no finisher).  Partials are read past L1: other CTAs of the same grid wrote them.
+WF_D double sum_fresh(const double* p, int n, int stride, double* red) {
+  double v = 0.0;
+#pragma unroll 16
+  for (int i = threadIdx.x; i < n; i += blockDim.x) v += __ldcg(p + (size_t)i * stride);
+  return block_sum(v, red);
+}
+// <p, A p> = partials [0, n1) (the m term, from the x pass) + [off2, off2 + n2) (the data term, from the z
+// turn); alpha = rr / <p, A p>.
+WF_D void fin_alpha(const double* partials, int n1, int off2, int n2, CgScal* sc, double* red) {
+  double v = 0.0;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n1; i += blockDim.x) v += __ldcg(partials + i);
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) v += __ldcg(partials + off2 + i);
+  const double pq = block_sum(v, red);
   if (threadIdx.x == 0) {
     sc->pq = pq;
     if (sc->defl == 2) {  // the start step of a deflated solve moves by exactly Z mu
@@ -990,15 +1005,10 @@ static __global__ void k_fin_alpha(const double* __restrict__ partials, int n1, 
     }
   }
 }
-
 // stop rule: rc2 * inv_vc <= max(tol2 * bb, rr_stop)
-static __global__ void k_fin_beta(const double* __restrict__ partials, int n, double inv_vc, CgScal* sc, Bat bt) {
-  __shared__ double red[32];
-  sc += blockIdx.x;
-  if (sc->done) return;
-  partials += blockIdx.x * bt.part;
-  const double rr = sum_partials(partials, n, 2, 0, red);
-  const double rc = sum_partials(partials, n, 2, 1, red);
+WF_D void fin_beta(const double* partials, int n, double inv_vc, CgScal* sc, double* red) {
+  const double rr = sum_fresh(partials, n, 2, red);
+  const double rc = sum_fresh(partials + 1, n, 2, red);
   if (threadIdx.x == 0) {
     const double rc2 = rc * inv_vc;
     sc->beta = rr / sc->rr;
@@ -1013,6 +1023,32 @@ static __global__ void k_fin_beta(const double* __restrict__ partials, int n, do
     else if (rc2 <= lim) sc->done = 1;
     else if (sc->iter >= sc->max_iter) sc->done = 2;
   }
+}
+// What the forward y pass, which does not need alpha, does beside its lines (n1 = 0: nothing): alpha from the n1 partial
+// sums of x pass 1 and the n2 of the z turn, and for a deflated iteration the coarse entries of r back to what
+// k_defl_mu saved (x pass 1 has used its own).  A single-CTA launch between the passes costs 3-8 us; a last-arrival
+// ticket in the z turn held every CTA for its fence (144^3: 17 -> 26 us).
+struct YFin {
+  int n1 = 0, off = 0, n2 = 0;  // x pass 1's partial sums [0, n1), the z turn's [off, off + n2)
+  const double* part = nullptr;
+  int nh = -1;                  // half-space modes of the coarse space, -1: none
+  float2* r = nullptr;
+  const float2* rsave = nullptr;
+  const int4* modes = nullptr;
+};
+static __global__ void k_fin_alpha(const double* __restrict__ partials, int n1, int off2, int n2, CgScal* sc, Bat bt) {
+  __shared__ double red[32];
+  chain_start();
+  sc += blockIdx.x;
+  if (finished(sc)) return;
+  fin_alpha(partials + blockIdx.x * bt.part, n1, off2, n2, sc, red);
+}
+static __global__ void k_fin_beta(const double* __restrict__ partials, int n, double inv_vc, CgScal* sc, Bat bt) {
+  __shared__ double red[32];
+  chain_start();
+  sc += blockIdx.x;
+  if (finished(sc)) return;
+  fin_beta(partials + blockIdx.x * bt.part, n, inv_vc, sc, red);
 }
 
 // sum of partials into sc->aux[slot] (slot >= 0, host reads it) or into sc->bb (slot < 0);
