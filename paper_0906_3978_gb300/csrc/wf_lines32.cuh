@@ -555,4 +555,152 @@ k_ln_zcoarse(const float2* __restrict__ spec, const float* __restrict__ D, const
   }
 }
 
+// ---- whole x-planes: the middle of an iteration in one kernel ---------------------------------------------------
+// Up to 72 launches and their ramps bound an iteration.  Here one CTA holds a plane (N x N/2 complex) in shared memory: the
+// inverse y transforms, the z turn and the forward y transforms move 3 spectra instead of 7 and are one launch
+// instead of three, and the coarse stage (y, z, the DFT along y at the coarse modes) is one instead of three.
+// A plane is stored as N padded rows; column and row lines work in place in it, with the same first radix along y
+// and z, so that the thread grids agree.  Mixed solve at 64^3: 4.33 -> 4.08 ms.  Larger planes leave one CTA
+// per SM, whose loads, transforms and stores do not overlap: 144^3 alone 8.80 -> 8.18 ms, but twelve systems of 64^3
+// to 192^3 together 56.7 -> 63.5, and the choice may not depend on the company a system keeps (same bits in any batch).
+template <int N> struct F32PlanePlan { using Y = LnRad<0, 0, 0>; using Z = LnRad<0, 0, 0>; };
+#define WF_PLAN(M, A, B, C, D, E) \
+  template <> struct F32PlanePlan<M> { using Y = LnRad<A, B, C>; using Z = LnRad<D, E, 1>; }
+WF_PLAN(16, 4, 4, 1, 4, 2);
+WF_PLAN(24, 4, 6, 1, 4, 3);
+WF_PLAN(32, 4, 8, 1, 4, 4);
+WF_PLAN(48, 6, 8, 1, 6, 4);
+WF_PLAN(64, 8, 8, 1, 8, 4);
+WF_PLAN(72, 6, 12, 1, 6, 6);
+#undef WF_PLAN
+constexpr int kPlaneMax = 72;
+template <int N_> struct LP {
+  using PY = typename F32PlanePlan<N_>::Y;
+  using PZ = typename F32PlanePlan<N_>::Z;
+  using Map = PadMapT<3>;
+  static constexpr int N = N_, H = N / 2, R1 = PY::r1, NY = N / R1, NZ = H / R1;
+  static constexpr int NT = H * NY, MINB = 768 / NT > 1 ? cmin(16, 768 / NT) : 1;
+  static constexpr int LS = ln_padded(H, 3, NZ, 16);  // slots of a row
+  static constexpr size_t SMEM = (size_t)(N * LS + N) * sizeof(cx<float>);
+  static_assert(PZ::r1 == R1 && N * NZ == NT && NT <= 1024 && PY::r1 * PY::r2 * PY::r3 == N && R1 * PZ::r2 == H, "plan");
+};
+template <int LS> struct RowMap {
+  WF_D int operator()(int p) const { return p * LS; }
+};
+
+// COARSE: T (read only) -> Gy[ky + K][kz][x], the DFT along y at |ky| <= K of the z turn's kz <= K (k_ycoarse's).
+// Otherwise: T -> FFT_y FFT_z (D IFFT_z IFFT_y T) in place, the partial sum of D T^2, and the last CTA's alpha
+// (YFin).  grid (N, 1, systems)
+template <int N, bool COARSE>
+__global__ void __launch_bounds__(LP<N>::NT, LP<N>::MINB)
+k_ln_plane(float2* __restrict__ T, const float* __restrict__ D, const float2* __restrict__ twtab,
+           double* __restrict__ partials, CgScal* __restrict__ sc, Bat bt, YFin fin, float2* __restrict__ gy, int K,
+           size_t gys) {
+  using C = cx<float>;
+  using G = LP<N>;
+  using Map = typename G::Map;
+  constexpr int H = G::H, R1 = G::R1, NY = G::NY, NZ = G::NZ, LS = G::LS;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  C* plane = reinterpret_cast<C*>(smem_raw);
+  float2* tw = reinterpret_cast<float2*>(plane + N * LS);
+  __shared__ double red[32];
+  const int z = blockIdx.z, tid = threadIdx.x, x = blockIdx.x;
+  const int kz = tid % H, yt = tid / H, y = tid / NZ, zt = tid % NZ;  // column line and row line of the thread
+  ln_load_tw<N>(tw, twtab, tid, G::NT);
+  chain_start();
+  if (sc && finished(sc + z)) return;
+  float2* t = T + z * bt.spec + (size_t)x * N * H;
+  C v[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q) v[q] = ld2(t + (size_t)(q * NY + yt) * H + kz);
+  __syncthreads();  // twiddles
+  ln_forward_nat<N, typename G::PY, +1, 1>(v, plane + Map{}(kz), RowMap<LS>{}, yt, tw);
+  AccF acc;
+  const float2* d = reinterpret_cast<const float2*>(D + z * bt.real) + ((size_t)x * N + y) * H;
+  C* s = plane + y * LS;
+  float2 dv[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q) dv[q] = __ldg(d + q * NZ + zt);
+  ln_inverse<H, typename G::PZ, +1, 2>(v, s, Map{}, zt, tw, [&](int k) { return ln_c2r<N>(s, Map{}, k, tw); });
+  float part = 0.f;
+#pragma unroll
+  for (int q = 0; q < R1; ++q) {
+    const C r = v[q];
+    v[q] = C{r.x * dv[q].x, r.y * dv[q].y};
+    if constexpr (!COARSE) {
+      part += v[q].x * r.x + v[q].y * r.y;
+      if (q % 2 == 1 || q == R1 - 1) {
+        acc.add(part);
+        part = 0.f;
+      }
+    }
+  }
+  __syncthreads();  // the inverse's last reads of the slots
+  ln_forward_nat<H, typename G::PZ, -1, 2>(v, s, Map{}, zt, tw);
+  if constexpr (COARSE) {
+    // kz <= K of every row (element 0 without the kz = N/2 plane), held by the row's first elements
+    const int KZ = K + 1;
+    constexpr int PER = (N * (kDeflMaxRadius + 1) + G::NT - 1) / G::NT;
+    C keep[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * G::NT;
+      if (e < N * KZ) {
+        keep[i] = ln_r2c<N>(plane + (e / KZ) * LS, Map{}, e % KZ, tw);
+        if (e % KZ == 0) keep[i].y = 0.f;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * G::NT;
+      if (e < N * KZ) plane[e] = keep[i];
+    }
+    __syncthreads();
+    // four lanes per output, each over a quarter of the rows
+    const int nout = (2 * K + 1) * KZ;
+    gy += z * gys;
+    for (int o4 = tid; o4 < (4 * nout + 31) / 32 * 32; o4 += G::NT) {
+      const int o = o4 / 4, q4 = o4 % 4, ky = o / KZ - K, kc = o % KZ, step = (ky + N) % N;
+      float sr = 0.f, si = 0.f;
+      if (o < nout) {
+        int e = (int)((unsigned)(q4 * (N / 4)) * (unsigned)step % N);
+        for (int row = q4 * (N / 4); row < (q4 + 1) * (N / 4); ++row) {
+          const C a = plane[row * KZ + kc];
+          const float2 w = tw[e];
+          sr += a.x * w.x - a.y * w.y;
+          si += a.x * w.y + a.y * w.x;
+          e += step;
+          if (e >= N) e -= N;
+        }
+      }
+      const unsigned m = __activemask();
+      sr += __shfl_xor_sync(m, sr, 1);
+      si += __shfl_xor_sync(m, si, 1);
+      sr += __shfl_xor_sync(m, sr, 2);
+      si += __shfl_xor_sync(m, si, 2);
+      if (q4 == 0 && o < nout) gy[(size_t)o * N + x] = make_float2(sr, si);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < R1; ++q) v[q] = ln_r2c<N>(s, Map{}, q * NZ + zt, tw);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < R1; ++q) s[Map{}(q * NZ + zt)] = v[q];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < R1; ++q) v[q] = plane[(q * NY + yt) * LS + Map{}(kz)];
+    __syncthreads();
+    ln_forward<N, typename G::PY, -1>(v, plane + Map{}(kz), RowMap<LS>{}, yt, tw,
+                                      [&](int k, C X, int) { st2(t + (size_t)k * H + kz, X); });
+    const double sum = block_sum_acc(acc, red);
+    partials += (size_t)z * bt.part;
+    if (tid == 0) partials[fin.off + x] = sum;
+    if (fin.n1 == 0 || !last_cta(&sc[z].tick[0], gridDim.x)) return;
+    for (int u = tid; u <= fin.nh; u += G::NT)
+      restore_entry<N>(fin.r + z * bt.spec, fin.rsave + (size_t)z * (2 * fin.nh + 1), fin.modes, fin.nh, u);
+    fin_alpha(partials, fin.n1, fin.off, gridDim.x, sc + z, red);
+  }
+}
+
 }  // namespace wf

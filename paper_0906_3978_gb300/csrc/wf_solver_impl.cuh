@@ -81,6 +81,7 @@ struct Spec {
   static constexpr int NPART = NX + NMID > 2 * NX ? NX + NMID : 2 * NX;
   static dim3 gxy(int nb) { return dim3(NH / NLxy, N, nb); }
   static dim3 gz(int nb) { return dim3(GZ, 1, nb); }
+  static_assert(NMID >= N, "a partial sum per plane");
   static Bat bat() { return Bat{SPEC, V, TAB, NPART}; }
 
   // launch-profile class of a pass: FP64-storage launches (the solves' FP64 residuals, the FP64
@@ -377,8 +378,32 @@ struct Spec {
   struct ZVariant {
     const char* name;
     cudaError_t (*setup)();
-    ZRun run;
+    ZRun run;            // null: the whole middle of the iteration (y, z, y) is k_ln_plane
   };
+  static constexpr bool PLANE = !F64 && N <= kPlaneMax;
+  static cudaError_t plane_setup() {
+    cudaError_t e = cudaSuccess;
+    if constexpr (PLANE) {
+      e = set_smem(k_ln_plane<N, false>, LP<N>::SMEM);
+      if (e == cudaSuccess) e = set_smem(k_ln_plane<N, true>, LP<N>::SMEM);
+    }
+    return e;
+  }
+  static bool whole_planes(const Ctx& c) {
+    if constexpr (PLANE) return pick(c, "zturn", zvariants()).run == nullptr;
+    return false;
+  }
+  // the middle of the iteration on T; fin.n1 > 0: with alpha
+  static void plane(Ctx& c, int nb, ST* T, const SS* D, const ST* tw, double* part, CgScal* sc, const YFin& fin,
+                    cudaStream_t st) {
+    if constexpr (PLANE) {
+      using G = LP<N>;
+      c.launch("plane", (2 * BS + sizeof(SS) * BV) * nb, st, [&] {
+        Ctx::chain(k_ln_plane<N, false>, dim3(N, 1, nb), G::NT, G::SMEM, st, T, D, tw, part, sc, bat(), fin, nullptr, 0,
+                   0);
+      });
+    }
+  }
   template <class G>
   struct ZLn {  // the line engine with geometry G
     static cudaError_t setup() { return set_smem(k_ln_zturn<G>, G::SMEM); }
@@ -403,6 +428,8 @@ struct Spec {
       if constexpr (F64) {
         out.push_back({"fixed", ZFix::setup, ZFix::run});
       } else {
+        // whole planes up to 72 (64^3: 4.33 -> 4.08 ms a solve), the passes above (k_ln_plane tells why)
+        if constexpr (PLANE) out.push_back({"plane", plane_setup, nullptr});
         out.push_back({"lines128", ZLn<GZ1>::setup, ZLn<GZ1>::run});
         if constexpr (N >= 128) out.push_back({"lines256", ZLn<GZ2>::setup, ZLn<GZ2>::run});
       }
@@ -487,7 +514,9 @@ struct Spec {
         fused = true;
       }
     }
-    if (!fused) {
+    if (!fused && whole_planes(c)) {
+      plane(c, nb, T, D, tw, part, sc, fin, st);
+    } else if (!fused) {
       ypass(c, nb, T, tw, sc, +1, st);
       fin.n2 = pick(c, "zturn", zvariants()).run(c, nb, T, D, tw, part + NX, sc, st);
       ypass(c, nb, T, tw, sc, -1, st, fin);
@@ -510,17 +539,28 @@ __global__ void k_make_D(const double* __restrict__ w, SSo* __restrict__ D, cons
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     D[i] = (SSo)(w[i] * f);
 }
-// partials[z * pstride + block] of sum(in) (SQ = false) or sum(in^2) (SQ = true)
+// partials[z * pstride + block] of sum(in) (SQ = false) or sum(in^2) (SQ = true).  Eight loads in flight per thread
+// and six CTAs per SM: latency bound one of each (512^3: 1.60 ms, now under 0.32).
 template <bool SQ>
 __global__ void k_sum(const double* __restrict__ in, size_t n, double* __restrict__ partials, int pstride) {
   __shared__ double red[32];
   const int z = blockIdx.y;
   in += z * n;
   AccD acc;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    if (SQ) acc.add_prod(in[i], in[i]);
-    else acc.add(in[i]);
+  const size_t step = (size_t)gridDim.x * blockDim.x;
+  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  auto add = [&](double v) {
+    if (SQ) acc.add_prod(v, v);
+    else acc.add(v);
+  };
+  for (; i + 7 * step < n; i += 8 * step) {
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = in[i + j * step];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) add(v[j]);
   }
+  for (; i < n; i += step) add(in[i]);
   const double s = block_sum(acc.get(), red);
   if (threadIdx.x == 0) partials[z * pstride + blockIdx.x] = s;
 }
@@ -651,18 +691,18 @@ struct GroupCommon : Group {
   }
 };
 
-// Per-system sums of w and b^2: two reductions into the partial slots [0,152) and [152,304),
-// enqueued with the copy of the scalars back to the host (no synchronisation) ...
+// Per-system sums of w and b^2: two reductions, enqueued with the copy of the scalars back to the host (no synchronisation) ...
 template <int N>
 static wf_status group_sums_begin(Ctx& c, GroupCommon<N>& g, int npart, cudaStream_t st) {
   const size_t V = GroupCommon<N>::V;
   g.h.assign(g.nb, CgScal{});
   WF_TRY(g.push_scalars(st));
   const Bat b{0, 0, 0, npart};
-  c.launch("reduce", 8.0 * V * g.nb, st, [&] { k_sum<false><<<dim3(152, g.nb), 256, 0, st>>>(g.W, V, g.part, npart); });
-  c.launch("fin", 0, st, [&] { k_fin_sum<<<g.nb, 1024, 0, st>>>(g.part, 152, 0, g.sc, b); });
-  c.launch("reduce", 8.0 * V * g.nb, st, [&] { k_sum<true><<<dim3(152, g.nb), 256, 0, st>>>(g.B, V, g.part, npart); });
-  c.launch("fin", 0, st, [&] { k_fin_sum<<<g.nb, 1024, 0, st>>>(g.part, 152, 1, g.sc, b); });
+  const int nblk = std::min(152 * 6, npart);  // partial sums fit a system's slots
+  c.launch("reduce", 8.0 * V * g.nb, st, [&] { k_sum<false><<<dim3(nblk, g.nb), 256, 0, st>>>(g.W, V, g.part, npart); });
+  c.launch("fin", 0, st, [&] { k_fin_sum<<<g.nb, 1024, 0, st>>>(g.part, nblk, 0, g.sc, b); });
+  c.launch("reduce", 8.0 * V * g.nb, st, [&] { k_sum<true><<<dim3(nblk, g.nb), 256, 0, st>>>(g.B, V, g.part, npart); });
+  c.launch("fin", 0, st, [&] { k_fin_sum<<<g.nb, 1024, 0, st>>>(g.part, nblk, 1, g.sc, b); });
   WF_CUDA(cudaGetLastError());
   return g.pull_scalars(st);
 }
@@ -1004,6 +1044,14 @@ struct GroupMixed : GroupCommon<N> {
     const int gw = (nh + 1 + 7) / 8;
     if constexpr (MODE == 1) {
       defl_xr(c, st, n3);
+      if (SF::whole_planes(c)) {
+        if constexpr (SF::PLANE)
+          c.launch("defl_plane", (SF::BS + 4 * SF::BV) * nb, st, [&] {
+            using G = LP<N>;
+            Ctx::chain(k_ln_plane<N, true>, dim3(N, 1, nb), G::NT, G::SMEM, st, T, D, tw32, nullptr, sc, bf, YFin{}, Gy, K,
+                       gys);
+          });
+      } else {
       SF::ypass(c, nb, T, tw32, sc, +1, st);
       c.launch("defl_z", (SF::BS + 4 * SF::BV) * nb, st, [&] {
         using G = typename SF::GZ1;
@@ -1013,6 +1061,7 @@ struct GroupMixed : GroupCommon<N> {
       c.launch("defl_y", 8.0 * gzs * nb, st, [&] {
         Ctx::chain(k_ycoarse<float, N>, dim3(N, nb), 256, ysm, st, Gz, tw32, Gy, K, sc, gzs, gys);
       });
+      }
     }
     c.launch("defl_x", 8.0 * gys * nb, st, [&] {
       Ctx::chain(k_xcoarse<float, N, MODE>, dim3(gw, nb), 256, 0, st, Gy, rh, ct, mt, tw32, dmodes, nh, K, gco, rco, sc,
@@ -1023,9 +1072,7 @@ struct GroupMixed : GroupCommon<N> {
                  out, rsave, dpart, sc, bf, doff);
     });
   }
-  // T = IFFT_x(c r), register-staged (a persistent form on tensor copies along x, the y pass's tile
-  // walk with the table multiply and partner column added, took 0.52 ms at 512^3 against 0.42: one
-  // CTA per SM cannot hide the table gathers and the strided partner loads)
+  // T = IFFT_x(c r); n3 > 0: beside it beta and the stop test of the iteration before
   void defl_xr(Ctx& c, cudaStream_t st, int n3) {
     const Bat bf = SF::bat();
     c.launch("defl_xr", 2 * SF::BS * nb, st, [&] {
@@ -1384,7 +1431,11 @@ wf_status tune_spec(Ctx& c, std::string& report) {
       CgScal* sc;
       const char* name;
       void run(Ctx& c, int nb, ST* buf, const ST* tw, const CgScal*, int, cudaStream_t st) const {
-        v->run(c, nb, buf, D, tw, part, sc, st);
+        // the whole middle of an iteration, since one variant is
+      if (!v->run) return SP::plane(c, nb, buf, D, tw, part, sc, YFin{}, st);
+      SP::ypass(c, nb, buf, tw, nullptr, +1, st);
+      v->run(c, nb, buf, D, tw, part, sc, st);
+      SP::ypass(c, nb, buf, tw, nullptr, -1, st);
       }
     };
     std::vector<ZAdapter> za;
