@@ -249,7 +249,7 @@ wf_status response_tables(const wf_grid& g, const wf_response* r, std::vector<do
                           std::vector<double>& ginv);
 // out = F^-1 diag(table[n2]) F in / n^3 (FP64 transforms; out may equal in)
 wf_status multiply_fourier(Ctx& c, int n, const double* in, double* out, const std::vector<double>& table,
-                           cudaStream_t st);
+                           cudaStream_t st, double kf = 0.0, double r_s = 0.0);
 // Solve every system (grouped by size and precision, groups interleaved on the device).
 // Returns WF_OK if all converged, else the first failing status; infos[i] filled for each.
 wf_status solve_many(Ctx& c, std::vector<SolveArgs*>& sys, std::vector<wf_solve_info*>& infos, cudaStream_t st);

@@ -66,6 +66,14 @@ k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, CgScal* __re
   ln_forward<N, FxPlan<N>, DIR>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X, int) { p[(size_t)k * NH] = fx_to2(X, f); });
 }
 
+// tab[n2] = exp(-(kf r_s)^2 n2 / 2), the argument rounded operation by operation in the definition's order
+static __global__ void k_gauss_table(double* __restrict__ tab, int n, double kf, double r_s) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  const double h = __dmul_rn(__dmul_rn(__dmul_rn(-0.5, kf), kf), (double)i);
+  tab[i] = exp(__dmul_rn(__dmul_rn(h, r_s), r_s));
+}
+
 // ---- Fourier tables as Q62 digits ----------------------------------------------------------------
 // tab[i] 2^-e as digits (high, low), in place; |tab[i]| < 2^e, e = exps[z estride].  grid (., systems)
 static __global__ void k_table_digits(double* __restrict__ tab, int len, const int* __restrict__ exps, int estride) {
@@ -427,7 +435,7 @@ k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double
 }
 
 // ==========================================================================================
-// The FP64 CG passes (the work of k_cg_xinv, k_cg_xupd and k_zturn): vector updates and sums in FP64,
+// The FP64 CG passes (the work of k_cg_xinv, k_cg_xupd and k_ln_zturn): vector updates and sums in FP64,
 // transforms in fixed point.  UNIT_M (every system preconditioned): m = 1 but at k = 0, where it is 0,
 // and the m table holds 1 / c^2 instead, which the residual estimate would otherwise divide for.  108^3 per
 // launch (events, with ~5 us of bracketing), FP64 butterflies -> here: x pass 1 58.8 -> 43 us, x pass 2 87 -> 43,

@@ -247,11 +247,11 @@ k_density_moments(const unsigned long long* __restrict__ hist, int n_bins, doubl
 // host side
 // ------------------------------------------------------------------------------------------
 wf_status multiply_fourier(Ctx& c, int n, const double* in, double* out, const std::vector<double>& table,
-                           cudaStream_t st) {
+                           cudaStream_t st, double kf, double r_s) {
   switch (n) {
 #define WF_CASE(N) \
   case N:          \
-    return fourier_multiply_n<N>(c, in, out, table, st);
+    return fourier_multiply_n<N>(c, in, out, table, kf, r_s, st);
     WF_SIZES(WF_CASE)
 #undef WF_CASE
     default:
@@ -264,10 +264,7 @@ static inline size_t n2_entries(int n) { return (size_t)3 * (n / 2) * (n / 2) + 
 
 wf_status smooth_run(Ctx& c, const wf_grid& g, const double* in, double r_s, double* out, cudaStream_t st) {
   if (!in || !out || !(r_s >= 0.0) || !std::isfinite(r_s)) return WF_ERR_ARG;
-  std::vector<double> t(n2_entries(g.n));
-  const double kf = 2.0 * 3.14159265358979323846 / g.box;
-  for (size_t n2 = 0; n2 < t.size(); ++n2) t[n2] = std::exp(-0.5 * kf * kf * (double)n2 * r_s * r_s);
-  return multiply_fourier(c, g.n, in, out, t, st);
+  return multiply_fourier(c, g.n, in, out, std::vector<double>(), st, 2.0 * 3.14159265358979323846 / g.box, r_s);
 }
 
 // <K D>_mu of Sec. 3.3.3 ("Redshift distortion operator"): the mean over mu in [0, 1] of

@@ -38,10 +38,11 @@ std::vector<int4> deflation_modes(int K);
 int deflation_ncp(int K);
 
 // out = F^-1 [table(|m|^2) F in] for one field of size N (instantiated with the solve drivers of
-// each size); table has 3 (N/2)^2 + 1 entries.
+// each size); table has 3 (N/2)^2 + 1 entries, or is empty: then it is the Gaussian exp(-kf^2 n2 r_s^2 / 2), made on
+// the device (its exponentials took the host 0.2 ms of the 0.83 ms of a smoothing at 256^3).
 template <int N>
-wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::vector<double>& table,
-                             cudaStream_t st);
+wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::vector<double>& table, double kf,
+                             double r_s, cudaStream_t st);
 
 // Time every launch variant of the spectral passes of grid size N in precision prec (the FP32
 // inner passes for WF_MIXED, the FP64 ones for WF_FP64), keep the fastest per pass in c.tuned and

@@ -1267,9 +1267,11 @@ struct GroupMixed : GroupCommon<N> {
 // B^-1 Z^-1 of Eq. eq:DEC.  The x pass applies the table as it applies the prior; the transforms
 // are the solver's FP64 passes.  in may equal out.
 template <int N>
-wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::vector<double>& table, cudaStream_t st) {
+wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::vector<double>& table, double kf,
+                             double r_s, cudaStream_t st) {
   using SD = Spec<FP64Arith, N>;
-  if ((int)table.size() != SD::TAB) return WF_ERR_ARG;
+  const bool gauss = table.empty();
+  if (!gauss && (int)table.size() != SD::TAB) return WF_ERR_ARG;
   int* err;
   WF_TRY(c.err_word(&err));
   WF_CUDA(SD::attrs());
@@ -1281,8 +1283,14 @@ wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::v
   WF_TRY(c.get("sm_e", sizeof(int), (void**)&exps));
   WF_TRY(c.get_pinned("sm_eh", sizeof(int), (void**)&hexp));
   double* gt;
-  WF_TRY(upload_tables<double>(c, "sm_g", table, &gt, st));
-  *hexp = table_exp(table.data(), table.size());
+  if (gauss) {
+    WF_TRY(c.get("sm_g", SD::TAB * sizeof(double), (void**)&gt));
+    c.launch("tables", 0, st, [&] { k_gauss_table<<<(SD::TAB + 255) / 256, 256, 0, st>>>(gt, SD::TAB, kf, r_s); });
+    *hexp = 1;  // the largest entry is 1
+  } else {
+    WF_TRY(upload_tables<double>(c, "sm_g", table, &gt, st));
+    *hexp = table_exp(table.data(), table.size());
+  }
   WF_CUDA(cudaMemcpyAsync(exps, hexp, sizeof(int), cudaMemcpyHostToDevice, st));
   c.launch("tables", 0, st, [&] { k_table_digits<<<dim3((SD::TAB + 255) / 256, 1), 256, 0, st>>>(gt, SD::TAB, exps, 1); });
   SD::zfwd(c, 1, in, T, nullptr, nullptr, nullptr, st);
