@@ -353,20 +353,27 @@ k_project_mask(const float4* __restrict__ pix, const unsigned long long* __restr
 // the host table rtab for count < kMaskRcp, else the correctly rounded reciprocal.  acc: the three words of
 // each cell
 constexpr int kMaskRcp = 4096;
+WF_D double mask_value(unsigned long long ss, unsigned long long sr, unsigned long long nc,
+                       const double* __restrict__ rtab) {
+  if (nc == 0) return 0.0;
+  const double rc = nc < (unsigned long long)kMaskRcp ? rtab[nc] : __drcp_rn(__ull2double_rn(nc));
+  return __dmul_rn(__dmul_rn(__dmul_rn(__ull2double_rn(ss), 0x1p-32), rc),
+                   __dmul_rn(__dmul_rn(__ull2double_rn(sr), 0x1p-32), rc));
+}
+// Two cells a thread (the cell count is even): three 16-byte loads of neighbouring words.  512^3: 1.17 ms, 1.32 with
+// 8-byte loads 24 bytes apart.
 __global__ void __launch_bounds__(256)
-k_mask_finish(const unsigned long long* __restrict__ acc, const double* __restrict__ rtab, size_t V,
+k_mask_finish(const ulonglong2* __restrict__ acc, const double* __restrict__ rtab, size_t V,
               double* __restrict__ w, long long* __restrict__ counts) {
-#pragma unroll 4
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < V; c += (size_t)gridDim.x * blockDim.x) {
-    const unsigned long long ss = acc[3 * c], sr = acc[3 * c + 1], nc = acc[3 * c + 2];
-    double v = 0.0;
-    if (nc) {
-      const double rc = nc < (unsigned long long)kMaskRcp ? rtab[nc] : __drcp_rn(__ull2double_rn(nc));
-      v = __dmul_rn(__dmul_rn(__dmul_rn(__ull2double_rn(ss), 0x1p-32), rc),
-                    __dmul_rn(__dmul_rn(__ull2double_rn(sr), 0x1p-32), rc));
+#pragma unroll 2
+  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < V / 2; c += (size_t)gridDim.x * blockDim.x) {
+    const ulonglong2 a = acc[3 * c], b = acc[3 * c + 1], d = acc[3 * c + 2];
+    w[2 * c] = mask_value(a.x, a.y, b.x, rtab);
+    w[2 * c + 1] = mask_value(b.y, d.x, d.y, rtab);
+    if (counts) {
+      counts[2 * c] = (long long)b.x;
+      counts[2 * c + 1] = (long long)d.y;
     }
-    w[c] = v;
-    if (counts) counts[c] = (long long)nc;
   }
 }
 
@@ -431,7 +438,7 @@ wf_status project_mask_run(Ctx& c, const wf_grid& g, const double* sky, int n_al
     k_project_mask<<<152 * 16, 256, 0, st>>>(pix, qsky, dqr, a, acc);
   });
   c.launch("mask_finish", 32.0 * (double)V, st, [&] {
-    k_mask_finish<<<152 * 8, 256, 0, st>>>(acc, drtab, V, w, reinterpret_cast<long long*>(counts));
+    k_mask_finish<<<152 * 8, 256, 0, st>>>(reinterpret_cast<const ulonglong2*>(acc), drtab, V, w, reinterpret_cast<long long*>(counts));
   });
   WF_CUDA(cudaGetLastError());
   int* hp = reinterpret_cast<int*>(c.host_pinned);
