@@ -22,8 +22,6 @@ struct df32 {
   float hi, lo;
 };
 
-WF_D df32 df_make(float h, float l) { return df32{h, l}; }
-
 // s + e = a + b exactly (Knuth two-sum, no magnitude assumption)
 WF_D void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -108,7 +106,6 @@ template <> struct RT<df32> {
 template <class R> struct __align__(2 * sizeof(R)) cx {
   R x, y;
 };
-template <class R> WF_D cx<R> mkc(R a, R b) { return cx<R>{a, b}; }
 template <class R> WF_D cx<R> operator+(cx<R> a, cx<R> b) { return cx<R>{a.x + b.x, a.y + b.y}; }
 template <class R> WF_D cx<R> operator-(cx<R> a, cx<R> b) { return cx<R>{a.x - b.x, a.y - b.y}; }
 template <class R> WF_D cx<R> operator*(cx<R> a, cx<R> b) {

@@ -235,8 +235,4 @@ WF_D void fft_line(cx<R>* col, int t, const cx<R>* tw, bool act = true) {
   fft_passes<R, M, 0, 1, TPL, DIR, TWS, RMAX>(col, Strided<LD>{}, t, tw, act);
 }
 
-// Threads per line for a line of length M: one radix-8-or-smaller butterfly group per thread
-// at elements-per-thread E.
-constexpr int tpl_for(int M, int E) { return M / E >= 1 ? M / E : 1; }
-
 }  // namespace wf

@@ -66,9 +66,6 @@ struct Bat {
 
 template <class R> constexpr int tile_lines() { return 128 / (int)sizeof(cx<R>); }
 template <class R> constexpr int elems_per_thread() { return sizeof(cx<R>) == 8 ? 16 : 8; }
-template <class R, int M> constexpr int tpl() {
-  return M / elems_per_thread<R>() >= 1 ? M / elems_per_thread<R>() : 1;
-}
 constexpr int cmin(int a, int b) { return a < b ? a : b; }
 // largest divisor of n that is <= cap (tile widths must divide the dimension they tile)
 constexpr int div_le(int n, int cap) {
