@@ -195,9 +195,10 @@ def oracle_sample(pr, iters, deadline_s=40.0, single_thread=True):
 
 
 def fp64_kernels(ctx, prof, n):
-    """The FP64-ALU-bound passes of the step (the three passes of the ideal low-pass and the passes of
-    the FP64 residual) against the device's FP64 rate measured here (wf_fp64_rate) and the nominal
-    1.25 TFLOP/s.  Algorithmic flops:
+    """The passes of the step with FP64 storage (the three passes of the ideal low-pass and the passes of
+    the FP64 residual): their transforms run in 64-bit fixed point, so the rate of their algorithmic flops is set
+    beside the device's FP64 FMA rate measured here (wf_fp64_rate; a fraction above 1 is what the integer pipe
+    gains) and the nominal 1.25 TFLOP/s.  Algorithmic flops:
     2.5 L log2 L per real transform of length L; each pass line takes a real transform of length 2n
     and an inverse of length n; the z pass has (2n)^2 lines, the y pass 2n n, the x pass n n.  The z
     pass skips the rows no galaxy reaches (their output is zero), so its figure counts flops it did
@@ -508,7 +509,7 @@ def batch_mocks(count=96, seed=2000):
 
 def bench_postproc(ctx, pr, s_rec, s_ref, w, b, nbar, defl=0):
     """Sec. 4.1 / 5.5 evaluation of the 512^3 reconstruction: Gaussian smoothing at r_S = 10, 20,
-    30 Mpc/h (FP64 transforms, FP64-ALU-bound), the quality measures of the mixed solution
+    30 Mpc/h (FP64 storage, fixed-point transforms), the quality measures of the mixed solution
     against the FP64 one, and the density statistics of the r_S = 10 field in the paper's radial
     shells and observed / unobserved regions (1 + delta bins of 0.03 from -1); also the solve with
     Z and B inside R and the projection of a sky map into the 3D mask."""
