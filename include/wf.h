@@ -94,7 +94,7 @@ typedef struct {
   int max_iter;       /* cap on CG iterations (inner iterations summed for WF_MIXED) */
   wf_precision prec;
   double inner_tol;   /* WF_MIXED: largest relative reduction asked of one inner solve (<= 0:
-                         1e-4; each step asks for half the remaining reduction, at most this) */
+                         1e-4; each step asks for a quarter of the remaining reduction, at most this) */
   int precond;        /* 1: CG in Fourier variables split-preconditioned by S^(1/2)
                          (same canonical system and residual); 0: plain CG on A */
   int deflate;        /* WF_MIXED only: 0 off; K in [1, 12] with 4 K < n: each inner CG is
