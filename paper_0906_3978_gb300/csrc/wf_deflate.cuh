@@ -210,87 +210,87 @@ k_defl_mu(const float* __restrict__ Einv, const float* __restrict__ gco, const f
   __syncthreads();
   const int warp = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   auto product = [&] {
-  if (warp > nh) return;
-  const int ra = warp < nh ? 1 + 2 * warp : 0;
-  const float4* rowa = reinterpret_cast<const float4*>(Einv + (size_t)ra * ncp);
-  const float4* rowb = reinterpret_cast<const float4*>(Einv + (size_t)(ra + 1) * ncp);
-  const float4* g4 = reinterpret_cast<const float4*>(gs);
-  // The products are summed exactly in double-float: the rows of E^-1 cancel heavily against g
-  // (its weak directions carry entries up to 1/lambda_min), and an FP32 sum of nc terms loses
-  // ~sqrt(nc) u of the terms' magnitude, which an ill-conditioned E turns into a stalled CG.
-  // one accumulator per vector component (four independent chains per row); the loads of four
-  // vectors of each row are issued before their products, to keep enough of them in flight
-  AccF aa[4], ab[4];
-  const bool two = warp < nh;
-  constexpr int U = 4;
-  const int nq = ncp / 4;  // a multiple of 32: ncp is a multiple of 128
-  for (int q0 = lane; q0 < nq; q0 += 32 * U) {
-    float4 av[U], bv[U];
+    if (warp > nh) return;
+    const int ra = warp < nh ? 1 + 2 * warp : 0;
+    const float4* rowa = reinterpret_cast<const float4*>(Einv + (size_t)ra * ncp);
+    const float4* rowb = reinterpret_cast<const float4*>(Einv + (size_t)(ra + 1) * ncp);
+    const float4* g4 = reinterpret_cast<const float4*>(gs);
+    // The products are summed exactly in double-float: the rows of E^-1 cancel heavily against g
+    // (its weak directions carry entries up to 1/lambda_min), and an FP32 sum of nc terms loses
+    // ~sqrt(nc) u of the terms' magnitude, which an ill-conditioned E turns into a stalled CG.
+    // one accumulator per vector component (four independent chains per row); the loads of four
+    // vectors of each row are issued before their products, to keep enough of them in flight
+    AccF aa[4], ab[4];
+    const bool two = warp < nh;
+    constexpr int U = 4;
+    const int nq = ncp / 4;  // a multiple of 32: ncp is a multiple of 128
+    for (int q0 = lane; q0 < nq; q0 += 32 * U) {
+      float4 av[U], bv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int q = q0 + 32 * u;
-      av[u] = q < nq ? __ldg(rowa + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-      bv[u] = (two && q < nq) ? __ldg(rowb + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+      for (int u = 0; u < U; ++u) {
+        const int q = q0 + 32 * u;
+        av[u] = q < nq ? __ldg(rowa + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+        bv[u] = (two && q < nq) ? __ldg(rowb + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int q = q0 + 32 * u;
-      if (q >= nq) break;
-      const float4 g = g4[q];
-      aa[0].add_prod(av[u].x, g.x);
-      aa[1].add_prod(av[u].y, g.y);
-      aa[2].add_prod(av[u].z, g.z);
-      aa[3].add_prod(av[u].w, g.w);
-      if (two) {
-        ab[0].add_prod(bv[u].x, g.x);
-        ab[1].add_prod(bv[u].y, g.y);
-        ab[2].add_prod(bv[u].z, g.z);
-        ab[3].add_prod(bv[u].w, g.w);
+      for (int u = 0; u < U; ++u) {
+        const int q = q0 + 32 * u;
+        if (q >= nq) break;
+        const float4 g = g4[q];
+        aa[0].add_prod(av[u].x, g.x);
+        aa[1].add_prod(av[u].y, g.y);
+        aa[2].add_prod(av[u].z, g.z);
+        aa[3].add_prod(av[u].w, g.w);
+        if (two) {
+          ab[0].add_prod(bv[u].x, g.x);
+          ab[1].add_prod(bv[u].y, g.y);
+          ab[2].add_prod(bv[u].z, g.z);
+          ab[3].add_prod(bv[u].w, g.w);
+        }
       }
     }
-  }
-  double da = (aa[0].get() + aa[1].get()) + (aa[2].get() + aa[3].get());
-  double db = (ab[0].get() + ab[1].get()) + (ab[2].get() + ab[3].get());
-  for (int o = 16; o > 0; o >>= 1) {
-    da += __shfl_xor_sync(0xffffffffu, da, o);
-    db += __shfl_xor_sync(0xffffffffu, db, o);
-  }
-  // a system whose coarse block failed the condition guard (k_defl_guard), or whose deflated inner
-  // solve failed (noco, set by the host), gets mu = 0: plain CG
-  const bool plain = off[z] || sc[z].noco;
-  const float sa = plain ? 0.f : (float)da, sb = plain ? 0.f : (float)db;
-  if (lane != 0) return;
-  if (warp < nh) {
-    const int4 md = modes[warp];
-    const float h = 0.70710678118654752f;
-    const cx<R> v{RT<R>::from_f(sa * h), RT<R>::from_f(sb * h)};
-    const size_t s1 = dslot<N>(md.x, md.y, md.z);
-    const size_t s2 = dslot<N>(-md.x, -md.y, 0);
-    if constexpr (MODE == 0) {
-      st_c(vec + s1, v);
-      if (md.z == 0) st_c(vec + s2, conj(v));
+    double da = (aa[0].get() + aa[1].get()) + (aa[2].get() + aa[3].get());
+    double db = (ab[0].get() + ab[1].get()) + (ab[2].get() + ab[3].get());
+    for (int o = 16; o > 0; o >>= 1) {
+      da += __shfl_xor_sync(0xffffffffu, da, o);
+      db += __shfl_xor_sync(0xffffffffu, db, o);
+    }
+    // a system whose coarse block failed the condition guard (k_defl_guard), or whose deflated inner
+    // solve failed (noco, set by the host), gets mu = 0: plain CG
+    const bool plain = off[z] || sc[z].noco;
+    const float sa = plain ? 0.f : (float)da, sb = plain ? 0.f : (float)db;
+    if (lane != 0) return;
+    if (warp < nh) {
+      const int4 md = modes[warp];
+      const float h = 0.70710678118654752f;
+      const cx<R> v{RT<R>::from_f(sa * h), RT<R>::from_f(sb * h)};
+      const size_t s1 = dslot<N>(md.x, md.y, md.z);
+      const size_t s2 = dslot<N>(-md.x, -md.y, 0);
+      if constexpr (MODE == 0) {
+        st_c(vec + s1, v);
+        if (md.z == 0) st_c(vec + s2, conj(v));
+      } else {
+        dpart[warp] = (double)rco[ra] * (double)sa + (double)rco[ra + 1] * (double)sb;
+        const ST o1 = vec[s1];
+        rsave[2 * warp] = o1;
+        st_c(vec + s1, ld_c<R>(&o1) - v);
+        if (md.z == 0) {
+          const ST o2 = vec[s2];
+          rsave[2 * warp + 1] = o2;
+          st_c(vec + s2, ld_c<R>(&o2) - conj(v));
+        }
+      }
     } else {
-      dpart[warp] = (double)rco[ra] * (double)sa + (double)rco[ra + 1] * (double)sb;
-      const ST o1 = vec[s1];
-      rsave[2 * warp] = o1;
-      st_c(vec + s1, ld_c<R>(&o1) - v);
-      if (md.z == 0) {
-        const ST o2 = vec[s2];
-        rsave[2 * warp + 1] = o2;
-        st_c(vec + s2, ld_c<R>(&o2) - conj(v));
+      const cx<R> v{RT<R>::from_f(sa), RT<R>::c(0.0)};
+      if constexpr (MODE == 0) {
+        st_c(vec, v);
+      } else {
+        dpart[nh] = (double)rco[0] * (double)sa;
+        const ST o = vec[0];
+        rsave[2 * nh] = o;
+        st_c(vec, ld_c<R>(&o) - v);
       }
     }
-  } else {
-    const cx<R> v{RT<R>::from_f(sa), RT<R>::c(0.0)};
-    if constexpr (MODE == 0) {
-      st_c(vec, v);
-    } else {
-      dpart[nh] = (double)rco[0] * (double)sa;
-      const ST o = vec[0];
-      rsave[2 * nh] = o;
-      st_c(vec, ld_c<R>(&o) - v);
-    }
-  }
   };
   product();
   if constexpr (MODE == 1) {  // the last CTA takes <r, z> and beta

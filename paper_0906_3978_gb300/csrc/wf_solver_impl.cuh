@@ -1054,15 +1054,15 @@ struct GroupMixed : GroupCommon<N> {
                        gys);
           });
       } else {
-      SF::ypass(c, nb, T, tw32, sc, +1, st);
-      c.launch("defl_z", (SF::BS + 4 * SF::BV) * nb, st, [&] {
-        using G = typename SF::GZ1;
-        Ctx::chain(k_ln_zcoarse<G>, dim3(G::GZ, 1, nb), G::NT, G::SMEM, st, T, D, tw32, Gz, K, sc, bf, gzs);
-      });
-      const size_t ysm = ((size_t)N * (K + 1) + N) * sizeof(float2);
-      c.launch("defl_y", 8.0 * gzs * nb, st, [&] {
-        Ctx::chain(k_ycoarse<float, N>, dim3(N, nb), 256, ysm, st, Gz, tw32, Gy, K, sc, gzs, gys);
-      });
+        SF::ypass(c, nb, T, tw32, sc, +1, st);
+        c.launch("defl_z", (SF::BS + 4 * SF::BV) * nb, st, [&] {
+          using G = typename SF::GZ1;
+          Ctx::chain(k_ln_zcoarse<G>, dim3(G::GZ, 1, nb), G::NT, G::SMEM, st, T, D, tw32, Gz, K, sc, bf, gzs);
+        });
+        const size_t ysm = ((size_t)N * (K + 1) + N) * sizeof(float2);
+        c.launch("defl_y", 8.0 * gzs * nb, st, [&] {
+          Ctx::chain(k_ycoarse<float, N>, dim3(N, nb), 256, ysm, st, Gz, tw32, Gy, K, sc, gzs, gys);
+        });
       }
     }
     c.launch("defl_x", 8.0 * gys * nb, st, [&] {
