@@ -18,15 +18,15 @@
 // basis is orthonormal for the CG inner product (the full-spectrum sum of Re(conj u v)).
 //
 // Per iteration (FP32 vectors, the packed half spectrum of wf_spectral.cuh):
-//   k_ln_xcr    T = IFFT_x(c r); then the solver's y pass, IFFT_y (wf_lines32.cuh)
-//   k_ln_zcoarse  IFFT_z, times D, FFT_z; keep kz <= K (the kz = 0 plane only)   -> Gz [N][N][K+1]
+//   k_xcr       T = IFFT_x(c r); then the solver's y pass, IFFT_y
+//   k_zcoarse   IFFT_z, times D, FFT_z; keep kz <= K (the kz = 0 plane only)   -> Gz [N][N][K+1]
 //   k_ycoarse   DFT along y at |ky| <= K                                      -> Gy [2K+1][K+1][N]
 //   k_xcoarse   DFT along x at the coarse modes; g = coords of (m - 1) r + c Gc, and coords of r
 //   k_defl_mu   mu = E^-1 g (one warp per mode); r -= Z mu kept aside for the x pass, which forms
 //               p = (r - Z mu) + beta p; partials of <r, Z mu>
 //               and, by its last CTA, <r, z> = <r, r> - <r, Z mu>; beta = <r, z> / <r, z>_prev; alpha's
 //               numerator
-//   (x pass 1)  then the forward y pass (or k_defl_restore) puts the saved coarse entries of r back
+//   (x pass 1)  then k_defl_alpha puts the saved coarse entries of r back
 #pragma once
 #include "wf_spectral.cuh"
 
@@ -40,13 +40,161 @@ template <int N> WF_D size_t dslot(int kx, int ky, int kz) {
 }
 
 // ------------------------------------------------------------------------------------------
+// x stage of the coarse projection: T = IFFT_x(c (.) r), the first pass of the inverse transform
+// of c r (the CG x pass 1 without its vector updates: r and the table gathers in flight together,
+// the packed column combined with its partner line at -ky).  grid (N/2 / NL, N, systems).
+// ------------------------------------------------------------------------------------------
+template <class R, int N, int RMAX = 8>
+__global__ void __launch_bounds__(XYG<R, N>::NT)
+k_xcr(const typename Store<R>::T* __restrict__ r, typename Store<R>::T* __restrict__ T,
+      const typename Store<R>::S* __restrict__ ctab, const typename Store<R>::T* __restrict__ twtab,
+      const CgScal* __restrict__ sc, Bat bt) {
+  using G = XYG<R, N>;
+  using SS = typename Store<R>::S;
+  using VT = typename G::VT;
+  constexpr int NH = G::NH;
+  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
+  cx<R>* tw = tile + G::M * G::LD;
+  const int z = blockIdx.z;
+  chain_start();
+  if (finished(sc + z)) return;
+  r += z * bt.spec;
+  T += z * bt.spec;
+  ctab += z * bt.tab;
+  const int tid = threadIdx.x;
+  const int kz0 = blockIdx.x * G::NL, ky = blockIdx.y;
+  const int ky_s = sfreq(ky, N);
+  load_tw<R, G::M, 2 * N>(tw, twtab, tid, G::NT);
+  const size_t rowstride = (size_t)N * NH;
+  const size_t base = (size_t)ky * NH + kz0;
+  constexpr int CH = 4;
+#pragma unroll
+  for (int k0 = 0; k0 < G::PER; k0 += CH) {
+    VT rv[CH];
+    SS cv[CH][G::VW];
+#pragma unroll
+    for (int k = 0; k < CH && k0 + k < G::PER; ++k) {
+      const int idx = tid + (k0 + k) * G::NT;
+      if (G::EVEN || idx < G::NVEC) {
+        const int i = idx / G::NV, c0 = (idx % G::NV) * G::VW;
+        rv[k] = *reinterpret_cast<const VT*>(r + base + (size_t)i * rowstride + c0);
+        const int kxs = sfreq(i, N);
+#pragma unroll
+        for (int u = 0; u < G::VW; ++u) {
+          const int kz = kz0 + c0 + u;
+          cv[k][u] = ctab[kxs * kxs + ky_s * ky_s + kz * kz];
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < CH && k0 + k < G::PER; ++k) {
+      const int idx = tid + (k0 + k) * G::NT;
+      if (G::EVEN || idx < G::NVEC) {
+        const int i = idx / G::NV, c0 = (idx % G::NV) * G::VW;
+        SS* rs = reinterpret_cast<SS*>(&rv[k]);
+#pragma unroll
+        for (int u = 0; u < G::VW; ++u)
+          if (kz0 + c0 + u != 0) {  // column kz = 0 stays raw for the packed-column combine
+            rs[2 * u] *= cv[k][u];
+            rs[2 * u + 1] *= cv[k][u];
+          }
+        vec_to_tile<G>(tile, i, c0, rv[k]);
+      }
+    }
+  }
+  if (kz0 == 0) {  // partner line of column 0: r at (kx, -ky, 0)
+    const size_t pb = (size_t)((N - ky) % N) * NH;
+    for (int i = tid; i < G::M; i += G::NT) tile[i * G::LD + G::NL] = ld_c<R>(r + pb + (size_t)i * rowstride);
+  }
+  __syncthreads();
+  if (kz0 == 0) combine_col0<R, N, G::LD, G::NL>(tile, ky_s, ctab, tid, G::NT);
+  fft_line<R, G::M, G::TPL, G::LD, +1, 1, cmin(RMAX, rmax_for(G::M, G::TPL))>(tile + tid % G::NL, tid / G::NL, tw);
+  tile_store<G>(tile, T + base, rowstride, tid);
+}
+
+// ------------------------------------------------------------------------------------------
+// z stage of the coarse projection (the z turn without its full store): each (x, y) line of the
+// y-transformed field is taken to real space, multiplied by D, transformed forward, and its
+// kz = 0..K coefficients are stored; element 0 keeps only the kz = 0 plane (its real part), so the
+// later x / y DFTs give that plane's coefficients directly.  grid (N*N / NL, 1, systems).
+// ------------------------------------------------------------------------------------------
+template <class R, int N>
+__global__ void __launch_bounds__(ZG<R, N>::NT)
+k_zcoarse(const typename Store<R>::T* __restrict__ spec, const typename Store<R>::S* __restrict__ D,
+          const typename Store<R>::T* __restrict__ twtab, typename Store<R>::T* __restrict__ gz, int K,
+          const CgScal* __restrict__ sc, Bat bt, size_t gzs) {
+  using G = ZG<R, N>;
+  using SS = typename Store<R>::S;
+  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
+  cx<R>* tw = tile + G::M * G::LD;  // 2N entries
+  const int z = blockIdx.z;
+  chain_start();
+  if (finished(sc + z)) return;
+  spec += z * bt.spec;
+  D += z * bt.real;
+  gz += z * gzs;
+  const int tid = threadIdx.x;
+  const size_t row0 = (size_t)blockIdx.x * G::NL;
+  if (tid < G::NL) prefetch_l2(D + (row0 + tid) * N, N * sizeof(SS));
+  for (int e = tid; e < 2 * N; e += G::NT) tw[e] = ld_c<R>(twtab + e);
+  zrows_load<G>(tile, spec, row0, tid);
+  __syncthreads();
+  const int l = tid % G::NL, t = tid / G::NL;
+  c2r_prep<R, N, G::LD>(tile + l, t, G::TPL, tw);
+  __syncthreads();
+  fft_line<R, G::M, G::TPL, G::LD, +1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
+  // real samples 2i, 2i+1 of line l sit in element i
+#pragma unroll 4
+  for (int k = 0; k < G::PER; ++k) {
+    const int idx = tid + k * G::NT;
+    if (!(G::EVEN || idx < G::NVEC)) continue;
+    const int ll = idx / G::NV, i = (idx % G::NV) * G::VW;
+    const SS* dp = D + (row0 + ll) * N + 2 * i;
+    if constexpr (G::VW == 2) {
+      const float4 d = *reinterpret_cast<const float4*>(dp);
+      cx<R> a = tile[i * G::LD + ll], b = tile[(i + 1) * G::LD + ll];
+      a.x = a.x * RT<R>::from_f(d.x);
+      a.y = a.y * RT<R>::from_f(d.y);
+      b.x = b.x * RT<R>::from_f(d.z);
+      b.y = b.y * RT<R>::from_f(d.w);
+      tile[i * G::LD + ll] = a;
+      tile[(i + 1) * G::LD + ll] = b;
+    } else {
+      const double2 d = *reinterpret_cast<const double2*>(dp);
+      cx<R> a = tile[i * G::LD + ll];
+      a.x = a.x * RT<R>::c(d.x);
+      a.y = a.y * RT<R>::c(d.y);
+      tile[i * G::LD + ll] = a;
+    }
+  }
+  __syncthreads();
+  fft_line<R, G::M, G::TPL, G::LD, -1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
+  r2c_post<R, N, G::LD>(tile + l, t, G::TPL, tw);
+  __syncthreads();
+  for (int e = tid; e < G::NL * (K + 1); e += G::NT) {
+    const int ll = e / (K + 1), i = e % (K + 1);
+    cx<R> v = tile[i * G::LD + ll];
+    if (i == 0) v.y = RT<R>::c(0.0);  // drop the kz = N/2 plane packed beside kz = 0
+    st_c(gz + (row0 + ll) * (K + 1) + i, v);
+  }
+}
+
+// ------------------------------------------------------------------------------------------
 // y stage: Gy[ky + K][kz][x] = sum_y exp(-2 pi i ky y / N) Gz[x][y][kz] for |ky| <= K.
-// grid (N, systems), 256 threads; shared memory N (K + 1) + N complex values.
+// With n3 > 0 one more CTA takes beta and the stop test of the iteration before from its n3 pairs of partial sums
+// (nothing before this kernel uses them; a launch of its own costs 3 us, and in k_xcr the sums' code took the registers
+// of its loads in flight: 512^3 solve 382 ms, here 344).
+// grid (N + (n3 > 0), systems), 256 threads; shared memory N (K + 1) + N complex values.
 // ------------------------------------------------------------------------------------------
 template <class R, int N>
 __global__ void __launch_bounds__(256)
 k_ycoarse(const typename Store<R>::T* __restrict__ gz, const typename Store<R>::T* __restrict__ twtab,
-          typename Store<R>::T* __restrict__ gy, int K, const CgScal* __restrict__ sc, size_t gzs, size_t gys) {
+          typename Store<R>::T* __restrict__ gy, int K, CgScal* __restrict__ sc, size_t gzs, size_t gys, Bat bt,
+          const double* __restrict__ part, int n3, double inv_vc) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int KZ = K + 1;
   cx<R>* a = reinterpret_cast<cx<R>*>(smem_raw);  // [N][K+1]
@@ -55,7 +203,11 @@ k_ycoarse(const typename Store<R>::T* __restrict__ gz, const typename Store<R>::
   for (int e = threadIdx.x; e < N; e += blockDim.x) tw[e] = ld_c<R>(twtab + 2 * e);
   chain_start();
   if (finished(sc + z)) return;
-  const int x = blockIdx.x;
+  int x = blockIdx.x;
+  if (n3 > 0 && x-- == 0) {
+    fin_beta(part + (size_t)z * bt.part, n3, inv_vc, sc + z, reinterpret_cast<double*>(smem_raw));
+    return;
+  }
   gz += z * gzs + (size_t)x * N * KZ;
   gy += z * gys;
   for (int e = threadIdx.x; e < N * KZ; e += blockDim.x) a[e] = ld_c<R>(gz + e);
@@ -149,16 +301,27 @@ k_xcoarse(const typename Store<R>::T* __restrict__ gy, const typename Store<R>::
   }
 }
 
-// the coarse entries of r as they were before k_defl_mu<MODE 1> (where the y pass does not put them back);
-// grid (ceil((nh + 1) / 256), systems)
+// entry u (u = nh: k = 0) of r and, on the kz = 0 plane, its conjugate's
+template <int N> WF_D void restore_entry(float2* r, const float2* rsave, const int4* modes, int nh, int u) {
+  if (u == nh) {
+    r[0] = rsave[2 * nh];
+    return;
+  }
+  const int4 md = modes[u];
+  r[dslot<N>(md.x, md.y, md.z)] = rsave[2 * u];
+  if (md.z == 0) r[dslot<N>(-md.x, -md.y, 0)] = rsave[2 * u + 1];
+}
+
+// alpha, and the coarse entries of r back to what k_defl_mu<MODE 1> saved (x pass 1 has used its own); grid = systems
 template <class R, int N>
-__global__ void k_defl_restore(typename Store<R>::T* __restrict__ r, const typename Store<R>::T* __restrict__ rsave,
-                               const int4* __restrict__ modes, int nh, const CgScal* __restrict__ sc, Bat bt) {
-  const int z = blockIdx.y;
+__global__ void k_defl_alpha(YFin fin, CgScal* sc, Bat bt) {
+  __shared__ double red[32];
+  const int z = blockIdx.x;
   chain_start();
   if (finished(sc + z)) return;
-  const int u = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (u <= nh) restore_entry<N>(r + z * bt.spec, rsave + (size_t)z * (2 * nh + 1), modes, nh, u);
+  for (int u = threadIdx.x; u <= fin.nh; u += blockDim.x)
+    restore_entry<N>(fin.r + z * bt.spec, fin.rsave + (size_t)z * (2 * fin.nh + 1), fin.modes, fin.nh, u);
+  fin_alpha(fin.part + (size_t)z * bt.part, fin.n1, fin.off, fin.n2, sc + z, red);
 }
 
 // <r, z> = <r, r> - <r, Z mu> (sc->rr holds <r, r> from the last x pass 2); beta = <r, z> over its

@@ -435,7 +435,7 @@ k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double
 }
 
 // ==========================================================================================
-// The FP64 CG passes (the work of k_cg_xinv, k_cg_xupd and k_ln_zturn): vector updates and sums in FP64,
+// The FP64 CG passes (the work of k_cg_xinv, k_cg_xupd and k_zturn): vector updates and sums in FP64,
 // transforms in fixed point.  UNIT_M (every system preconditioned): m = 1 but at k = 0, where it is 0,
 // and the m table holds 1 / c^2 instead, which the residual estimate would otherwise divide for.  108^3 per
 // launch (events, with ~5 us of bracketing), FP64 butterflies -> here: x pass 1 58.8 -> 43 us, x pass 2 87 -> 43,

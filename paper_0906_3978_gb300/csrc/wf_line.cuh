@@ -1,32 +1,13 @@
 // wf_line.cuh -- transforms of one line held by a group of threads, exchanged through shared memory between
 // two or three passes.  A line of M = R1 R2 R3 (R3 = 1: two passes) belongs to N1 = M / R1 threads; thread t
 // enters with the elements n1 N1 + t in registers, so a caller loads them straight from memory, and the
-// last pass hands its results out of registers.  Written over the complex type C (FP32 complex, or the
-// 64-bit fixed point of wf_fix.cuh) with twiddles of type W.
+// last pass hands its results out of registers.  Written over the complex type C (the 64-bit fixed point of
+// wf_fix.cuh) with twiddles of type W.
 #pragma once
 #include "wf_common.cuh"
 
 namespace wf {
 
-// the engine's operations on FP32 complex values
-template <int DIR> WF_D cx<float> ln_mul_i(cx<float> a) { return mul_si<DIR>(a); }
-template <int DIR> WF_D cx<float> ln_twid(cx<float> a, float2 w) {
-  return DIR < 0 ? cx<float>{a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x}
-                 : cx<float>{a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y};
-}
-WF_D cx<float> ln_r2(cx<float> a) { return scale(a, 0.70710678118654752f); }
-WF_D cx<float> ln_s3(cx<float> a) { return scale(a, 0.86602540378443865f); }
-WF_D cx<float> ln_half(cx<float> a) { return scale(a, 0.5f); }
-template <int DIR> WF_D cx<float> ln_rot9(cx<float> a, int m) {  // a exp(DIR 2 pi i m / 9), m = 1, 2, 4
-  const float c = m == 1 ? 0.76604444311897804f : m == 2 ? 0.17364817766693035f : -0.93969262078590838f;
-  const float s = m == 1 ? 0.64278760968653933f : m == 2 ? 0.98480775301220806f : 0.34202014332566873f;
-  return ln_twid<DIR>(a, make_float2(c, -s));
-}
-template <int DIR, int m> WF_D cx<float> ln_rot16(cx<float> a) {  // a exp(DIR 2 pi i m / 16), m = 1, 3, 9
-  const float c = m == 1 ? 0.92387953251128676f : m == 3 ? 0.38268343236508977f : -0.92387953251128676f;
-  const float s = m == 1 ? 0.38268343236508977f : m == 3 ? 0.92387953251128676f : -0.38268343236508977f;
-  return ln_twid<DIR>(a, make_float2(c, -s));
-}
 struct fxc;
 template <int DIR> WF_D fxc ln_mul_i(fxc a);
 template <int DIR> WF_D fxc ln_twid(fxc a, int4 w);
@@ -106,29 +87,6 @@ template <int RAD, int DIR, class C> WF_D void ln_dft(C* v) {
     t = v[5];
     v[5] = v[7];
     v[7] = t;
-  } else if constexpr (RAD == 16) {
-    // 4 x 4: columns n = 4 n1 + n2, twiddles W16^(n2 k1), rows; k = k1 + 4 k2
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) ln_dft4<DIR>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);
-    v[5] = ln_rot16<DIR, 1>(v[5]);
-    v[6] = ln_r2(v[6] + ln_mul_i<DIR>(v[6]));
-    v[7] = ln_rot16<DIR, 3>(v[7]);
-    v[9] = ln_r2(v[9] + ln_mul_i<DIR>(v[9]));
-    v[10] = ln_mul_i<DIR>(v[10]);
-    v[11] = ln_r2(ln_mul_i<DIR>(v[11]) - v[11]);
-    v[13] = ln_rot16<DIR, 3>(v[13]);
-    v[14] = ln_r2(ln_mul_i<DIR>(v[14]) - v[14]);
-    v[15] = ln_rot16<DIR, 9>(v[15]);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) ln_dft4<DIR>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = i + 1; j < 4; ++j) {
-        const C t = v[4 * i + j];
-        v[4 * i + j] = v[4 * j + i];
-        v[4 * j + i] = t;
-      }
   } else {
     static_assert(RAD == 12, "radix");
     // 4 x 3 without twiddles: n = 3 n1 + 4 n2, k = 9 k1 + 4 k2 (mod 12)
@@ -361,49 +319,6 @@ constexpr int ln_padded(int m, int sh, int n1, int banks) {
   int l = m + (m >> sh);
   while (n1 < banks && l % banks != n1 % banks) ++l;
   return l;
-}
-
-// Sum over the CTA of the threads' double-float accumulators; valid in thread 0.  Each warp adds its 32 values
-// exactly, as integers in units of 2^-57 of the largest (three reductions of limbs), and only the warps' sums
-// meet in FP64: a tree of FP64 shuffles over all threads keeps GB300's FP64 pipe busy for ~1 us per CTA.
-// The result does not depend on any order.  red holds >= 32 doubles.
-WF_D long long acc_fixed(float f, int E) {  // f 2^(33 - (E - 150)) truncated, for exponents up to E
-  const unsigned u = __float_as_uint(f);
-  const int e = (u >> 23) & 0xff, sh = 33 - (E - e);
-  const long long m = e ? (long long)((u & 0x7fffffu) | 0x800000u) : 0;
-  const long long v = sh >= 0 ? m << sh : (sh > -24 ? m >> -sh : 0);
-  return (int)u < 0 ? -v : v;
-}
-WF_D double block_sum_acc(const AccF& a, double* red) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5, nl = warp_lanes();
-  const unsigned mask = lane_mask(nl);
-  const int E = (int)(__reduce_max_sync(mask, __float_as_uint(a.hi) & 0x7fffffffu) >> 23);
-  const long long v = acc_fixed(a.hi, E) + acc_fixed(a.lo, E);
-  const int s0 = __reduce_add_sync(mask, (int)(v & 0x1fffff));
-  const int s1 = __reduce_add_sync(mask, (int)((v >> 21) & 0x1fffff));
-  const int s2 = __reduce_add_sync(mask, (int)(v >> 42));
-  long long* sums = reinterpret_cast<long long*>(red);
-  __shared__ int exps[32];
-  __syncthreads();
-  if (l == 0) {
-    sums[w] = (long long)s0 + ((long long)s1 << 21) + ((long long)s2 << 42);
-    exps[w] = E;
-  }
-  __syncthreads();
-  double r = 0.0;
-  if (w == 0) {
-    for (int i = l; i < nw; i += nl) {  // one round but in a CTA of a single partial warp
-      const int k = exps[i] - 150 - 33;  // the units; a non-finite accumulator makes the sum a NaN
-      r += exps[i] == 0xff ? __longlong_as_double(0x7ff8000000000000ll)
-                           : __ll2double_rn(sums[i]) * __hiloint2double((k + 1023) << 20, 0);
-    }
-    for (int o = 16; o > 0; o >>= 1)
-      if (o < nw) {
-        const double t = __shfl_down_sync(mask, r, o);
-        if (l + o < nl) r += t;
-      }
-  }
-  return r;
 }
 
 }  // namespace wf

@@ -808,6 +808,81 @@ WF_D void zrows_store(const cx<R>* tile, typename G::ST* g, size_t row0, int tid
 }
 
 // ------------------------------------------------------------------------------------------
+// z turn (middle of A p): each (x, y) line: packed -> real (C2R), times D(x, y, z), -> packed.
+// D = nbar w / V_c carries the 1/V_c of the inverse transform.  grid (N*N / NL).
+// ------------------------------------------------------------------------------------------
+template <class R, int N, int EZ = z_elems<R, N>()>
+__global__ void __launch_bounds__(ZG<R, N, EZ>::NT)
+k_zturn(typename Store<R>::T* __restrict__ spec, const typename Store<R>::S* __restrict__ D,
+        const typename Store<R>::T* __restrict__ twtab, double* __restrict__ partials, const CgScal* __restrict__ sc,
+        Bat bt) {
+  using G = ZG<R, N, EZ>;
+  using SS = typename Store<R>::S;
+  static_assert(std::is_same<R, SS>::value, "the CG passes compute in their storage type");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
+  cx<R>* tw = tile + G::M * G::LD;  // 2N entries
+  __shared__ double red[32];
+  const int z = blockIdx.z;
+  chain_start();
+  if (sc && finished(sc + z)) return;
+  spec += z * bt.spec;
+  D += z * bt.real;
+  partials += z * bt.part;
+  const int tid = threadIdx.x;
+  const size_t row0 = (size_t)blockIdx.x * G::NL;
+  // the D rows go to L2 while the rows are transformed
+  if (tid < G::NL) prefetch_l2(D + (row0 + tid) * N, N * sizeof(SS));
+  for (int e = tid; e < 2 * N; e += G::NT) tw[e] = ld_c<R>(twtab + e);
+  zrows_load<G>(tile, spec, row0, tid);
+  __syncthreads();
+  const int l = tid % G::NL, t = tid / G::NL;
+  c2r_prep<R, N, G::LD>(tile + l, t, G::TPL, tw);
+  __syncthreads();
+  fft_line<R, G::M, G::TPL, G::LD, +1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
+  // real samples 2i, 2i+1 of line l sit in element i: multiply by D, VW elements at a time,
+  // and sum D T^2 (the <c p, D (c p)> term of <p, A p>)
+  using DV = typename std::conditional<G::VW == 2, float4, double2>::type;  // 2 VW reals of D
+  typename AccFor<SS>::T acc;
+#pragma unroll 4
+  for (int k = 0; k < G::PER; ++k) {
+    const int idx = tid + k * G::NT;
+    if (!(G::EVEN || idx < G::NVEC)) continue;
+    const int ll = idx / G::NV, i = (idx % G::NV) * G::VW;
+    const SS* dp = D + (row0 + ll) * N + 2 * i;
+    if constexpr (G::VW == 2) {
+      const float4 d = *reinterpret_cast<const float4*>(dp);
+      cx<R> a = tile[i * G::LD + ll], b = tile[(i + 1) * G::LD + ll];
+      const cx<R> a0 = a, b0 = b;
+      a.x = a.x * RT<R>::from_f(d.x);
+      a.y = a.y * RT<R>::from_f(d.y);
+      b.x = b.x * RT<R>::from_f(d.z);
+      b.y = b.y * RT<R>::from_f(d.w);
+      // D T^2 >= 0: the vector's four terms are summed first (in R = the storage type)
+      acc.add((SS)(a.x * a0.x + a.y * a0.y + b.x * b0.x + b.y * b0.y));
+      tile[i * G::LD + ll] = a;
+      tile[(i + 1) * G::LD + ll] = b;
+    } else {
+      const double2 d = *reinterpret_cast<const double2*>(dp);
+      cx<R> a = tile[i * G::LD + ll];
+      const cx<R> a0 = a;
+      a.x = a.x * RT<R>::c(d.x);
+      a.y = a.y * RT<R>::c(d.y);
+      acc.add((SS)(a.x * a0.x + a.y * a0.y));
+      tile[i * G::LD + ll] = a;
+    }
+  }
+  (void)sizeof(DV);
+  __syncthreads();
+  fft_line<R, G::M, G::TPL, G::LD, -1, 4, rmax_for(G::M, G::TPL)>(tile + l, t, tw);
+  r2c_post<R, N, G::LD>(tile + l, t, G::TPL, tw);
+  __syncthreads();
+  zrows_store<G>(tile, spec, row0, tid);
+  const double sum = block_sum(acc.get(), red);
+  if (tid == 0) partials[blockIdx.x] = sum;
+}
+
+// ------------------------------------------------------------------------------------------
 // z forward: real rows (FP64) -> packed spectrum rows.  Optional partial of sum(in^2).
 // ------------------------------------------------------------------------------------------
 template <class R, int N, bool SQ>
@@ -1021,10 +1096,11 @@ WF_D void fin_beta(const double* partials, int n, double inv_vc, CgScal* sc, dou
     else if (sc->iter >= sc->max_iter) sc->done = 2;
   }
 }
-// What the forward y pass, which does not need alpha, does beside its lines (n1 = 0: nothing): alpha from the n1 partial
-// sums of x pass 1 and the n2 of the z turn, and for a deflated iteration the coarse entries of r back to what
-// k_defl_mu saved (x pass 1 has used its own).  A single-CTA launch between the passes costs 3-8 us; a last-arrival
-// ticket in the z turn held every CTA for its fence (144^3: 17 -> 26 us).
+// What is due between the z turn and x pass 2 (n1 = 0: nothing): alpha from the n1 partial sums of x pass 1 and the n2 of
+// the z turn, and for a deflated iteration the coarse entries of r back to what k_defl_mu saved (x pass 1 has
+// used its own).  The forward y pass in fixed point, which does not need alpha, takes it in a CTA row of its own; the
+// persistent y pass has none to spare, so k_fin_alpha or k_defl_alpha runs before it.  A last-arrival ticket in
+// the z turn held every CTA for its fence (144^3: 17 -> 26 us).
 struct YFin {
   int n1 = 0, off = 0, n2 = 0;  // x pass 1's partial sums [0, n1), the z turn's [off, off + n2)
   const double* part = nullptr;
