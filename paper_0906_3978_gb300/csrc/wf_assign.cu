@@ -153,6 +153,12 @@ template <int N> struct LpShift {
   }
 };
 
+template <bool A16> WF_D ulonglong2 ld_pair(const ulonglong2* p) {
+  if constexpr (A16) return __ldg(p);
+  const unsigned long long* q = reinterpret_cast<const unsigned long long*>(p);
+  return make_ulonglong2(__ldg(q), __ldg(q + 1));
+}
+
 // z axis: rows of 2N integers (units of the grid) in pairs -> rows of N doubles.  Thread t of a pair
 // holds elements n1 (N / R1) + t, so a warp reads and writes consecutive 16- and 8-byte pieces of a row.  Pairs
 // of an all-zero CTA (most of the grid outside the survey) are written as zeros at once.  Bound by integer
@@ -165,7 +171,8 @@ template <int N> struct LpZ {
   static constexpr int LS = ln_padded(N, 3, TPL, 8);
   static constexpr size_t SMEM = (size_t)(NP * LS + N + NP * (TPL + kNyqParts)) * 16;
 };
-template <int N>
+// A16: the grid (a caller's fine_out) lies on a 16-byte boundary; otherwise its values are loaded one by one.
+template <int N, bool A16>
 __global__ void __launch_bounds__(LpZ<N>::NT, N >= 128 ? 3 : 0)
 k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out, double unit,
             const int4* __restrict__ twtab, const int4* __restrict__ phtab) {
@@ -185,8 +192,8 @@ k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out,
   unsigned long long any = 0;
 #pragma unroll
   for (int r = 0; r < R1; ++r) {
-    a[r] = __ldg(r0 + r * N1 + t);
-    b[r] = __ldg(r1 + r * N1 + t);
+    a[r] = ld_pair<A16>(r0 + r * N1 + t);
+    b[r] = ld_pair<A16>(r1 + r * N1 + t);
   }
 #pragma unroll
   for (int r = 0; r < R1; ++r) any |= (a[r].x | a[r].y) | (b[r].x | b[r].y);
@@ -264,11 +271,12 @@ k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out,
 // SM below 256 (216^3: y 0.34 -> 0.285 ms), which spilled to 4.08 ms at 512^3.
 template <int N> struct LpC {
   static constexpr int R1 = fx_plan(N).r1, TPL = N / R1;
-    static constexpr int NL = div_le(N / 2, N >= 256 ? 4 : 8);
+  static constexpr int NL = div_le(N / 2, N >= 256 ? 4 : 8);
   static constexpr int NT = NL * TPL;
   static constexpr size_t SMEM = (size_t)(N * NL + N + NL * (TPL + kNyqParts)) * 16;
 };
-template <int N, int AXIS>
+// A16: the output (AXIS 2: a caller's n_obs) lies on a 16-byte boundary.
+template <int N, int AXIS, bool A16>
 __global__ void __launch_bounds__(LpC<N>::NT, N >= 128 && N < 256 ? 3 : 0)
 k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4* __restrict__ twtab,
             const int4* __restrict__ phtab) {
@@ -346,8 +354,13 @@ k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4*
   for (int r = 0; r < R1; ++r) {
     const size_t m = r * N1 + t;
     const double2 ev = __ldg(reinterpret_cast<const double2*>(src + (2 * m) * stride));
-    *reinterpret_cast<double2*>(dst + m * ostride) =
-        make_double2(fma(__ll2double_rn(v[r].x), c, ev.x), fma(__ll2double_rn(v[r].y), c, ev.y));
+    const double2 y = make_double2(fma(__ll2double_rn(v[r].x), c, ev.x), fma(__ll2double_rn(v[r].y), c, ev.y));
+    if constexpr (A16) {
+      *reinterpret_cast<double2*>(dst + m * ostride) = y;
+    } else {
+      dst[m * ostride] = y.x;
+      dst[m * ostride + 1] = y.y;
+    }
   }
 }
 
@@ -368,18 +381,21 @@ static wf_status lowpass_sized(Ctx& c, const unsigned long long* fine, double* n
   double *t1, *t2;
   WF_TRY(c.get("lp_t1", (size_t)4 * N * N * N * sizeof(double), (void**)&t1));
   WF_TRY(c.get("lp_t2", (size_t)2 * N * N * N * sizeof(double), (void**)&t2));
-  WF_CUDA(smem_attr(k_lowpass_z<N>, Z::SMEM));
-  WF_CUDA(smem_attr(k_lowpass_c<N, 1>, C::SMEM));
-  WF_CUDA(smem_attr(k_lowpass_c<N, 2>, C::SMEM));
+  auto kz = (uintptr_t)fine % 16 == 0 ? k_lowpass_z<N, true> : k_lowpass_z<N, false>;
+  auto ky = k_lowpass_c<N, 1, true>;
+  auto kx = (uintptr_t)n_obs % 16 == 0 ? k_lowpass_c<N, 2, true> : k_lowpass_c<N, 2, false>;
+  WF_CUDA(smem_attr(kz, Z::SMEM));
+  WF_CUDA(smem_attr(ky, C::SMEM));
+  WF_CUDA(smem_attr(kx, C::SMEM));
   const double V = (double)N * N * N;
   c.launch("lowpass_z", 8 * (8 * V + 4 * V), st,
-           [&] { k_lowpass_z<N><<<2 * N * N / Z::NP, Z::NT, Z::SMEM, st>>>(fine, t1, unit, tw, half); });
+           [&] { kz<<<2 * N * N / Z::NP, Z::NT, Z::SMEM, st>>>(fine, t1, unit, tw, half); });
   WF_CUDA(cudaGetLastError());
   c.launch("lowpass_y", 8 * (4 * V + 2 * V), st,
-           [&] { k_lowpass_c<N, 1><<<dim3(N / 2 / C::NL, 2 * N), C::NT, C::SMEM, st>>>(t1, t2, tw, half); });
+           [&] { ky<<<dim3(N / 2 / C::NL, 2 * N), C::NT, C::SMEM, st>>>(t1, t2, tw, half); });
   WF_CUDA(cudaGetLastError());
   c.launch("lowpass_x", 8 * (2 * V + V), st,
-           [&] { k_lowpass_c<N, 2><<<dim3(N / 2 / C::NL, N), C::NT, C::SMEM, st>>>(t2, n_obs, tw, half); });
+           [&] { kx<<<dim3(N / 2 / C::NL, N), C::NT, C::SMEM, st>>>(t2, n_obs, tw, half); });
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
