@@ -62,9 +62,9 @@ WF_D double sel_value(const SelParams& s, const double4* __restrict__ holes, dou
 }
 
 // The window at the nodes.  The plain formula costs ~75 FP64 operations a node, all on the 1/64-rate pipe
-// (256^3: 1.97 ms, here 0.82).  The cone and hole tests are first taken in FP32: a node whose margin exceeds
-// 2^-20 r (|a_x| + |a_y| + |a_z| + |cos|), more than twice the FP32 error of dot and cos r (each a few
-// 2^-24 relative, the approximate square root 2^-22), is decided there, and only the others repeat the exact
+// (256^3: 1.97 ms, here 0.85).  The cone and hole tests are first taken in FP32: a node whose margin exceeds
+// 2^-20 r (|a_x| + |a_y| + |a_z| + |cos|), 16 units of 2^-24 where the roundings of dot and cos r (the approximate
+// square root's 2^-22 among them) add up to about 10, is decided there, and only the others repeat the exact
 // test of sel_value, operation by operation.  What depends on one axis alone (offset, its square, its term of
 // the axis product, each rounded as in the definition) comes from tables of the CTA, and the value of an
 // observed node takes the FP64 functions of wf_fp64fn.cuh (~30 operations).  Lengths beyond 1e12 or below
@@ -132,8 +132,8 @@ k_window(int n, SelParams s, const double4* __restrict__ holes, double* __restri
             const double r = sqrt_fast(r2);
             double t = r * ip0;
             t = fma(fma(-t, s.p0, r), ip0, t);
-            const double x = s.kind == 1 ? -(t * t) : s.p1 * (log_fast(t, fn.lg) + (1.0 - t));
-            val = fabs(x) < 700.0 ? exp_fast(x, fn.ex) : exp(x);
+            const double x = s.kind == 1 ? -(t * t) : s.p1 * (log_fast(t, fn) + (1.0 - t));
+            val = fabs(x) < 700.0 ? exp_fast(x, fn) : exp(x);
           }
           acc.add(val);
         }
