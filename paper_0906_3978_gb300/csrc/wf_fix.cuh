@@ -12,8 +12,8 @@
 // of rounding noise a transform adds, ~1e-17 relative at M = 512, where FP64 butterflies leave ~2e-16.
 // What remains is the rounding of the FP64 values that are stored.  A line's scale comes from its own
 // largest exponent and sum of squares, so lines of any magnitude keep their digits; the statistics are
-// integers, so the result does not depend on the order in which threads add to them.  Lines whose
-// largest value lies below 2^-800 keep an absolute resolution of about 2^-860 only, and a line with an
+// integers, so the result does not depend on the order in which threads add to them.  Scalings beyond
+// 2^+-900, which an exponent field may not hold in one step, take two FP64 multiplications.  A line with an
 // infinity or NaN becomes NaN throughout (FP64 butterflies spread either over the line as well).
 #pragma once
 #include "wf_line.cuh"
@@ -124,9 +124,17 @@ template <int M> struct FxPlan {
 WF_D int fx_exp(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
 // an upper bound of |d| 2^(12 - (emax - 1023)), 13 bits and one, for exponents up to emax
 WF_D unsigned fx_top(double d, int emax) {
-  const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff, s = emax - e + 8;
-  return e == 0 || s > 31 ? (unsigned)((hi & 0x7fffffff) != 0 || __double2loint(d) != 0)
-                          : ((unsigned)((hi & 0xfffff) | 0x100000) >> s) + 1u;
+  const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff, s = emax - max(e, 1) + 8;
+  const unsigned m = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
+  return s > 31 || m == 0 ? (unsigned)((m | (unsigned)__double2loint(d)) != 0) : (m >> s) + 1u;
+}
+// 2^e for -1022 <= e <= 1023
+WF_D double fx_pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+constexpr int kFxStep = 900;  // scalings up to 2^+-kFxStep are integer additions to exponent fields
+// d 2^e for any e; the result under- or overflows as it should
+WF_D double fx_scaled(double d, int e) {
+  e = min(max(e, -2044), 2044);
+  return d * fx_pow2(e / 2) * fx_pow2(e - e / 2);
 }
 // d 2^k rounded to an integer (0 where the exponent leaves the normal range downwards)
 WF_D long long fx_from(double d, int k) {
@@ -134,11 +142,8 @@ WF_D long long fx_from(double d, int k) {
   if (e == 0 || e + k <= 0) return 0;
   return __double2ll_rn(__hiloint2double(hi + (k << 20), __double2loint(d)));
 }
-// 2^e for -1022 <= e <= 1023
-WF_D double fx_pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 // The power of two k that takes a line of M complex values to sqrt(M) ||z||_2 2^k <= 2^62: emax the
-// largest biased exponent of the line (at least kFxMinExp), q >= (sum of fx_top^2) / 128
-constexpr int kFxMinExp = 223;
+// largest biased exponent of the line (at least 1), q >= (sum of fx_top^2) / 128
 WF_D int fx_scale(int emax, unsigned q, int M) {
   const unsigned long long s = (unsigned long long)q * 128ull * (unsigned)M;
   const int b = 64 - __clzll((long long)s);  // sqrt(s) < 2^(b / 2)
@@ -146,15 +151,17 @@ WF_D int fx_scale(int emax, unsigned q, int M) {
 }
 
 
-// A line's scale: its values are integers in units of 2^-k; nan: the exponent bits that make every
-// result of a line with a non-finite element a NaN
+// A line's scale: its values are integers in units of 2^-k, made from the registers' values by 2^kin; nan: the
+// exponent bits that make every result of a line with a non-finite element a NaN
 struct FxScale {
-  int k;
+  int k, kin;
   unsigned nan;
 };
 // The scale of the line whose elements are spread over the threads' raw[]; se, sq: the line's words in
-// shared memory, kFxMinExp and 0 before (visible to all).  Two barriers.
-template <int NV> WF_D FxScale fx_line_scale(const double2 (&raw)[NV], int* se, unsigned* sq, int M) {
+// shared memory, kFxMinExp and 0 before (visible to all).  Two barriers.  A line of zeros gets k = 0; the
+// values of a line of tiny ones, subnormals among them, are multiplied by 2^600 in the registers.
+constexpr int kFxMinExp = 1;
+template <int NV> WF_D FxScale fx_line_scale(double2 (&raw)[NV], int* se, unsigned* sq, int M) {
   static_assert(2 * NV <= 62, "the sum of squares of a thread fits 32 bits");
   int mx = 0;
 #pragma unroll
@@ -170,15 +177,22 @@ template <int NV> WF_D FxScale fx_line_scale(const double2 (&raw)[NV], int* se, 
   }
   if (q) atomicAdd(sq, (q >> 7) + 1u);
   __syncthreads();
-  return FxScale{fx_scale(emax, *sq + 1u, M), emax == 0x7ff ? 0x7ff80000u : 0u};
+  const unsigned s = *sq;
+  FxScale f{s ? fx_scale(emax, s + 1u, M) : 0, 0, emax == 0x7ff ? 0x7ff80000u : 0u};
+  f.kin = f.k;
+  if (f.k > kFxStep) {
+    f.kin = f.k - 600;
+#pragma unroll
+    for (int r = 0; r < NV; ++r) raw[r] = make_double2(raw[r].x * 0x1p600, raw[r].y * 0x1p600);
+  }
+  return f;
 }
-WF_D fxc fx_from2(double2 d, FxScale f) { return fxc{fx_from(d.x, f.k), fx_from(d.y, f.k)}; }
-// v 2^-(k + sh).  The power of two goes to the exponent field by an integer addition (values near the top
-// of the range, where it could overflow, take a multiplication).
+WF_D fxc fx_from2(double2 d, FxScale f) { return fxc{fx_from(d.x, f.kin), fx_from(d.y, f.kin)}; }
+// v 2^-(k + sh).  The power of two goes to the exponent field by an integer addition within 2^+-kFxStep.
 WF_D double fx_to(long long v, FxScale f, int sh = 0) {
   const int k = f.k + sh;
   double d = __ll2double_rn(v);
-  if (k < -900) d *= fx_pow2(-k);
+  if ((unsigned)(k + kFxStep) > 2u * kFxStep) d = fx_scaled(d, -k);
   else if (v != 0) d = __hiloint2double(__double2hiint(d) - (k << 20), __double2loint(d));
   return __hiloint2double(__double2hiint(d) | (int)f.nan, __double2loint(d));
 }

@@ -75,12 +75,15 @@ static __global__ void k_gauss_table(double* __restrict__ tab, int n, double kf,
 }
 
 // ---- Fourier tables as Q62 digits ----------------------------------------------------------------
-// tab[i] 2^-e as digits (high, low), in place; |tab[i]| < 2^e, e = exps[z estride].  grid (., systems)
+// tab[i] 2^-e as digits (high, low), in place; |tab[i]| < 2^e, e = exps[z estride].  One exponent serves a table, so
+// an entry below 2^-9 of the largest has fewer bits than its FP64 value: the error of a product stays below
+// 2^-62 max|tab| of the line's norm, where the transforms' FP64 storage leaves 2^-53 of it times the largest
+// entry.  exps[] = kFxNanTab: a table with an infinity or NaN, whose every product is a NaN.  grid (., systems)
 static __global__ void k_table_digits(double* __restrict__ tab, int len, const int* __restrict__ exps, int estride) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= len) return;
   tab += (size_t)blockIdx.y * len;
-  long long q = __double2ll_rn(tab[i] * fx_pow2(62 - exps[blockIdx.y * estride]));
+  long long q = __double2ll_rn(fx_scaled(tab[i], 62 - exps[blockIdx.y * estride]));
   const int l = (int)q;
   reinterpret_cast<int2*>(tab)[i] = make_int2((int)((q - l) >> 32), l);
 }
@@ -133,12 +136,13 @@ k_fx_xmul(const double2* __restrict__ in, double2* __restrict__ out, const int2*
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const int ls = pair && l < 2 ? 0 : l;  // the two lines of a pair share a scale
-  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
   constexpr int H2 = fx_mid(N);
-  const int sh = -(H2 + exps[z * estride]);
+  const int te = exps[z * estride], sh = -(H2 + te);
+  if (te == kFxNanTab) f.nan = 0x7ff80000u;
   if (!pair) {
     const int kz = blockIdx.x * NL + l, k0 = ky_s * ky_s + kz * kz;
     ln_convolve<N, FxPlan<N>>(v, slots + l, ColMap<NL>{}, t, tw, [&](int k, fxc X) {

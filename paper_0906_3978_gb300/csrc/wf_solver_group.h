@@ -37,6 +37,8 @@ Group* make_group_n(int n, int prec);
 std::vector<int4> deflation_modes(int K);
 int deflation_ncp(int K);
 
+// exponent of a Fourier table with a non-finite entry (k_table_digits)
+constexpr int kFxNanTab = 1 << 20;
 // out = F^-1 [table(|m|^2) F in] for one field of size N (instantiated with the solve drivers of
 // each size); table has 3 (N/2)^2 + 1 entries, or is empty: then it is the Gaussian exp(-kf^2 n2 r_s^2 / 2), made on
 // the device (its exponentials took the host 0.2 ms of the 0.83 ms of a smoothing at 256^3).

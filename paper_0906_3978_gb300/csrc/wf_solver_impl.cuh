@@ -544,10 +544,13 @@ static void make_tables(const std::vector<double>& sinv, bool precond, double c0
 // Smallest e with every entry of v below 2^e in modulus (the power of two of a table's digits)
 static inline int table_exp(const double* v, size_t n) {
   double m = 0.0;
-  for (size_t i = 0; i < n; ++i) m = std::max(m, std::fabs(v[i]));
+  for (size_t i = 0; i < n; ++i) {
+    if (!std::isfinite(v[i])) return kFxNanTab;
+    m = std::max(m, std::fabs(v[i]));
+  }
   int e = 0;
   std::frexp(m, &e);
-  return std::max(-900, std::min(e, 1000));
+  return e;
 }
 
 // Device table `name` from v, converted to T, through a page-locked staging buffer of the same
@@ -1222,7 +1225,9 @@ wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::v
   if (gauss) {
     WF_TRY(c.get("sm_g", SD::TAB * sizeof(double), (void**)&gt));
     c.launch("tables", 0, st, [&] { k_gauss_table<<<(SD::TAB + 255) / 256, 256, 0, st>>>(gt, SD::TAB, kf, r_s); });
-    *hexp = 1;  // the largest entry is 1
+    // the largest entry is 1; an exponent's infinity times 0 makes the first or the last one a NaN
+    const double h = -0.5 * kf * kf;
+    *hexp = std::isnan(h * 0.0 * r_s * r_s) || std::isnan(h * (double)(SD::TAB - 1) * r_s * r_s) ? kFxNanTab : 1;
   } else {
     WF_TRY(upload_tables<double>(c, "sm_g", table, &gt, st));
     *hexp = table_exp(table.data(), table.size());
