@@ -35,7 +35,7 @@ def test_radial_law_rms(n, kind, params):
     t = r / np.longdouble(p0)
     law = np.exp(-t * t) if kind == 1 else np.exp(np.longdouble(p1) * (np.log(t) + (1 - t)))
     dx, dy, dz = (torch.from_numpy(x).to(DEV) for x in d)
-    td = torch.sqrt((dx * dx + dy * dy) + dz * dz) / p0
+    td = torch.sqrt((dx * dx + dy * dy) + dz * dz) / torch.full_like(dx, p0)  # (a scalar divisor is multiplied by 1 / p0)
     lib = torch.exp(-(td * td)) if kind == 1 else torch.exp(p1 * (torch.log(td) + (1.0 - td)))
     rms = [float(np.sqrt(np.mean(((v.astype(np.longdouble) - law) / law).astype(np.float64) ** 2)))
            for v in (w[at], lib.cpu().numpy())]
