@@ -199,14 +199,14 @@ def fp64_kernels(ctx, prof, n):
     the FP64 residual): their transforms run in 64-bit fixed point, so the rate of their algorithmic flops is set
     beside the device's FP64 FMA rate measured here (wf_fp64_rate; a fraction above 1 is what the integer pipe
     gains) and the nominal 1.25 TFLOP/s.  Algorithmic flops:
-    2.5 L log2 L per real transform of length L; each pass line takes a real transform of length 2n
-    and an inverse of length n; the z pass has (2n)^2 lines, the y pass 2n n, the x pass n n.  The z
-    pass skips the rows no galaxy reaches (their output is zero), so its figure counts flops it did
-    not need to do."""
+    5 L log2 L per complex transform of length L; a low-pass transforms the odd samples of its lines alone, two lines
+    of 2n as one complex line of n, forward and back; the z pass has (2n)^2 lines, the y pass 2n n, the x
+    pass n n.  The z pass skips the rows no galaxy reaches (their output is zero), so its figure counts flops it
+    did not need to do."""
     peak = ctx.fp64_rate()
-    f_line = 2.5 * 2 * n * math.log2(2 * n) + 2.5 * n * math.log2(n)
+    f_line = 5.0 * n * math.log2(n)
     lines = {"lowpass_z": (2 * n) ** 2, "lowpass_y": 2 * n * n, "lowpass_x": n * n}
-    # the FP64 residual's passes (FP64 storage and arithmetic): per launch, the y pass takes n n/2
+    # the FP64 residual's passes (FP64 storage): per launch, the y pass takes n n/2
     # complex transforms of length n (5 n log2 n each), the x pass with the Fourier table two of them
     # (forward and inverse), the z passes n^2 real transforms of length n (2.5 n log2 n each)
     cplx = 5.0 * n * math.log2(n)
