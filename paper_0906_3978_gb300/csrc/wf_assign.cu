@@ -229,7 +229,7 @@ k_lowpass_z(const unsigned long long* __restrict__ in, double* __restrict__ out,
   __syncthreads();
   // sqrt(N) ||(e, o)|| 2^k <= 2^62
   const unsigned long long sq = (unsigned long long)s_q[l] * 128ull * (unsigned)N;
-  const int k = 62 + (13 - len) - ((64 - __clzll((long long)sq) + 1) >> 1);
+  const int k = len ? 62 + (13 - len) - ((64 - __clzll((long long)sq) + 1) >> 1) : 0;  // (0: a pair of zeros)
   auto fix = [&](unsigned long long v) { return (long long)(k >= 0 ? v << k : v >> -k); };
   fxc v[R1];
   {

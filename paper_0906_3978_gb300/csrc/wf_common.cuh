@@ -1,12 +1,7 @@
 // wf_common.cuh -- arithmetic types, complex helpers and reductions shared by the kernels.
 //
-// Three real types carry the spectral arithmetic:
-//   double  FP64 (1/64-rate units on GB300: used where FP64 storage meets FP64 arithmetic)
-//   float   FP32 (the inner solves of the mixed-precision path)
-//   df32    a double-float pair (hi + lo, |lo| <= ulp(hi)/2, ~48-bit significand) evaluated on
-//           the FP32 units with error-free transforms (Knuth two-sum, FMA two-product, as in
-//           Dekker 1971 / the "double-double" literature); used to transform FP64-stored fields
-//           at FP32-unit throughput.
+// Two real types carry the spectral arithmetic: double (the 1/64-rate unit) and float; FP64-stored fields also go
+// through 64-bit fixed point (wf_fix.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -15,58 +10,12 @@
 #define WF_HD __host__ __device__ __forceinline__
 #define WF_D __device__ __forceinline__
 
-// ------------------------------------------------------------------------------------------
-// double-float
-// ------------------------------------------------------------------------------------------
-struct df32 {
-  float hi, lo;
-};
-
 // s + e = a + b exactly (Knuth two-sum, no magnitude assumption)
 WF_D void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
-// s + e = a + b exactly when |a| >= |b| (Dekker fast two-sum)
-WF_D void fast_two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  e = __fsub_rn(b, __fsub_rn(s, a));
-}
-// accurate double-float sum (relative error ~2^-46 even under cancellation)
-WF_D df32 operator+(df32 a, df32 b) {
-  float s, e, t, f;
-  two_sum(a.hi, b.hi, s, e);
-  two_sum(a.lo, b.lo, t, f);
-  e = __fadd_rn(e, t);
-  fast_two_sum(s, e, s, e);
-  e = __fadd_rn(e, f);
-  fast_two_sum(s, e, s, e);
-  return df32{s, e};
-}
-WF_D df32 operator-(df32 a) { return df32{-a.hi, -a.lo}; }
-WF_D df32 operator-(df32 a, df32 b) { return a + (-b); }
-WF_D df32 operator*(df32 a, df32 b) {
-  float p = __fmul_rn(a.hi, b.hi);
-  float e = __fmaf_rn(a.hi, b.hi, -p);          // exact error of the product
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  float s, t;
-  fast_two_sum(p, e, s, t);
-  return df32{s, t};
-}
-WF_D df32& operator+=(df32& a, df32 b) { return a = a + b; }
-WF_D df32& operator-=(df32& a, df32 b) { return a = a - b; }
-WF_D df32& operator*=(df32& a, df32 b) { return a = a * b; }
-
-// FP64 <-> df32 (hi = nearest float, lo = nearest float of the remainder)
-WF_D df32 df_from_double(double v) {
-  float h = __double2float_rn(v);
-  float l = __double2float_rn(v - (double)h);
-  return df32{h, l};
-}
-WF_D double df_to_double(df32 a) { return (double)a.hi + (double)a.lo; }
-
 // Ask L2 to fetch [p, p + bytes) from HBM ahead of its use (a bulk prefetch: no registers or
 // shared memory held, no completion to wait for).  p and bytes must be multiples of 16.
 WF_D void prefetch_l2(const void* p, unsigned bytes) {
@@ -83,7 +32,6 @@ template <> struct RT<double> {
   WF_D static double to_d(double v) { return v; }
   WF_D static double from_f(float v) { return (double)v; }
   WF_D static float to_f(double v) { return (float)v; }
-  WF_D static double mul(double a, double b) { return a * b; }
 };
 template <> struct RT<float> {
   WF_HD static float c(double v) { return (float)v; }
@@ -92,14 +40,6 @@ template <> struct RT<float> {
   WF_D static float from_f(float v) { return v; }
   WF_D static float to_f(float v) { return v; }
 };
-template <> struct RT<df32> {
-  WF_D static df32 c(double v) { return df_from_double(v); }
-  WF_D static df32 from_d(double v) { return df_from_double(v); }
-  WF_D static double to_d(df32 v) { return df_to_double(v); }
-  WF_D static df32 from_f(float v) { return df32{v, 0.f}; }
-  WF_D static float to_f(df32 v) { return v.hi + v.lo; }
-};
-
 // ------------------------------------------------------------------------------------------
 // complex over a real type
 // ------------------------------------------------------------------------------------------
@@ -132,7 +72,7 @@ template <class R> WF_D cx<R> ld_c(const float2* p) {
 template <class R> WF_D void st_c(double2* p, cx<R> v) { *p = make_double2(RT<R>::to_d(v.x), RT<R>::to_d(v.y)); }
 template <class R> WF_D void st_c(float2* p, cx<R> v) { *p = make_float2(RT<R>::to_f(v.x), RT<R>::to_f(v.y)); }
 
-// storage complex type for an arithmetic type: FP64 storage for double and df32, FP32 for float
+// storage complex type for an arithmetic type
 template <class R> struct Store { using T = double2; using S = double; };
 template <> struct Store<float> { using T = float2; using S = float; };
 

@@ -458,7 +458,7 @@ k_defl_mu(const float* __restrict__ Einv, const float* __restrict__ gco, const f
   product();
   if constexpr (MODE == 1) {  // the last CTA takes <r, z> and beta
     __syncthreads();          // every warp's entry of dpart
-    if (last_cta(&sc[z].tick[2], gridDim.x)) fin_defl(dpart, nh, sc + z, red);
+    if (last_cta(&sc[z].tick, gridDim.x)) fin_defl(dpart, nh, sc + z, red);
   }
 }
 

@@ -329,11 +329,11 @@ template <int N, class MAP> WF_D fxc fx_c2r(const fxc* s, const MAP& map, int k,
 // ||Z||_2 <= 2 sqrt(2) ||X||_2, its partial sums are below sqrt(8 H) ||X||_2.
 template <int N> constexpr int fx_c2r_count() { return 8 * (N / 2); }
 
-// z forward: real rows -> packed spectrum rows; optional partial of sum(in^2).  grid (GZ, 1, systems)
-template <int N, bool SQ>
+// z forward: real rows -> packed spectrum rows.  grid (GZ, 1, systems)
+template <int N>
 __global__ void __launch_bounds__(FxZ<N>::NT)
 k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* __restrict__ twtab,
-          double* __restrict__ partials, const CgScal* __restrict__ sc, Bat bt) {
+          const CgScal* __restrict__ sc, Bat bt) {
   using G = FxZ<N>;
   constexpr int R1 = G::R1, N1 = G::N1, H = G::H;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -341,7 +341,6 @@ k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* 
   int4* tw = reinterpret_cast<int4*>(slots + G::NL * G::LS);  // exp(-2 pi i e / N)
   __shared__ int se[G::NL];
   __shared__ unsigned sq[G::NL];
-  __shared__ double red[32];
   const int z = blockIdx.z, tid = threadIdx.x, l = tid / N1, t = tid % N1;
   if (sc && sc[z].done) return;
   const size_t row = (size_t)blockIdx.x * G::NL + l;
@@ -360,16 +359,6 @@ k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* 
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
-  if constexpr (SQ) {
-    AccD acc;
-#pragma unroll
-    for (int r = 0; r < R1; ++r) {
-      acc.add_prod(raw[r].x, raw[r].x);
-      acc.add_prod(raw[r].y, raw[r].y);
-    }
-    const double q = block_sum(acc.get(), red);
-    if (tid == 0) partials[(size_t)z * bt.part + blockIdx.x] = q;
-  }
   ln_forward_nat<H, FxPlan<H>, -1, 2>(v, s, PadMap{}, t, tw);
   double2* dst = out + z * bt.spec + row * H;
   for (int k = t; k < H; k += N1) dst[k] = fx_to2(fx_r2c<N>(s, PadMap{}, k, tw), f);

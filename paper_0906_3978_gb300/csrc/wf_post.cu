@@ -104,8 +104,7 @@ __global__ void k_compare_fin(const double* __restrict__ partials, int nblk, dou
 struct DensArgs {
   int n, n_shells, n_bins;
   double H, ox, oy, oz, lo, width, inv_width;
-  double shells[16];     // the shells' radii
-  long long r2_from[16]; // bits of the smallest double whose square root is at least that radius
+  long long r2_from[16]; // bits of the smallest double whose square root is at least a shell's radius
 };
 
 // Bound by the FP64 pipe: a division, a floor and a square root a node made it 55 operations (256^3: 1.46 ms); 8
@@ -358,10 +357,9 @@ wf_status density_run(Ctx& c, const wf_grid& g, const double* delta, const doubl
   a.lo = lo;
   a.width = width;
   a.inv_width = std::isnormal(1.0 / width) ? 1.0 / width : NAN;  // NAN: every bin by division
-  for (int i = 0; i < 16; ++i) a.shells[i] = i < 2 * n_shells ? shells[i] : 0.0;
   for (int i = 0; i < 2 * n_shells; ++i)
     if (std::isnan(shells[i])) return WF_ERR_ARG;
-  for (int i = 0; i < 16; ++i) a.r2_from[i] = shell_from(a.shells[i]);
+  for (int i = 0; i < 16; ++i) a.r2_from[i] = shell_from(i < 2 * n_shells ? shells[i] : 0.0);
   const int nb2 = n_bins + 2, slots = n_shells * 2 * nb2;
   unsigned long long *dh, *hh;
   double *dm, *hm;

@@ -85,7 +85,6 @@ struct Spec {
   static constexpr int NPART = NX + NMID > 2 * NX ? NX + NMID : 2 * NX;
   static dim3 gxy(int nb) { return dim3(NH / NLxy, N, nb); }
   static dim3 gz(int nb) { return dim3(GZ, 1, nb); }
-  static_assert(NMID >= N, "a partial sum per plane");
   static Bat bat() { return Bat{SPEC, V, TAB, NPART}; }
 
   // launch-profile class of a pass: FP64-storage launches (the solves' FP64 residuals, the FP64
@@ -108,11 +107,11 @@ struct Spec {
       WF_A((k_fx_xmul<N>), fx_xmul_smem<N>());
       WF_A((k_fx_xfwd<N>), fx_xmul_smem<N>());
       WF_A((k_fx_xinv<N>), FC::SMEM);
-      WF_A((k_fx_zfwd<N, false>), FZ::SMEM);
+      WF_A((k_fx_zfwd<N>), FZ::SMEM);
       WF_A((k_fx_zinv<N, ZI_STORE>), FZ::SMEM);
       WF_A((k_fx_zinv<N, ZI_RESID>), FZ::SMEM);
       if constexpr (BUTTERFLY_RESID) {
-        WF_A((k_zfwd<R, N, false>), SMz);
+        WF_A((k_zfwd<R, N>), SMz);
         WF_A((k_xmul<R, N, true, true, false>), SMxy);
         WF_A((k_zinv<R, N, ZI_RESID>), SMz);
         if (e == cudaSuccess) e = YV<NLT, 2, 8>::setup();
@@ -120,7 +119,7 @@ struct Spec {
     } else {
       WF_A((k_xmul<R, N, true, false, true>), SMxy);
       WF_A((k_xmul<R, N, false, true, false>), SMxy);
-      WF_A((k_zfwd<R, N, false>), SMz);
+      WF_A((k_zfwd<R, N>), SMz);
       WF_A((k_zinv<R, N, ZI_ACCUM>), SMz);
     }
     if constexpr (std::is_same<R, float>::value) {
@@ -254,7 +253,7 @@ struct Spec {
     }
     static int xinv(Ctx& c, int nb, ST* r, ST* P0, ST* P1, ST* x, ST* T, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
-      c.launch(cls("cg_xinv", "cg_xinv_f64"), 6 * BS * nb, st, [&] {
+      c.launch("cg_xinv", 6 * BS * nb, st, [&] {
         if (unit_m)
           Ctx::chain(k_cg_xinv<R, N, true, RMAX>, gxy(nb), NTx, SMxy, st, r, P0, P1, x, T, ctab, mtab, tw, part, sc, bat());
         else
@@ -264,7 +263,7 @@ struct Spec {
     }
     static int xupd(Ctx& c, int nb, const ST* T, ST* r, ST* P0, ST* P1, const SS* ctab, const SS* mtab, bool unit_m,
                     const ST* tw, double* part, CgScal* sc, cudaStream_t st) {
-      c.launch(cls("cg_xupd", "cg_xupd_f64"), 4 * BS * nb, st, [&] {
+      c.launch("cg_xupd", 4 * BS * nb, st, [&] {
         if (unit_m)
           Ctx::chain(k_cg_xupd<R, N, true, RMAX>, gxy(nb), NTx, SMxy, st, T, r, P0, P1, ctab, mtab, tw, part, sc, bat());
         else
@@ -406,12 +405,11 @@ struct Spec {
           in, out, reinterpret_cast<const int2*>(tab), exps, estride, c.fixed(N), bat());
     });
   }
-  static void zfwd(Ctx& c, int nb, const double* in, ST* out, const ST* tw, double* part, const CgScal* sc,
-                   cudaStream_t st) {
+  static void zfwd(Ctx& c, int nb, const double* in, ST* out, const ST* tw, const CgScal* sc, cudaStream_t st) {
     c.launch(cls("zfwd", "zfwd_f64"), (BS + 8 * BV) * nb, st, [&] {
       if constexpr (F64)
-        k_fx_zfwd<N, false><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(in, out, c.fixed(N), part, sc, bat());
-      else k_zfwd<R, N, false><<<gz(nb), NTz, SMz, st>>>(in, out, tw, part, sc, bat());
+        k_fx_zfwd<N><<<dim3(FZ::GZ, 1, nb), FZ::NT, FZ::SMEM, st>>>(in, out, c.fixed(N), sc, bat());
+      else k_zfwd<R, N><<<gz(nb), NTz, SMz, st>>>(in, out, tw, sc, bat());
     });
   }
   template <int MODE>
@@ -435,7 +433,7 @@ struct Spec {
       using Y = YV<NLT, 2, 8>;
       const Bat bt = bat();
       c.launch("zfwd_f64", (BS + 8 * BV) * nb, st,
-               [&] { k_zfwd<R, N, false><<<gz(nb), NTz, SMz, st>>>(s, T, tw, part, nullptr, bt); });
+               [&] { k_zfwd<R, N><<<gz(nb), NTz, SMz, st>>>(s, T, tw, nullptr, bt); });
       Y::run(c, nb, T, tw, nullptr, -1, st, YFin{});
       c.launch("xmul_f64", 2 * BS * nb, st, [&] {
         k_xmul<R, N, true, true, false><<<gxy(nb), NTx, SMxy, st>>>(T, T2, stab, tw, part, nullptr, bt);
@@ -446,7 +444,7 @@ struct Spec {
       });
       return GZ;
     } else {
-      zfwd(c, nb, s, T, tw, part, nullptr, st);
+      zfwd(c, nb, s, T, tw, nullptr, st);
       ypass(c, nb, T, tw, nullptr, -1, st);
       fmul(c, nb, T, T2, stab, exps, estride, st);
       ypass(c, nb, T2, tw, nullptr, +1, st);
@@ -787,7 +785,7 @@ struct GroupFP64 : GroupCommon<N> {
   // r = C F(rhs) for every system; p = 0; reset the recurrences of the running systems
   wf_status start_cg(Ctx& c, const double* rhs, cudaStream_t st) {
     const size_t SPEC = SP::SPEC;
-    SP::zfwd(c, nb, rhs, T, tw, part, nullptr, st);
+    SP::zfwd(c, nb, rhs, T, tw, nullptr, st);
     SP::ypass(c, nb, T, tw, nullptr, -1, st);
     SP::template xmul<true, false, true>(c, nb, T, rh, ct, tw, part, nullptr, st);
     const Bat b = SP::bat();
@@ -814,7 +812,7 @@ struct GroupFP64 : GroupCommon<N> {
       SP::ypass(c, nb, T, tw, nullptr, +1, st);
       SP::template zinv<ZI_STORE>(c, nb, T, S, nullptr, nullptr, nullptr, inv_vc, tw, part, nullptr, st);
       // residual b - A s
-      SP::zfwd(c, nb, S, T, tw, part, nullptr, st);
+      SP::zfwd(c, nb, S, T, tw, nullptr, st);
       SP::ypass(c, nb, T, tw, nullptr, -1, st);
       SP::fmul(c, nb, T, T2, stab, &sc->texp, this->kScalInts, st);
       SP::ypass(c, nb, T2, tw, nullptr, +1, st);
@@ -974,7 +972,7 @@ struct GroupMixed : GroupCommon<N> {
     std::vector<double> ones((size_t)nb * SF::TAB, 1.0);
     float* tone;
     WF_TRY(upload_tables<float>(c, key + "t1", ones, &tone, st));
-    SF::zfwd(c, nb, W, T, tw32, part, nullptr, st);
+    SF::zfwd(c, nb, W, T, tw32, nullptr, st);
     SF::ypass(c, nb, T, tw32, nullptr, -1, st);
     SF::template xmul<true, false, true>(c, nb, T, P0, tone, tw32, part, nullptr, st);
     const int C = 4 * K + 1;
@@ -1114,7 +1112,7 @@ struct GroupMixed : GroupCommon<N> {
       }
       WF_TRY(this->push_scalars(st));
       const size_t SPEC = SF::SPEC;
-      SF::zfwd(c, nb, RES, T, tw32, part, nullptr, st);
+      SF::zfwd(c, nb, RES, T, tw32, nullptr, st);
       SF::ypass(c, nb, T, tw32, nullptr, -1, st);
       SF::template xmul<true, false, true>(c, nb, T, rh, ct, tw32, part, nullptr, st);
       c.launch("fin", 0, st, [&] { k_fin_init<<<nb, 1024, 0, st>>>(part, SF::GXY, sc, bf); });
@@ -1234,7 +1232,7 @@ wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::v
   }
   WF_CUDA(cudaMemcpyAsync(exps, hexp, sizeof(int), cudaMemcpyHostToDevice, st));
   c.launch("tables", 0, st, [&] { k_table_digits<<<dim3((SD::TAB + 255) / 256, 1), 256, 0, st>>>(gt, SD::TAB, exps, 1); });
-  SD::zfwd(c, 1, in, T, nullptr, nullptr, nullptr, st);
+  SD::zfwd(c, 1, in, T, nullptr, nullptr, st);
   SD::ypass(c, 1, T, nullptr, nullptr, -1, st);
   SD::fmul(c, 1, T, T2, gt, exps, 1, st);
   SD::ypass(c, 1, T2, nullptr, nullptr, +1, st);

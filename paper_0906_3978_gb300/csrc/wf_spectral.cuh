@@ -50,10 +50,13 @@ struct __align__(16) CgScal {
   int defl;           // deflated inner solves: 2 start step (alpha = 1) pending, 1 first iteration
   int noco;           // deflated groups: 1 = this system runs its inner solves without the coarse space
   int texp;           // power of two of the FP64 prior table's digits (k_fx_xmul)
-  unsigned tick[4];   // arrivals of the CTAs of a kernel that ends with a finisher (0 between kernels)
+  unsigned tick;      // arrivals of the CTAs of a kernel that ends with a finisher (0 between kernels)
 };
 // sc->done, read after chain_start(): a volatile read, which is not moved across the wait (the loads that follow
-// the test of it are then not moved either)
+// the test of it are then not moved either).  In the kernels where one CTA takes beta or alpha beside the others'
+// work (k_ycoarse, k_fx_ypass) that CTA may set done while threads of the others test it, and these may split: the
+// ones that return do not count at the barriers that follow (and no shuffle follows), and what the others leave half
+// made, T or the coarse coefficients, is not read once done is set.
 WF_D bool finished(const CgScal* sc) { return *(const volatile int*)&sc->done != 0; }
 
 // Distances between consecutive systems of a batch (elements of each array type).
@@ -65,7 +68,6 @@ struct Bat {
 };
 
 template <class R> constexpr int tile_lines() { return 128 / (int)sizeof(cx<R>); }
-template <class R> constexpr int elems_per_thread() { return sizeof(cx<R>) == 8 ? 16 : 8; }
 constexpr int cmin(int a, int b) { return a < b ? a : b; }
 // largest divisor of n that is <= cap (tile widths must divide the dimension they tile)
 constexpr int div_le(int n, int cap) {
@@ -883,28 +885,24 @@ k_zturn(typename Store<R>::T* __restrict__ spec, const typename Store<R>::S* __r
 }
 
 // ------------------------------------------------------------------------------------------
-// z forward: real rows (FP64) -> packed spectrum rows.  Optional partial of sum(in^2).
+// z forward: real rows (FP64) -> packed spectrum rows.
 // ------------------------------------------------------------------------------------------
-template <class R, int N, bool SQ>
+template <class R, int N>
 __global__ void __launch_bounds__(ZG<R, N>::NT)
 k_zfwd(const double* __restrict__ in, typename Store<R>::T* __restrict__ out,
-       const typename Store<R>::T* __restrict__ twtab, double* __restrict__ partials, const CgScal* __restrict__ sc,
-       Bat bt) {
+       const typename Store<R>::T* __restrict__ twtab, const CgScal* __restrict__ sc, Bat bt) {
   using G = ZG<R, N>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   cx<R>* tile = reinterpret_cast<cx<R>*>(smem_raw);
   cx<R>* tw = tile + G::M * G::LD;
-  __shared__ double red[32];
   const int z = blockIdx.z;
   if (sc && sc[z].done) return;
   in += z * bt.real;
   out += z * bt.spec;
-  partials += z * bt.part;
   const int tid = threadIdx.x;
   const size_t row0 = (size_t)blockIdx.x * G::NL;
   for (int e = tid; e < 2 * N; e += G::NT) tw[e] = ld_c<R>(twtab + e);
   const double2* in2 = reinterpret_cast<const double2*>(in);
-  AccD acc;
   constexpr int NE = G::NL * G::M, PE = (NE + G::NT - 1) / G::NT;
   double2 buf[PE];
 #pragma unroll
@@ -917,10 +915,6 @@ k_zfwd(const double* __restrict__ in, typename Store<R>::T* __restrict__ out,
     const int idx = tid + k * G::NT;
     if (!(NE % G::NT == 0 || idx < NE)) continue;
     tile[(idx % G::M) * G::LD + idx / G::M] = ld_c<R>(&buf[k]);
-    if constexpr (SQ) {
-      acc.add_prod(buf[k].x, buf[k].x);
-      acc.add_prod(buf[k].y, buf[k].y);
-    }
   }
   __syncthreads();
   const int l = tid % G::NL, t = tid / G::NL;
@@ -928,15 +922,11 @@ k_zfwd(const double* __restrict__ in, typename Store<R>::T* __restrict__ out,
   r2c_post<R, N, G::LD>(tile + l, t, G::TPL, tw);
   __syncthreads();
   zrows_store<G>(tile, out, row0, tid);
-  if constexpr (SQ) {
-    const double s = block_sum(acc.get(), red);
-    if (tid == 0) partials[blockIdx.x] = s;
-  }
 }
 
 // ------------------------------------------------------------------------------------------
 // z inverse: packed spectrum rows -> real rows (FP64), value v = scale * C2R(in), then
-//   ZI_STORE: out = v
+//   ZI_STORE: out = v (k_fx_zinv alone)
 //   ZI_RESID: out = b - (v + nbar w s), partial sum(out^2)
 //   ZI_ACCUM: out += v
 // ------------------------------------------------------------------------------------------
@@ -1046,9 +1036,9 @@ static __global__ void k_fin_init(const double* __restrict__ partials, int n, Cg
   }
 }
 
-// The sums and scalar updates at the end of a CG iteration's halves, by the threads of one CTA: the last to
-// finish of the pass that produced the partial sums (last_cta), or a kernel of its own (k_fin_*, after the
-// passes that have no finisher).  Partials are read past L1: other CTAs of the same grid wrote them.
+// The sums and scalar updates at the end of a CG iteration's halves, by the threads of one CTA: the last to finish of
+// k_defl_mu (last_cta), a CTA beside a later pass that does not need them (k_fx_ypass, k_ycoarse), or a kernel of its
+// own (k_fin_*, k_defl_alpha).  Partials are read past L1: other CTAs of the same grid may have written them.
 WF_D double sum_fresh(const double* p, int n, int stride, double* red) {
   double v = 0.0;
 #pragma unroll 16
