@@ -10,6 +10,7 @@
 // library (rms over a 30-degree survey at 64^3 to 128^3: 2.29 to 2.60 units of 2^-53, the library 2.27 to 2.59; one-word tables 2.43 to 2.79).
 #pragma once
 #include "wf_common.cuh"
+#include "wf_fntab.cuh"
 
 namespace wf {
 
@@ -47,39 +48,26 @@ WF_D double sqrt_fast(double d) {
 // ---- logarithm -----------------------------------------------------------------------------------
 // x = 2^k m with m in [3/4, 3/2); interval j of 128 gives c ~ 1/m and T = -log c (c = 1, T = 0 beside m = 1, so
 // that log keeps its relative accuracy there); log x = k log 2 + T + log1p(m c - 1)
-constexpr int kLogTab = 128, kExpTab = 64;
-using LogTable = double2[kLogTab];  // (c, T); intervals of 1/256 from 3/4 to 1, of 1/128 from 1 to 3/2
+// The rows come from memory (wf_fntab.cuh): making them with the math library's functions took each CTA 2 to 3 us
+// of the FP64 pipe, more than the nodes of a small grid.
+struct LogTable {
+  double2 lg[kLogTab];  // (c, T = -log c)
+};
 struct FnTables {
-  LogTable lg;
+  double c[kLogTab];
   double2 th[kLogTab];  // T as a multiple of 2^-40 and the rest
   double2 ex[kExpTab];  // 2^(j / 64) and what its rounding left
 };
 // fill the tables (in shared memory); a barrier has to follow
-WF_D void make_log_table(LogTable& lg, int tid, int nt) {
-  for (int j = tid; j < kLogTab; j += nt) {
-    const double mid = j < 64 ? 0.75 + (j + 0.5) / 256.0 : 1.0 + (j - 64 + 0.5) / 128.0;
-    const double c = j == 63 || j == 64 ? 1.0 : rint(4096.0 / mid) / 4096.0;
-    lg[j] = make_double2(c, c == 1.0 ? 0.0 : -log(c));
-  }
+WF_D void load_log_table(LogTable& t, int tid, int nt) {
+  for (int j = tid; j < kLogTab; j += nt) t.lg[j] = make_double2(kLogRows[j].c, kLogRows[j].th + kLogRows[j].tl);
 }
-WF_D void make_fn_tables(FnTables& t, int tid, int nt) {
-  make_log_table(t.lg, tid, nt);
+WF_D void load_fn_tables(FnTables& t, int tid, int nt) {
   for (int j = tid; j < kLogTab; j += nt) {
-    const double T = t.lg[j].y, hi = rint(T * 0x1p40) * 0x1p-40;
-    t.th[j] = make_double2(hi, T - hi);
+    t.c[j] = kLogRows[j].c;
+    t.th[j] = make_double2(kLogRows[j].th, kLogRows[j].tl);
   }
-  for (int j = tid; j < kExpTab; j += nt) {
-    // hi = 2^(j/64) (1 + d): d from hi^64 / 2^j, whose squarings run in two words
-    const double hi = exp2(j / 64.0);
-    double p = hi, q = 0.0;
-    for (int i = 0; i < 6; ++i) {
-      const double s = p * p, e = fma(p, p, -s) + 2.0 * p * q;
-      p = s + e;
-      q = e - (p - s);
-    }
-    const double two_j = (double)(1ull << j);
-    t.ex[j] = make_double2(hi, -hi * (((p - two_j) + q) / (64.0 * two_j)));
-  }
+  for (int j = tid; j < kExpTab; j += nt) t.ex[j] = kExpRows[j];
 }
 // log1p(r) for |r| <= 2^-6.9
 WF_D double log1p_short(double r) {
@@ -97,7 +85,7 @@ WF_D double log_fast(double x, const FnTables& t) {
   const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
   const int j = (ix >> 13) & (kLogTab - 1);
   const double2 th = t.th[j];
-  const double kd = small_int(k), l = log1p_short(fma(m, t.lg[j].x, -1.0));
+  const double kd = small_int(k), l = log1p_short(fma(m, t.c[j], -1.0));
   return fma(kd, 0x1.62e42fefa4p-1, th.x) + (l + fma(kd, -0x1.8432a1b0e2634p-43, th.y));  // log 2 in two parts
 }
 // exp(x) for -700 <= x <= 700 (12 FP64 operations)

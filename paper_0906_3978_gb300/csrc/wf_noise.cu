@@ -84,7 +84,7 @@ k_window(int n, SelParams s, const double4* __restrict__ holes, double* __restri
   FnTables& fn = *reinterpret_cast<FnTables*>(smem_raw);
   AxisTab* tab = reinterpret_cast<AxisTab*>(smem_raw + sizeof(FnTables));
   const int tid = threadIdx.x, lane = tid & 31;
-  make_fn_tables(fn, tid, blockDim.x);
+  load_fn_tables(fn, tid, blockDim.x);
   for (int e = tid; e < 3 * n; e += blockDim.x) {
     const int a = e / n, i = e - a * n;
     const double d = __dsub_rn(__dmul_rn((double)i, s.H), a == 0 ? s.ox : a == 1 ? s.oy : s.oz);
@@ -145,6 +145,8 @@ k_window(int n, SelParams s, const double4* __restrict__ holes, double* __restri
   if (threadIdx.x == 0) partials[blockIdx.x] = sum;
 }
 constexpr int kWindowBlocks = 152 * 4;
+// blocks of a window: no more than its rows keep busy
+constexpr int window_blocks(int n) { return n * n < 8 * kWindowBlocks ? n * n / 8 : kWindowBlocks; }
 
 // The selection at arbitrary positions pos[3 i] (the completeness at a galaxy), or its
 // reciprocal (0 where w = 0), the galaxy mass of the inverse-weighting estimator.
@@ -508,7 +510,7 @@ wf_status noise_run(Ctx& c, const wf_grid& g, const wf_selection& sel, const dou
   double4* dh;
   WF_TRY(c.get("holes", hh.size() * sizeof(double4), (void**)&dh));
   WF_CUDA(cudaMemcpyAsync(dh, hh.data(), hh.size() * sizeof(double4), cudaMemcpyHostToDevice, st));
-  const int grid = 152 * 8, wgrid = kWindowBlocks;
+  const int grid = 152 * 8, wgrid = window_blocks(n);
   double *part, *scal;
   WF_TRY(c.get("noise_part", grid * sizeof(double), (void**)&part));
   WF_TRY(c.get("noise_scal", 4 * sizeof(double), (void**)&scal));
@@ -650,9 +652,9 @@ extern "C" wf_status wf_build_noise_noalloc(const wf_grid* grid, const wf_select
   const size_t V = (size_t)n * n * n;
   static_assert(kWindowBlocks <= kNoallocParts, "partial sums");
   WF_CUDA(cudaFuncSetAttribute(k_window, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)window_smem(kWindowMaxN)));
-  k_window<<<kWindowBlocks, 256, window_smem(n), st>>>(n, s, dh, w, part);
+  k_window<<<window_blocks(n), 256, window_smem(n), st>>>(n, s, dh, w, part);
   WF_CUDA(cudaGetLastError());
-  k_nbar<<<1, 1024, 0, st>>>(part, kWindowBlocks, (double)n_gal, scal);
+  k_nbar<<<1, 1024, 0, st>>>(part, window_blocks(n), (double)n_gal, scal);
   WF_CUDA(cudaGetLastError());
   k_data<<<kNoallocParts, 256, 0, st>>>(n_obs, w, scal, d, b, V);
   WF_CUDA(cudaGetLastError());

@@ -58,8 +58,8 @@ WF_D double log_ratio(double a, double b, const double2* __restrict__ lg) {
 __global__ void __launch_bounds__(256)
 k_compare(const double* __restrict__ rec, const double* __restrict__ tru, size_t n, double* __restrict__ partials) {
   __shared__ double red[32];
-  __shared__ LogTable lg;
-  make_log_table(lg, threadIdx.x, blockDim.x);
+  __shared__ LogTable tab;
+  load_log_table(tab, threadIdx.x, blockDim.x);
   __syncthreads();
   AccD tr, tt, rr, d2, kl;
   int excl = 0;
@@ -71,7 +71,7 @@ k_compare(const double* __restrict__ rec, const double* __restrict__ tru, size_t
     const double d = r - t;
     d2.add_prod(d, d);
     const double a = 1.0 + r, b = 1.0 + t;
-    if (plain_range(a) && plain_range(b)) kl.add_prod(a, log_ratio(a, b, lg));
+    if (plain_range(a) && plain_range(b)) kl.add_prod(a, log_ratio(a, b, tab.lg));
     else if (a > 0.0 && b > 0.0) kl.add(a * log(a / b));
     else ++excl;
   }
