@@ -135,7 +135,6 @@ __global__ void k_q48_to_double(const unsigned long long* __restrict__ fine, dou
 // the shift table's factor 2^a / N.
 // ------------------------------------------------------------------------------------------
 constexpr int kNyqParts = 8;  // partial sums of A that the bin N/2 adds
-constexpr int kLpMinExp = 223;  // smallest exponent of a line (2^-800: counts and masses are multiples of 2^-48)
 
 // The multiplier between the transforms: bin k of the line (digits ph[k]); bin N/2 takes -A, the sum
 // of the line's kNyqParts partial sums at ny[0], ny[st], ...
@@ -302,7 +301,7 @@ k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4*
     o[r] = __ldg(reinterpret_cast<const double2*>(src + (2 * m + 1) * stride));
   }
   if (tid < NL) {
-    s_e[tid] = kLpMinExp;
+    s_e[tid] = FxScale::kMin;
     s_q[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
@@ -318,7 +317,7 @@ k_lowpass_c(const double* __restrict__ in, double* __restrict__ out, const int4*
       s.y += odd ? -e[r].y : e[r].y;
     }
     pa[t * NL + l] = s;
-    if (mx > kLpMinExp) atomicMax(&s_e[l], mx);
+    if (mx > FxScale::kMin) atomicMax(&s_e[l], mx);
   }
   __syncthreads();
   const int emax = s_e[l];

@@ -12,10 +12,11 @@
 // of rounding noise a transform adds, ~1e-17 relative at M = 512, where FP64 butterflies leave ~2e-16.
 // What remains is the rounding of the FP64 values that are stored.  A line's scale comes from its own
 // largest exponent and sum of squares, so lines of any magnitude keep their digits; the statistics are
-// integers, so the result does not depend on the order in which threads add to them.  Scalings beyond
-// 2^+-900, which an exponent field may not hold in one step, take two FP64 multiplications.  A line with an
+// integers, so the result does not depend on the order in which threads add to them.  A line with an
 // infinity or NaN becomes NaN throughout (FP64 butterflies spread either over the line as well).
 #pragma once
+#include <type_traits>
+
 #include "wf_line.cuh"
 
 namespace wf {
@@ -122,15 +123,21 @@ template <int M> struct FxPlan {
 
 // ---- scaling -----------------------------------------------------------------------------------
 WF_D int fx_exp(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
-// an upper bound of |d| 2^(12 - (emax - 1023)), 13 bits and one, for exponents up to emax
-WF_D unsigned fx_top(double d, int emax) {
-  const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff, s = emax - max(e, 1) + 8;
-  const unsigned m = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
-  return s > 31 || m == 0 ? (unsigned)((m | (unsigned)__double2loint(d)) != 0) : (m >> s) + 1u;
+// an upper bound of |d| 2^(12 - (emax - 1023)), 13 bits and one, for exponents up to emax (where SUB is false, a
+// subnormal's is 1: emax is at least 14)
+template <bool SUB = false> WF_D unsigned fx_top(double d, int emax) {
+  const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff;
+  if constexpr (SUB) {
+    const int s = emax - max(e, 1) + 8;
+    const unsigned m = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
+    return s > 31 || m == 0 ? (unsigned)((m | (unsigned)__double2loint(d)) != 0) : (m >> s) + 1u;
+  }
+  const int s = emax - e + 8;
+  return e == 0 || s > 31 ? (unsigned)((hi & 0x7fffffff) != 0 || __double2loint(d) != 0)
+                          : ((unsigned)((hi & 0xfffff) | 0x100000) >> s) + 1u;
 }
 // 2^e for -1022 <= e <= 1023
 WF_D double fx_pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-constexpr int kFxStep = 900;  // scalings up to 2^+-kFxStep are integer additions to exponent fields
 // d 2^e for any e; the result under- or overflows as it should
 WF_D double fx_scaled(double d, int e) {
   e = min(max(e, -2044), 2044);
@@ -143,60 +150,83 @@ WF_D long long fx_from(double d, int k) {
   return __double2ll_rn(__hiloint2double(hi + (k << 20), __double2loint(d)));
 }
 // The power of two k that takes a line of M complex values to sqrt(M) ||z||_2 2^k <= 2^62: emax the
-// largest biased exponent of the line (at least 1), q >= (sum of fx_top^2) / 128
+// largest biased exponent of the line, q >= (sum of fx_top^2) / 128
 WF_D int fx_scale(int emax, unsigned q, int M) {
   const unsigned long long s = (unsigned long long)q * 128ull * (unsigned)M;
   const int b = 64 - __clzll((long long)s);  // sqrt(s) < 2^(b / 2)
   return 62 - (emax - 1023) + 12 - ((b + 1) >> 1);
 }
 
-
-// A line's scale: its values are integers in units of 2^-k, made from the registers' values by 2^kin; nan: the
-// exponent bits that make every result of a line with a non-finite element a NaN
+// A line's scale: its values are integers in units of 2^-k; nan: the exponent bits that make every
+// result of a line with a non-finite element a NaN.  kMin: the smallest exponent a line is taken to have: 2^-800,
+// below which values keep the resolution of 2^-860.
 struct FxScale {
+  static constexpr int kMin = 223;
+  int k;
+  unsigned nan;
+};
+// The same for the whole FP64 range, in the passes of a filter on a caller's field and of a residual: integers are made
+// from the registers' values by 2^kin, and scalings past 2^+-kFxStep, which an exponent field may not hold, are
+// multiplications.  (In the passes of a CG iteration, whose smallest values are sqrt(the smallest norm), it
+// costs 3 to 5% of an FP64 solve and can change nothing.)
+constexpr int kFxStep = 900;
+struct FxWide {
+  static constexpr int kMin = 1;
   int k, kin;
   unsigned nan;
 };
 // The scale of the line whose elements are spread over the threads' raw[]; se, sq: the line's words in
-// shared memory, kFxMinExp and 0 before (visible to all).  Two barriers.  A line of zeros gets k = 0; the
-// values of a line of tiny ones, subnormals among them, are multiplied by 2^600 in the registers.
-constexpr int kFxMinExp = 1;
-template <int NV> WF_D FxScale fx_line_scale(double2 (&raw)[NV], int* se, unsigned* sq, int M) {
+// shared memory, S::kMin and 0 before (visible to all).  Two barriers.  In the wide form a line of zeros gets k = 0,
+// and the values of a line of tiny ones, subnormals among them, are multiplied by 2^600 in the registers.
+template <class S = FxScale, int NV> WF_D S fx_line_scale(double2 (&raw)[NV], int* se, unsigned* sq, int M) {
   static_assert(2 * NV <= 62, "the sum of squares of a thread fits 32 bits");
+  constexpr bool WIDE = std::is_same<S, FxWide>::value;
   int mx = 0;
 #pragma unroll
   for (int r = 0; r < NV; ++r) mx = max(mx, max(fx_exp(raw[r].x), fx_exp(raw[r].y)));
-  if (mx > kFxMinExp) atomicMax(se, mx);
+  if (mx > S::kMin) atomicMax(se, mx);
   __syncthreads();
   const int emax = *se;
   unsigned q = 0;
 #pragma unroll
   for (int r = 0; r < NV; ++r) {
-    const unsigned h0 = fx_top(raw[r].x, emax), h1 = fx_top(raw[r].y, emax);
+    const unsigned h0 = fx_top<WIDE>(raw[r].x, emax), h1 = fx_top<WIDE>(raw[r].y, emax);
     q += h0 * h0 + h1 * h1;
   }
   if (q) atomicAdd(sq, (q >> 7) + 1u);
   __syncthreads();
-  const unsigned s = *sq;
-  FxScale f{s ? fx_scale(emax, s + 1u, M) : 0, 0, emax == 0x7ff ? 0x7ff80000u : 0u};
-  f.kin = f.k;
-  if (f.k > kFxStep) {
-    f.kin = f.k - 600;
+  const unsigned nan = emax == 0x7ff ? 0x7ff80000u : 0u;
+  if constexpr (WIDE) {
+    const unsigned s = *sq;
+    FxWide f{s ? fx_scale(emax, s + 1u, M) : 0, 0, nan};
+    f.kin = f.k;
+    if (f.k > kFxStep) {
+      f.kin = f.k - 600;
 #pragma unroll
-    for (int r = 0; r < NV; ++r) raw[r] = make_double2(raw[r].x * 0x1p600, raw[r].y * 0x1p600);
+      for (int r = 0; r < NV; ++r) raw[r] = make_double2(raw[r].x * 0x1p600, raw[r].y * 0x1p600);
+    }
+    return f;
+  } else {
+    return FxScale{fx_scale(emax, *sq + 1u, M), nan};
   }
-  return f;
 }
-WF_D fxc fx_from2(double2 d, FxScale f) { return fxc{fx_from(d.x, f.kin), fx_from(d.y, f.kin)}; }
-// v 2^-(k + sh).  The power of two goes to the exponent field by an integer addition within 2^+-kFxStep.
-WF_D double fx_to(long long v, FxScale f, int sh = 0) {
+WF_D fxc fx_from2(double2 d, FxScale f) { return fxc{fx_from(d.x, f.k), fx_from(d.y, f.k)}; }
+WF_D fxc fx_from2(double2 d, FxWide f) { return fxc{fx_from(d.x, f.kin), fx_from(d.y, f.kin)}; }
+// v 2^-(k + sh).  The power of two goes to the exponent field by an integer addition (values near the top
+// of the range, where it could overflow, take a multiplication).
+template <class S> WF_D double fx_to(long long v, S f, int sh = 0) {
   const int k = f.k + sh;
   double d = __ll2double_rn(v);
-  if ((unsigned)(k + kFxStep) > 2u * kFxStep) d = fx_scaled(d, -k);
-  else if (v != 0) d = __hiloint2double(__double2hiint(d) - (k << 20), __double2loint(d));
+  if constexpr (std::is_same<S, FxWide>::value) {
+    if ((unsigned)(k + kFxStep) > 2u * kFxStep) d = fx_scaled(d, -k);
+    else if (v != 0) d = __hiloint2double(__double2hiint(d) - (k << 20), __double2loint(d));
+  } else {
+    if (k < -900) d *= fx_pow2(-k);
+    else if (v != 0) d = __hiloint2double(__double2hiint(d) - (k << 20), __double2loint(d));
+  }
   return __hiloint2double(__double2hiint(d) | (int)f.nan, __double2loint(d));
 }
-WF_D double2 fx_to2(fxc v, FxScale f, int sh = 0) { return make_double2(fx_to(v.x, f, sh), fx_to(v.y, f, sh)); }
+template <class S> WF_D double2 fx_to2(fxc v, S f, int sh = 0) { return make_double2(fx_to(v.x, f, sh), fx_to(v.y, f, sh)); }
 WF_D long long fx_rshift(long long v, int s) { return (v + (1ll << (s - 1))) >> s; }  // s >= 1, rounded
 
 constexpr int fx_floor_log2(int n) { return n < 2 ? 0 : 1 + fx_floor_log2(n / 2); }

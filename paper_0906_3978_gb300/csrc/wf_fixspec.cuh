@@ -27,8 +27,8 @@ template <int N> struct FxC {
 };
 
 // y pass: complex transform along y of every (x, kz) line, in place.  With fin.n1 > 0 the first row of CTAs takes alpha
-// (YFin).  grid (N/2 / NL, N + (fin.n1 > 0), systems)
-template <int N, int DIR>
+// (YFin).  S: the lines' range.  grid (N/2 / NL, N + (fin.n1 > 0), systems)
+template <int N, int DIR, class S>
 __global__ void __launch_bounds__(FxC<N>::NT)
 k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, CgScal* __restrict__ sc, Bat bt, YFin fin) {
   using G = FxC<N>;
@@ -55,11 +55,11 @@ k_fx_ypass(double2* __restrict__ T, const int4* __restrict__ twtab, CgScal* __re
 #pragma unroll
   for (int r = 0; r < R1; ++r) raw[r] = p[(size_t)(r * N1 + t) * NH];
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = S::kMin;
     sq[tid] = 0;
   }
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  const S f = fx_line_scale<S>(raw, &se[l], &sq[l], N);
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
@@ -130,13 +130,13 @@ k_fx_xmul(const double2* __restrict__ in, double2* __restrict__ out, const int2*
   for (int r = 0; r < R1; ++r)
     raw[r] = live ? __ldg(in + base + (size_t)(r * N1 + t) * rowstride) : make_double2(0.0, 0.0);
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxWide::kMin;
     sq[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const int ls = pair && l < 2 ? 0 : l;  // the two lines of a pair share a scale
-  FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  FxWide f = fx_line_scale<FxWide>(raw, &se[ls], &sq[ls], N);
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
@@ -205,13 +205,13 @@ k_fx_xfwd(const double2* __restrict__ in, double2* __restrict__ out, const doubl
   for (int r = 0; r < R1; ++r)
     raw[r] = live ? __ldg(in + base + (size_t)(r * N1 + t) * rowstride) : make_double2(0.0, 0.0);
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxScale::kMin;
     sq[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
   const int ls = pair && l < 2 ? 0 : l;
-  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  const FxScale f = fx_line_scale<FxScale>(raw, &se[ls], &sq[ls], N);
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
@@ -282,12 +282,12 @@ k_fx_xinv(const double2* __restrict__ in, double2* __restrict__ out, const doubl
     }
   }
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxScale::kMin;
     sq[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  const FxScale f = fx_line_scale<FxScale>(raw, &se[l], &sq[l], N);
   fxc v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], f);
@@ -349,12 +349,12 @@ k_fx_zfwd(const double* __restrict__ in, double2* __restrict__ out, const int4* 
 #pragma unroll
   for (int r = 0; r < R1; ++r) raw[r] = __ldg(src + r * N1 + t);
   if (tid < G::NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxWide::kMin;
     sq[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], H);
+  const FxWide f = fx_line_scale<FxWide>(raw, &se[l], &sq[l], H);
   fxc* s = slots + l * G::LS;
   fxc v[R1];
 #pragma unroll
@@ -389,12 +389,12 @@ k_fx_zinv(const double2* __restrict__ in, double* __restrict__ out, const double
 #pragma unroll
   for (int r = 0; r < R1; ++r) raw[r] = __ldg(src + r * N1 + t);
   if (tid < G::NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxWide::kMin;
     sq[tid] = 0;
   }
   fx_load_tw<N>(tw, twtab, tid, G::NT);
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], fx_c2r_count<N>());
+  const FxWide f = fx_line_scale<FxWide>(raw, &se[l], &sq[l], fx_c2r_count<N>());
   fxc* sl = slots + l * G::LS;
 #pragma unroll
   for (int r = 0; r < R1; ++r) sl[PadMap{}(r * N1 + t)] = fx_from2(raw[r], f);
@@ -534,11 +534,11 @@ k_fx_cg_xinv(const double2* __restrict__ r, double2* P0, double2* P1, double2* _
     }
   }
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxScale::kMin;
     sq[tid] = 0;
   }
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], N);
+  const FxScale f = fx_line_scale<FxScale>(raw, &se[l], &sq[l], N);
   fxc v[R1];
 #pragma unroll
   for (int q = 0; q < R1; ++q) v[q] = fx_from2(raw[q], f);
@@ -591,12 +591,12 @@ k_fx_cg_xupd(const double2* __restrict__ T, double2* __restrict__ r, const doubl
   for (int q = 0; q < R1; ++q)
     raw[q] = live ? __ldg(T + base + (size_t)(q * N1 + t) * rowstride) : make_double2(0.0, 0.0);
   if (tid < NL) {
-    se[tid] = kFxMinExp;
+    se[tid] = FxScale::kMin;
     sq[tid] = 0;
   }
   __syncthreads();
   const int ls = pair && l < 2 ? 0 : l;
-  const FxScale f = fx_line_scale(raw, &se[ls], &sq[ls], N);
+  const FxScale f = fx_line_scale<FxScale>(raw, &se[ls], &sq[ls], N);
   fxc v[R1];
 #pragma unroll
   for (int q = 0; q < R1; ++q) v[q] = fx_from2(raw[q], f);
@@ -694,11 +694,11 @@ k_fx_zturn(double2* __restrict__ spec, const double* __restrict__ D, const int4*
 #pragma unroll
   for (int r = 0; r < R1; ++r) raw[r] = line[r * N1 + t];
   for (int i = tid; i < 2 * G::NL; i += G::NT) {
-    se[i] = kFxMinExp;
+    se[i] = FxScale::kMin;
     sq[i] = 0;
   }
   __syncthreads();
-  const FxScale f = fx_line_scale(raw, &se[l], &sq[l], fx_c2r_count<N>());
+  const FxScale f = fx_line_scale<FxScale>(raw, &se[l], &sq[l], fx_c2r_count<N>());
   fxc* sl = slots + l * G::LS;
 #pragma unroll
   for (int r = 0; r < R1; ++r) sl[PadMap{}(r * N1 + t)] = fx_from2(raw[r], f);
@@ -713,7 +713,7 @@ k_fx_zturn(double2* __restrict__ spec, const double* __restrict__ D, const int4*
     raw[r] = make_double2(T.x * dv.x, T.y * dv.y);
     acc = fma(raw[r].x, T.x, fma(raw[r].y, T.y, acc));
   }
-  const FxScale g = fx_line_scale(raw, &se[G::NL + l], &sq[G::NL + l], H);
+  const FxScale g = fx_line_scale<FxScale>(raw, &se[G::NL + l], &sq[G::NL + l], H);
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = fx_from2(raw[r], g);
   ln_forward_nat<H, FxPlan<H>, -1, 2>(v, sl, PadMap{}, t, tw);

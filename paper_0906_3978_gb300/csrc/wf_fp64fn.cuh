@@ -7,7 +7,8 @@
 // brings the argument within 2^-7 (log) or 2^-7.5 (exp) of 1 or 0, where the Taylor series of degree 7 or 5
 // reaches 2^-56.  All sign, exponent and index work is integer arithmetic.  Table values carry a second word, so
 // that a function's error is its last rounding and little more: the window's values err no more than with the math
-// library (rms over a 30-degree survey at 64^3 to 128^3: 2.29 to 2.60 units of 2^-53, the library 2.27 to 2.59; one-word tables 2.43 to 2.79).
+// library (rms over a 30-degree survey at 64^3 to 128^3: 2.27 to 2.59 units of 2^-53, as with the library;
+// one-word tables 2.43 to 2.79).
 #pragma once
 #include "wf_common.cuh"
 #include "wf_fntab.cuh"

@@ -62,7 +62,7 @@ WF_D double sel_value(const SelParams& s, const double4* __restrict__ holes, dou
 }
 
 // The window at the nodes.  The plain formula costs ~75 FP64 operations a node, all on the 1/64-rate pipe
-// (256^3: 1.97 ms, here 0.85).  The cone and hole tests are first taken in FP32: a node whose margin exceeds
+// (256^3: 1.97 ms, here 0.82).  The cone and hole tests are first taken in FP32: a node whose margin exceeds
 // 2^-20 r (|a_x| + |a_y| + |a_z| + |cos|), 16 units of 2^-24 where the roundings of dot and cos r (the approximate
 // square root's 2^-22 among them) add up to about 10, is decided there, and only the others repeat the exact
 // test of sel_value, operation by operation.  What depends on one axis alone (offset, its square, its term of

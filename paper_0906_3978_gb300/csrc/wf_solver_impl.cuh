@@ -110,6 +110,7 @@ struct Spec {
       WF_A((k_fx_zfwd<N>), FZ::SMEM);
       WF_A((k_fx_zinv<N, ZI_STORE>), FZ::SMEM);
       WF_A((k_fx_zinv<N, ZI_RESID>), FZ::SMEM);
+      if (e == cudaSuccess) e = YFix<FxWide>::setup();
       if constexpr (BUTTERFLY_RESID) {
         WF_A((k_zfwd<R, N>), SMz);
         WF_A((k_xmul<R, N, true, true, false>), SMxy);
@@ -196,17 +197,18 @@ struct Spec {
     }
   };
   // the FP64 y pass (fixed point); tw is unused, its twiddles come from the context
+  template <class S>
   struct YFix {
     static cudaError_t setup() {
-      cudaError_t e = set_smem(k_fx_ypass<N, -1>, FC::SMEM);
-      return e == cudaSuccess ? set_smem(k_fx_ypass<N, +1>, FC::SMEM) : e;
+      cudaError_t e = set_smem(k_fx_ypass<N, -1, S>, FC::SMEM);
+      return e == cudaSuccess ? set_smem(k_fx_ypass<N, +1, S>, FC::SMEM) : e;
     }
     static void run(Ctx& c, int nb, ST* t, const ST*, CgScal* sc, int dir, cudaStream_t st, const YFin& fin) {
       double2* T = reinterpret_cast<double2*>(t);
       const dim3 grid(FC::KB, N + (fin.n1 > 0), nb);
       c.launch("ypass_f64", 2 * BS * nb, st, [&] {
-        if (dir < 0) Ctx::chain(k_fx_ypass<N, -1>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
-        else Ctx::chain(k_fx_ypass<N, +1>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
+        if (dir < 0) Ctx::chain(k_fx_ypass<N, -1, S>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
+        else Ctx::chain(k_fx_ypass<N, +1, S>, grid, FC::NT, FC::SMEM, st, T, c.fixed(N), sc, bat(), fin);
       });
     }
   };
@@ -214,7 +216,7 @@ struct Spec {
     static const std::vector<PassVariant> v = [] {
       std::vector<PassVariant> out;
       if constexpr (F64) {
-        out.push_back({"fixed", YFix::setup, YFix::run});
+        out.push_back({"fixed", YFix<FxScale>::setup, YFix<FxScale>::run});
       } else {
         // variant 0 decides how a mixed solve rounds (kInnerMargin): its radices stay
         out.push_back({"nl_s2_r8", YV<NLT, 2, 8>::setup, YV<NLT, 2, 8>::run});
@@ -1233,9 +1235,10 @@ wf_status fourier_multiply_n(Ctx& c, const double* in, double* out, const std::v
   WF_CUDA(cudaMemcpyAsync(exps, hexp, sizeof(int), cudaMemcpyHostToDevice, st));
   c.launch("tables", 0, st, [&] { k_table_digits<<<dim3((SD::TAB + 255) / 256, 1), 256, 0, st>>>(gt, SD::TAB, exps, 1); });
   SD::zfwd(c, 1, in, T, nullptr, nullptr, st);
-  SD::ypass(c, 1, T, nullptr, nullptr, -1, st);
+  using Y = typename SD::template YFix<FxWide>;  // a caller's field may have any magnitude
+  Y::run(c, 1, T, nullptr, nullptr, -1, st, YFin{});
   SD::fmul(c, 1, T, T2, gt, exps, 1, st);
-  SD::ypass(c, 1, T2, nullptr, nullptr, +1, st);
+  Y::run(c, 1, T2, nullptr, nullptr, +1, st, YFin{});
   SD::template zinv<ZI_STORE>(c, 1, T2, out, nullptr, nullptr, nullptr, 1.0 / (double)SD::V, nullptr, nullptr, nullptr,
                               st);
   WF_CUDA(cudaGetLastError());
